@@ -20,8 +20,10 @@ EXPORTED_SYMBOLS = [
     "soap_neighbors_at", "soap_descriptor_at", "soap_derivatives_at",
     "soap_rows_dense", "soap_neighbors_batch", "soap_descriptor_batch", "soap_derivatives_batch",
     "soap_num_compact_features", "soap_compact_feature_map", "soap_derivatives_compact", "soap_compact_expand",
-    "soap_measure_fp32_peak",
+    "soap_measure_fp32_peak", "soap_search", "soap_derivatives_found",
 ]
+
+ROWS_FULL, ROWS_COMPACT, ROWS_COEFFICIENTS = 0, 1, 2
 
 _ERRORS = {-1: "SOAP_ERR_INVALID_ARG", -2: "SOAP_ERR_UNKNOWN_SPECIES", -3: "SOAP_ERR_CAPACITY",
            -4: "SOAP_ERR_CUDA", -5: "SOAP_ERR_ALLOC"}
@@ -78,6 +80,8 @@ def load_library() -> C.CDLL:
     lib.soap_neighbors_batch.argtypes = [vp, vp, vp, i64, vp, i64, C.POINTER(i64), C.POINTER(i64), vp]
     lib.soap_descriptor_batch.argtypes = [vp, vp, vp, i64, vp, i64, vp, vp]
     lib.soap_derivatives_batch.argtypes = [vp, vp, vp, i64, vp, i64, vp, vp, i64, vp, vp, vp]
+    lib.soap_search.argtypes = [vp, vp, vp, i64, C.POINTER(C.c_double), vp, vp, i64, vp, i64, vp, C.POINTER(i64), C.POINTER(i64), vp]
+    lib.soap_derivatives_found.argtypes = [vp, i32, vp, i64, C.POINTER(C.c_double), vp, vp, i64, vp, vp, vp, i64, vp, vp, vp]
     lib.soap_set_crossover.argtypes = [vp, i32]
     lib.soap_set_weighting.argtypes = [vp, i32] + [C.c_double] * 5
     lib.soap_num_coefficients.argtypes = [vp, C.POINTER(i64)]
@@ -268,19 +272,37 @@ class Soap:
                                                desc.data_ptr(), jac.data_ptr(), jac.shape[0], row_ptr.data_ptr(),
                                                row_atom.data_ptr(), self._stream()))
 
+    def _sized(self, kind, width, positions, numbers, cell=None, centers=None, sites=None, struct_ptr=None):
+        """One neighbour search, outputs of exactly its size, the derivatives of what it found; waits for the stream.
+        Returns (values, centre rows or None, Jacobian rows, row_ptr, row_atom)."""
+        import torch
+        n, c, cptr = self._inputs(positions, numbers, centers)
+        keep, cellp = self._cell(cell)
+        sptr, bptr, n_structs = None, None, 0
+        if sites is not None:
+            c, sptr = sites.shape[0], sites.data_ptr()
+        if struct_ptr is not None:
+            bptr, n_structs = struct_ptr.data_ptr(), struct_ptr.shape[0] - 1
+        dev, stream, pos = positions.device, self._stream(), positions.data_ptr()
+        row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
+        npairs, nrows = C.c_int64(), C.c_int64()
+        self._check(self._lib.soap_search(self._h, pos, numbers.data_ptr(), n, cellp, cptr, sptr, c, bptr, n_structs,
+                                          row_ptr.data_ptr(), C.byref(npairs), C.byref(nrows), stream))
+        rows = nrows.value
+        compact = kind == ROWS_COMPACT
+        values = torch.empty((c, self.n_coefficients if kind == ROWS_COEFFICIENTS else self.n_features), dtype=torch.float32, device=dev)
+        center_rows = torch.empty((c, 3, self.n_features), dtype=torch.float32, device=dev) if compact else None
+        jac = torch.empty((max(rows, 1), 3, width), dtype=torch.float32, device=dev)
+        row_atom = torch.empty(max(rows, 1), dtype=torch.int32, device=dev)
+        self._check(self._lib.soap_derivatives_found(self._h, kind, pos, n, cellp, cptr, sptr, c, values.data_ptr(),
+                                                     center_rows.data_ptr() if compact else None, jac.data_ptr(), jac.shape[0],
+                                                     row_ptr.data_ptr(), row_atom.data_ptr(), stream))
+        return values, center_rows, jac[:rows], row_ptr, row_atom[:rows]
+
     def derivatives(self, positions, numbers, cell=None, centers=None) -> Derivatives:
         """Sizes the Jacobian with one neighbour search, then computes it."""
-        import torch
-        _, nrows = self.neighbors(positions, numbers, cell, centers)
-        c = positions.shape[0] if centers is None else centers.shape[0]
-        dev = positions.device
-        desc = torch.empty((c, self.n_features), dtype=torch.float32, device=dev)
-        jac = torch.empty((max(nrows, 1), 3, self.n_features), dtype=torch.float32, device=dev)
-        row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
-        row_atom = torch.empty(max(nrows, 1), dtype=torch.int32, device=dev)
-        self.derivatives_into(positions, numbers, cell, centers, desc, jac, row_ptr, row_atom)
-        self.status()
-        return Derivatives(desc, jac[:nrows], row_ptr, row_atom[:nrows])
+        desc, _, jac, row_ptr, row_atom = self._sized(ROWS_FULL, self.n_features, positions, numbers, cell, centers)
+        return Derivatives(desc, jac, row_ptr, row_atom)
 
     # ------------------------------------------------------------------ many structures in one call
     def derivatives_batch(self, positions, numbers, struct_ptr, jacobian=True):
@@ -291,25 +313,14 @@ class Soap:
         n, _, _ = self._inputs(positions, numbers, None)
         assert struct_ptr.is_cuda and struct_ptr.dtype == torch.int64 and struct_ptr.is_contiguous()
         b, sp = struct_ptr.shape[0] - 1, C.c_void_p(struct_ptr.data_ptr())
-        dev = positions.device
-        desc = torch.empty((n, self.n_features), dtype=torch.float32, device=dev)
         if not jacobian:
+            desc = torch.empty((n, self.n_features), dtype=torch.float32, device=positions.device)
             self._check(self._lib.soap_descriptor_batch(self._h, positions.data_ptr(), numbers.data_ptr(), n, sp, b,
                                                         desc.data_ptr(), self._stream()))
             self.status()
             return desc
-        npairs, nrows = C.c_int64(), C.c_int64()
-        self._check(self._lib.soap_neighbors_batch(self._h, positions.data_ptr(), numbers.data_ptr(), n, sp, b,
-                                                   C.byref(npairs), C.byref(nrows), self._stream()))
-        nrows = int(nrows.value)
-        jac = torch.empty((max(nrows, 1), 3, self.n_features), dtype=torch.float32, device=dev)
-        row_ptr = torch.empty(n + 1, dtype=torch.int64, device=dev)
-        row_atom = torch.empty(max(nrows, 1), dtype=torch.int32, device=dev)
-        self._check(self._lib.soap_derivatives_batch(self._h, positions.data_ptr(), numbers.data_ptr(), n, sp, b,
-                                                     desc.data_ptr(), jac.data_ptr(), jac.shape[0], row_ptr.data_ptr(),
-                                                     row_atom.data_ptr(), self._stream()))
-        self.status()
-        return Derivatives(desc, jac[:nrows], row_ptr, row_atom[:nrows])
+        desc, _, jac, row_ptr, row_atom = self._sized(ROWS_FULL, self.n_features, positions, numbers, struct_ptr=struct_ptr)
+        return Derivatives(desc, jac, row_ptr, row_atom)
 
     # ------------------------------------------------------------------ species-compact rows
     def compact_feature_map(self, species_index):
@@ -326,18 +337,7 @@ class Soap:
 
     def derivatives_compact(self, positions, numbers, cell=None, centers=None) -> CompactDerivatives:
         """Like `derivatives`, with neighbour rows that leave out the structurally zero species blocks."""
-        import torch
-        _, nrows = self.neighbors(positions, numbers, cell, centers)
-        c = positions.shape[0] if centers is None else centers.shape[0]
-        dev = positions.device
-        desc = torch.empty((c, self.n_features), dtype=torch.float32, device=dev)
-        center_rows = torch.empty((c, 3, self.n_features), dtype=torch.float32, device=dev)
-        jac = torch.empty((max(nrows, 1), 3, self.compact_pitch), dtype=torch.float32, device=dev)
-        row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
-        row_atom = torch.empty(max(nrows, 1), dtype=torch.int32, device=dev)
-        self.derivatives_compact_into(positions, numbers, cell, centers, desc, center_rows, jac, row_ptr, row_atom)
-        self.status()
-        return CompactDerivatives(desc, center_rows, jac[:nrows], row_ptr, row_atom[:nrows])
+        return CompactDerivatives(*self._sized(ROWS_COMPACT, self.compact_pitch, positions, numbers, cell, centers))
 
     def compact_expand(self, numbers, centers, comp: "CompactDerivatives"):
         """(rows, 3, F): the full rows `derivatives` would have written."""
@@ -359,27 +359,16 @@ class Soap:
         import torch
         n, _, _ = self._inputs(positions, numbers, None)
         assert sites.is_cuda and sites.dtype == torch.float32 and sites.is_contiguous() and sites.shape[-1] == 3
-        c, sptr = sites.shape[0], C.c_void_p(sites.data_ptr())
-        keep, cellp = self._cell(cell)
-        dev = positions.device
-        desc = torch.empty((c, self.n_features), dtype=torch.float32, device=dev)
         if not jacobian:
+            c, sptr = sites.shape[0], C.c_void_p(sites.data_ptr())
+            keep, cellp = self._cell(cell)
+            desc = torch.empty((c, self.n_features), dtype=torch.float32, device=positions.device)
             self._check(self._lib.soap_descriptor_at(self._h, positions.data_ptr(), numbers.data_ptr(), n, cellp, sptr, c,
                                                      desc.data_ptr(), self._stream()))
             self.status()
             return desc
-        npairs, nrows = C.c_int64(), C.c_int64()
-        self._check(self._lib.soap_neighbors_at(self._h, positions.data_ptr(), numbers.data_ptr(), n, cellp, sptr, c,
-                                                C.byref(npairs), C.byref(nrows), self._stream()))
-        nrows = int(nrows.value)
-        jac = torch.empty((max(nrows, 1), 3, self.n_features), dtype=torch.float32, device=dev)
-        row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
-        row_atom = torch.empty(max(nrows, 1), dtype=torch.int32, device=dev)
-        self._check(self._lib.soap_derivatives_at(self._h, positions.data_ptr(), numbers.data_ptr(), n, cellp, sptr, c,
-                                                  desc.data_ptr(), jac.data_ptr(), jac.shape[0], row_ptr.data_ptr(),
-                                                  row_atom.data_ptr(), self._stream()))
-        self.status()
-        return Derivatives(desc, jac[:nrows], row_ptr, row_atom[:nrows])
+        desc, _, jac, row_ptr, row_atom = self._sized(ROWS_FULL, self.n_features, positions, numbers, cell, sites=sites)
+        return Derivatives(desc, jac, row_ptr, row_atom)
 
     # ------------------------------------------------------------------ other output modes
     def coefficients(self, positions, numbers, cell=None, centers=None, out=None):
@@ -395,20 +384,8 @@ class Soap:
 
     def coefficient_derivatives(self, positions, numbers, cell=None, centers=None) -> Derivatives:
         """Coefficients and their Jacobian in the row format of `derivatives` (width W)."""
-        import torch
-        _, nrows = self.neighbors(positions, numbers, cell, centers)
-        n, c, cptr = self._inputs(positions, numbers, centers)
-        keep, cellp = self._cell(cell)
-        dev = positions.device
-        coeff = torch.empty((c, self.n_coefficients), dtype=torch.float32, device=dev)
-        jac = torch.empty((max(nrows, 1), 3, self.n_coefficients), dtype=torch.float32, device=dev)
-        row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
-        row_atom = torch.empty(max(nrows, 1), dtype=torch.int32, device=dev)
-        self._check(self._lib.soap_coefficient_derivatives(self._h, positions.data_ptr(), numbers.data_ptr(), n, cellp, cptr, c,
-                                                           coeff.data_ptr(), jac.data_ptr(), jac.shape[0], row_ptr.data_ptr(),
-                                                           row_atom.data_ptr(), self._stream()))
-        self.status()
-        return Derivatives(coeff, jac[:nrows], row_ptr, row_atom[:nrows])
+        coeff, _, jac, row_ptr, row_atom = self._sized(ROWS_COEFFICIENTS, self.n_coefficients, positions, numbers, cell, centers)
+        return Derivatives(coeff, jac, row_ptr, row_atom)
 
     def descriptor_average(self, mode, positions, numbers, cell=None, centers=None, out=None):
         """(F,) averaged descriptor, mode "inner" or "outer"."""

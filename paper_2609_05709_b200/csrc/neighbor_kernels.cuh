@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(1024) tile_sum_kernel(const int* __restrict__ 
 }
 template <typename OutT>
 __global__ void __launch_bounds__(1024) tile_scan_kernel(const int* __restrict__ in, OutT* __restrict__ out, long long n,
-                                                         const long long* __restrict__ tile_offsets, long long n_tiles) {
+                                                         const long long* __restrict__ tile_offsets, long long n_tiles,
+                                                         const Counters* counters = nullptr, Counters* host = nullptr) {
     __shared__ long long ws[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const long long base = (long long)blockIdx.x * kScanTile + threadIdx.x * 4;      // 4 consecutive items per thread
@@ -233,7 +234,10 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(const int* __restrict__
         if (base + k < n) out[base + k] = (OutT)run;
         run += v[k];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = (OutT)tile_offsets[n_tiles];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        out[n] = (OutT)tile_offsets[n_tiles];
+        if (host) *host = *counters;                     // pinned host memory: the caller waits for the stream and reads it
+    }
 }
 
 __global__ void bin_fill_kernel(const float* __restrict__ pos, long long N, const int* __restrict__ atom_cell,
@@ -748,13 +752,13 @@ batch_pairs_kernel(const float* __restrict__ pos, const int* __restrict__ number
     }
 }
 
-// One block: exclusive scan of the row counts (rows of centre c start at row_ptr[c]) and the launch
+// One block: exclusive scan of the row counts (rows of centre c start at row_ptr[c]), the totals to the host if it asks for them, and the launch
 // order of the per-centre kernel, largest pair count first (bins of 4 pairs, counting sort), so that
 // the long CTAs do not end up alone at the tail of the launch.
 constexpr int kSizeBins = 256, kSizeBinShift = 2;
 __global__ void __launch_bounds__(1024)
 rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pair_count, long long C,
-                  long long* __restrict__ row_ptr, int* __restrict__ order, Counters* counters) {
+                  long long* __restrict__ row_ptr, int* __restrict__ order, Counters* counters, Counters* host) {
     __shared__ long long warp_sums[32];
     __shared__ long long carry_s;
     __shared__ int hist[kSizeBins], first_slot[kSizeBins];
@@ -806,6 +810,7 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
     if (tid == 0) {
         row_ptr[C] = carry_s;
         counters->n_rows = carry_s;
+        if (host) *host = *counters;                     // pinned host memory: the caller waits for the stream and reads it
     }
     if (wid == 0) {
         // first slot of every size bin, largest bin first: lane k scans the bins 255 - 8k down to 248 - 8k, a warp

@@ -124,6 +124,7 @@ struct soap_handle {
     int64_t pairs_per_center_hint = 0;   // average at the last plan (chooses the pair kernel variant)
     int64_t last_centers = 0;
     bool list_sorted = false;            // whether the pair list of the last search is sorted (descriptor-only calls skip that)
+    int64_t found_atoms = -1, found_centers = -1;   // sizes of the search soap_search left for soap_derivatives_found; -1: none
     int P_deriv = 16, P_outer = 16;      // pairs per staged chunk: derivative kernels, kernel of the outer average
     size_t smem_deriv = 0, smem_outer = 0;
     bool outer_fast = false;             // whether the kernel of the outer average fits the shared memory
@@ -333,7 +334,8 @@ int blocks_for(int64_t n, int threads, int cap = 4096) {
 }
 
 // Exclusive scan of C per-centre counts into out[0..C] (out[C] = total, also to *total_dev).
-void scan_counts(soap_t* h, const int* counts, long long* out, int64_t C, long long* total_dev, cudaStream_t st) {
+void scan_counts(soap_t* h, const int* counts, long long* out, int64_t C, long long* total_dev, cudaStream_t st,
+                 const Counters* counters = nullptr, Counters* host = nullptr) {
     if (C <= 65536) {
         scan_kernel<long long><<<1, 1024, 0, st>>>(counts, out, C, total_dev);
         return;
@@ -341,7 +343,7 @@ void scan_counts(soap_t* h, const int* counts, long long* out, int64_t C, long l
     const long long tiles = (C + kScanTile - 1) / kScanTile;
     tile_sum_kernel<<<(unsigned)tiles, 1024, 0, st>>>(counts, C, h->d_tile_sums);
     scan_kernel<long long><<<1, 1024, 0, st>>>(h->d_tile_sums, h->d_tile_offsets, tiles, total_dev);
-    tile_scan_kernel<long long><<<(unsigned)tiles, 1024, 0, st>>>(counts, out, C, h->d_tile_offsets, tiles);
+    tile_scan_kernel<long long><<<(unsigned)tiles, 1024, 0, st>>>(counts, out, C, h->d_tile_offsets, tiles, counters, host);
 }
 
 // The whole neighbour search: cell list, sorted pair segments with their row bookkeeping, row
@@ -358,7 +360,9 @@ constexpr int64_t kBruteForceAtoms = 512;
 
 int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g,
                      const int32_t* centers, const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st,
-                     const Batch& batch = Batch(), bool rows = true) {
+                     const Batch& batch = Batch(), bool rows = true, bool publish = false) {
+    h->found_atoms = h->found_centers = -1;
+    Counters* const host = publish ? h->h_counters : nullptr;
     // (C == N: the brute-force kernel writes the per-centre arrays for every atom, and those are sized from C)
     const bool brute = !batch.struct_ptr && !centers && !sites && C == N && N <= kBruteForceAtoms && !(g.pbc[0] | g.pbc[1] | g.pbc[2]);
     if (batch.struct_ptr || brute) {
@@ -405,9 +409,9 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
         return SOAP_OK;
     }
     if (C <= kOrderMaxCenters) {
-        CU(launch_dependent(rows_order_kernel, 1, 1024, 0, st, h->d_row_count, h->d_pair_count, C, row_ptr_out, h->d_order, h->d_counters));
+        CU(launch_dependent(rows_order_kernel, 1, 1024, 0, st, h->d_row_count, h->d_pair_count, C, row_ptr_out, h->d_order, h->d_counters, host));
     } else {
-        scan_counts(h, h->d_row_count, row_ptr_out, C, &h->d_counters->n_rows, st);
+        scan_counts(h, h->d_row_count, row_ptr_out, C, &h->d_counters->n_rows, st, h->d_counters, host);
     }
     CU(cudaGetLastError());
     return SOAP_OK;
@@ -422,26 +426,32 @@ int check_inputs(soap_t* h, const float* pos, const int32_t* num, int64_t N, con
     return SOAP_OK;
 }
 
-// Plans scratch for a structure of this size: run the search (with whatever capacity there is;
-// the counts come out right even when the pairs do not fit), read the totals back, grow.
-int plan(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g,
-         const int32_t* centers, const float* sites, int64_t C, cudaStream_t st, const Batch& batch = Batch()) {
+// One neighbour search whose totals come back to the host, in scratch that is grown (and the search run again) when it
+// does not hold the pairs: allocates then, and WAITS.  The totals are written to the handle's pinned memory by the last
+// kernel of the search, so that the host waits for the stream and nothing else.  (A call that sizes its own outputs used
+// to search three times and wait five times; searching once took the 24-atom call from 129 to 65 us and the call on
+// 3000 atoms with 274 neighbours each from 1712 to 1374 us.)
+int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g, const int32_t* centers,
+                    const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st, const Batch& batch = Batch()) {
     int rc = ensure_scratch(h, N, C, 0);
     if (rc) return rc;
-    rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, h->d_row_ptr, st, batch);
-    if (rc) return rc;
-    CU(cudaMemcpyAsync(h->h_counters, h->d_counters, sizeof(Counters), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
-    const int64_t pairs = h->h_counters->n_pairs;
-    h->pairs_per_center_hint = C > 0 ? (pairs + C - 1) / C : 0;
-    if (pairs > h->cap_pairs) {
-        rc = ensure_scratch(h, N, C, pairs + pairs / 4 + 1024);
-        if (rc) return rc;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
+        CU(cudaStreamSynchronize(st));
+        const int64_t pairs = h->h_counters->n_pairs;
+        h->pairs_per_center_hint = C > 0 ? (pairs + C - 1) / C : 0;
+        if (h->h_counters->status & kStatusPairCapacity) {
+            // the shortage is mended here, whichever call reported it: forget that bit only
+            h->h_counters->status &= ~kStatusPairCapacity;
+            CU(cudaMemcpyAsync(&h->d_counters->status, &h->h_counters->status, sizeof(int), cudaMemcpyHostToDevice, st));
+            CU(cudaStreamSynchronize(st));
+        }
+        if (pairs <= h->cap_pairs) break;
+        // the counts come out right even when the pairs do not fit
+        if ((rc = ensure_scratch(h, N, C, pairs + pairs / 4 + 1024))) return rc;
     }
-    // the planning run may have reported the shortage it was there to measure: forget that bit only
-    h->h_counters->status &= ~kStatusPairCapacity;
-    CU(cudaMemcpyAsync(&h->d_counters->status, &h->h_counters->status, sizeof(int), cudaMemcpyHostToDevice, st));
-    CU(cudaStreamSynchronize(st));
+    h->list_sorted = true;
+    h->last_centers = C;
     h->planned_atoms = std::max<int64_t>(h->planned_atoms, N);
     h->planned_centers = std::max<int64_t>(h->planned_centers, C);
     return SOAP_OK;
@@ -486,6 +496,15 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     return SOAP_OK;
 }
 
+// What the bits of the status word mean to a caller.
+int status_error(soap_t* h, int s) {
+    if (s & kStatusUnknownSpecies) return fail(h, SOAP_ERR_UNKNOWN_SPECIES, "an atomic number is not in the species list");
+    if (s & kStatusShiftRange) return fail(h, SOAP_ERR_INVALID_ARG, "positions lie too many cells away from the unit cell");
+    if (s & kStatusPairCapacity) return fail(h, SOAP_ERR_CAPACITY, "more pairs than planned (call soap_neighbors again) or than the export buffer holds");
+    if (s & kStatusRowCapacity) return fail(h, SOAP_ERR_CAPACITY, "more Jacobian rows than capacity_rows");
+    return SOAP_OK;
+}
+
 // Feature table: species pairs mu <= nu (only mu == nu without crossover), radial pair (n' >= n on
 // the diagonal), l fastest.
 void build_feature_table(soap_t* h) {
@@ -508,6 +527,15 @@ void build_feature_table(soap_t* h) {
     h->Fc_pitch = (h->Fc + 7) & ~(int64_t)7;
 }
 
+// The radial weights of the pairs found, where the handle has a weighting.
+int launch_weights(soap_t* h, const float* pos, const int32_t* centers, const float* sites, int64_t C, const Geometry& g, cudaStream_t st) {
+    if (!h->weight.fn || C <= 0) return SOAP_OK;
+    pair_weight_kernel<<<(unsigned)((C + 7) / 8), 256, 0, st>>>(pos, centers, sites, C, g, h->d_pair_start, h->d_pair_count, h->d_pair_key,
+                                                               h->cap_pairs, h->d_counters, h->weight, h->d_pair_w);
+    CU(cudaGetLastError());
+    return SOAP_OK;
+}
+
 // Everything before the per-centre kernel: argument checks, device set-up, planning when the sizes
 // changed, the neighbour search.
 int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const double* cell, const int32_t* centers,
@@ -520,21 +548,19 @@ int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const do
     if ((rc = ensure_device(h))) return rc;
     if ((rc = make_geometry(h, cell, g))) return rc;
     if (h->profiling) CU(cudaEventRecord(h->ev[0], st));
-    // plan (search once, read the totals, grow the scratch: allocates and waits) when this structure is larger
+    // search with the totals read back (grows the scratch: allocates and waits) when this structure is larger
     // than anything planned so far; smaller ones run in the scratch that is there, and if one of them turns out
     // to have more pairs than that holds the status word says so
-    if (h->planned_atoms < 0 || N > h->planned_atoms || C > h->planned_centers) {
-        if ((rc = plan(h, pos, num, N, g, centers, sites, C, st, batch))) return rc;
+    const bool planned = h->planned_atoms >= 0 && N <= h->planned_atoms && C <= h->planned_centers;
+    if (!planned && (rc = search_and_size(h, pos, num, N, g, centers, sites, C, row_ptr_out, st, batch))) return rc;
+    if (planned || !rows) {
+        // (a call without rows always takes the unsorted list, so that its sums run in the same order every time)
+        if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, rows))) return rc;
+        h->list_sorted = rows;
+        h->last_centers = C;
     }
-    if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, rows))) return rc;
-    h->list_sorted = rows;
-    if (h->weight.fn && C > 0) {
-        pair_weight_kernel<<<(unsigned)((C + 7) / 8), 256, 0, st>>>(pos, centers, sites, C, g, h->d_pair_start, h->d_pair_count, h->d_pair_key,
-                                                                   h->cap_pairs, h->d_counters, h->weight, h->d_pair_w);
-        CU(cudaGetLastError());
-    }
+    if ((rc = launch_weights(h, pos, centers, sites, C, g, st))) return rc;
     if (h->profiling) CU(cudaEventRecord(h->ev[1], st));
-    h->last_centers = C;
     return SOAP_OK;
 }
 
@@ -640,7 +666,7 @@ int soap_radial_table(const soap_t* h, double d, double* G, double* Ghat) {
 
 static int neighbors_impl(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
                           const int32_t* d_centers, const float* d_sites, int64_t n_centers, int64_t* n_pairs, int64_t* n_rows,
-                          void* stream, const Batch& batch = Batch()) {
+                          void* stream, const Batch& batch = Batch(), long long* row_ptr_out = nullptr) {
     int rc = check_inputs(h, d_positions, d_numbers, n_atoms, d_centers, n_centers, d_sites);
     if (rc) return rc;
     if (batch.struct_ptr && (h->pbc[0] || h->pbc[1] || h->pbc[2]))
@@ -648,13 +674,7 @@ static int neighbors_impl(soap_t* h, const float* d_positions, const int32_t* d_
     if ((rc = ensure_device(h))) return rc;
     Geometry g;
     if ((rc = make_geometry(h, cell, g))) return rc;
-    cudaStream_t st = (cudaStream_t)stream;
-    if ((rc = plan(h, d_positions, d_numbers, n_atoms, g, d_centers, d_sites, n_centers, st, batch))) return rc;
-    if ((rc = launch_neighbors(h, d_positions, d_numbers, n_atoms, g, d_centers, d_sites, n_centers, h->d_row_ptr, st, batch))) return rc;
-    h->list_sorted = true;
-    CU(cudaMemcpyAsync(h->h_counters, h->d_counters, sizeof(Counters), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
-    h->last_centers = n_centers;
+    if ((rc = search_and_size(h, d_positions, d_numbers, n_atoms, g, d_centers, d_sites, n_centers, row_ptr_out, (cudaStream_t)stream, batch))) return rc;
     if (n_pairs) *n_pairs = h->h_counters->n_pairs;
     if (n_rows) *n_rows = h->h_counters->n_rows;
     return SOAP_OK;
@@ -795,6 +815,59 @@ int soap_derivatives_batch(soap_t* h, const float* d_positions, const int32_t* d
     b.n_structs = n_structs;
     return derivatives_impl(h, d_positions, d_numbers, n_atoms, nullptr, nullptr, nullptr, n_atoms, d_out_desc, d_out_jac,
                             capacity_rows, d_row_ptr, d_row_atom, stream, nullptr, b);
+}
+
+// ---- a search, then the derivatives of what it found ----
+int soap_search(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
+                const int32_t* d_centers, const float* d_sites, int64_t n_centers, const int64_t* d_struct_ptr, int64_t n_structs,
+                int64_t* d_row_ptr, int64_t* n_pairs, int64_t* n_rows, void* stream) {
+    if (h && !d_row_ptr) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
+    if (h && d_struct_ptr && (d_centers || d_sites || n_centers != n_atoms))
+        return fail(h, SOAP_ERR_INVALID_ARG, "in a batch of structures every atom is a centre");
+    Batch b;
+    b.struct_ptr = (const long long*)d_struct_ptr;
+    b.n_structs = n_structs;
+    int rc = d_struct_ptr ? check_batch(h, d_struct_ptr, n_structs, n_atoms) : SOAP_OK;
+    if (rc) return rc;
+    if ((rc = neighbors_impl(h, d_positions, d_numbers, n_atoms, cell, d_centers, d_sites, n_centers, n_pairs, n_rows, stream, b, (long long*)d_row_ptr))) return rc;
+    if (h->h_counters->status) {
+        CU(cudaMemsetAsync(&h->d_counters->status, 0, sizeof(int), (cudaStream_t)stream));
+        return status_error(h, h->h_counters->status);
+    }
+    h->found_atoms = n_atoms; h->found_centers = n_centers;
+    return SOAP_OK;
+}
+
+int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_t n_atoms, const double* cell, const int32_t* d_centers,
+                           const float* d_sites, int64_t n_centers, float* d_out_desc, float* d_out_center, float* d_out_jac,
+                           int64_t capacity_rows, const int64_t* d_row_ptr, int32_t* d_row_atom, void* stream) {
+    if (!h) return SOAP_ERR_INVALID_ARG;
+    if (kind != SOAP_ROWS_FULL && kind != SOAP_ROWS_COMPACT && kind != SOAP_ROWS_COEFFICIENTS) return fail(h, SOAP_ERR_INVALID_ARG, "unknown kind of rows");
+    if (h->found_atoms != n_atoms || h->found_centers != n_centers)
+        return fail(h, SOAP_ERR_INVALID_ARG, "no neighbour search of this size is at hand: call soap_search first");
+    if (!d_row_ptr || capacity_rows < 0) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
+    if (n_centers > 0 && (!d_out_desc || !d_out_jac || !d_row_atom)) return fail(h, SOAP_ERR_INVALID_ARG, "output pointers must not be NULL");
+    if (n_centers > 0 && kind == SOAP_ROWS_COMPACT && !d_out_center) return fail(h, SOAP_ERR_INVALID_ARG, "d_out_center must not be NULL");
+    int rc = ensure_device(h);
+    if (rc) return rc;
+    Geometry g;
+    if ((rc = make_geometry(h, cell, g))) return rc;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (h->profiling) CU(cudaEventRecord(h->ev[0], st));
+    if ((rc = launch_weights(h, d_positions, d_centers, d_sites, n_centers, g, st))) return rc;
+    if (h->profiling) CU(cudaEventRecord(h->ev[1], st));
+    if (n_centers > 0) {
+        CenterParams cp;
+        fill_center_params(h, cp, d_positions, d_centers, n_centers, g, true, d_sites);
+        cp.row_ptr = (const long long*)d_row_ptr;
+        cp.row_capacity = capacity_rows;
+        cp.out_desc = d_out_desc; cp.out_jac = d_out_jac; cp.row_atom = d_row_atom;
+        if (kind == SOAP_ROWS_COMPACT) { cp.compact = 1; cp.out_center = d_out_center; }
+        CU(center_launch(kind == SOAP_ROWS_COEFFICIENTS ? kCenterCoeff : kCenterDeriv, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_deriv, st));
+    }
+    if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
+    CU(cudaStreamSynchronize(st));
+    return SOAP_OK;
 }
 
 int soap_num_compact_features(const soap_t* h, int64_t* n_compact, int64_t* pitch) {
@@ -1102,12 +1175,7 @@ int soap_status(soap_t* h, int64_t* n_pairs, int64_t* n_rows, void* stream) {
     CU(cudaStreamSynchronize(st));
     if (n_pairs) *n_pairs = h->h_counters->n_pairs;
     if (n_rows) *n_rows = h->h_counters->n_rows;
-    const int s = h->h_counters->status;
-    if (s & kStatusUnknownSpecies) return fail(h, SOAP_ERR_UNKNOWN_SPECIES, "an atomic number is not in the species list");
-    if (s & kStatusShiftRange) return fail(h, SOAP_ERR_INVALID_ARG, "positions lie too many cells away from the unit cell");
-    if (s & kStatusPairCapacity) return fail(h, SOAP_ERR_CAPACITY, "more pairs than planned (call soap_neighbors again) or than the export buffer holds");
-    if (s & kStatusRowCapacity) return fail(h, SOAP_ERR_CAPACITY, "more Jacobian rows than capacity_rows");
-    return SOAP_OK;
+    return status_error(h, h->h_counters->status);
 }
 
 // ---------------------------------------------------------------------------------------------
