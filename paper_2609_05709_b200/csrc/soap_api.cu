@@ -222,14 +222,16 @@ int plan_smem(soap_t* h) {
         return bytes <= (size_t)max_smem;
     };
     if (!plan_chunk(0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
-    CU(center_set_smem(kCenterDeriv, h->l_max, h->n_max, (int)h->smem_deriv));
-    CU(center_set_smem(kCenterCoeff, h->l_max, h->n_max, (int)h->smem_deriv));
-    CU(center_set_smem(kCenterInner, h->l_max, h->n_max, (int)h->smem_deriv));
+    // (a kernel's limit is the process's, not the handle's: every handle sets the device's maximum, so that none takes away
+    // what another one launches with)
+    CU(center_set_smem(kCenterDeriv, h->l_max, h->n_max, max_smem));
+    CU(center_set_smem(kCenterCoeff, h->l_max, h->n_max, max_smem));
+    CU(center_set_smem(kCenterInner, h->l_max, h->n_max, max_smem));
     // the kernel of the outer average keeps, per warp, a copy of a neighbouring centre's coefficients behind the usual
     // layout; a basis too large for that takes the general path (per-pair rows in a workspace)
     const int LMP = ((h->l_max + 1) * (h->l_max + 1)) | 1;
     h->outer_fast = plan_chunk((size_t)kWarps * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
-    if (h->outer_fast) CU(center_set_smem(kCenterOuter, h->l_max, h->n_max, (int)h->smem_outer));
+    if (h->outer_fast) CU(center_set_smem(kCenterOuter, h->l_max, h->n_max, max_smem));
     return SOAP_OK;
 }
 
