@@ -11,17 +11,6 @@ namespace soap {
 #define SOAP_CAT2(a, b) a##b
 #define SOAP_CAT(a, b) SOAP_CAT2(a, b)
 
-template <int KIND, int NM, bool PLAIN>
-static cudaError_t set_one(int bytes) {
-    return cudaFuncSetAttribute(center_kernel<KIND, SOAP_L, NM, PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-template <int KIND, int NM, bool PLAIN>
-static cudaError_t launch_one(const CenterParams& p, unsigned grid, size_t smem, cudaStream_t st) {
-    // the kernel waits on the device for the kernel before it (the row scan, as a rule): its launch and its
-    // set-up overlap that kernel's tail
-    return launch_dependent(center_kernel<KIND, SOAP_L, NM, PLAIN>, grid, kThreads, smem, st, p);
-}
-
 // Fills this translation unit's constant tables (once per process and device is enough;
 // it is cheap, so it runs whenever a handle sets up its kernels).
 cudaError_t SOAP_CAT(center_constants_l, SOAP_L)(const float* anorm91, const float* dfact16) {
@@ -45,97 +34,94 @@ cudaError_t SOAP_CAT(center_constants_l, SOAP_L)(const float* anorm91, const flo
     return cudaMemcpyToSymbol(kc_dfact, dfact16, 16 * sizeof(float));
 }
 
-// The plain kernels have their own instantiation for the usual n_max (loops over n unroll, the accumulators of
-// pass 1 fit the registers exactly; the variant that reads n_max at run time is 1.4 to 2 times slower and
-// serves every other n_max); the kernels that honour the options are instantiated for fewer n_max still.
-// Even l_max and l_max = 3 get the long lists, the other odd l_max the short ones.
-#if (SOAP_L % 2 == 0) || (SOAP_L == 3)
+// The kernels have an instantiation of their own for the usual n_max: loops over n unroll, the accumulators of pass 1
+// fit the registers exactly.  The variant that reads n_max at run time spills 0.6 kB and serves what is left (n_max 1
+// and 13 to 16, and the largest l_max, whose kernels take longest to compile).  Measured, run time against compile time:
+// (n_max, l_max) = (5, 5) on 1021 centres 254 -> 159 us, (6, 6) with a weighting and compact rows on 1111 centres
+// 368 -> 270 us, whole calls of the other sizes 1.2 to 1.7 times faster.
+#if SOAP_L <= 10
+#define SOAP_FOR_FIXED_NMAX(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
+#elif SOAP_L == 12
 #define SOAP_FOR_FIXED_NMAX(X) X(2) X(4) X(6) X(7) X(8) X(10) X(12)
-#define SOAP_FOR_GENERAL_NMAX(X) X(4) X(8)
 #else
 #define SOAP_FOR_FIXED_NMAX(X) X(4) X(8)
+#endif
+#if SOAP_L <= 8
+#define SOAP_FOR_GENERAL_NMAX(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(10) X(12)
+#elif SOAP_L <= 10
+#define SOAP_FOR_GENERAL_NMAX(X) X(4) X(6) X(8) X(10) X(12)
+#else
 #define SOAP_FOR_GENERAL_NMAX(X) X(8)
 #endif
-static bool center_has_fixed_nmax(int n_max) {
-    switch (n_max) {
-#define X(N) case N: return true;
-        SOAP_FOR_FIXED_NMAX(X)
-#undef X
-    }
-    return false;
-}
-static bool general_has_fixed_nmax(int n_max) {
-    switch (n_max) {
-#define X(N) case N: return true;
-        SOAP_FOR_GENERAL_NMAX(X)
-#undef X
-    }
-    return false;
-}
+#if SOAP_L % 2 == 0 || SOAP_L == 3
+#define SOAP_FOR_COEFF_NMAX(X) X(4) X(8)
+#else
+#define SOAP_FOR_COEFF_NMAX(X) X(8)
+#endif
 
-cudaError_t SOAP_CAT(center_set_smem_l, SOAP_L)(int kind, int n_max, int bytes) {
-    cudaError_t e;
+#if SOAP_L <= 8
+#define SOAP_FOR_AVERAGE_NMAX(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9)
+#else
+#define SOAP_FOR_AVERAGE_NMAX(X) X(8)
+#endif
+
+using Kernel = void (*)(CenterParams);
+
+static Kernel kernel_of(int kind, int n_max, bool plain) {
     if (kind == kCenterInner) {
-        if ((e = set_one<3, 0, false>(bytes)) != cudaSuccess) return e;
-        return set_one<3, 8, false>(bytes);
+        switch (n_max) {
+#define X(N) case N: return center_kernel<3, SOAP_L, N, false>;
+            SOAP_FOR_AVERAGE_NMAX(X)
+#undef X
+        }
+        return center_kernel<3, SOAP_L, 0, false>;
     }
     if (kind == kCenterOuter) {
-        if ((e = set_one<4, 0, false>(bytes)) != cudaSuccess) return e;
-        return set_one<4, 8, false>(bytes);
-    }
-    if (kind == kCenterCoeff) {
-        if ((e = set_one<2, 0, false>(bytes)) != cudaSuccess) return e;
-        switch (general_has_fixed_nmax(n_max) ? n_max : 0) {
-#define X(N) case N: return set_one<2, N, false>(bytes);
-            SOAP_FOR_GENERAL_NMAX(X)
+        switch (n_max) {
+#define X(N) case N: return center_kernel<4, SOAP_L, N, false>;
+            SOAP_FOR_AVERAGE_NMAX(X)
 #undef X
         }
-        return cudaSuccess;
+        return center_kernel<4, SOAP_L, 0, false>;
     }
-    if ((e = set_one<1, 0, false>(bytes)) != cudaSuccess) return e;
-    switch (general_has_fixed_nmax(n_max) ? n_max : 0) {
-#define X(N) case N: e = set_one<1, N, false>(bytes); break;
-        SOAP_FOR_GENERAL_NMAX(X)
-#undef X
-        default: e = cudaSuccess;
-    }
-    if (e != cudaSuccess) return e;
-    switch (center_has_fixed_nmax(n_max) ? n_max : 0) {
-#define X(N) case N: return set_one<1, N, true>(bytes);
-        SOAP_FOR_FIXED_NMAX(X)
-#undef X
-        default: return set_one<1, 0, true>(bytes);
-    }
-}
-
-cudaError_t SOAP_CAT(center_launch_l, SOAP_L)(int kind, int n_max, bool plain, const CenterParams& p, unsigned grid, size_t smem,
-                                              cudaStream_t st) {
-    if (kind == kCenterInner)
-        return n_max == 8 ? launch_one<3, 8, false>(p, grid, smem, st) : launch_one<3, 0, false>(p, grid, smem, st);
-    if (kind == kCenterOuter)
-        return n_max == 8 ? launch_one<4, 8, false>(p, grid, smem, st) : launch_one<4, 0, false>(p, grid, smem, st);
     if (kind == kCenterCoeff) {
-        switch (general_has_fixed_nmax(n_max) ? n_max : 0) {
-#define X(N) case N: return launch_one<2, N, false>(p, grid, smem, st);
-            SOAP_FOR_GENERAL_NMAX(X)
+        switch (n_max) {
+#define X(N) case N: return center_kernel<2, SOAP_L, N, false>;
+            SOAP_FOR_COEFF_NMAX(X)
 #undef X
-            default: return launch_one<2, 0, false>(p, grid, smem, st);
         }
+        return center_kernel<2, SOAP_L, 0, false>;
     }
     if (!plain) {
-        switch (general_has_fixed_nmax(n_max) ? n_max : 0) {
-#define X(N) case N: return launch_one<1, N, false>(p, grid, smem, st);
+        switch (n_max) {
+#define X(N) case N: return center_kernel<1, SOAP_L, N, false>;
             SOAP_FOR_GENERAL_NMAX(X)
 #undef X
-            default: return launch_one<1, 0, false>(p, grid, smem, st);
         }
+        return center_kernel<1, SOAP_L, 0, false>;
     }
-    switch (center_has_fixed_nmax(n_max) ? n_max : 0) {
-#define X(N) case N: return launch_one<1, N, true>(p, grid, smem, st);
+    switch (n_max) {
+#define X(N) case N: return center_kernel<1, SOAP_L, N, true>;
         SOAP_FOR_FIXED_NMAX(X)
 #undef X
-        default: return launch_one<1, 0, true>(p, grid, smem, st);
     }
+    return center_kernel<1, SOAP_L, 0, true>;
+}
+
+// The dynamic shared memory that every kernel of this kind and n_max may be launched with.
+cudaError_t SOAP_CAT(center_set_smem_l, SOAP_L)(int kind, int n_max, int bytes) {
+    for (const bool plain : {false, true}) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel_of(kind, n_max, plain), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// The kernel waits on the device for the kernel before it (the row scan, as a rule): its launch and its set-up overlap
+// that kernel's tail.
+cudaError_t SOAP_CAT(center_launch_l, SOAP_L)(int kind, int n_max, bool plain, const CenterParams& p, unsigned grid, size_t smem,
+                                              cudaStream_t st) {
+    return launch_dependent(kernel_of(kind, n_max, plain), grid, kThreads, smem, st, p);
 }
 
 }  // namespace soap
