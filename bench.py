@@ -46,12 +46,12 @@ UNIT = "atoms/s"
 
 
 def kernels_per_step(n_atoms, n_centers, periodic=False):
-    """Kernel launches of one soap_derivatives call over all atoms: the cell-list build (one launch up to
-    16384 atoms, five above; none for a non-periodic structure of up to 512 atoms, which takes the
-    brute-force pair kernel), the pair kernel, the row scan with the launch order (one launch up to 65536
-    centres, three above) and the fused per-centre kernel."""
-    build = 0 if (n_atoms <= 512 and not periodic) else (1 if n_atoms <= 16384 else 5)
-    return build + 1 + (1 if n_centers <= 65536 else 3) + 1
+    """Kernel launches of one soap_derivatives call over all atoms: the search of a non-periodic structure of up to 512
+    atoms is one launch; else the cell list (one launch up to 65536 atoms, seven above), the pair kernel and the row
+    scan with the launch order (one launch up to 65536 centres, three above); then the fused per-centre kernel."""
+    if n_atoms <= 512 and not periodic:
+        return 2
+    return (1 if n_atoms <= 65536 else 7) + 1 + (1 if n_centers <= 65536 else 3) + 1
 
 
 # DRAM traffic of the fused kernel: ONE ncu capture on the 300-molecule cluster (profiles/center_kernel_water300.md),

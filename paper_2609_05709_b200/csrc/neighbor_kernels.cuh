@@ -9,9 +9,28 @@
 // does not depend on the binning and can be compared bit for bit with a
 // reference.  Pairs of a centre come out sorted by (atom, n_a, n_b, n_c).
 #pragma once
+#include <cooperative_groups.h>
+
 #include "soap_device.cuh"
 
 namespace soap {
+
+#ifdef __CUDACC__
+// launch of a grid that is one thread-block cluster; `dependent`: it begins with grid_dependency_wait() and may overlap
+// the tail of its predecessor
+template <class... KArgs, class... Args>
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int ctas, int threads, cudaStream_t st, bool dependent, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = ctas; cfg.blockDim = threads; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = dependent ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+#endif
 
 // ---- order-preserving encoding of doubles for atomicMax ---------------------
 __device__ inline unsigned long long enc_double(double x) {
@@ -57,53 +76,44 @@ __global__ void species_bbox_kernel(const float* __restrict__ pos, const int* __
     if (bad) atomicOr(&counters->status, kStatusUnknownSpecies);
 }
 
-// One thread: choose the bin grid.  Bin width (measured perpendicular to the
-// cell faces) is at least r_cut (1 + 1e-6) wherever more than one bin fits, so a
-// stencil of +-1 bin covers the sphere; short periodic axes get one bin and a
-// wider stencil of images.
-__device__ inline GridParams choose_grid(const double hi_in[3], const double lo_in[3], const Geometry& geom, long long N, int cell_cap) {
-    GridParams g;
+// Choose the bin grid; called by a whole warp, one lane per axis, the result in `g` (shared or global memory).  Bin
+// width (measured perpendicular to the cell faces) is at least r_cut (1 + 1e-6) wherever more than one bin fits, so a
+// stencil of +-1 bin covers the sphere; short periodic axes get one bin and a wider stencil of images.
+__device__ inline void choose_grid(double hi, double lo, const Geometry& geom, long long N, int cell_cap, GridParams* g) {
+    const int a = threadIdx.x & 31;                       // lanes 3 .. 31 repeat axis 2
+    const int ax = min(a, 2);
     const double rc = geom.r_cut * (1.0 + 1e-6);
-    double want[3];
-    for (int a = 0; a < 3; ++a) {
-        g.periodic[a] = geom.pbc[a];
-        if (geom.pbc[a]) {
-            g.smin[a] = 0.0;
-            want[a] = floor(geom.height[a] / rc);
-        } else {
-            double hi = N > 0 ? hi_in[a] : 0.0, lo = N > 0 ? lo_in[a] : 0.0;
-            g.smin[a] = lo;
-            want[a] = floor((hi - lo) * geom.height[a] / rc);
-        }
-        if (!(want[a] >= 1.0)) want[a] = 1.0;
-        if (want[a] > 1024.0) want[a] = 1024.0;
-    }
+    const bool periodic = geom.pbc[ax] != 0;
+    if (N <= 0) { hi = 0.0; lo = 0.0; }
+    const double span = hi - lo;
+    double want = periodic ? floor(geom.height[ax] / rc) : floor(span * geom.height[ax] / rc);
+    if (!(want >= 1.0)) want = 1.0;
+    if (want > 1024.0) want = 1024.0;
     // respect the scratch capacity: shrink the grid uniformly
-    for (int it = 0; it < 64 && want[0] * want[1] * want[2] > (double)cell_cap; ++it)
-        for (int a = 0; a < 3; ++a) want[a] = fmax(1.0, floor(want[a] * 0.8));
-    for (int a = 0; a < 3; ++a) {
-        g.nb[a] = (int)want[a];
-        if (geom.pbc[a]) {
-            g.sscale[a] = (double)g.nb[a];
-            double width = geom.height[a] / g.nb[a];
-            g.R[a] = (int)ceil(rc / width);
-        } else {
-            double hi = N > 0 ? hi_in[a] : 0.0;
-            double span = hi - g.smin[a];
-            g.sscale[a] = span > 0 ? g.nb[a] / span : 0.0;
-            g.R[a] = g.nb[a] > 1 ? 1 : 0;
-        }
+    auto of = [&](int axis) { return __shfl_sync(0xffffffffu, want, axis); };
+    for (int it = 0; it < 64; ++it) {
+        const double w0 = of(0), w1 = of(1), w2 = of(2);
+        if (!(w0 * w1 * w2 > (double)cell_cap)) break;
+        want = fmax(1.0, floor(want * 0.8));
     }
-    g.n_cells = g.nb[0] * g.nb[1] * g.nb[2];
-    return g;
+    const int nb = (int)want;
+    const int n0 = __shfl_sync(0xffffffffu, nb, 0), n1 = __shfl_sync(0xffffffffu, nb, 1), n2 = __shfl_sync(0xffffffffu, nb, 2);
+    if (a < 3) {
+        g->nb[a] = nb;
+        g->periodic[a] = periodic;
+        g->smin[a] = periodic ? 0.0 : lo;
+        g->sscale[a] = periodic ? (double)nb : (span > 0 ? nb / span : 0.0);
+        g->R[a] = periodic ? (int)ceil(rc / (geom.height[a] / nb)) : (nb > 1 ? 1 : 0);
+    }
+    if (a == 0) g->n_cells = n0 * n1 * n2;
+    __syncwarp();
 }
 
-__global__ void grid_setup_kernel(const unsigned long long* bbox, Geometry geom, long long N, int cell_cap, GridParams* out,
+__global__ void __launch_bounds__(32) grid_setup_kernel(const unsigned long long* bbox, Geometry geom, long long N, int cell_cap, GridParams* out,
                                   Counters* counters) {
-    if (counters) { counters->n_pairs = 0; counters->n_rows = 0; }      // the pair cursor of this call
-    double hi[3], lo[3];
-    for (int a = 0; a < 3; ++a) { hi[a] = dec_double(bbox[a]); lo[a] = -dec_double(bbox[3 + a]); }
-    *out = choose_grid(hi, lo, geom, N, cell_cap);
+    if (counters && threadIdx.x == 0) { counters->n_pairs = 0; counters->n_rows = 0; }      // the pair cursor of this call
+    const int a = min((int)threadIdx.x, 2);
+    choose_grid(dec_double(bbox[a]), -dec_double(bbox[3 + a]), geom, N, cell_cap, out);
 }
 
 __device__ inline void bin_of(const Geometry& geom, const GridParams& g, float x, float y, float z, int b[3], int w[3]) {
@@ -255,7 +265,7 @@ __global__ void bin_fill_kernel(const float* __restrict__ pos, long long N, cons
 // the atoms by bin in ONE launch of a single CTA (five dependent launches otherwise; at a few
 // thousand atoms the launches, not the work, set the time).
 constexpr int kPrepThreads = 1024;
-constexpr long long kSmallPrepAtoms = 16384;
+constexpr long long kSmallPrepAtoms = 4096;
 constexpr int kPrepSmemCells = 4096;
 __global__ void __launch_bounds__(kPrepThreads)
 small_prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long long N, Geometry geom,
@@ -299,14 +309,15 @@ small_prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        double h3[3], l3[3];
-        for (int a = 0; a < 3; ++a) { h3[a] = red[a][0]; l3[a] = -red[3 + a][0]; }
-        sg = choose_grid(h3, l3, geom, N, cell_cap);
-        *grid_out = sg;
-        carry_s = 0;
-        counters->n_pairs = 0;                                            // the pair cursor of this call
-        counters->n_rows = 0;
+    if (wid == 0) {
+        const int a = min(lane, 2);
+        choose_grid(red[a][0], -red[3 + a][0], geom, N, cell_cap, &sg);
+        if (lane == 0) {
+            *grid_out = sg;
+            carry_s = 0;
+            counters->n_pairs = 0;                                            // the pair cursor of this call
+            counters->n_rows = 0;
+        }
     }
     __syncthreads();
     const GridParams g = sg;
@@ -367,6 +378,135 @@ small_prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers
         const int slot = starts[cell] + atomicSub(&cnt[cell], 1) - 1;
         s_pos[slot] = make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __int_as_float((int)i));
         s_wrap[slot] = atom_wrap[i];
+    }
+}
+
+// Structures of kSmallPrepAtoms to kPrepAtoms atoms: the same steps, species lookup, bounding box, grid choice, binning, bin scan and the sort of
+// the atoms by bin, in ONE launch of a thread-block cluster (seven dependent launches otherwise; up to some ten thousand
+// atoms the launches, not the work, set the time).  The CTAs exchange the bounding box and the totals of the bin scan
+// through each other's shared memory; the bin counters are in global memory, zero before and after the call (the scan
+// clears what it reads).  Below kSmallPrepAtoms one CTA with its counters on chip is as fast or faster (1111 atoms 11.0
+// against 12.0 us, 3000 atoms 14.5 us both); at 30,000 atoms this takes 20 us, the seven launches 31 us and
+// their gaps.
+constexpr int kPrepCtas = 8, kPrepPerThread = 8;
+constexpr long long kPrepAtoms = (long long)kPrepThreads * kPrepCtas * kPrepPerThread;
+__global__ void __launch_bounds__(kPrepThreads)
+prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long long N, Geometry geom,
+            const int* __restrict__ z_lut, int* __restrict__ species_idx, int cell_cap, GridParams* grid_out,
+            int* __restrict__ atom_cell, int* __restrict__ atom_wrap, int* cell_count, int* cell_start,
+            float4* __restrict__ s_pos, int* __restrict__ s_wrap, Counters* counters) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ double red[6][32], box[6];
+    __shared__ GridParams sg;
+    __shared__ int warp_sums[32], cta_total;
+    grid_dependency_launch();                                                // the pair kernel may move in and wait
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
+    const int stride = ctas * kPrepThreads, first = rank * kPrepThreads + tid, n = (int)N;
+    // ---- species and bounding box of the fractional coordinates ----
+    double m[6] = {-1e300, -1e300, -1e300, -1e300, -1e300, -1e300};           // max s, max -s
+    bool bad = false;
+    for (int i = first; i < n; i += stride) {
+        const int z = numbers[i];
+        int s = (z >= 0 && z < 128) ? z_lut[z] : -1;
+        if (s < 0) { bad = true; s = 0; }
+        species_idx[i] = s;
+        double f[3];
+        frac_coords(geom, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], f);
+        for (int a = 0; a < 3; ++a) { m[a] = fmax(m[a], f[a]); m[3 + a] = fmax(m[3 + a], -f[a]); }
+    }
+    if (bad) atomicOr(&counters->status, kStatusUnknownSpecies);
+    for (int a = 0; a < 6; ++a) {
+        for (int o = 16; o > 0; o >>= 1) m[a] = fmax(m[a], __shfl_xor_sync(0xffffffffu, m[a], o));
+        if (lane == 0) red[a][wid] = m[a];
+    }
+    __syncthreads();
+    if (wid < 6) {
+        double v = red[wid][lane];
+        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if (lane == 0) box[wid] = v;
+    }
+    cluster.sync();
+    if (wid == 0) {
+        // every CTA makes the same choice from the boxes of all of them
+        const int a = min(lane, 2);
+        double hi = -1e300, lo = -1e300;
+        for (int r = 0; r < ctas; ++r) {
+            const double* other = cluster.map_shared_rank(box, r);
+            hi = fmax(hi, other[a]); lo = fmax(lo, other[3 + a]);
+        }
+        choose_grid(hi, -lo, geom, N, cell_cap, &sg);
+        if (rank == 0 && lane == 0) {
+            *grid_out = sg;
+            counters->n_pairs = 0;                                            // the pair cursor of this call
+            counters->n_rows = 0;
+        }
+    }
+    __syncthreads();
+    const GridParams g = sg;
+    // ---- bin counts; the count an atom finds is its place within the bin ----
+    int cell[kPrepPerThread], place[kPrepPerThread];
+#pragma unroll
+    for (int k = 0; k < kPrepPerThread; ++k) {
+        const int i = first + k * stride;
+        cell[k] = place[k] = 0;
+        if (i < n) {
+            int b[3], w[3];
+            bin_of(geom, g, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], b, w);
+            if (abs(w[0]) > 100 || abs(w[1]) > 100 || abs(w[2]) > 100) {      // positions absurdly far outside the cell
+                atomicOr(&counters->status, kStatusShiftRange);
+                w[0] = w[1] = w[2] = 0;
+            }
+            cell[k] = (b[2] * g.nb[1] + b[1]) * g.nb[0] + b[0];
+            atom_cell[i] = cell[k];
+            atom_wrap[i] = pack3(w);
+            place[k] = atomicAdd(&cell_count[cell[k]], 1);
+        }
+    }
+    cluster.sync();
+    // ---- exclusive scan of the bin counts: a contiguous range of bins per CTA and per thread ----
+    const int per_cta = (g.n_cells + ctas - 1) / ctas, c_end = min(g.n_cells, (rank + 1) * per_cta);
+    const int per_thread = (per_cta + kPrepThreads - 1) / kPrepThreads;
+    const int c0 = min(c_end, rank * per_cta + tid * per_thread), c1 = min(c_end, c0 + per_thread);
+    int mine = 0;
+    for (int c = c0; c < c1; ++c) mine += cell_count[c];
+    int incl = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_sums[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        int w = warp_sums[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        warp_sums[lane] = w;
+        if (lane == 31) cta_total = w;
+    }
+    cluster.sync();
+    int at = (wid > 0 ? warp_sums[wid - 1] : 0) + incl - mine;
+    for (int r = 0; r < rank; ++r) at += *cluster.map_shared_rank(&cta_total, r);
+    for (int c = c0; c < c1; ++c) {
+        const int v = cell_count[c];
+        cell_start[c] = at;
+        cell_count[c] = 0;
+        at += v;
+    }
+    if (rank == 0 && tid == 0) cell_start[g.n_cells] = n;
+    cluster.sync();
+    // ---- atoms sorted by bin ----
+#pragma unroll
+    for (int k = 0; k < kPrepPerThread; ++k) {
+        const int i = first + k * stride;
+        if (i < n) {
+            const int slot = cell_start[cell[k]] + place[k];
+            s_pos[slot] = make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __int_as_float(i));
+            s_wrap[slot] = atom_wrap[i];
+        }
     }
 }
 
@@ -553,8 +693,10 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
              long long pair_capacity, unsigned long long* pair_tmp, unsigned long long* pair_key, int* __restrict__ pair_row,
              long long* __restrict__ pair_start, int* __restrict__ pair_count, int* __restrict__ row_count,
              int* __restrict__ self_row, Counters* counters) {
+    constexpr int BUCKETS = KEYS < 256 ? KEYS : 256;
     __shared__ unsigned long long s_raw[kFillWarps][KEYS];
-    __shared__ unsigned long long s_sorted[kFillWarps][KEYS];
+    __shared__ unsigned long long s_sorted[kFillWarps][ROWS ? KEYS : 1];
+    __shared__ __align__(16) int s_bucket[kFillWarps][ROWS ? BUCKETS : 4];
     grid_dependency_launch();
     grid_dependency_wait();                                                  // the cell list of the kernel before
     const GridParams g = *gp;
@@ -614,40 +756,75 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
                                at0 += __popc(m);
                            });
     }
-    volatile unsigned long long* raw = in_smem ? s_raw[wid] : pair_tmp + base;
-    volatile unsigned long long* sorted = in_smem ? s_sorted[wid] : pair_key + base;
     __syncwarp();
     if (!ROWS) {
+        const unsigned long long* raw = in_smem ? s_raw[wid] : pair_tmp + base;
         for (int q = lane; q < k; q += 32) pair_key[base + q] = raw[q];
         return;
     }
-    // rank sort (keys are distinct), two keys per lane and trip so that every key read serves two comparisons;
-    // without a periodic axis all keys carry the same lattice translation and the atom fields alone decide
+    // ---- sort by (atom, translation): the keys are distinct ----
+    volatile unsigned long long* sorted = in_smem ? s_raw[wid] : pair_key + base;
     bool self_in = false;
-    const bool atoms_only = !(geom.pbc[0] | geom.pbc[1] | geom.pbc[2]);
-    for (int q = lane; q < k; q += 64) {
-        const bool two = q + 32 < k;
-        const unsigned long long key0 = raw[q], key1 = two ? raw[q + 32] : ~0ull;
-        int rank0 = 0, rank1 = 0;
-        if (atoms_only) {
-            const unsigned a0 = (unsigned)(key0 >> 24), a1 = (unsigned)(key1 >> 24);
-            for (int r = 0; r < k; ++r) {
-                const unsigned a = (unsigned)(raw[r] >> 24);
-                rank0 += a < a0; rank1 += a < a1;
-            }
-        } else {
-            for (int r = 0; r < k; ++r) {
-                const unsigned long long v = raw[r];
-                rank0 += v < key0; rank1 += v < key1;
-            }
+    if (in_smem) {
+        // Buckets of equal width between the smallest and the largest atom: one or two keys each as a rule, which are
+        // ranked within their bucket (a rank sort over all k keys takes k^2 / 32 steps of a warp: 110 against 39 us for
+        // the kernel on 3000 centres of 274 pairs, 16.8 against 14.6 us with 68 pairs each)
+        unsigned long long* const raw = s_raw[wid];
+        unsigned long long* const grouped = s_sorted[wid];
+        int* const bucket_at = s_bucket[wid];
+        unsigned lo = 0xffffffffu, hi = 0;
+        for (int q = lane; q < k; q += 32) {
+            const unsigned a = (unsigned)(raw[q] >> 24);
+            lo = min(lo, a); hi = max(hi, a);
         }
-        sorted[rank0] = key0;
-        if (in_smem) pair_key[base + rank0] = key0;
-        self_in |= key_atom(key0) == i;
-        if (two) {
-            sorted[rank1] = key1;
-            if (in_smem) pair_key[base + rank1] = key1;
-            self_in |= key_atom(key1) == i;
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        const float scale = (float)BUCKETS / (float)(hi - lo + 1u);                   // conversion and product keep the order
+        auto bucket_of = [&](unsigned long long key) { return min(BUCKETS - 1, (int)((float)((unsigned)(key >> 24) - lo) * scale)); };
+        constexpr int PER_LANE = BUCKETS / 32;
+        int4* const mine = reinterpret_cast<int4*>(bucket_at) + lane * (PER_LANE / 4);
+#pragma unroll
+        for (int v = 0; v < PER_LANE / 4; ++v) mine[v] = make_int4(0, 0, 0, 0);
+        __syncwarp();
+        for (int q = lane; q < k; q += 32) atomicAdd(&bucket_at[bucket_of(raw[q])], 1);
+        __syncwarp();
+        int4 cnt[PER_LANE / 4];
+        int sum = 0;
+#pragma unroll
+        for (int v = 0; v < PER_LANE / 4; ++v) { cnt[v] = mine[v]; sum += cnt[v].x + cnt[v].y + cnt[v].z + cnt[v].w; }
+        int at = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += y;
+        }
+        at -= sum;
+#pragma unroll
+        for (int v = 0; v < PER_LANE / 4; ++v) {
+            mine[v] = make_int4(at, at + cnt[v].x, at + cnt[v].x + cnt[v].y, at + cnt[v].x + cnt[v].y + cnt[v].z);
+            at += cnt[v].x + cnt[v].y + cnt[v].z + cnt[v].w;
+        }
+        __syncwarp();
+        for (int q = lane; q < k; q += 32) {
+            const unsigned long long key = raw[q];
+            grouped[atomicAdd(&bucket_at[bucket_of(key)], 1)] = key;
+        }
+        __syncwarp();                                                                  // bucket b now ends at bucket_at[b]
+        for (int q = lane; q < k; q += 32) {
+            const unsigned long long key = grouped[q];
+            const int b = bucket_of(key), end = bucket_at[b];
+            int rank = b > 0 ? bucket_at[b - 1] : 0;
+            for (int r = rank; r < end; ++r) rank += grouped[r] < key;
+            raw[rank] = key;
+            self_in |= key_atom(key) == i;
+        }
+    } else {
+        const volatile unsigned long long* raw = pair_tmp + base;
+        for (int q = lane; q < k; q += 32) {
+            const unsigned long long key = raw[q];
+            int rank = 0;
+            for (int r = 0; r < k; ++r) rank += raw[r] < key;
+            sorted[rank] = key;
+            self_in |= key_atom(key) == i;
         }
     }
     self_in = __any_sync(0xffffffffu, self_in);
@@ -658,7 +835,9 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
         const int q = q0 + lane;
         int atom = -1, prev = -2;
         if (q < k) {
-            atom = key_atom(sorted[q]);
+            const unsigned long long key = sorted[q];
+            if (in_smem) pair_key[base + q] = key;
+            atom = key_atom(key);
             prev = q > 0 ? key_atom(sorted[q - 1]) : -1;
         }
         const bool isnew = q < k && atom != prev;
@@ -752,87 +931,238 @@ batch_pairs_kernel(const float* __restrict__ pos, const int* __restrict__ number
     }
 }
 
-// One block: exclusive scan of the row counts (rows of centre c start at row_ptr[c]), the totals to the host if it asks for them, and the launch
-// order of the per-centre kernel, largest pair count first (bins of 4 pairs, counting sort), so that
-// the long CTAs do not end up alone at the tail of the launch.
-constexpr int kSizeBins = 256, kSizeBinShift = 2;
-__global__ void __launch_bounds__(1024)
-rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pair_count, long long C,
-                  long long* __restrict__ row_ptr, int* __restrict__ order, Counters* counters, Counters* host) {
-    __shared__ long long warp_sums[32];
-    __shared__ long long carry_s;
-    __shared__ int hist[kSizeBins], first_slot[kSizeBins];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+// The test 0 < |d|^2 < r_cut^2 on the raw fp32 inputs, every operation rounded to fp64 on its own: what a pair is.
+__device__ inline bool inside_exact(const Geometry& geom, float4 pj, float xi, float yi, float zi) {
+    const double dx = __dsub_rn((double)pj.x, (double)xi), dy = __dsub_rn((double)pj.y, (double)yi), dz = __dsub_rn((double)pj.z, (double)zi);
+    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    return d2 < geom.rc2 && d2 > 0.0;
+}
+// The same answer, decided in fp32 wherever that is safe: the fp32 value of |d|^2 is off by at most 5 roundings (each
+// difference one, counted twice by the square; the square; two sums), 5 x 2^-24 of itself, and the differences are zero
+// when the coordinates are equal and only then; a band of +-2^-20 around r_cut^2 goes to the exact test.
+__device__ __forceinline__ bool inside(const Geometry& geom, float rc2_lo, float rc2_hi, float4 pj, float xi, float yi, float zi) {
+    const float dx = pj.x - xi, dy = pj.y - yi, dz = pj.z - zi;
+    const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+    if (d2 < rc2_lo) return dx != 0.f || dy != 0.f || dz != 0.f;
+    return d2 < rc2_hi && inside_exact(geom, pj, xi, yi, zi);
+}
+
+// The whole search of one non-periodic structure of up to kBruteForceAtoms atoms with every atom a centre, in ONE launch
+// of a thread-block cluster: every CTA holds all positions in shared memory, its warps take the centres of a contiguous
+// range and run over all atoms (neighbours come out in atom order, nothing is sorted); the pair totals of the CTAs
+// before it come from their shared memory, so segments and row pointers are written directly.  At these sizes a call
+// is a handful of launches and nothing else (24 atoms: memset, pair kernel and row scan took 10.7 us, this takes
+// 7.7 us).  Writes what pairs_kernel and rows_order_kernel write, except a launch order.
+constexpr int kBruteThreads = 1024, kBruteWarps = kBruteThreads / 32, kBruteCtas = 8, kBrutePerWarp = 2;
+constexpr int kBruteForceAtoms = kBruteWarps * kBruteCtas * kBrutePerWarp, kBrutePerCta = kBruteWarps * kBrutePerWarp;
+__global__ void __launch_bounds__(kBruteThreads)
+brute_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, const int* __restrict__ z_lut, int* __restrict__ species_idx,
+             int n, Geometry geom, long long pair_capacity, unsigned long long* __restrict__ pair_key, int* __restrict__ pair_row,
+             long long* __restrict__ pair_start, int* __restrict__ pair_count, int* __restrict__ self_row,
+             long long* __restrict__ row_ptr, Counters* counters, Counters* host) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ float4 s_atom[kBruteForceAtoms];
+    __shared__ int s_count[kBrutePerCta], cta_total;
     grid_dependency_launch();
-    if (tid == 0) carry_s = 0;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
+    const int per_cta = (n + ctas - 1) / ctas, c_lo = min(n, rank * per_cta), c_hi = min(n, c_lo + per_cta);
+    for (int i = tid; i < n; i += kBruteThreads) s_atom[i] = make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], 0.f);
+    if (c_lo + tid < c_hi) {
+        const int z = numbers[c_lo + tid];
+        int s = (z >= 0 && z < 128) ? z_lut[z] : -1;
+        if (s < 0) { atomicOr(&counters->status, kStatusUnknownSpecies); s = 0; }
+        species_idx[c_lo + tid] = s;
+    }
+    if (tid < kBrutePerCta) s_count[tid] = 0;
+    __syncthreads();
+    // ---- who sees whom: lane t of a warp keeps the mask of the atoms 32 t .. 32 t + 31 ----
+    const float rc2_lo = (float)geom.rc2 * (1.f - 0x1p-20f), rc2_hi = (float)geom.rc2 * (1.f + 0x1p-20f);
+    unsigned mask[kBrutePerWarp];
+#pragma unroll
+    for (int k = 0; k < kBrutePerWarp; ++k) {
+        const int i = c_lo + wid + k * kBruteWarps;
+        mask[k] = 0;
+        if (i < c_hi) {
+            const float4 pi = s_atom[i];
+            int count = 0;
+            for (int t = 0; 32 * t < n; ++t) {
+                const int j = 32 * t + lane;
+                const unsigned m = __ballot_sync(0xffffffffu, j < n && inside(geom, rc2_lo, rc2_hi, s_atom[j], pi.x, pi.y, pi.z));
+                if (lane == t) mask[k] = m;
+                count += __popc(m);
+            }
+            if (lane == 0) s_count[i - c_lo] = count;
+        }
+    }
+    __syncthreads();
+    // ---- first pair of every centre: exclusive scan over this CTA's centres, on top of the CTAs before it ----
+    if (wid == 0) {
+        constexpr int PER_LANE = kBrutePerCta / 32;
+        int v[PER_LANE], sum = 0;
+#pragma unroll
+        for (int k = 0; k < PER_LANE; ++k) { v[k] = s_count[lane * PER_LANE + k]; sum += v[k]; }
+        int at = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += y;
+        }
+        if (lane == 31) cta_total = at;
+        at -= sum;
+#pragma unroll
+        for (int k = 0; k < PER_LANE; ++k) { s_count[lane * PER_LANE + k] = at; at += v[k]; }
+    }
+    cluster.sync();
+    int before = 0, total = 0;
+    for (int r = 0; r < ctas; ++r) {
+        const int v = *cluster.map_shared_rank(&cta_total, r);
+        if (r < rank) before += v;
+        total += v;
+    }
+    cluster.sync();                                                          // nobody reads this CTA's shared memory any more
+    const bool fits = total <= pair_capacity;
+    if (rank == 0 && tid == 0) {
+        if (!fits) atomicOr(&counters->status, kStatusPairCapacity);
+        counters->n_pairs = total;
+        counters->n_rows = total + n;                                        // the neighbours and the centres themselves
+        row_ptr[n] = total + n;
+        if (host) { __threadfence(); *host = *counters; }                    // pinned host memory: the caller waits for the stream and reads it
+    }
+#pragma unroll
+    for (int k = 0; k < kBrutePerWarp; ++k) {
+        const int i = c_lo + wid + k * kBruteWarps;
+        if (i >= c_hi) continue;
+        const int base = before + s_count[i - c_lo];
+        int at = base, below = 0;
+        for (int t = 0; 32 * t < n; ++t) {
+            const unsigned m = __shfl_sync(0xffffffffu, mask[k], t);
+            const int j = 32 * t + lane;
+            if (fits && (m >> lane & 1)) {
+                const int q = at + __popc(m & ((1u << lane) - 1));
+                pair_key[q] = ((unsigned long long)j << 24) | 0x808080ull;
+                pair_row[q] = q - base + (j > i ? 1 : 0);                    // rows in atom order, the centre's own among them
+            }
+            at += __popc(m);
+            below += __popc(__ballot_sync(0xffffffffu, (m >> lane & 1) && j < i));
+        }
+        if (lane == 0) {
+            pair_start[i] = base;
+            pair_count[i] = fits ? at - base : 0;
+            row_ptr[i] = base + i;
+            self_row[i] = below;
+        }
+    }
+}
+
+// One cluster: exclusive scan of the row counts (rows of centre c start at row_ptr[c]), the totals to the host if it
+// asks for them, and the launch order of the per-centre kernel, largest pair count first (bins of 4 pairs, counting
+// sort), so that the long CTAs do not end up alone at the tail of the launch.  Every CTA takes a contiguous range of
+// centres; sums and bin counts of the others come from their shared memory.  Up to kRowsPerCta centres one CTA does it,
+// above that eight (36,000 centres: 46 us with one, 13 us with eight).
+constexpr int kSizeBins = 256, kSizeBinShift = 2;
+constexpr int kRowsCtas = 8, kRowsPerThread = 8, kRowsPerCta = 4096;
+__global__ void __launch_bounds__(1024)
+rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pair_count, int C,
+                  long long* __restrict__ row_ptr, int* __restrict__ order, Counters* counters, Counters* host) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ int warp_sums[32], cta_sum;
+    __shared__ int hist[kSizeBins], total[kSizeBins], first_slot[kSizeBins];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
+    grid_dependency_launch();
     if (tid < kSizeBins) hist[tid] = 0;
+    // a contiguous range per CTA, consecutive centres per thread
+    const int per_cta = (C + ctas - 1) / ctas, per_thread = (per_cta + 1023) / 1024;       // at most kRowsPerThread
+    const int c_hi = min(C, (rank + 1) * per_cta), i0 = rank * per_cta + tid * per_thread;
     grid_dependency_wait();                                                  // the counts of the pair kernel
     __syncthreads();
-    // four consecutive centres per thread and trip: a few thousand centres are one trip, four barriers
-    constexpr int kPerThread = 4;
-    for (long long base = 0; base < C; base += 1024 * kPerThread) {
-        const long long i0 = base + (long long)tid * kPerThread;
-        long long v[kPerThread], x = 0;
+    int v[kRowsPerThread], bin[kRowsPerThread], mine = 0;
 #pragma unroll
-        for (int k = 0; k < kPerThread; ++k) {
-            const long long i = i0 + k;
-            v[k] = i < C ? (long long)row_count[i] : 0;
-            if (i < C) atomicAdd(&hist[min(pair_count[i] >> kSizeBinShift, kSizeBins - 1)], 1);
-            x += v[k];
+    for (int k = 0; k < kRowsPerThread; ++k) {
+        v[k] = bin[k] = 0;
+        if (k < per_thread && i0 + k < c_hi) {
+            v[k] = row_count[i0 + k];
+            bin[k] = min(pair_count[i0 + k] >> kSizeBinShift, kSizeBins - 1);
+            atomicAdd(&hist[bin[k]], 1);
         }
-        const long long mine = x;
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) warp_sums[wid] = x;
-        __syncthreads();
-        if (wid == 0) {
-            long long sacc = warp_sums[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long y = __shfl_up_sync(0xffffffffu, sacc, o);
-                if (lane >= o) sacc += y;
-            }
-            warp_sums[lane] = sacc;
-        }
-        __syncthreads();
-        const long long carry = carry_s;
-        long long at = carry + (wid > 0 ? warp_sums[wid - 1] : 0) + x - mine;
-#pragma unroll
-        for (int k = 0; k < kPerThread; ++k) {
-            if (i0 + k < C) row_ptr[i0 + k] = at;
-            at += v[k];
-        }
-        __syncthreads();
-        if (tid == 1023) carry_s = carry + warp_sums[31];
-        __syncthreads();
+        mine += v[k];
     }
-    if (tid == 0) {
-        row_ptr[C] = carry_s;
-        counters->n_rows = carry_s;
-        if (host) *host = *counters;                     // pinned host memory: the caller waits for the stream and reads it
+    int incl = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_sums[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        int w = warp_sums[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        warp_sums[lane] = w;
+        if (lane == 31) cta_sum = w;
+    }
+    int before = 0;                                                          // centres of this thread's bin in the CTAs before this one
+    long long base = 0, rows = 0;                                            // rows of the CTAs before this one, of all
+    if (ctas > 1) {
+        cluster.sync();
+        if (tid < kSizeBins) {
+            int all = 0;
+            for (int r = 0; r < ctas; ++r) {
+                const int h = cluster.map_shared_rank(hist, r)[tid];
+                if (r < rank) before += h;
+                all += h;
+            }
+            total[tid] = all;
+        }
+        for (int r = 0; r < ctas; ++r) {
+            const int t = *cluster.map_shared_rank(&cta_sum, r);
+            if (r < rank) base += t;
+            rows += t;
+        }
+        cluster.sync();                                                      // (also: nobody reads this CTA's shared memory any more)
+    } else {
+        __syncthreads();
+        rows = cta_sum;
+    }
+    if (rank == 0 && tid == 1023) {
+        row_ptr[C] = rows;
+        counters->n_rows = rows;
+        if (host) *host = *counters;                                         // pinned host memory: the caller waits for the stream and reads it
     }
     if (wid == 0) {
         // first slot of every size bin, largest bin first: lane k scans the bins 255 - 8k down to 248 - 8k, a warp
         // scan adds what the lanes before it hold
         constexpr int per_lane = kSizeBins / 32;
+        const int* const count = ctas > 1 ? total : hist;
         const int top = kSizeBins - 1 - lane * per_lane;
-        int mine = 0;
-        for (int k = 0; k < per_lane; ++k) mine += hist[top - k];
-        int incl = mine;
+        int sum = 0;
+        for (int k = 0; k < per_lane; ++k) sum += count[top - k];
+        int at = sum;
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
+            const int y = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += y;
         }
-        int run = incl - mine;
-        for (int k = 0; k < per_lane; ++k) { first_slot[top - k] = run; run += hist[top - k]; }
+        int run = at - sum;
+        for (int k = 0; k < per_lane; ++k) { first_slot[top - k] = run; run += count[top - k]; }
     }
     __syncthreads();
-    if (order)
-        for (long long i = tid; i < C; i += 1024) {
-            const int b = min(pair_count[i] >> kSizeBinShift, kSizeBins - 1);
-            order[atomicAdd(&first_slot[b], 1)] = (int)i;
+    if (ctas > 1) {
+        if (tid < kSizeBins) first_slot[tid] += before;
+        __syncthreads();
+    }
+    long long at = base + (wid > 0 ? warp_sums[wid - 1] : 0) + incl - mine;
+#pragma unroll
+    for (int k = 0; k < kRowsPerThread; ++k) {
+        if (k < per_thread && i0 + k < c_hi) {
+            row_ptr[i0 + k] = at;
+            order[atomicAdd(&first_slot[bin[k]], 1)] = i0 + k;
         }
+        at += v[k];
+    }
 }
 
 // Compact copy of the pair list (the pair arrays are addressed by segment): one warp per centre.

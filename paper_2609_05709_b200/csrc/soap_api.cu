@@ -124,6 +124,7 @@ struct soap_handle {
     int64_t pairs_per_center_hint = 0;   // average at the last plan (chooses the pair kernel variant)
     int64_t last_centers = 0;
     bool list_sorted = false;            // whether the pair list of the last search is sorted (descriptor-only calls skip that)
+    bool ordered = false;                // whether the last search with rows left a launch order
     int64_t found_atoms = -1, found_centers = -1;   // sizes of the search soap_search left for soap_derivatives_found; -1: none
     int P_deriv = 16, P_outer = 16;      // pairs per staged chunk: derivative kernels, kernel of the outer average
     size_t smem_deriv = 0, smem_outer = 0;
@@ -291,7 +292,7 @@ int ensure_device(soap_t* h) {
     return SOAP_OK;
 }
 
-int ensure_scratch(soap_t* h, int64_t N, int64_t C, int64_t pairs) {
+int ensure_scratch(soap_t* h, int64_t N, int64_t C, int64_t pairs, cudaStream_t st) {
     if (N > h->cap_atoms || h->cap_atoms == 0) {
         int64_t cap = N + N / 8 + 256;
         CU(regrow(&h->d_species_idx, cap));
@@ -304,6 +305,7 @@ int ensure_scratch(soap_t* h, int64_t N, int64_t C, int64_t pairs) {
         CU(regrow(&h->d_cell_start, cells + 1));
         CU(regrow(&h->d_cell_tile_sums, cells / kScanTile + 2));
         CU(regrow(&h->d_cell_tile_offsets, cells / kScanTile + 3));
+        CU(cudaMemsetAsync(h->d_cell_count, 0, (cells + 1) * sizeof(int), st));      // zero between calls
         h->cap_cells = cells;
         h->cap_atoms = cap;
     }
@@ -356,18 +358,24 @@ struct Batch {
     const long long* struct_ptr = nullptr;
     int64_t n_structs = 0;
 };
-// A single small non-periodic structure with every atom a centre takes the same brute-force pair kernel (one
-// launch instead of the two that build and walk a cell list).
-constexpr int64_t kBruteForceAtoms = 512;
-
 int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g,
                      const int32_t* centers, const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st,
                      const Batch& batch = Batch(), bool rows = true, bool publish = false) {
     h->found_atoms = h->found_centers = -1;
     Counters* const host = publish ? h->h_counters : nullptr;
+    // A small non-periodic structure with every atom a centre is searched by brute force, without a cell list.
     // (C == N: the brute-force kernel writes the per-centre arrays for every atom, and those are sized from C)
     const bool brute = !batch.struct_ptr && !centers && !sites && C == N && N <= kBruteForceAtoms && !(g.pbc[0] | g.pbc[1] | g.pbc[2]);
-    if (batch.struct_ptr || brute) {
+    if (brute) {
+        // one launch of one cluster: no row scan, no launch order (these centres fit the device at once)
+        const int ctas = N <= kBrutePerCta / 2 ? 1 : N <= kBrutePerCta ? 2 : N <= 2 * kBrutePerCta ? 4 : kBruteCtas;
+        CU(launch_cluster(brute_kernel, ctas, kBruteThreads, st, false, pos, num, h->d_zlut, h->d_species_idx, (int)N, g, h->cap_pairs,
+                          h->d_pair_key, h->d_pair_row, h->d_pair_start, h->d_pair_count, h->d_self_row, row_ptr_out, h->d_counters, host));
+        h->ordered = false;
+        CU(cudaGetLastError());
+        return SOAP_OK;
+    }
+    if (batch.struct_ptr) {
         CU(cudaMemsetAsync(&h->d_counters->n_pairs, 0, 2 * sizeof(long long), st));      // pair cursor and row total
         if (N > 0) batch_pairs_kernel<<<(unsigned)((N + kFillWarps - 1) / kFillWarps), kFillWarps * 32, 0, st>>>(
             pos, num, h->d_zlut, h->d_species_idx, batch.struct_ptr, batch.n_structs, N, g.rc2, h->cap_pairs, h->d_pair_key,
@@ -376,11 +384,14 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
         small_prep_kernel<<<1, kPrepThreads, 0, st>>>(pos, num, N, g, h->d_zlut, h->d_species_idx, (int)h->cap_cells, h->d_grid,
                                                       h->d_atom_cell, h->d_atom_wrap, h->d_cell_count, h->d_cell_start,
                                                       h->d_s_pos, h->d_s_wrap, h->d_counters);
+    } else if (N <= kPrepAtoms) {
+        CU(launch_cluster(prep_kernel, kPrepCtas, kPrepThreads, st, false, pos, num, N, g, h->d_zlut, h->d_species_idx, (int)h->cap_cells,
+                          h->d_grid, h->d_atom_cell, h->d_atom_wrap, h->d_cell_count, h->d_cell_start, h->d_s_pos, h->d_s_wrap, h->d_counters));
     } else {
         CU(cudaMemsetAsync(h->d_bbox, 0, 64, st));
         CU(cudaMemsetAsync(h->d_cell_count, 0, (h->cap_cells + 1) * sizeof(int), st));
         species_bbox_kernel<<<blocks_for(N, 256, 1024), 256, 0, st>>>(pos, num, N, g, h->d_zlut, h->d_species_idx, h->d_bbox, h->d_counters);
-        grid_setup_kernel<<<1, 1, 0, st>>>(h->d_bbox, g, N, (int)h->cap_cells, h->d_grid, h->d_counters);
+        grid_setup_kernel<<<1, 32, 0, st>>>(h->d_bbox, g, N, (int)h->cap_cells, h->d_grid, h->d_counters);
         bin_count_kernel<<<blocks_for(N, 256), 256, 0, st>>>(pos, N, g, h->d_grid, h->d_atom_cell, h->d_atom_wrap, h->d_cell_count, h->d_counters);
         {
             // exclusive scan of the bin counts over the whole (zero-filled) capacity, tile by tile
@@ -391,7 +402,7 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
         }
         bin_fill_kernel<<<blocks_for(N, 256), 256, 0, st>>>(pos, N, h->d_atom_cell, h->d_atom_wrap, h->d_cell_start, h->d_cell_count, h->d_s_pos, h->d_s_wrap);
     }
-    if (C > 0 && !batch.struct_ptr && !brute) {
+    if (C > 0 && !batch.struct_ptr) {
         // few pairs per centre at the last plan: the variant with the small on-chip key buffers (more warps resident);
         // descriptor-only calls take the variants without sorting and row bookkeeping
         const bool small_keys = h->pairs_per_center_hint > 0 && h->pairs_per_center_hint <= kFillSmemKeysSmall * 3 / 4;
@@ -405,13 +416,15 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
         else CU(launch_dependent(pairs_kernel<kFillSmemKeys, false>, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
 #undef SOAP_PAIRS_ARGS
     }
-    if (!rows && !batch.struct_ptr && !brute) {
+    if (!rows) {
         // no Jacobian rows wanted: no row pointers, no launch order
         CU(cudaGetLastError());
         return SOAP_OK;
     }
-    if (C <= kOrderMaxCenters) {
-        CU(launch_dependent(rows_order_kernel, 1, 1024, 0, st, h->d_row_count, h->d_pair_count, C, row_ptr_out, h->d_order, h->d_counters, host));
+    h->ordered = C <= kOrderMaxCenters;
+    if (h->ordered) {
+        CU(launch_cluster(rows_order_kernel, C <= kRowsPerCta ? 1 : kRowsCtas, 1024, st, true, h->d_row_count, h->d_pair_count, (int)C, row_ptr_out, h->d_order,
+                          h->d_counters, host));
     } else {
         scan_counts(h, h->d_row_count, row_ptr_out, C, &h->d_counters->n_rows, st, h->d_counters, host);
     }
@@ -435,7 +448,7 @@ int check_inputs(soap_t* h, const float* pos, const int32_t* num, int64_t N, con
 // 3000 atoms with 274 neighbours each from 1712 to 1374 us.)
 int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g, const int32_t* centers,
                     const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st, const Batch& batch = Batch()) {
-    int rc = ensure_scratch(h, N, C, 0);
+    int rc = ensure_scratch(h, N, C, 0, st);
     if (rc) return rc;
     for (int attempt = 0; attempt < 2; ++attempt) {
         if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
@@ -450,7 +463,7 @@ int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, 
         }
         if (pairs <= h->cap_pairs) break;
         // the counts come out right even when the pairs do not fit
-        if ((rc = ensure_scratch(h, N, C, pairs + pairs / 4 + 1024))) return rc;
+        if ((rc = ensure_scratch(h, N, C, pairs + pairs / 4 + 1024, st))) return rc;
     }
     h->list_sorted = true;
     h->last_centers = C;
@@ -461,7 +474,7 @@ int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, 
 
 void fill_center_params(soap_t* h, CenterParams& cp, const float* pos, const int32_t* centers, int64_t C,
                         const Geometry& g, bool deriv, const float* sites = nullptr) {
-    cp.pos = pos; cp.centers = centers; cp.sites = sites; cp.order = C <= kOrderMaxCenters ? h->d_order : nullptr; cp.species_idx = h->d_species_idx; cp.n_centers = C; cp.geom = g;
+    cp.pos = pos; cp.centers = centers; cp.sites = sites; cp.order = h->ordered ? h->d_order : nullptr; cp.species_idx = h->d_species_idx; cp.n_centers = C; cp.geom = g;
     cp.pair_start = h->d_pair_start; cp.pair_count = h->d_pair_count; cp.pair_key = h->d_pair_key; cp.pair_row = h->d_pair_row;
     cp.row_ptr = h->d_row_ptr; cp.self_row = h->d_self_row;
     cp.pair_capacity = h->cap_pairs; cp.row_capacity = 0; cp.counters = h->d_counters;
@@ -1272,7 +1285,7 @@ int soap_neighbor_counts_static(const float* d_positions, int64_t n_atoms, doubl
     if ((e = cudaMemsetAsync(base, 0, StaticLayout::header, st)) != cudaSuccess) return say(SOAP_ERR_CUDA, cudaGetErrorString(e));
     if ((e = cudaMemsetAsync(cell_count, 0, sizeof(int) * (kStaticMaxCells + 1), st)) != cudaSuccess) return say(SOAP_ERR_CUDA, cudaGetErrorString(e));
     bbox_only_kernel<<<blocks_for(N, 256, 256), 256, 0, st>>>(d_positions, N, g, bbox);
-    grid_setup_kernel<<<1, 1, 0, st>>>(bbox, g, N, kStaticMaxCells, grid, nullptr);
+    grid_setup_kernel<<<1, 32, 0, st>>>(bbox, g, N, kStaticMaxCells, grid, nullptr);
     bin_count_kernel<<<blocks_for(N, 256), 256, 0, st>>>(d_positions, N, g, grid, atom_cell, atom_wrap, cell_count, counters);
     scan_kernel<int><<<1, 1024, 0, st>>>(cell_count, cell_start, kStaticMaxCells, nullptr, &grid->n_cells);
     bin_fill_kernel<<<blocks_for(N, 256), 256, 0, st>>>(d_positions, N, atom_cell, atom_wrap, cell_start, cell_count, s_pos, s_wrap);

@@ -29,7 +29,7 @@ def into(soap, pos, num, cell, c, rows):
     return out
 
 
-# the brute-force search (up to 512 atoms), the single-CTA cell list (up to 16384) and the tiled one
+# the brute-force search (up to 512 atoms) and the cell lists of one CTA (up to 4096), of a cluster and of many launches
 @pytest.mark.parametrize("molecules", [1, 8, 171, 400, 5600])
 def test_sized_call_equals_the_call_into_buffers(pkg, molecules):
     s = water_cluster(molecules, 1)
@@ -88,3 +88,49 @@ def test_derivatives_of_a_search_need_that_search(pkg):
     soap.descriptor(pos, num, s.cell)                      # a call in between
     with pytest.raises(pkg.SoapError):
         found(60)
+
+
+def all_pairs(pos, r_cut):
+    """(pair_ptr, pair_atom) of a non-periodic structure: a k-d tree in fp64, neighbours in atom order."""
+    from scipy.spatial import cKDTree
+    x = pos.astype(np.float64)
+    lists = cKDTree(x).query_ball_point(x, r_cut, return_sorted=True)
+    lists = [[j for j in l if j != i] for i, l in enumerate(lists)]
+    return np.concatenate([[0], np.cumsum([len(l) for l in lists])]), np.array([j for l in lists for j in l], np.int64)
+
+
+def check_search(pkg, pos, r_cut):
+    ptr, atom = all_pairs(pos, r_cut)
+    soap = pkg.Soap([1], r_cut, 1, 0, 0.5)
+    p, num = torch.from_numpy(pos).cuda(), torch.ones(len(pos), dtype=torch.int32, device="cuda")
+    for _ in range(2):                                       # the second call knows how many pairs a centre has
+        got_ptr, got_atom, _ = soap.neighbor_list(p, num)
+        assert np.array_equal(got_ptr.cpu().numpy(), ptr) and np.array_equal(got_atom.cpu().numpy(), atom)
+        d = soap.derivatives(p, num)
+        assert np.array_equal(d.row_ptr.cpu().numpy(), ptr + np.arange(len(pos) + 1))
+        row_atom = d.row_atom.cpu().numpy()
+        for i in (0, len(pos) // 2, len(pos) - 1):
+            a, b = ptr[i] + i, ptr[i + 1] + i + 1
+            assert np.array_equal(row_atom[a:b], np.sort(np.append(atom[ptr[i]:ptr[i + 1]], i)))
+
+
+# one, two, four and eight CTAs of the brute-force search; one CTA, a cluster and many launches for the cell list;
+# one CTA and a cluster for the row pointers, and the tiled scan
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 65, 127, 129, 255, 257, 511, 512, 513, 4095, 4096, 4097, 8193, 65536, 65537])
+def test_sizes_at_which_the_search_changes(pkg, n):
+    rng = np.random.default_rng(n)
+    edge = (n / 0.6) ** (1 / 3)
+    check_search(pkg, (rng.random((n, 3)) * edge).astype(np.float32), 1.7)
+
+
+@pytest.mark.parametrize("n_ball,spread", [(100, 1), (128, 1), (129, 40), (300, 150), (512, 1), (513, 90), (300, 100000)])
+def test_sort_of_a_centre_s_pairs(pkg, n_ball, spread):
+    """Neighbours whose indices are consecutive, evenly spread, or crowded at one end of a long range."""
+    rng = np.random.default_rng(spread)
+    n = max(20000, n_ball * min(spread, 150) + 1)
+    pos = (rng.random((n, 3)) * 1000.0 + 50.0).astype(np.float32)
+    ids = np.arange(n_ball) * (spread if spread <= 150 else 1)
+    if spread > 150:
+        ids[-1] = n - 1
+    pos[ids] = (rng.random((n_ball, 3)) * 1.0).astype(np.float32)
+    check_search(pkg, pos, 2.5)
