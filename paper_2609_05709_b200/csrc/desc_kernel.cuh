@@ -6,10 +6,11 @@
 //   * the radial table (value polynomials, re-laid as [interval][l][n / 2][6][2]) sits in shared memory
 //     once per CTA when it fits; a lane evaluates two adjacent n at once from three conflict-free 16-byte
 //     loads and five packed multiply-adds (fma.rn.f32x2: one issue slot for two multiply-adds);
-//   * the pairs of a centre (up to 64 at a time) have their geometry formed in registers, are ranked by species with ballots, and staged 16 at a time in
-//     species order: solid
-//     harmonics with a lane per pair from the fully unrolled Q_l^m recursion, radial factors with
-//     lanes on the channels (l, n);
+//   * the pairs of a centre (up to 64 at a time) have their geometry formed in registers, are ranked by species with
+//     ballots, and staged 16 or 32 at a time in species order: solid harmonics with a lane per pair from the fully
+//     unrolled Q_l^m recursion, radial factors with the lanes side by side on the list of all (pair, two channels) of
+//     the chunk (a round per pair left half of the lanes idle at l_max 3: 324,000 atoms at (4, 3) 2.03 -> 1.47 ms,
+//     215,000 at (6, 4) 2.90 -> 2.33 ms, with the chunks of 32);
 //   * accumulation c[l,m][n] += S_lm G_nl is register-tiled: a lane owns four consecutive m of one l
 //     times all n (an outer product of 4 x n_max per pair from one 16-byte load of S and n_max/4 of
 //     G); with at most 16 such tiles the two half-warps work on two pairs at once.  Sums stay in
@@ -17,16 +18,17 @@
 //     once per species; the staging rows are laid out so that all these loads are conflict-free;
 //   * Eq. 4 is the Gram matrix of that tile per l: lanes take 4 x 4 blocks of (species, n) pairs,
 //     two 16-byte loads per 16 multiply-adds, and the feature row is put together in shared memory
-//     and written out in order.
+//     and handed to the copy engine.
+// At (8, 6) on 30,000 atoms the kernel takes 246 us; the shared-memory pipe is 77 % busy, the issue slots 57 %.
 // Nothing but the pair list is read from HBM and nothing but the descriptor row is written.
 #pragma once
 #include "soap_device.cuh"
 
 namespace soap {
 
-constexpr int kDescChunk = 16;                    // pairs staged at once by a warp
 constexpr int kDescGroup = 64;                    // pairs whose geometry a warp holds in registers (two per lane)
 constexpr int kDescMaxWarps = 16;                 // warps per CTA (one CTA per SM)
+constexpr int kDescTeamWarps = 4;                 // most warps of a CTA that works on one centre
 
 // harmonic normalisation up to l = 12, filled by desc_constants(): a_lm (sqrt2 folded in for m > 0), index l(l+1)/2 + m
 __device__ __constant__ float kd_norm[91] = {0};
@@ -50,30 +52,47 @@ __host__ __device__ constexpr int desc_s_row(int l_max) { return 4 * (desc_tiles
 __host__ __device__ constexpr int desc_g_l(int np) { return np == 16 ? 20 : np; }
 __host__ __device__ constexpr int desc_g_swap(int np, int l) { return np == 8 ? (l >> 2) & 1 : 0; }
 
-// 16-byte chunks per row of the centre's coefficient tile c[lm][species, n]: S NP / 4 rounded up to a power of two.
-// Chunk k of row r sits at position (k + r / 4) mod that number, so that the lanes of a warp, which own rows four
-// apart, do not all hit one group of banks when they store their sums.
-__host__ __device__ constexpr int desc_c_chunks(int S, int np) {
-    int rc = 1;
-    while (rc < S * np / 4) rc <<= 1;
-    return rc;
-}
+// The centre's coefficient tile c[lm][species, n]: S NP / 4 16-byte chunks per row, and one more chunk of room after every
+// four rows: the lanes of a warp, which own rows four apart, then do not all hit one group of banks when they store
+// their sums.
+__host__ __device__ constexpr int desc_c_at(int row, int row_chunks) { return row * row_chunks + (row >> 2); }
+__host__ __device__ constexpr int desc_c_words(int S, int np, int lm) { return 4 * (desc_c_at(lm - 1, S * np / 4) + S * np / 4); }
 
-// Shared memory in 4-byte words: [table (optional)] then one region per warp:
-//   c [LM][4 desc_c_chunks] | S staging [chunk][s_row] | G staging [chunk][L1 g_l] | pair staging [chunk][8 or 5]
+// Pairs staged at once by a warp: 32 where a staged pair is small, so that every lane has a pair's harmonics to form
+// (80 words: sixteen warps still fit beside the table for two species), else 16; a team deals its chunks out to its warps
+// and takes 16.
+__host__ __device__ constexpr int desc_chunk(int l_max, int np, bool team) { return !team && desc_s_row(l_max) + (l_max + 1) * desc_g_l(np) <= 80 ? 32 : 16; }
+
+// Blocks of 4 x 4 (species, n) pairs that Eq. 4 is computed in, and whether their places in the feature row are decoded
+// once per CTA into a table (few blocks: up to S n_max = 32) or by every lane for every centre
+__host__ __device__ constexpr int desc_blocks(int S, int np, bool crossover) {
+    const int ta = S * np / 4, tb = np / 4;
+    return crossover ? ta * (ta + 1) / 2 : S * (tb * (tb + 1) / 2);
+}
+constexpr int kDescTableBlocks = 36;
+struct DescBlock {
+    int rowoff[4];             // row i of the block starts at this feature (+ j (l_max+1) + l)
+    int ta, tb;                // its column tiles
+    unsigned valid;            // bit 4 i + j: whether (i, j) is a feature (n below n_max, n' >= n inside a diagonal species block)
+    int pad;
+};
+
+// Shared memory in 4-byte words: [table (optional)] [block table (few blocks)] then one region per warp:
+//   c [LM] rows | S staging [chunk][s_row] | G staging [chunk][L1 g_l] | pair staging [chunk][8 or 5]
 // The feature row is assembled on top of the staging area when it fits there.  With the table in shared memory (the
 // plain build on many centres) a staged pair is five words (dx, dy, dz, t; interval | species << 16) instead of
 // eight (dx, dy, dz, r; interval, t, species, weight): at the benchmark's basis that is what lets a 16th warp fit.
 struct DescLayout {
-    int table, warp0, per_warp, c, sS, sG, ring, slab_words, total;
+    int table, blocks, warp0, per_warp, c, sS, sG, ring, slab_words, total;
 };
-__host__ __device__ inline DescLayout make_desc_layout(int S, int np, int l_max, int warps, int table_words) {
-    const int L1 = l_max + 1, LM = L1 * L1;
+__host__ __device__ inline DescLayout make_desc_layout(int S, int np, int l_max, int warps, int table_words, bool team) {
+    const int L1 = l_max + 1, LM = L1 * L1, n_blocks = desc_blocks(S, np, true), kDescChunk = desc_chunk(l_max, np, team);
     DescLayout o;
     o.table = 0;
-    o.warp0 = (table_words + 3) & ~3;
+    o.blocks = (table_words + 3) & ~3;
+    o.warp0 = o.blocks + (n_blocks <= kDescTableBlocks ? n_blocks * (int)(sizeof(DescBlock) / 4) : 0);
     int off = 0;
-    o.c = off; off += LM * 4 * desc_c_chunks(S, np);
+    o.c = off; off += desc_c_words(S, np, LM);
     o.sS = off; off += kDescChunk * desc_s_row(l_max);
     o.sG = off; off += kDescChunk * L1 * desc_g_l(np);
     o.ring = off; off += kDescChunk * (table_words ? 5 : 8);
@@ -128,8 +147,10 @@ __device__ __forceinline__ void harmonics_tiles(float x, float y, float z, float
 
 // NP: n_max rounded up to a multiple of four.  PLAIN: the default configuration (atom centres, no weighting, every
 // species pair, power spectrum out).  TS: the radial table is in shared memory.
-template <int L, int NP, bool PLAIN, bool TS>
-__global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const CenterParams p) {
+// TEAM: few centres, a CTA per centre: its warps take the chunks of pairs in turn, each into a tile of its own, and the
+// tiles are added up; the blocks of Eq. 4 are spread over all of them.
+template <int L, int NP, bool PLAIN, bool TS, bool TEAM>
+__global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 32, TEAM ? 16 / kDescTeamWarps : 1) desc_kernel(const CenterParams p) {
     constexpr int L1 = L + 1, LM = L1 * L1;
     constexpr int NCHP = L1 * NP;                                        // channels (l, n), n padded
     constexpr int SROW = desc_s_row(L), GL = desc_g_l(NP), GROW = L1 * GL;
@@ -138,7 +159,8 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
     constexpr int TPL = (T + LANES_T - 1) / LANES_T;                     // tiles per lane (1, or 2 from l_max = 10 on)
     constexpr int NB = (TPL * NP * 4 <= 64) ? NP : 64 / (4 * TPL);      // n handled per pass (at most 64 accumulators)
     constexpr int NPASS = (NP + NB - 1) / NB;
-    constexpr int CPAIRS = NCHP / 2, ROUNDS = (CPAIRS + 31) / 32;       // lanes take pairs of adjacent n
+    constexpr int CPAIRS = NCHP / 2;                                     // channel pairs: two adjacent n of one l
+    constexpr int kDescChunk = desc_chunk(L, NP, TEAM);
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const bool o_cross = PLAIN || p.crossover, o_emit = !PLAIN && p.emit_coeff;
@@ -147,31 +169,69 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
     const float2* const o_pw = PLAIN ? nullptr : p.pair_w;
     const float o_w0 = PLAIN ? 1.f : p.w0;
     const int S = p.S, NMAX = p.n_max, F = p.F;
-    const DescLayout lay = make_desc_layout(S, NP, L, warps, TS ? p.n_intervals * NCHP * 6 : 0);
+    const DescLayout lay = make_desc_layout(S, NP, L, warps, TS ? p.n_intervals * NCHP * 6 : 0, TEAM);
 
     if (TS) {
         const float4* src = reinterpret_cast<const float4*>(p.table_ln);
         float4* dst = reinterpret_cast<float4*>(smem);
         const int n4 = p.n_intervals * NCHP * 6 / 4;
         for (int e = threadIdx.x; e < n4; e += blockDim.x) dst[e] = __ldg(src + e);
+        if (desc_blocks(S, NP, true) > kDescTableBlocks) __syncthreads();
+    }
+    // ---- the blocks of Eq. 4: where they lie in the tile and in the feature row (the same for every l and centre) ----
+    constexpr int TB = NP / 4;                                           // 4-wide column tiles per species
+    const int TA = S * TB, NTP = desc_blocks(S, NP, o_cross);
+    const bool tabled = desc_blocks(S, NP, true) <= kDescTableBlocks;
+    DescBlock* const blocks = reinterpret_cast<DescBlock*>(smem + lay.blocks);
+    auto decode_block = [&](int rem) {
+        DescBlock o;
+        int ta = 0, tb;
+        if (o_cross) {
+            while (rem >= TA - ta) { rem -= TA - ta; ++ta; }
+            tb = ta + rem;
+        } else {
+            const int sb = rem / (TB * (TB + 1) / 2);
+            rem -= sb * (TB * (TB + 1) / 2);
+            while (rem >= TB - ta) { rem -= TB - ta; ++ta; }
+            tb = sb * TB + ta + rem;
+            ta += sb * TB;
+        }
+        const int TRI = (NMAX * (NMAX + 1) / 2) * L1, SQ = NMAX * NMAX * L1;
+        const int mu = (4 * ta) / NP, nu = (4 * tb) / NP, na = 4 * ta - mu * NP, nb = 4 * tb - nu * NP;
+        const int before = o_cross ? mu * S - mu * (mu - 1) / 2 + (nu - mu) : mu, diag = o_cross ? mu + (nu > mu ? 1 : 0) : mu;
+        const int base = diag * TRI + (before - diag) * SQ;
+        o.ta = ta; o.tb = tb; o.valid = 0; o.pad = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int n1 = na + i;
+            o.rowoff[i] = base + (mu < nu ? n1 * NMAX + nb : n1 * NMAX - n1 * (n1 - 1) / 2 - n1 + nb) * L1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (n1 < NMAX && nb + j < NMAX && (mu < nu || n1 <= nb + j)) o.valid |= 1u << (4 * i + j);
+        }
+        return o;
+    };
+    if (tabled) {
+        if ((int)threadIdx.x < NTP) blocks[threadIdx.x] = decode_block(threadIdx.x);
+        if ((int)blockDim.x < NTP)
+            for (int e = threadIdx.x + blockDim.x; e < NTP; e += blockDim.x) blocks[e] = decode_block(e);
         __syncthreads();
     }
-    // the table is this handle's own; everything below reads what the kernels before this one wrote
+    // the tables are this handle's own; everything below reads what the kernels before this one wrote
     grid_dependency_wait();
     // a failed neighbour build: write nothing
     if (p.counters->n_pairs > p.pair_capacity) return;
 
     float* const wbase = smem + lay.warp0 + wid * lay.per_warp;
-    float* const c_t = wbase + lay.c;                                               // [LM][4 RC], chunks rotated by row / 4
-    const int RC = desc_c_chunks(S, NP), rc_mask = RC - 1;
-    auto c_chunk = [&](int r, int k) { return r * RC + ((k + (r >> 2)) & rc_mask); };        // 16-byte chunk k of row r
+    float* const c_t = wbase + lay.c;                                               // [LM] rows of RC chunks, skewed
+    const int RC = S * NP / 4;
+    auto c_chunk = [&](int r, int k) { return desc_c_at(r, RC) + k; };              // 16-byte chunk k of row r
     auto c_word = [&](int r, int col) { return 4 * c_chunk(r, col >> 2) + (col & 3); };
     float4* const sS4 = reinterpret_cast<float4*>(wbase + lay.sS);                  // [chunk][SROW / 4] tiles of four m
     float* const sG = wbase + lay.sG;                                               // [chunk][L1][GL]
     float4* const ring_d = reinterpret_cast<float4*>(wbase + lay.ring);             // [chunk] dx, dy, dz, r
     int4* const ring_i = reinterpret_cast<int4*>(wbase + lay.ring + 4 * kDescChunk);// [chunk] interval, t, species, weight
     int* const ring_q = reinterpret_cast<int*>(wbase + lay.ring + 4 * kDescChunk);  // TS: [chunk] interval | species << 16, and t in ring_d.w
-    float* const slab = wbase + lay.sS;
     const float4* const tab = TS ? reinterpret_cast<const float4*>(smem) : reinterpret_cast<const float4*>(p.table_ln);
 
     // the tiles of this lane: l, tile index, first row (l^2 + 4 j) and number of valid rows
@@ -185,14 +245,11 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
         while (t >= (2 * l + 4) / 4) { t -= (2 * l + 4) / 4; ++l; }
         t_l[tp] = l; t_lm0[tp] = l * l + 4 * t; t_kv[tp] = min(4, 2 * l + 1 - 4 * t);
     }
-    // where this lane puts the radial factors it evaluates: the channel pair cp = l NP/2 + n/2 of round rr goes to
-    // words l GL + n, l GL + n + 1
-    int g_word[ROUNDS];
-#pragma unroll
-    for (int rr = 0; rr < ROUNDS; ++rr) {
-        const int cp = rr * 32 + lane, l = cp / (NP / 2), n = 2 * (cp - l * (NP / 2));
-        g_word[rr] = l * GL + 4 * ((n >> 2) ^ desc_g_swap(NP, l)) + (n & 3);
-    }
+    // where the radial factors of the channel pair cp = l NP/2 + n/2 go in a pair's staging row: words l GL + n, l GL + n + 1
+    auto g_word = [](int cp) {
+        const int l = cp / (NP / 2);
+        return (2 * cp + l * (GL - NP)) ^ (4 * desc_g_swap(NP, l));
+    };
     const bool periodic = p.geom.pbc[0] | p.geom.pbc[1] | p.geom.pbc[2];
     const long long n_work = o_cbar ? 1 : p.n_centers;
 
@@ -231,18 +288,21 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
         }
     };
     // Full rounds give every warp of the grid one centre, CTA by CTA; the centres of the last, partial round are
-    // dealt out across the CTAs first, so that every SM gets its share of them instead of a few SMs a full round
-    const long long w_stride = (long long)gridDim.x * warps, full_rounds = n_work / w_stride;
+    // dealt out across the CTAs first, so that every SM gets its share of them instead of a few SMs a full round.
+    // (A team: the CTA's own centre.)
+    auto wait_row = []() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); };   // this thread's row copies have read the slab
+    const long long w_stride = TEAM ? gridDim.x : (long long)gridDim.x * warps, full_rounds = n_work / w_stride;
     for (long long round = 0; round <= full_rounds; ++round) {
-        const long long c_idx = round * w_stride + (round < full_rounds ? (long long)blockIdx.x * warps + wid
-                                                                         : (long long)wid * gridDim.x + blockIdx.x);
+        const long long c_idx = TEAM ? round * w_stride + blockIdx.x
+                                     : round * w_stride + (round < full_rounds ? (long long)blockIdx.x * warps + wid
+                                                                               : (long long)wid * gridDim.x + blockIdx.x);
         if (c_idx >= n_work) break;
         const Head hd = load_head(c_idx);
         Raw raw;
         const float xi = hd.xi, yi = hd.yi, zi = hd.zi;
         const int zi_species = hd.zsp, k_pairs = hd.k_pairs;
 
-        for (int e = lane; e < LM * RC; e += 32) reinterpret_cast<float4*>(c_t)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e = lane; e < desc_c_at(LM - 1, RC) + RC; e += 32) reinterpret_cast<float4*>(c_t)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
 
         for (int g0 = 0; g0 < k_pairs; g0 += kDescGroup) {
@@ -272,8 +332,12 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
                         dy += sh[0] * p.geom.cell[1] + sh[1] * p.geom.cell[4] + sh[2] * p.geom.cell[7];
                         dz += sh[0] * p.geom.cell[2] + sh[1] * p.geom.cell[5] + sh[2] * p.geom.cell[8];
                     }
-                    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-                    // interval and offset in the radial table, in fp64 so that the offset keeps its digits
+                    // interval and offset in the radial table, in fp64 so that the offset keeps its digits: r is the fp32
+                    // root r0 (relative error 2^-23) and one Newton step on it, whose residual is formed in fp64 and
+                    // whose own error is 2^-47
+                    const double d2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                    const float r0 = sqrtf(fmaxf((float)d2, 1e-30f));
+                    const double r = (double)r0 + (double)((float)fma(-(double)r0, (double)r0, d2) * __fdividef(0.5f, r0));
                     const double u = r * p.inv_h;
                     const int qi = min((int)u, p.n_intervals - 1);
                     dd[b] = make_float4((float)dx, (float)dy, (float)dz, (float)r);
@@ -292,9 +356,16 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
                     }
             }
 
+            if (!TEAM) {
+                if (lane == 0) wait_row();                                   // the row of the centre before has left the staging area
+                __syncwarp();
+            }
 #pragma unroll 1
             for (int ip = 0; ip < NPASS; ++ip) {
                 const int n0 = ip * NB;
+                // Packed multiply-adds take two products at once: (h_k g_n, h_k+1 g_n+1) into acc[..][k][n/2] and, with the two
+                // h swapped, (h_k+1 g_n, h_k g_n+1) into acc[..][k+1][n/2] (k even): two swaps per tile instead of four copies
+                // of an h into both halves of a register pair
                 float2 acc[TPL][4][NB / 2];
 #pragma unroll
                 for (int tp = 0; tp < TPL; ++tp)
@@ -302,24 +373,32 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
                     for (int k = 0; k < 4; ++k)
 #pragma unroll
                         for (int n = 0; n < NB / 2; ++n) acc[tp][k][n] = make_float2(0.f, 0.f);
+                auto sum_of = [&](int tp, int k, int n) {
+                    const float2 even = acc[tp][k & ~1][n / 2], odd = acc[tp][k | 1][n / 2];
+                    return (k & 1) == (n & 1) ? ((n & 1) ? even.y : even.x) : ((n & 1) ? odd.y : odd.x);
+                };
                 int cur = -1;
                 const bool single = k_pairs <= kDescGroup;            // one group: every (row, species) is written once
 
                 // sums of species s (columns n0 .. n0 + NB - 1) are added to the centre's tile; the two half-warps add up first
                 auto flush = [&](int s) {
 #pragma unroll
-                    for (int tp = 0; tp < TPL; ++tp)
+                    for (int tp = 0; tp < TPL; ++tp) {
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
+                        for (int k2 = 0; k2 < (HALVES == 2 ? 2 : 4); ++k2) {
+                            // (with two half-warps a lane keeps rows 0, 1 or rows 2, 3 of the tile and sends the others)
                             float v[NB];
 #pragma unroll
                             for (int n = 0; n < NB; ++n) {
-                                v[n] = (n & 1) ? acc[tp][k][n / 2].y : acc[tp][k][n / 2].x;
-                                if (HALVES == 2) v[n] += __shfl_xor_sync(0xffffffffu, v[n], 16);
+                                if (HALVES == 2) {
+                                    const float low = sum_of(tp, k2, n), high = sum_of(tp, k2 + 2, n);
+                                    v[n] = (half ? high : low) + __shfl_xor_sync(0xffffffffu, half ? low : high, 16);
+                                } else {
+                                    v[n] = sum_of(tp, k2, n);
+                                }
                             }
-#pragma unroll
-                            for (int n = 0; n < NB / 2; ++n) acc[tp][k][n] = make_float2(0.f, 0.f);
-                            if (k < t_kv[tp] && (HALVES == 1 || (k >> 1) == half)) {
+                            const int k = HALVES == 2 ? k2 + 2 * half : k2;
+                            if (k < t_kv[tp]) {
                                 float4* const c4w = reinterpret_cast<float4*>(c_t);
                                 const int r = t_lm0[tp] + k, k0 = (s * NP + n0) / 4;
 #pragma unroll
@@ -335,9 +414,14 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
                                     }
                             }
                         }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+#pragma unroll
+                            for (int n = 0; n < NB / 2; ++n) acc[tp][k][n] = make_float2(0.f, 0.f);
+                    }
                 };
 
-                for (int c0 = 0; c0 < kg; c0 += kDescChunk) {
+                for (int c0 = TEAM ? wid * kDescChunk : 0; c0 < kg; c0 += TEAM ? warps * kDescChunk : kDescChunk) {
                     const int n_stage = min(kDescChunk, kg - c0);
                     // the pairs at sorted positions c0 .. c0 + 15 go to the staging slots
 #pragma unroll
@@ -357,31 +441,29 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
                         const float4 d = ring_d[lane];
                         harmonics_tiles<L>(d.x, d.y, d.z, TS ? fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)) : d.w * d.w, sS4 + lane * (SROW / 4));
                     }
-                    // radial factors: lanes on the channels, pairs in turn
+                    // radial factors: the lanes walk down the (pair, channel pair) list side by side, a warp's width at a time
+                    {
+                        int pr = lane / CPAIRS, cp = lane - pr * CPAIRS;
 #pragma unroll 4
-                    for (int pr = 0; pr < n_stage; ++pr) {
-                        int4 gi;
-                        if (TS) { gi = make_int4(ring_q[pr] & 0xffff, __float_as_int(ring_d[pr].w), 0, 0); }
-                        else gi = ring_i[pr];
-                        const float t = __int_as_float(gi.y);
-                        const float2 tt = make_float2(t, t);
-                        const float4* row = tab + (size_t)gi.x * (NCHP * 6 / 4);
-#pragma unroll
-                        for (int rr = 0; rr < ROUNDS; ++rr) {
-                            const int cp = rr * 32 + lane;
-                            if (ROUNDS * 32 == CPAIRS || cp < CPAIRS) {
-                                // coefficients of t^0 .. t^5 of two adjacent n, interleaved: (c0, c0', c1, c1'), (c2, c2', c3, c3'), (c4, c4', c5, c5')
-                                const float4 A = TS ? row[cp * 3] : __ldg(row + cp * 3);
-                                const float4 B = TS ? row[cp * 3 + 1] : __ldg(row + cp * 3 + 1);
-                                const float4 C = TS ? row[cp * 3 + 2] : __ldg(row + cp * 3 + 2);
-                                float2 v = __ffma2_rn(make_float2(C.z, C.w), tt, make_float2(C.x, C.y));
-                                v = __ffma2_rn(v, tt, make_float2(B.z, B.w));
-                                v = __ffma2_rn(v, tt, make_float2(B.x, B.y));
-                                v = __ffma2_rn(v, tt, make_float2(A.z, A.w));
-                                v = __ffma2_rn(v, tt, make_float2(A.x, A.y));
-                                if (!PLAIN) { const float wgt = __int_as_float(gi.w); v.x *= wgt; v.y *= wgt; }
-                                *reinterpret_cast<float2*>(sG + pr * GROW + g_word[rr]) = v;
-                            }
+                        for (int e = lane; e < n_stage * CPAIRS; e += 32) {
+                            int4 gi;
+                            if (TS) { gi = make_int4(ring_q[pr] & 0xffff, __float_as_int(ring_d[pr].w), 0, 0); }
+                            else gi = ring_i[pr];
+                            const float t = __int_as_float(gi.y);
+                            const float2 tt = make_float2(t, t);
+                            // coefficients of t^0 .. t^5 of two adjacent n, interleaved: (c0, c0', c1, c1'), (c2, c2', c3, c3'), (c4, c4', c5, c5')
+                            const float4* row = tab + (unsigned)(gi.x * CPAIRS + cp) * 3u;
+                            const float4 A = TS ? row[0] : __ldg(row), B = TS ? row[1] : __ldg(row + 1), C = TS ? row[2] : __ldg(row + 2);
+                            float2 v = __ffma2_rn(make_float2(C.z, C.w), tt, make_float2(C.x, C.y));
+                            v = __ffma2_rn(v, tt, make_float2(B.z, B.w));
+                            v = __ffma2_rn(v, tt, make_float2(B.x, B.y));
+                            v = __ffma2_rn(v, tt, make_float2(A.z, A.w));
+                            v = __ffma2_rn(v, tt, make_float2(A.x, A.y));
+                            if (!PLAIN) { const float wgt = __int_as_float(gi.w); v.x *= wgt; v.y *= wgt; }
+                            *reinterpret_cast<float2*>(sG + pr * GROW + g_word(cp)) = v;
+                            // 32 further down the list
+                            pr += 32 / CPAIRS; cp += 32 % CPAIRS;
+                            if (cp >= CPAIRS) { cp -= CPAIRS; ++pr; }
                         }
                     }
                     __syncwarp();
@@ -401,8 +483,8 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
 #pragma unroll
                             for (int tp = 0; tp < TPL; ++tp) {
                                 const float4 h4 = sp4[t_idx[tp]];
-                                const float2 h[4] = {make_float2(h4.x, h4.x), make_float2(h4.y, h4.y), make_float2(h4.z, h4.z),
-                                                     make_float2(h4.w, h4.w)};
+                                const float2 h[4] = {make_float2(h4.x, h4.y), make_float2(h4.y, h4.x), make_float2(h4.z, h4.w),
+                                                     make_float2(h4.w, h4.z)};
 #pragma unroll
                                 for (int n4 = 0; n4 < NB / 4; ++n4) {
                                     if (NPASS > 1 && n0 + 4 * n4 >= NP) break;
@@ -423,8 +505,26 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
             }
         }
 
+        if (!TEAM && k_pairs == 0) {
+            if (lane == 0) wait_row();
+            __syncwarp();
+        }
+        float4* const sum4 = reinterpret_cast<float4*>(TEAM ? smem + lay.warp0 + lay.c : c_t);       // the tile of the centre
+        if (TEAM) {
+            // the tiles of the team add up in the first warp's, in a fixed order
+            __syncthreads();
+            for (int e = threadIdx.x; e < desc_c_at(LM - 1, RC) + RC; e += blockDim.x) {
+                float4 v = sum4[e];
+                for (int w = 1; w < warps; ++w) {
+                    const float4 o = sum4[e + w * (lay.per_warp / 4)];
+                    v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+                }
+                sum4[e] = v;
+            }
+            __syncthreads();
+        }
         // on-site term: the centre's own Gaussian, l = 0 only (second term of Eq. 13)
-        if (!o_cbar && !o_sites && lane < NMAX) c_t[c_word(0, zi_species * NP + lane)] += o_w0 * __ldg(p.self_term + lane);
+        if ((!TEAM || wid == 0) && !o_cbar && !o_sites && lane < NMAX) c_t[c_word(0, zi_species * NP + lane)] += o_w0 * __ldg(p.self_term + lane);
         if (o_cbar) {
             // given mean coefficients (inner average) take the place of the centre's own: index (mu n_max + n) LM + lm
             for (int e = lane; e < S * NMAX * LM; e += 32) {
@@ -432,102 +532,92 @@ __global__ void __launch_bounds__(kDescMaxWarps * 32, 1) desc_kernel(const Cente
                 c_t[c_word(lm, mu * NP + n)] = __ldg(o_cbar + e);
             }
         }
-        __syncwarp();
+        if (TEAM) __syncthreads(); else __syncwarp();
         if (o_emit) {
             // coefficient mode: the tile itself is the result, index (mu n_max + n) (l_max+1)^2 + l^2 + l + m
             float* crow = p.out_desc + (size_t)c_idx * (S * NMAX * LM);
-            for (int e = lane; e < S * NMAX * LM; e += 32) {
+            const float* const tile = reinterpret_cast<const float*>(sum4);
+            for (int e = TEAM ? (int)threadIdx.x : lane; e < S * NMAX * LM; e += TEAM ? (int)blockDim.x : 32) {
                 const int row = e / LM, lm = e - row * LM, mu = row / NMAX, n = row - mu * NMAX;
-                crow[e] = c_t[c_word(lm, mu * NP + n)];
+                crow[e] = tile[c_word(lm, mu * NP + n)];
             }
-            __syncwarp();
+            if (TEAM) __syncthreads(); else __syncwarp();
             continue;
         }
 
         // ---- power spectrum (Eq. 4): per l the Gram matrix of the tile's rows over (species, n) ----
         float* const desc_row = p.out_desc + (o_cbar ? (size_t)0 : (size_t)c_idx * F);
         const bool staged = F <= lay.slab_words;
+        float* const slab = TEAM ? smem + lay.warp0 + lay.sS : wbase + lay.sS;
         float* const dst = staged ? slab : desc_row;
         // Lanes take blocks of 4 x 4 (species, n) pairs (ta <= tb in units of four columns); a block's place in the
-        // feature row does not depend on l, so it is decoded once, and the lanes then walk down the l (with few
-        // blocks, several l side by side: group g of the lanes takes l = l_max - g, l_max - g - G, ...).
-        constexpr int TB = NP / 4;                                   // 4-wide column tiles per species
-        const int TA = S * TB;
-        const int NTP = o_cross ? TA * (TA + 1) / 2 : S * (TB * (TB + 1) / 2);
-        const int G = NTP <= 16 ? 32 / NTP : 1;                      // l's side by side
-        const int TRI = (NMAX * (NMAX + 1) / 2) * L1, SQ = NMAX * NMAX * L1;
-        const float4* const c4 = reinterpret_cast<const float4*>(c_t);
-        for (int tp0 = 0; tp0 < NTP; tp0 += 32) {
-            const int grp = G > 1 ? lane / NTP : 0;
-            int rem = G > 1 ? lane - grp * NTP : tp0 + lane;
+        // feature row does not depend on l, and the lanes walk down the l (with few blocks, several l side by side:
+        // group g of the lanes takes l = l_max - g, l_max - g - G, ...).
+        const int lanes = TEAM ? (int)blockDim.x : 32, me = TEAM ? (int)threadIdx.x : lane;
+        const int G = 2 * NTP <= lanes ? min(lanes / NTP, L1) : 1;   // l's side by side
+        for (int tp0 = 0; tp0 < NTP; tp0 += lanes) {
+            const int grp = G > 1 ? me / NTP : 0, rem = G > 1 ? me - grp * NTP : tp0 + me;
             const bool active = grp < G && rem < NTP;
-            if (!active) rem = 0;
-            int ta = 0, tb = 0;
-            if (o_cross) {
-                while (rem >= TA - ta) { rem -= TA - ta; ++ta; }
-                tb = ta + rem;
-            } else {
-                const int sb = rem / (TB * (TB + 1) / 2);
-                rem -= sb * (TB * (TB + 1) / 2);
-                while (rem >= TB - ta) { rem -= TB - ta; ++ta; }
-                tb = sb * TB + ta + rem;
-                ta += sb * TB;
-            }
-            // row i of the block starts at feature offset rowoff[i] (+ j (l_max+1) + l); bit 4 i + j of `valid` says
-            // whether (i, j) is a feature at all (n below n_max, and n' >= n inside a diagonal species block)
-            const int mu = (4 * ta) / NP, nu = (4 * tb) / NP, na = 4 * ta - mu * NP, nb = 4 * tb - nu * NP;
-            int rowoff[4];
-            unsigned valid = 0;
-            {
-                const int before = o_cross ? mu * S - mu * (mu - 1) / 2 + (nu - mu) : mu, diag = o_cross ? mu + (nu > mu ? 1 : 0) : mu;
-                const int base = diag * TRI + (before - diag) * SQ;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int n1 = na + i;
-                    rowoff[i] = base + (mu < nu ? n1 * NMAX + nb : n1 * NMAX - n1 * (n1 - 1) / 2 - n1 + nb) * L1;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (active && n1 < NMAX && nb + j < NMAX && (mu < nu || n1 <= nb + j)) valid |= 1u << (4 * i + j);
-                }
-            }
+            const DescBlock blk = tabled ? blocks[active ? rem : 0] : decode_block(active ? rem : 0);
+            const unsigned valid = active ? blk.valid : 0u;
             for (int l0 = L; l0 >= 0; l0 -= G) {
                 const int l = l0 - grp;                                // this lane's l (may fall below zero in the last trip)
                 const int steps = (active && l >= 0) ? 2 * l + 1 : 0;
+                // sums of (a_i b_j, a_i+1 b_j+1) in g[i][j / 2] and, with the two b swapped, (a_i b_j+1, a_i+1 b_j) in
+                // g[i + 1][j / 2] (i, j even)
                 float2 g[4][2];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) g[i][0] = g[i][1] = make_float2(0.f, 0.f);
-                const int r0 = l >= 0 ? l * l : 0;
-                for (int m = 0; m < steps; ++m) {
-                    const float4 A = c4[c_chunk(r0 + m, ta)];
-                    const float4 B = c4[c_chunk(r0 + m, tb)];
-                    const float2 b01 = make_float2(B.x, B.y), b23 = make_float2(B.z, B.w);
-                    const float av[4] = {A.x, A.y, A.z, A.w};
+                int r = l >= 0 ? l * l : 0;
+                const float4 *pa = sum4 + blk.ta, *pb = sum4 + blk.tb;
+                for (int m = 0; m < steps; ++m, ++r) {
+                    const int at = desc_c_at(r, RC);
+                    const float4 A = pa[at], B = pb[at];
+                    const float2 a01 = make_float2(A.x, A.y), a23 = make_float2(A.z, A.w);
+                    const float2 b[2] = {make_float2(B.x, B.y), make_float2(B.z, B.w)}, bs[2] = {make_float2(B.y, B.x), make_float2(B.w, B.z)};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 aa = make_float2(av[i], av[i]);
-                        g[i][0] = __ffma2_rn(aa, b01, g[i][0]);
-                        g[i][1] = __ffma2_rn(aa, b23, g[i][1]);
+                    for (int j = 0; j < 2; ++j) {
+                        g[0][j] = __ffma2_rn(a01, b[j], g[0][j]);
+                        g[1][j] = __ffma2_rn(a01, bs[j], g[1][j]);
+                        g[2][j] = __ffma2_rn(a23, b[j], g[2][j]);
+                        g[3][j] = __ffma2_rn(a23, bs[j], g[3][j]);
                     }
                 }
                 if (steps) {
                     const float kl = __ldg(p.kl + l);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        float* o = dst + rowoff[i] + l;
-                        if (valid & (1u << (4 * i))) o[0] = kl * g[i][0].x;
-                        if (valid & (2u << (4 * i))) o[L1] = kl * g[i][0].y;
-                        if (valid & (4u << (4 * i))) o[2 * L1] = kl * g[i][1].x;
-                        if (valid & (8u << (4 * i))) o[3 * L1] = kl * g[i][1].y;
+                        float* o = dst + blk.rowoff[i] + l;
+                        // (i, j): the even rows of a pair sit in the first halves
+                        const float2 u = g[i & 2][0], us = g[(i & 2) + 1][0], w = g[i & 2][1], ws = g[(i & 2) + 1][1];
+                        const float v[4] = {(i & 1) ? us.y : u.x, (i & 1) ? u.y : us.x, (i & 1) ? ws.y : w.x, (i & 1) ? w.y : ws.x};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (valid & (1u << (4 * i + j))) o[j * L1] = kl * v[j];
                     }
                 }
             }
         }
-        __syncwarp();
+        if (TEAM) __syncthreads(); else __syncwarp();
         if (staged) {
-            for (int e = lane; e < F; e += 32) desc_row[e] = slab[e];
-            __syncwarp();
+            // the copy engine takes the row where its place allows that (16-byte boundaries); the slab is not written
+            // again before the copy has read it
+            if ((F & 3) == 0 && (reinterpret_cast<size_t>(p.out_desc) & 15) == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                if (TEAM) __syncthreads(); else __syncwarp();
+                if (me == 0) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                                 :: "l"(desc_row), "r"((unsigned)__cvta_generic_to_shared(slab)), "r"(4u * (unsigned)F) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    if (TEAM) wait_row();
+                }
+            } else {
+                for (int e = me; e < F; e += lanes) desc_row[e] = slab[e];
+            }
+            if (TEAM) __syncthreads(); else __syncwarp();
         }
     }
+    if (!TEAM && lane == 0) wait_row();                                      // the slab must outlive the copies that read it
 }
 
 }  // namespace soap

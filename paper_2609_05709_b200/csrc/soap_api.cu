@@ -64,10 +64,10 @@ cudaError_t desc_set_smem(int l_max, int np, int bytes) {
     }
     return cudaErrorInvalidValue;
 }
-cudaError_t desc_launch(int l_max, int np, bool plain, bool table_in_smem, const CenterParams& p, unsigned grid, unsigned block,
+cudaError_t desc_launch(int l_max, int np, bool plain, bool table_in_smem, bool team, const CenterParams& p, unsigned grid, unsigned block,
                         size_t smem, cudaStream_t st) {
     switch (l_max) {
-#define X(LV) case LV: return desc_launch_l##LV(np, plain, table_in_smem, p, grid, block, smem, st);
+#define X(LV) case LV: return desc_launch_l##LV(np, plain, table_in_smem, team, p, grid, block, smem, st);
         X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
 #undef X
     }
@@ -200,7 +200,7 @@ int plan_smem(soap_t* h) {
     int max_smem = 0;
     CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     h->max_smem = max_smem;
-    h->desc_warp_bytes = (size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0).per_warp * 4;
+    h->desc_warp_bytes = (size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0, false).per_warp * 4;
     if (h->desc_warp_bytes > (size_t)max_smem) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
     CU(desc_set_smem(h->l_max, desc_np(h->n_max), max_smem));
     // pairs per staged chunk of the derivative kernels: the largest that still leaves room for three CTAs per SM,
@@ -490,24 +490,37 @@ void fill_center_params(soap_t* h, CenterParams& cp, const float* pos, const int
 
 // Launch of the descriptor-only kernel: persistent CTAs (one per SM) whose warps take the centres in turn.
 // The radial table goes to shared memory when it leaves room for at least six warps and there is enough
-// work to pay for staging it; small jobs use fewer warps per CTA so that they spread over the SMs.
+// work to pay for staging it; small jobs use fewer warps per CTA so that they spread over the SMs, the smallest
+// several warps per centre.
 int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     if (n_work <= 0) return SOAP_OK;
     cp.table_ln = h->d_table_ln;
     cp.inv_h = h->basis.inv_h_values; cp.n_intervals = h->basis.n_intervals_values;      // the value table has intervals of its own
     const bool plain = center_params_plain(cp);
-    const int warps_fit = (int)std::min<size_t>(kDescMaxWarps, (size_t)h->max_smem / h->desc_warp_bytes);
+    // Few centres: a team of warps per centre, four if the CTAs then run side by side in one wave (four of them fit an
+    // SM's registers), else two (eight; up to five centres per SM: beyond that a warp per centre is the faster one on half
+    // of the sizes).  Whole calls, (n_max, l_max) = (8, 6): 120 atoms 27 -> 17 us, 431 atoms of four species 66 -> 38 us,
+    // 600 atoms 31.2 -> 29.2 us; (12, 8), 600 atoms 60 -> 43 us.
+    for (const int team_warps : {kDescTeamWarps, 2}) {
+        const size_t bytes = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, team_warps, 0, true).total * 4;
+        const int64_t per_sm = std::min<int64_t>(team_warps == 2 ? 5 : 16 / kDescTeamWarps, (int64_t)(228 * 1024 / (bytes + 1024)));
+        if (n_work > per_sm * h->sm_count || bytes > (size_t)h->max_smem) continue;
+        CU(desc_launch(h->l_max, h->desc_np, plain, false, true, cp, (unsigned)n_work, (unsigned)team_warps * 32, bytes, st));
+        return SOAP_OK;
+    }
+    const size_t fixed = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, 1, 0, false).warp0 * 4;
+    const int warps_fit = (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed) / h->desc_warp_bytes);
     // (with the table in shared memory a warp's region is a little smaller: its staged pairs are five words, not eight)
-    const size_t table_pad = (h->desc_table_bytes + 15) & ~(size_t)15;
-    const size_t warp_bytes_ts = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, 1, (int)(h->desc_table_bytes / 4)).per_warp * 4;
-    const int warps_ts = h->desc_table_bytes > 0 && table_pad + warp_bytes_ts <= (size_t)h->max_smem
-                             ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - table_pad) / warp_bytes_ts) : 0;
+    const DescLayout with_table = make_desc_layout(h->S, h->desc_np, h->l_max, 1, (int)(h->desc_table_bytes / 4), false);
+    const size_t fixed_ts = (size_t)with_table.warp0 * 4, warp_bytes_ts = (size_t)with_table.per_warp * 4;
+    const int warps_ts = h->desc_table_bytes > 0 && fixed_ts + warp_bytes_ts <= (size_t)h->max_smem
+                             ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed_ts) / warp_bytes_ts) : 0;
     const bool ts = plain && warps_ts >= 6 && n_work >= (int64_t)4 * h->sm_count;
     int warps = ts ? warps_ts : warps_fit;
     warps = (int)std::max<int64_t>(1, std::min<int64_t>(warps, (n_work + h->sm_count - 1) / h->sm_count));
     const unsigned grid = (unsigned)std::min<int64_t>(h->sm_count, (n_work + warps - 1) / warps);
-    const size_t smem = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, warps, ts ? (int)(h->desc_table_bytes / 4) : 0).total * 4;
-    CU(desc_launch(h->l_max, h->desc_np, plain, ts, cp, grid, (unsigned)warps * 32, smem, st));
+    const size_t smem = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, warps, ts ? (int)(h->desc_table_bytes / 4) : 0, false).total * 4;
+    CU(desc_launch(h->l_max, h->desc_np, plain, ts, false, cp, grid, (unsigned)warps * 32, smem, st));
     return SOAP_OK;
 }
 

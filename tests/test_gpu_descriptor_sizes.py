@@ -1,0 +1,77 @@
+"""The descriptor kernel where its dispatch changes: teams of four and of two warps per centre, a warp per centre, the
+table in shared memory; chunks of 16 and of 32 pairs; feature rows that the copy engine takes and rows that it cannot."""
+import numpy as np
+import pytest
+
+from oracle.soap import GTO, SoapOracle
+from soap_inputs import multispecies_box, water_cluster
+from test_gpu_parity import DESC_TOL
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_05709_b200 as p
+    return p
+
+
+def col_err(a, ref):
+    """Largest error over the column's largest magnitude, which counts as 1e-3 of the output's largest entry at least: the
+    bound include/soap.h states for few centres, whose columns can all be small at once."""
+    a = np.asarray(a, np.float64)
+    return float((np.abs(a - ref).max(axis=0) / np.maximum(np.abs(ref).max(axis=0), 1e-3 * np.abs(ref).max())).max())
+
+
+def check(pkg, s, args, sample, centers=None):
+    soap, oracle = pkg.Soap(*args), SoapOracle(*args)
+    pos, num = torch.from_numpy(s.positions).cuda(), torch.from_numpy(s.numbers).cuda()
+    cen = None if centers is None else torch.tensor(centers, dtype=torch.int32, device="cuda")
+    got = soap.descriptor(pos, num, s.cell, cen)
+    soap.status()
+    of = [k if centers is None else centers[k] for k in sample]
+    ref = oracle.descriptor(s.positions, s.numbers, s.cell, of)
+    assert bool(torch.isfinite(got).all())
+    assert col_err(got[list(sample)].cpu().numpy(), ref) < DESC_TOL
+    return got
+
+
+# with 148 SMs: up to 592 centres a team of four, up to 740 a team of two, then a warp per centre
+@pytest.mark.parametrize("n_centers", [1, 147, 592, 593, 740, 741, 1200])
+@pytest.mark.parametrize("n_max,l_max", [(8, 6), (3, 2), (5, 4), (12, 7)])
+def test_centre_counts(pkg, n_centers, n_max, l_max):
+    s = water_cluster(400, 1)
+    args = ([1, 8], 5.0, n_max, l_max, 0.5, GTO)
+    rng = np.random.default_rng(n_centers)
+    centers = rng.permutation(s.n_atoms)[:n_centers].tolist()
+    sample = sorted({0, n_centers // 3, n_centers // 2, n_centers - 1})
+    a = check(pkg, s, args, sample, centers)
+    full = check(pkg, s, args, [0, 600, 1199])
+    # one row by different kernels: sums in another order
+    scale = full.abs().max(dim=0).values.clamp_min(1e-3 * float(full.abs().max()))
+    assert float(((a - full[centers]).abs() / scale).max()) < DESC_TOL
+
+
+@pytest.mark.parametrize("n_species", [1, 3, 8])
+@pytest.mark.parametrize("n_max,l_max", [(1, 0), (4, 1), (7, 3), (8, 4), (4, 8), (13, 2), (2, 12)])
+def test_bases_and_species_counts(pkg, n_species, n_max, l_max):
+    """Tiles of one to eight species (three: a tile whose rows are no power of two), more blocks than the table of blocks holds."""
+    s = multispecies_box(60, 2)
+    species = [1, 6, 7, 8, 9, 14, 16, 17][:n_species]
+    s.numbers = np.random.default_rng(1).choice(species, size=s.n_atoms).astype(np.int32)
+    args = (species, 4.0, n_max, l_max, 0.5, GTO, (True, True, True))
+    check(pkg, s, args, [0, 17, 59])
+
+
+def test_centres_with_no_one_few_and_very_many_neighbours(pkg):
+    """A lone atom, a pair, and several groups of 64 pairs in one call, on many and on few centres."""
+    rng = np.random.default_rng(0)
+    for n_ball in (150, 800):
+        s = water_cluster(1, 0)
+        ball = rng.random((n_ball, 3)) * 2.2
+        s.positions = np.concatenate([ball, [[50, 0, 0], [80, 0, 0], [81, 0, 0]]]).astype(np.float32)
+        s.numbers = rng.choice([1, 8], size=n_ball + 3).astype(np.int32)
+        check(pkg, s, ([1, 8], 4.0, 6, 5, 0.5, GTO), [0, n_ball - 1, n_ball, n_ball + 1, n_ball + 2])
