@@ -9,9 +9,10 @@
 //   grad_j c^Z_nlm  = G_nl grad S_lm + Ghat_nl d S_lm,  Ghat = G'/|d|  (Eq. 14 / 23)
 // with S_lm = r^l Y_lm the real solid harmonic and G_nl, G'_nl read from the
 // degree-5 tables.
-//   Staging (whole CTA, a chunk of up to 32 pairs): radial factors with a warp per
-//   pair and lanes on channels; solid harmonics with lanes on pairs and warps on
-//   the columns m of the recursion, so that control flow is uniform.
+//   Staging (whole CTA, a chunk of up to 32 pairs, 96 for small bases): radial factors
+//   with the threads side by side on the list of (pair, two channels); solid harmonics
+//   with lanes on pairs and warps on the columns m of the recursion, so that control
+//   flow is uniform.
 //   Pass 1 accumulates c and D = sum_j grad_j c with thread-owned elements; the
 //   centre's own Jacobian row is minus the sum over its neighbours (translation
 //   invariance, text below Eq. 5), which is a contraction of D with c.
@@ -38,18 +39,17 @@ __device__ __constant__ float2 kc_norm[91] = {0};    // [(l,m)] a_lm = sqrt((2l+
 __device__ __constant__ float4 kc_step[91] = {0};    // [(l,m)] coefficients that advance columns m and m+1 from l to l+1
 __device__ __constant__ float kc_dfact[16] = {0};    // [m] (2m-1)!!
 
-// Degree-5 table lookup: value and derivative with respect to the interval coordinate t.
-__device__ __forceinline__ void radial_lookup(const float* __restrict__ table, int qi, int n_ch, int ch, float t,
-                                              float& v, float& dv) {
-    // 32-bit index arithmetic: the table has at most 4096 x 208 x 6 floats
-    const float2* cf = reinterpret_cast<const float2*>(table) + (unsigned)(qi * n_ch + ch) * 3u;
-    const float2 a = __ldg(cf), b = __ldg(cf + 1), c = __ldg(cf + 2);
-    v = c.y; dv = 0.f;
-    dv = fmaf(dv, t, v); v = fmaf(v, t, c.x);
-    dv = fmaf(dv, t, v); v = fmaf(v, t, b.y);
-    dv = fmaf(dv, t, v); v = fmaf(v, t, b.x);
-    dv = fmaf(dv, t, v); v = fmaf(v, t, a.y);
-    dv = fmaf(dv, t, v); v = fmaf(v, t, a.x);
+// Degree-5 table lookup of two adjacent n of one l, whose coefficients lie interleaved: values and derivatives with
+// respect to the interval coordinate t, by packed multiply-adds.
+__device__ __forceinline__ void radial_lookup2(const float4* __restrict__ cf, float t, float2& v, float2& dv) {
+    const float4 a = __ldg(cf), b = __ldg(cf + 1), c = __ldg(cf + 2);             // (c0, c0', c1, c1'), (c2, ..), (c4, c4', c5, c5')
+    const float2 tt = make_float2(t, t);
+    dv = make_float2(c.z, c.w);
+    v = __ffma2_rn(dv, tt, make_float2(c.x, c.y));
+    dv = __ffma2_rn(dv, tt, v); v = __ffma2_rn(v, tt, make_float2(b.z, b.w));
+    dv = __ffma2_rn(dv, tt, v); v = __ffma2_rn(v, tt, make_float2(b.x, b.y));
+    dv = __ffma2_rn(dv, tt, v); v = __ffma2_rn(v, tt, make_float2(a.z, a.w));
+    dv = __ffma2_rn(dv, tt, v); v = __ffma2_rn(v, tt, make_float2(a.x, a.y));
 }
 
 // Real solid harmonics of one pair per lane, one column m of
@@ -106,6 +106,7 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 // (every atom a centre; given the coefficients of all centres; one row per atom, no per-pair rows).
 // PLAIN: the default configuration (every species pair, atom centres, no weighting, full rows, own
 // coefficients); the options are then compile-time constants and their code drops out.
+// The CTA has 256 threads, or 128 for small bases on many centres (KIND 1 and 2; launch_deriv in soap_api.cu has the rule).
 template <int KIND, int L, int NMAX_T, bool PLAIN>
 __global__ void __launch_bounds__(kThreads, kMinCtas)
 center_kernel(const CenterParams p) {
@@ -121,39 +122,50 @@ center_kernel(const CenterParams p) {
     const float o_scale = o_atom_rows ? p.own_scale : 1.f;
     constexpr int L1 = L + 1, LM = L1 * L1, LMP = LM | 1;      // odd row stride: no shared-memory bank conflicts
     constexpr int NMAX_BOUND = NMAX_T ? NMAX_T : 16;
-    // pass-1 ownership: W_LM warps cover the lm index, SLOTS such groups split the n index
-    constexpr int W_LM = (LM + 31) / 32;
-    constexpr int SLOTS_FULL = kWarps / W_LM, SLOT_DIV = 2;
-    constexpr int SLOTS = SLOTS_FULL / SLOT_DIV > 0 ? SLOTS_FULL / SLOT_DIV : 1;
+    // pass-1 ownership: LM_SPAN threads cover the lm index (half a warp or less when that is enough), SLOTS such groups split
+    // the n index.  Fewer groups mean fewer instructions in all (the harmonics of a pair are read once per group), more of
+    // them shorter chains; at most 8 functions per thread, so that one trip over the pairs does (a second trip stages
+    // everything again: at l_max 8 to 10 two groups instead of one are 1.14 to 1.19 times faster with n_max 9 to 12, 1.03 to
+    // 1.07 times with 6 to 8)
+    constexpr int LM_SPAN = pass1_span(L), SLOTS = pass1_slots(L, NMAX_BOUND);
     constexpr int NPT_RAW = (NMAX_BOUND + SLOTS - 1) / SLOTS;      // radial functions per thread ...
     constexpr int NPT = NPT_RAW < 8 ? NPT_RAW : 8;                // ... at most 8 at a time (register budget)
     extern __shared__ __align__(16) float smem[];
+    const int threads = KIND <= 2 ? (int)blockDim.x : kThreads, warps = threads >> 5;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int S = p.S, NMAX = NMAX_T ? NMAX_T : p.n_max, NCH = NMAX * L1, NE = NMAX * LM;
     const int CT = S * NMAX * LMP, P = p.P, F = p.F;
-    const SmemLayout lay = make_layout(S, NMAX, L, P, true, o_pw != nullptr);
+    const SmemLayout lay = make_layout(S, NMAX, L, P, warps, o_pw != nullptr);
+    constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
+    // words pairs (G, Ghat) per staged pair: the channels, and with a row table a zero behind them
+    constexpr bool kRowTable = KIND == 1 && NMAX_T != 0 && row_table_wanted(NMAX_T, L);
+    const int GP = NCH + (row_table_wanted(NMAX, L) ? 1 : 0);
+    const int CP = NMAX_T ? CP_T : (NMAX + 1) / 2 * L1;                     // channel pairs: (l, two adjacent n)
     float* c_t = smem + lay.c;                                             // [S][NMAX][LMP]
-    float4* geo_d = reinterpret_cast<float4*>(smem + lay.geo);             // [GP] dx, dy, dz, r
+    float4* geo_d = reinterpret_cast<float4*>(smem + lay.geo);             // [GP] dx, dy, dz, (table intervals per A) / r
     int4* geo_i = reinterpret_cast<int4*>(smem + lay.geo + 4 * kGeoPairs);   // [GP] interval, t bits, species|moving<<8, row word
     int* geo_j = reinterpret_cast<int*>(smem + lay.geo + 8 * kGeoPairs);     // [GP] neighbour atom
     float2* geo_w = reinterpret_cast<float2*>(smem + lay.geo + kGeoWords);   // [GP] (w, w'/d), only with a radial weighting
     float* D_t = smem + lay.D;                                             // [3][CT]    (pass 1 and the centre's row)
     float4* sSD4 = reinterpret_cast<float4*>(smem + lay.sSD);              // [P][LMP]   (S, dSx, dSy, dSz)
-    float2* sG2 = reinterpret_cast<float2*>(smem + lay.sG);                // [P][NCH]   (G, Ghat)
+    float2* sG2 = reinterpret_cast<float2*>(smem + lay.sG);                // [P][GP]    (G, Ghat)
 
     // ---- set-up that needs nothing from the kernels before this one (it may run while they finish) ----
-    for (int e = tid; e < CT * 4; e += kThreads) {
+    for (int e = tid; e < CT * 4; e += threads) {
         if (e < CT) c_t[e] = 0.f; else D_t[e - CT] = 0.f;
     }
     // zeros for the bulk copies of pass 2 (made visible to the copy engine; the barriers of pass 1 order them)
     const float* zero_buf = smem + lay.zero;
-    for (int e = tid; e < kZeroWords; e += kThreads) smem[lay.zero + e] = 0.f;
+    const int zero_w = zero_words(S, NMAX, L);
+    for (int e = tid; e < zero_w; e += threads) smem[lay.zero + e] = 0.f;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (kRowTable)
+        for (int e = tid; e < P; e += threads) sG2[e * GP + NCH] = make_float2(0.f, 0.f);
 
     // same-species blocks: feature index -> (n1 L1 + l) | (n2 L1 + l) << 8, rows n1 of (NMAX - n1) L1 entries
     unsigned short* tri_dec = reinterpret_cast<unsigned short*>(smem + lay.tri);
     if (!CC)
-        for (int e = tid; e < (NMAX * (NMAX + 1) / 2) * L1; e += kThreads) {
+        for (int e = tid; e < (NMAX * (NMAX + 1) / 2) * L1; e += threads) {
             int n1 = 0, r = e;
             while (r >= (NMAX - n1) * L1) { r -= (NMAX - n1) * L1; ++n1; }
             const int n2 = n1 + r / L1, l = r % L1;
@@ -165,7 +177,7 @@ center_kernel(const CenterParams p) {
     constexpr bool kCrossTable = KIND != 2 && NMAX_T > 8 && NMAX_T <= 12 && ((NMAX_BOUND * L1) & 3) != 0;
     unsigned short* x_dec = reinterpret_cast<unsigned short*>(smem + lay.xdec);
     if (kCrossTable && S > 1)
-        for (int e = tid; e < NMAX * NCH; e += kThreads) {
+        for (int e = tid; e < NMAX * NCH; e += threads) {
             const int n1 = e / NCH, j = e - n1 * NCH;
             x_dec[e] = (unsigned short)((n1 * L1 + j % L1) | (j << 8));
         }
@@ -192,7 +204,7 @@ center_kernel(const CenterParams p) {
     const int geo_batch = geo_batches > 1 ? min(kGeoPairs, (((k_pairs + geo_batches - 1) / geo_batches) + 7) & ~7) : kGeoPairs;
 
     // pass-1 ownership of this thread: one lm, and the radial functions slot, slot + SLOTS, ...
-    const int own_slot = wid / W_LM, own_lm = (wid - own_slot * W_LM) * 32 + lane;
+    const int own_slot = tid / LM_SPAN, own_lm = tid % LM_SPAN;
     const bool owner = own_slot < SLOTS && own_lm < LM;
     const int own_l = owner ? __ldg(p.l_of_lm + own_lm) : 0;
 
@@ -201,7 +213,7 @@ center_kernel(const CenterParams p) {
     //      are the pairs of species s.  Returns whether any pair of the batch shares its row with
     //      another or is an image of the centre ----
     int* seg = reinterpret_cast<int*>(smem + lay.geo + 9 * kGeoPairs);       // [kMaxSpecies + 1]
-    int* seg_warp = seg + kMaxSpecies + 1;                                   // [4 warps][kMaxSpecies]
+    int* seg_warp = seg + kMaxSpecies + 1;                                   // [warps][kMaxSpecies]
     auto stage_geometry = [&](int g0, int gc) -> bool {
         int special = 0, sp = -1, rank = 0, rw = 0, j = 0;
         float4 dd = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -223,7 +235,7 @@ center_kernel(const CenterParams p) {
                     dz += s[0] * p.geom.cell[2] + s[1] * p.geom.cell[5] + s[2] * p.geom.cell[8];
                 }
                 const double r = sqrt(dx * dx + dy * dy + dz * dz);
-                dd = make_float4((float)dx, (float)dy, (float)dz, (float)r);
+                dd = make_float4((float)dx, (float)dy, (float)dz, (float)p.inv_h / (float)r);
                 rw = p.pair_row[pair_base + g0 + tid];
                 if (o_pw) wgt = o_pw[pair_base + g0 + tid];
                 special = rw & (kRowSelfImage | kRowContinuation);
@@ -261,45 +273,45 @@ center_kernel(const CenterParams p) {
         return any_special;
     };
 
+    // ---- radial factors of channel pair cp of the staged pair g, to the staging row `to` ----
+    auto stage_radial = [&](int g, int cp, float2* to) {
+        const int4 gi = geo_i[g];
+        const float rinv_h = geo_d[g].w;
+        const int l = NMAX_T ? cp / ((NMAX_T + 1) / 2) : cp / ((NMAX + 1) / 2), n = 2 * (cp - l * ((NMAX + 1) / 2));
+        float2 v, dv;
+        radial_lookup2(reinterpret_cast<const float4*>(p.table) + (unsigned)(gi.x * CP + cp) * 3u, __int_as_float(gi.y), v, dv);
+        float2 lo = make_float2(v.x, dv.x * rinv_h), hi = make_float2(v.y, dv.y * rinv_h);
+        if (o_pw) {
+            // radial weighting: G -> w G, Ghat -> w Ghat + (w'/d) G
+            const float2 w = geo_w[g];
+            lo = make_float2(v.x * w.x, fmaf(lo.y, w.x, v.x * w.y));
+            hi = make_float2(v.y * w.x, fmaf(hi.y, w.x, v.y * w.y));
+        }
+        to[n * L1 + l] = lo;
+        if ((NMAX_T != 0 && (NMAX_T & 1) == 0) || n + 1 < NMAX) to[(n + 1) * L1 + l] = hi;
+    };
+    auto harmonics_of = [&](int g, int m, float4* to) {
+        const float4 d = geo_d[g];
+        harmonics_column(L, m, d.x, d.y, d.z, fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)), to);
+    };
     // ---- radial factors and solid harmonics of the pairs g .. g + pc - 1 of the staged geometry ----
     auto stage_chunk = [&](int g, int pc) {
-        for (int pr = wid; pr < pc; pr += kWarps) {
-            const int4 gi = geo_i[g + pr];
-            const float t = __int_as_float(gi.y);
-            const float rinv_h = (float)p.inv_h / geo_d[g + pr].w;
-            if (o_pw) {
-                // radial weighting: G -> w G, Ghat -> w Ghat + (w'/d) G
-                const float2 w = geo_w[g + pr];
-                for (int ch = lane; ch < NCH; ch += 32) {
-                    float v, dv;
-                    radial_lookup(p.table, gi.x, NCH, ch, t, v, dv);
-                    sG2[pr * NCH + ch] = make_float2(v * w.x, fmaf(dv * rinv_h, w.x, v * w.y));
-                }
-                continue;
-            }
-            for (int ch = lane; ch < NCH; ch += 32) {
-                float v, dv;
-                radial_lookup(p.table, gi.x, NCH, ch, t, v, dv);
-                sG2[pr * NCH + ch] = make_float2(v, dv * rinv_h);
-            }
+        // the threads side by side on the list of all (pair, channel pair): no lane is idle, whatever the basis
+        for (int e = tid; e < pc * CP; e += threads) {
+            const int pr = NMAX_T ? e / CP_T : e / CP;
+            stage_radial(g + pr, e - pr * CP, sG2 + pr * GP);
         }
         if (P >= 32) {
             // a warp per column: m is the same for all its lanes, so the recursion's coefficients are uniform reads
-            if (lane < pc) {
-                const float4 d = geo_d[g + lane];
-                for (int m = wid; m <= L; m += kWarps)
-                    harmonics_column(L, m, d.x, d.y, d.z, d.w * d.w, sSD4 + lane * LMP);
-            }
+            for (int m = wid; m <= L; m += warps)
+                for (int pr = lane; pr < pc; pr += 32) harmonics_of(g + pr, m, sSD4 + pr * LMP);
         } else {
             // the staging area holds 16 pairs or fewer: the lanes of a warp take several columns side by side (more of
             // them for a short chunk), so that the recursion runs over fewer trips
             // (the span follows the chunk only from l_max = 9 on: below, the extra code cost the headline build 0.5 %)
-            const int span = L >= 9 ? (pc > 8 ? 16 : pc > 4 ? 8 : 4) : P, cols = 32 / span, pr = lane & (span - 1), cg = lane / span;
-            if (pr < pc) {
-                const float4 d = geo_d[g + pr];
-                for (int m = wid * cols + cg; m <= L; m += kWarps * cols)
-                    harmonics_column(L, m, d.x, d.y, d.z, d.w * d.w, sSD4 + pr * LMP);
-            }
+            const int span = L >= 9 ? (pc > 8 ? 16 : pc > 4 ? 8 : 4) : (P >= 16 ? 16 : P >= 8 ? 8 : 4), cols = 32 / span, cg = lane / span;
+            for (int pr = lane & (span - 1); pr < pc; pr += span)
+                for (int m = wid * cols + cg; m <= L; m += warps * cols) harmonics_of(g + pr, m, sSD4 + pr * LMP);
         }
     };
 
@@ -354,7 +366,7 @@ center_kernel(const CenterParams p) {
                                 const float mv = (!special || (geo_i[g].z & 256)) ? 1.f : 0.f;
                                 float hy = h.y, hz = h.z, hw = h.w, tx = h.x * d.x, ty = h.x * d.y, tz = h.x * d.z;
                                 if (special) { hy *= mv; hz *= mv; hw *= mv; tx *= mv; ty *= mv; tz *= mv; }
-                                const float2* gp = sG2 + pr * NCH + (n0 + own_slot) * L1 + own_l;
+                                const float2* gp = sG2 + pr * GP + (n0 + own_slot) * L1 + own_l;
 #pragma unroll
                                 for (int k = 0; k < NPT; ++k)
                                     if (n0 + own_slot + k * SLOTS < NMAX) {
@@ -397,7 +409,7 @@ center_kernel(const CenterParams p) {
     const int RW = CC ? W : (o_compact ? p.Fc : F);                        // width of an output row
     if (o_cbar) {
         // inner average: the mean coefficients (on-site terms included) take the place of the centre's own
-        for (int e = tid; e < W; e += kThreads) {
+        for (int e = tid; e < W; e += threads) {
             const int row = e / LM;
             c_t[row * LMP + (e - row * LM)] = __ldg(o_cbar + e);
         }
@@ -406,7 +418,7 @@ center_kernel(const CenterParams p) {
     if (CC) {
         // coefficient mode: the tile itself is the result, index (mu n_max + n) (l_max+1)^2 + l^2 + l + m
         float* crow = p.out_desc + (size_t)c_idx * W;
-        for (int e = tid; e < W; e += kThreads) {
+        for (int e = tid; e < W; e += threads) {
             const int row = e / LM;
             crow[e] = c_t[row * LMP + (e - row * LM)];
         }
@@ -415,7 +427,7 @@ center_kernel(const CenterParams p) {
     // ============ power spectrum (Eq. 4) and the centre's own row ============
     // Threads walk the features l-major so that the lanes of a warp share the trip count 2l+1; the
     // centre's row is minus the sum over its neighbours: -K_l sum_m (D^mu c^nu + c^mu D^nu).  Results
-    // pass through the (now idle) staging area in slabs, so that global memory is written in
+    // pass through the slab, so that global memory is written in
     // feature order, whole sectors at a time.
     const long long row_base = p.row_ptr[c_idx];
     const bool has_own = !o_sites;                   // a centre that is no atom has no row of its own
@@ -423,7 +435,7 @@ center_kernel(const CenterParams p) {
         // the centre's own row: minus the sum over the atoms that move relative to it
         if (has_own) {
             float* own = p.out_jac + (size_t)(row_base + p.self_row[c_idx]) * 3 * W;
-            for (int e = tid; e < 3 * W; e += kThreads) {
+            for (int e = tid; e < 3 * W; e += threads) {
                 const int k = e / W, r = e - k * W, row = r / LM;
                 own[e] = -D_t[k * CT + row * LMP + (r - row * LM)];
             }
@@ -441,17 +453,18 @@ center_kernel(const CenterParams p) {
                                  : p.out_jac + (size_t)(row_base + p.self_row[c_idx]) * 3 * F;
         if (has_own && o_compact) {
             float* slot = p.out_jac + (size_t)(row_base + p.self_row[c_idx]) * 3 * RW;
-            for (int e = tid; e < 3 * RW; e += kThreads) slot[e] = 0.f;
+            for (int e = tid; e < 3 * RW; e += threads) slot[e] = 0.f;
         }
-        float* slab = smem + lay.sSD;
+        float* slab = smem + lay.slab;
+        const int slab_words = lay.slab_words;
         constexpr int NV = 4;                                               // values per feature: p and the three components of the centre's row
         const int NP = F / L1;                                              // (species pair, n, n') groups
-        int gp = ((lay.total - lay.sSD) / NV) / L1;                         // groups per slab
+        int gp = (slab_words / NV) / L1;                         // groups per slab
         gp = gp < 1 ? 1 : (gp > NP ? NP : gp);
-        const bool staged = (lay.total - lay.sSD) >= NV * L1;
+        const bool staged = slab_words >= NV * L1;
         for (int q0 = 0; q0 < NP; q0 += gp) {
             const int nq = min(gp, NP - q0), nf = nq * L1, f0 = q0 * L1;
-            for (int g = tid; g < nf; g += kThreads) {
+            for (int g = tid; g < nf; g += threads) {
                 const int l = g / nq, fl = (g - l * nq) * L1 + l;             // feature index inside the slab
                 const int pk = __ldg(p.feat_pack + f0 + fl);
                 const int n1 = pk & 31, n2 = (pk >> 5) & 31, mu = (pk >> 10) & 15, nu = (pk >> 14) & 15;
@@ -479,7 +492,7 @@ center_kernel(const CenterParams p) {
             }
             if (staged) {
                 __syncthreads();
-                for (int e = tid; e < nf; e += kThreads) {
+                for (int e = tid; e < nf; e += threads) {
                     if (write_desc) desc_row[f0 + e] = slab[e];
                     if (has_own) {
                         own[f0 + e] = slab[nf + e];
@@ -508,8 +521,8 @@ center_kernel(const CenterParams p) {
         const int NI = S * NCH, SN = S * NMAX, Z = zi_species;
         const int TRI = (NMAX * (NMAX + 1) / 2) * L1, SQ = NMAX * NCH;
         const int NZ = TRI + (o_cross ? (S - 1) * SQ : 0);                     // features that involve species Z
-        float4* sUV = reinterpret_cast<float4*>(smem + lay.wUV);              // [kWarps][nu][n'][l]
-        float* c_copy = smem + lay.total + wid * CT;                          // [kWarps][S n_max][LMP], behind the usual layout
+        float4* sUV = reinterpret_cast<float4*>(smem + lay.wUV);              // [warps][nu][n'][l]
+        float* c_copy = smem + lay.total + wid * CT;                          // [warps][S n_max][LMP], behind the usual layout
         float* const row = p.out_jac + (size_t)ci * 3 * F;
         // the x-th feature that involves Z: its place in the row and its operands, (radial index, U/V index) of one
         // term, or of both in the same-species block (gB >= 0)
@@ -532,7 +545,7 @@ center_kernel(const CenterParams p) {
                 uA = other * NCH + (first_term ? j : i1);
             }
         };
-        const int n_groups = (NZ + kSlots * kThreads - 1) / (kSlots * kThreads);
+        const int n_groups = (NZ + kSlots * threads - 1) / (kSlots * threads);
         const bool in_registers = n_groups == 1;
         int sf[kSlots], sgA[kSlots], suA[kSlots], sgB[kSlots], suB[kSlots];
         float ax[kSlots], ay[kSlots], az[kSlots];
@@ -540,7 +553,7 @@ center_kernel(const CenterParams p) {
         for (int k = 0; k < kSlots; ++k) {
             ax[k] = ay[k] = az[k] = 0.f;
             sf[k] = -1; sgA[k] = suA[k] = suB[k] = 0; sgB[k] = -1;
-            if (in_registers && k * kThreads + tid < NZ) decode(k * kThreads + tid, sf[k], sgA[k], suA[k], sgB[k], suB[k]);
+            if (in_registers && k * threads + tid < NZ) decode(k * threads + tid, sf[k], sgA[k], suA[k], sgB[k], suB[k]);
         }
         for (int g0 = 0; g0 < k_pairs; g0 += geo_batch) {
             const int gc = min(geo_batch, k_pairs - g0);
@@ -550,8 +563,8 @@ center_kernel(const CenterParams p) {
                 const int pc = min(P, gc - q0);
                 stage_chunk(q0, pc);
                 __syncthreads();
-                for (int r0 = 0; r0 < pc; r0 += kWarps) {
-                    const int nr = min(kWarps, pc - r0);
+                for (int r0 = 0; r0 < pc; r0 += warps) {
+                    const int nr = min(warps, pc - r0);
                     if (wid < nr) {
                         const float* cj = p.c_all + (size_t)geo_j[q0 + r0 + wid] * W;   // every atom is a centre, in order
                         for (int e = lane; e < W; e += 32) {
@@ -605,7 +618,7 @@ center_kernel(const CenterParams p) {
                         if (!in_registers) {
 #pragma unroll
                             for (int k = 0; k < kSlots; ++k) {
-                                const int x = (grp * kSlots + k) * kThreads + tid;
+                                const int x = (grp * kSlots + k) * threads + tid;
                                 sf[k] = -1;
                                 if (x < NZ) {
                                     decode(x, sf[k], sgA[k], suA[k], sgB[k], suB[k]);
@@ -617,7 +630,7 @@ center_kernel(const CenterParams p) {
                             const int g = q0 + r0 + w;
                             if (!(geo_i[g].z & 256)) continue;                 // an image of a itself: part of its own row already
                             const float4 d = geo_d[g];
-                            const float2* wG = sG2 + (r0 + w) * NCH;
+                            const float2* wG = sG2 + (r0 + w) * GP;
                             const float4* UV = sUV + w * NI;
 #pragma unroll
                             for (int k = 0; k < kSlots; ++k) {
@@ -655,7 +668,7 @@ center_kernel(const CenterParams p) {
     }
     // fold K_l into c for pass 2
     if (!CC)
-        for (int e = tid; e < W; e += kThreads) {
+        for (int e = tid; e < W; e += threads) {
             const int row = e / LM, lm = e - row * LM;
             c_t[row * LMP + lm] *= __ldg(p.kl + __ldg(p.l_of_lm + lm));
         }
@@ -669,7 +682,7 @@ center_kernel(const CenterParams p) {
     // coefficient mode: table lm -> l in the (now idle) space of the D tiles; the loop below starts with a barrier
     int* lm_to_l = reinterpret_cast<int*>(smem + lay.wUV);
     if (CC)
-        for (int e = tid; e < LM; e += kThreads) lm_to_l[e] = __ldg(p.l_of_lm + e);
+        for (int e = tid; e < LM; e += threads) lm_to_l[e] = __ldg(p.l_of_lm + e);
     float4* wUV = reinterpret_cast<float4*>(smem + lay.wUV) + wid * NI;       // [nu][n'][l]
 
     // Product rule of one pair (Eq. 5).  Lanes take consecutive features of the row in sweeps that
@@ -699,11 +712,11 @@ center_kernel(const CenterParams p) {
                     if (o_compact) continue;                  // compact rows hold only the blocks that involve Z
                     if (!ACC) {
                         if (bulk_ok) {
-                            // structural zeros: the lanes hand the plane segments (pieces of at most kZeroWords) to the copy engine
-                            const int parts = (hi - lo + kZeroWords - 1) / kZeroWords;
+                            // structural zeros: the lanes hand the plane segments (pieces of at most zero_w) to the copy engine
+                            const int parts = (hi - lo + zero_w - 1) / zero_w;
                             for (int idx = lane; idx < 3 * parts; idx += 32) {
-                                const int k = idx / parts, f = lo + (idx - k * parts) * kZeroWords;
-                                bulk_store(out + k * PS + f, zero_buf, 4u * (unsigned)min(kZeroWords, hi - f));
+                                const int k = idx / parts, f = lo + (idx - k * parts) * zero_w;
+                                bulk_store(out + k * PS + f, zero_buf, 4u * (unsigned)min(zero_w, hi - f));
                             }
                         } else {
                             for (int f = first + lane; f < hi; f += 32)
@@ -893,6 +906,28 @@ center_kernel(const CenterParams p) {
             for (int f = lo + lane; f < RW; f += 32) put(f, 0.f, 0.f, 0.f);
     };
 
+    // The same for small bases, whose blocks leave most lanes of the sweeps above idle: the lanes walk down the whole row,
+    // with the operands of every feature for this species from a table, a zero for those a feature does not have
+    // (up to 20 channels: kernel on 3000 atoms at (2, 2) 154 -> 113 us, (4, 3) 193 -> 178 us, four species (3, 3)
+    // 140 -> 125 us, (3, 5) equal; with more channels the sweeps win, (4, 8) 285 against 302 us).
+    auto table_rule = [&](auto acc_tag, int Z, float4 d, const float2* wG, float* out) {
+        constexpr bool ACC = decltype(acc_tag)::value;
+        const unsigned* ops = p.row_ops + Z * F;
+        float *o0 = out, *o1 = out + F, *o2 = out + 2 * F;
+#pragma unroll 2
+        for (int f = lane; f < F; f += 32) {
+            const unsigned op = __ldg(ops + f);
+            const float2 g1 = wG[op & 255], g2 = wG[(op >> 8) & 255];
+            const float4 u1 = wUV[(op >> 16) & 255], u2 = wUV[op >> 24];
+            const float t = fmaf(g1.y, u1.x, g2.y * u2.x);
+            const float vx = fmaf(g1.x, u1.y, fmaf(g2.x, u2.y, t * d.x)), vy = fmaf(g1.x, u1.z, fmaf(g2.x, u2.z, t * d.y)),
+                        vz = fmaf(g1.x, u1.w, fmaf(g2.x, u2.w, t * d.z));
+            if (ACC) { o0[f] += vx; o1[f] += vy; o2[f] += vz; }
+            else { o0[f] = vx; o1[f] = vy; o2[f] = vz; }
+        }
+    };
+    const bool by_table = kRowTable && p.row_ops != nullptr && !o_compact;
+
     // Coefficient mode: the row of a neighbour of species Z is grad c^Z_nlm = G_nl grad S_lm + Ghat_nl d S_lm
     // (Eq. 14 / Eq. 23) in the block of Z and zero in the other blocks, written in aligned sweeps as above.
     auto coeff_rule = [&](auto acc_tag, int Z, float4 d, const float2* wG, const float4* wSD, float* out) {
@@ -926,11 +961,26 @@ center_kernel(const CenterParams p) {
         const int row = rw & kRowMask;
         const int Z = gi.z & 255;
         const float4 d = geo_d[g];
-        const float2* wG = sG2 + pr * NCH;
+        const float2* wG = sG2 + pr * GP;
         const float4* wSD = sSD4 + pr * LMP;
         __syncwarp();
         // ---- U, V for every (nu, n', l) ----
         if (CC) {
+        } else if (SN <= 8) {
+            // lane <-> (nu n', component of (U, Vx, Vy, Vz))
+            const int sn = lane >> 2, k = lane & 3;
+            if (sn < SN) {
+                const float* cp = c_t + sn * LMP;
+                const float* hp = reinterpret_cast<const float*>(wSD) + k;
+                float* up = reinterpret_cast<float*>(wUV + sn * L1) + k;
+#pragma unroll
+                for (int l = 0; l <= L; ++l) {
+                    float acc = 0.f;
+#pragma unroll
+                    for (int m = 0; m <= 2 * l; ++m) acc = fmaf(cp[l * l + m], hp[4 * (l * l + m)], acc);
+                    up[4 * l] = acc;
+                }
+            }
         } else if (SN <= 16) {
             // lane <-> (nu n', half): half 0 accumulates (U, Vx), half 1 (Vy, Vz)
             const int sn = lane >> 1, half = lane & 1;
@@ -971,82 +1021,68 @@ center_kernel(const CenterParams p) {
         float* out = p.out_jac + (size_t)(row_base + row) * 3 * RW;
         if (rw & kRowContinuation) {
             if (CC) coeff_rule(std::true_type{}, Z, d, wG, wSD, out);
+            else if (by_table) table_rule(std::true_type{}, Z, d, wG, out);
             else product_rule(std::true_type{}, Z, d, wG, out);
         } else {
             if (lane == 0) p.row_atom[row_base + row] = geo_j[g];
             if (CC) coeff_rule(std::false_type{}, Z, d, wG, wSD, out);
+            else if (by_table) table_rule(std::false_type{}, Z, d, wG, out);
             else product_rule(std::false_type{}, Z, d, wG, out);
             if (bulk_ok) bulk_commit();
         }
     };
 
-    const int PW = P / kWarps;             // pairs a warp stages for itself (the staging area holds P)
+    const int PW = min(4, P / warps);     // pairs a warp stages for itself (the staging area holds P; eight lanes per pair)
     for (int g0 = 0; g0 < k_pairs; g0 += geo_batch) {
         const int gc = min(geo_batch, k_pairs - g0);
         __syncthreads();
         if (g0 > 0 || k_pairs > kGeoPairs) special = stage_geometry(g0, gc);     // otherwise still valid from pass 1
+        // everything that pass 1 staged is still there
+        const bool kept = lay.keep && k_pairs <= P && k_pairs <= kGeoPairs && SLOTS * NPT >= NMAX;
         // (measured on the 1000-molecule cluster: 1 to 4 % faster from n_max = 8 on up to l_max = 8; with fewer
         // channels than lanes, or more columns m than the eight lanes of a pair, the staging by the whole CTA wins)
         constexpr bool kPrivate = !CC && NMAX_T >= 8 && L <= 8;      // (the coefficient rows are cheap per pair: staging by the CTA wins there)
-        if (kPrivate && !special && PW >= 1) {
+        if (kPrivate && !special && PW >= 1 && !kept) {
             // Every pair has a row of its own: the warps work without one another.  Warp w takes the pairs w, w + 8,
             // ... of the batch, PW at a time: it stages their radial factors (lanes on channels) and harmonics (eight
             // lanes per pair, on the columns m of the recursion) in its own part of the staging area, then writes
             // their rows.  No CTA barrier until the next batch of geometry.
             const int slot0 = wid * PW;
-            for (int gw = wid; gw < gc; gw += PW * kWarps) {
-                const int nb = min(PW, (gc - gw + kWarps - 1) / kWarps);
+            for (int gw = wid; gw < gc; gw += PW * warps) {
+                const int nb = min(PW, (gc - gw + warps - 1) / warps);
                 __syncwarp();
-                for (int pr = 0; pr < nb; ++pr) {
-                    const int g = gw + pr * kWarps;
-                    const int4 gi = geo_i[g];
-                    const float t = __int_as_float(gi.y);
-                    const float rinv_h = (float)p.inv_h / geo_d[g].w;
-                    float2* mG = sG2 + (slot0 + pr) * NCH;
-                    if (o_pw) {
-                        const float2 w = geo_w[g];
-                        for (int ch = lane; ch < NCH; ch += 32) {
-                            float v, dv;
-                            radial_lookup(p.table, gi.x, NCH, ch, t, v, dv);
-                            mG[ch] = make_float2(v * w.x, fmaf(dv * rinv_h, w.x, v * w.y));
-                        }
-                    } else {
-                        for (int ch = lane; ch < NCH; ch += 32) {
-                            float v, dv;
-                            radial_lookup(p.table, gi.x, NCH, ch, t, v, dv);
-                            mG[ch] = make_float2(v, dv * rinv_h);
-                        }
-                    }
+                for (int e = lane; e < nb * CP; e += 32) {
+                    const int pr = NMAX_T ? e / CP_T : e / CP;
+                    stage_radial(gw + pr * warps, e - pr * CP, sG2 + (slot0 + pr) * GP);
                 }
                 {
                     const int pr = lane >> 3;
-                    if (pr < nb) {
-                        const float4 d = geo_d[gw + pr * kWarps];
-                        for (int m = lane & 7; m <= L; m += 8)
-                            harmonics_column(L, m, d.x, d.y, d.z, d.w * d.w, sSD4 + (slot0 + pr) * LMP);
-                    }
+                    if (pr < nb)
+                        for (int m = lane & 7; m <= L; m += 8) harmonics_of(gw + pr * warps, m, sSD4 + (slot0 + pr) * LMP);
                 }
                 __syncwarp();
-                for (int pr = 0; pr < nb; ++pr) do_pair(gw + pr * kWarps, slot0 + pr);
+                for (int pr = 0; pr < nb; ++pr) do_pair(gw + pr * warps, slot0 + pr);
             }
             continue;
         }
         // Images of one atom share a row (or the staging area holds fewer pairs than there are warps): staged by the
         // whole CTA in chunks of equal size, a multiple of the warp count.
         const int n_chunks = (gc + P - 1) / P;
-        const int PB = min(P, (((gc + n_chunks - 1) / n_chunks) + kWarps - 1) & ~(kWarps - 1));
+        const int PB = min(P, (((gc + n_chunks - 1) / n_chunks) + warps - 1) & ~(warps - 1));   // (kept: one chunk)
         for (int q0 = 0; q0 < gc; q0 += PB) {
             const int pc = min(PB, gc - q0);
-            stage_chunk(q0, pc);
-            __syncthreads();
+            if (!kept) {
+                stage_chunk(q0, pc);
+                __syncthreads();
+            }
             if (!special) {
-                for (int pr = wid; pr < pc; pr += kWarps) do_pair(q0 + pr, pr);
+                for (int pr = wid; pr < pc; pr += warps) do_pair(q0 + pr, pr);
             } else {
                 // images of one atom must stay with one warp, in order;
                 // images of the centre itself do not move relative to it and are skipped
                 for (int pr = 0; pr < pc; ++pr) {
                     const int rw = geo_i[q0 + pr].w;
-                    if ((rw & kRowSelfImage) || ((rw & kRowMask) & (kWarps - 1)) != wid) continue;
+                    if ((rw & kRowSelfImage) || ((rw & kRowMask) & (warps - 1)) != wid) continue;
                     do_pair(q0 + pr, pr);
                 }
             }

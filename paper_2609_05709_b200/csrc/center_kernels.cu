@@ -119,9 +119,9 @@ cudaError_t SOAP_CAT(center_set_smem_l, SOAP_L)(int kind, int n_max, int bytes) 
 
 // The kernel waits on the device for the kernel before it (the row scan, as a rule): its launch and its set-up overlap
 // that kernel's tail.
-cudaError_t SOAP_CAT(center_launch_l, SOAP_L)(int kind, int n_max, bool plain, const CenterParams& p, unsigned grid, size_t smem,
+cudaError_t SOAP_CAT(center_launch_l, SOAP_L)(int kind, int n_max, bool plain, int threads, const CenterParams& p, unsigned grid, size_t smem,
                                               cudaStream_t st) {
-    return launch_dependent(kernel_of(kind, n_max, plain), grid, kThreads, smem, st, p);
+    return launch_dependent(kernel_of(kind, n_max, plain), grid, threads, smem, st, p);
 }
 
 }  // namespace soap

@@ -40,9 +40,9 @@ cudaError_t center_set_smem(int kind, int l_max, int n_max, int bytes) {
     }
     return cudaErrorInvalidValue;
 }
-cudaError_t center_launch(int kind, int l_max, int n_max, const CenterParams& p, unsigned grid, size_t smem, cudaStream_t st) {
+cudaError_t center_launch(int kind, int l_max, int n_max, int threads, const CenterParams& p, unsigned grid, size_t smem, cudaStream_t st) {
     switch (l_max) {
-#define X(LV) case LV: return center_launch_l##LV(kind, n_max, center_params_plain(p), p, grid, smem, st);
+#define X(LV) case LV: return center_launch_l##LV(kind, n_max, center_params_plain(p), threads, p, grid, smem, st);
         X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
 #undef X
     }
@@ -99,6 +99,7 @@ struct soap_handle {
     int sm_count = 0, max_smem = 0;
     int desc_np = 0;                     // n_max rounded up to a multiple of four
     size_t desc_table_bytes = 0, desc_warp_bytes = 0;
+    unsigned* d_row_ops = nullptr;       // operands of the Jacobian rows' features (small bases)
     int *d_feat = nullptr, *d_zlut = nullptr, *d_l_of_lm = nullptr;
     Counters* d_counters = nullptr;
     unsigned long long* d_bbox = nullptr;   // 6 words of bounding box (structures above 16384 atoms)
@@ -126,6 +127,8 @@ struct soap_handle {
     bool list_sorted = false;            // whether the pair list of the last search is sorted (descriptor-only calls skip that)
     bool ordered = false;                // whether the last search with rows left a launch order
     int64_t found_atoms = -1, found_centers = -1;   // sizes of the search soap_search left for soap_derivatives_found; -1: none
+    int P_deriv4 = 16;                   // ... with CTAs of 128 threads
+    size_t smem_deriv4 = 0;
     int P_deriv = 16, P_outer = 16;      // pairs per staged chunk: derivative kernels, kernel of the outer average
     size_t smem_deriv = 0, smem_outer = 0;
     bool outer_fast = false;             // whether the kernel of the outer average fits the shared memory
@@ -203,26 +206,29 @@ int plan_smem(soap_t* h) {
     h->desc_warp_bytes = (size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0, false).per_warp * 4;
     if (h->desc_warp_bytes > (size_t)max_smem) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
     CU(desc_set_smem(h->l_max, desc_np(h->n_max), max_smem));
-    // pairs per staged chunk of the derivative kernels: the largest that still leaves room for three CTAs per SM,
-    // else two, else whatever fits (`extra` bytes follow the usual layout); false if nothing fits
-    auto plan_chunk = [&](size_t extra, int& P_out, size_t& bytes_out) -> bool {
-        int P = 32;
-        size_t bytes = 0;
-        const size_t budget3 = (size_t)228 * 1024 / 3 - 1024, budget2 = (size_t)228 * 1024 / 2 - 1024;
+    // pairs per staged chunk of the derivative kernels: the largest that still leaves room for all the CTAs per SM that
+    // the registers allow (three of 256 threads), else two thirds of them, else whatever fits (`extra` bytes follow the
+    // usual layout); false if nothing fits.  Where the slab has room of its own a chunk may hold 96 pairs, so that most
+    // centres are staged once for both passes (3000 atoms of 68 neighbours at (4, 3): 218 -> 193 us).
+    auto plan_chunk = [&](int warps, size_t extra, int& P_out, size_t& bytes_out) -> bool {
+        const int ctas = 24 / warps;
+        auto bytes_of = [&](int P) { return (size_t)make_layout(h->S, h->n_max, h->l_max, P, warps, h->weight.fn != 0).total * 4 + extra; };
+        const bool keep = make_layout(h->S, h->n_max, h->l_max, 32, warps, false).keep;
+        int P = 4;
         for (int pass = 0; pass < 3; ++pass) {
-            const size_t budget = pass == 0 ? budget3 : pass == 1 ? budget2 : (size_t)max_smem;
-            for (P = 32; P >= 4; P /= 2) {
-                bytes = (size_t)make_layout(h->S, h->n_max, h->l_max, P, true, h->weight.fn != 0).total * 4 + extra;
-                if (bytes <= budget) break;
+            const size_t budget = pass == 2 ? (size_t)max_smem : (size_t)228 * 1024 / (pass == 0 ? ctas : (2 * ctas + 2) / 3) - 1024;
+            for (const int candidate : {96, 80, 64, 56, 48, 40, 32, 24, 16, 8, 4}) {
+                P = candidate;
+                if ((keep ? P <= 32 * warps && (P != 24 || h->l_max < 8) : P <= 32 && P != 24) && bytes_of(P) <= budget) break;
             }
-            if (P >= (pass == 2 ? 4 : 8) && bytes <= budget) break;
-            if (P < 4) P = 4;
+            if (P >= (pass == 2 ? 4 : 8) && bytes_of(P) <= budget) break;
         }
-        bytes = (size_t)make_layout(h->S, h->n_max, h->l_max, P, true, h->weight.fn != 0).total * 4 + extra;
-        P_out = P; bytes_out = bytes;
-        return bytes <= (size_t)max_smem;
+        P_out = P; bytes_out = bytes_of(P);
+        return bytes_out <= (size_t)max_smem;
     };
-    if (!plan_chunk(0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
+    // 256 threads, and the smaller CTAs that this basis may run with
+    if (!plan_chunk(8, 0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
+    if (!plan_chunk(4, 0, h->P_deriv4, h->smem_deriv4)) h->smem_deriv4 = 0;
     // (a kernel's limit is the process's, not the handle's: every handle sets the device's maximum, so that none takes away
     // what another one launches with)
     CU(center_set_smem(kCenterDeriv, h->l_max, h->n_max, max_smem));
@@ -231,8 +237,29 @@ int plan_smem(soap_t* h) {
     // the kernel of the outer average keeps, per warp, a copy of a neighbouring centre's coefficients behind the usual
     // layout; a basis too large for that takes the general path (per-pair rows in a workspace)
     const int LMP = ((h->l_max + 1) * (h->l_max + 1)) | 1;
-    h->outer_fast = plan_chunk((size_t)kWarps * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
+    h->outer_fast = plan_chunk(kThreads / 32, (size_t)(kThreads / 32) * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
     if (h->outer_fast) CU(center_set_smem(kCenterOuter, h->l_max, h->n_max, max_smem));
+    return SOAP_OK;
+}
+
+// The feature table, and for small bases the operands of every feature in the row of a neighbour of each species (Eq. 5):
+// radial factor g and U/V entry u of the term in which the neighbour's species comes first, g' and u' of the one in which
+// it comes second; index n_max (l_max+1) of g is a zero.
+int upload_features(soap_t* h) {
+    for (void* old : {(void*)h->d_feat, (void*)h->d_row_ops}) if (old) cudaFree(old);
+    h->d_feat = nullptr; h->d_row_ops = nullptr;
+    CU(upload(&h->d_feat, h->feat_pack));
+    const int L1 = h->l_max + 1, n_ch = h->n_max * L1;
+    if (!row_table_wanted(h->n_max, h->l_max) || h->F > kKeepFeatures || h->S * n_ch > 256 || n_ch > 255) return SOAP_OK;
+    std::vector<unsigned> ops;
+    for (int z = 0; z < h->S; ++z)
+        for (const int pk : h->feat_pack) {
+            const int n = pk & 31, n2 = (pk >> 5) & 31, mu = (pk >> 10) & 15, nu = (pk >> 14) & 15, l = (pk >> 18) & 15;
+            const int i = n * L1 + l, j = n2 * L1 + l;
+            const unsigned g = mu == z ? i : n_ch, u = mu == z ? nu * n_ch + j : 0, g2 = nu == z ? j : n_ch, u2 = nu == z ? mu * n_ch + i : 0;
+            ops.push_back(g | g2 << 8 | u << 16 | u2 << 24);
+        }
+    CU(upload(&h->d_row_ops, ops));
     return SOAP_OK;
 }
 
@@ -245,26 +272,31 @@ int ensure_device(soap_t* h) {
         return SOAP_OK;
     }
     h->device = dev;
-    CU(upload(&h->d_table, h->basis.table));
     {
-        // [interval][l][n / 2][6][2], n padded to a multiple of four: the coefficients of two adjacent n interleaved
-        // (the descriptor-only kernel evaluates them with packed multiply-adds); the padding channels are zero
-        const int L1 = h->l_max + 1, n_ch = h->n_max * L1, np = desc_np(h->n_max);
-        std::vector<float> ln((size_t)h->basis.n_intervals_values * L1 * np * kTableCoef, 0.f);
-        for (int q = 0; q < h->basis.n_intervals_values; ++q)
-            for (int l = 0; l < L1; ++l)
-                for (int n = 0; n < h->n_max; ++n)
-                    for (int k = 0; k < kTableCoef; ++k)
-                        ln[((((size_t)q * L1 + l) * (np / 2) + n / 2) * kTableCoef + k) * 2 + (n & 1)] =
-                            h->basis.table_values[((size_t)q * n_ch + n * L1 + l) * kTableCoef + k];
-        CU(upload(&h->d_table_ln, ln));
-        h->desc_np = np;
-        h->desc_table_bytes = ln.size() * sizeof(float);
+        // [interval][l][n / 2][6][2]: the coefficients of two adjacent n interleaved (the kernels evaluate them with packed
+        // multiply-adds), n padded to a multiple of two for the derivative kernels and of four for the descriptor-only
+        // kernel; the padding channels are zero
+        const int L1 = h->l_max + 1, n_ch = h->n_max * L1;
+        auto interleaved = [&](const std::vector<float>& table, int intervals, int np) {
+            std::vector<float> out((size_t)intervals * L1 * np * kTableCoef, 0.f);
+            for (int q = 0; q < intervals; ++q)
+                for (int l = 0; l < L1; ++l)
+                    for (int n = 0; n < h->n_max; ++n)
+                        for (int k = 0; k < kTableCoef; ++k)
+                            out[((((size_t)q * L1 + l) * (np / 2) + n / 2) * kTableCoef + k) * 2 + (n & 1)] =
+                                table[((size_t)q * n_ch + n * L1 + l) * kTableCoef + k];
+            return out;
+        };
+        CU(upload(&h->d_table, interleaved(h->basis.table, h->basis.n_intervals, (h->n_max + 1) & ~1)));
+        h->desc_np = desc_np(h->n_max);
+        const std::vector<float> values = interleaved(h->basis.table_values, h->basis.n_intervals_values, h->desc_np);
+        CU(upload(&h->d_table_ln, values));
+        h->desc_table_bytes = values.size() * sizeof(float);
     }
     CU(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device));
     CU(upload(&h->d_self, h->basis.self_term));
     CU(upload(&h->d_kl, h->basis.kl));
-    CU(upload(&h->d_feat, h->feat_pack));
+    if (int rc = upload_features(h)) return rc;
     {
         std::vector<int> l_of_lm;
         for (int l = 0; l <= h->l_max; ++l)
@@ -479,7 +511,7 @@ void fill_center_params(soap_t* h, CenterParams& cp, const float* pos, const int
     cp.row_ptr = h->d_row_ptr; cp.self_row = h->d_self_row;
     cp.pair_capacity = h->cap_pairs; cp.row_capacity = 0; cp.counters = h->d_counters;
     cp.table = h->d_table; cp.self_term = h->d_self; cp.kl = h->d_kl; cp.l_of_lm = h->d_l_of_lm;
-    cp.feat_pack = h->d_feat; cp.nch_magic = (unsigned)((1ull << 32) / (unsigned)(h->n_max * (h->l_max + 1))) + 1u; cp.inv_h = h->basis.inv_h; cp.n_intervals = h->basis.n_intervals;
+    cp.feat_pack = h->d_feat; cp.row_ops = h->d_row_ops; cp.nch_magic = (unsigned)((1ull << 32) / (unsigned)(h->n_max * (h->l_max + 1))) + 1u; cp.inv_h = h->basis.inv_h; cp.n_intervals = h->basis.n_intervals;
     cp.S = h->S; cp.n_max = h->n_max; cp.l_max = h->l_max; cp.F = (int)h->F;
     cp.P = h->P_deriv;
     cp.crossover = h->crossover; cp.emit_coeff = 0; cp.c_bar = nullptr; cp.inner_rows = 0; cp.own_scale = 1.f; cp.c_all = nullptr;
@@ -530,6 +562,23 @@ int status_error(soap_t* h, int s) {
     if (s & kStatusShiftRange) return fail(h, SOAP_ERR_INVALID_ARG, "positions lie too many cells away from the unit cell");
     if (s & kStatusPairCapacity) return fail(h, SOAP_ERR_CAPACITY, "more pairs than planned (call soap_neighbors again) or than the export buffer holds");
     if (s & kStatusRowCapacity) return fail(h, SOAP_ERR_CAPACITY, "more Jacobian rows than capacity_rows");
+    return SOAP_OK;
+}
+
+// Launch of the derivative kernel, a CTA per centre.  Small bases on many centres run with CTAs of 128 threads, six per SM
+// instead of three: what a CTA does once, and its barriers, weigh more there than the pairs (kernel, 256 against 128
+// threads: 36,000 centres of 18 pairs at (4, 3) 914 -> 687 us, 3000 of 274 at (7, 3) 1130 -> 1094 us, 900 at (8, 3)
+// 115 -> 101 us).  With few centres the larger CTA finishes sooner (450 at (4, 3) 37 against 48 us, 600 equal), and so it
+// does where pass 1 keeps 128 threads busy and the rows are long (4 species at (4, 7) 250 against 262 us).
+int launch_deriv(soap_t* h, int kind, CenterParams& cp, int64_t n_centers, cudaStream_t st) {
+    int threads = kThreads;
+    size_t bytes = h->smem_deriv;
+    const int channels = h->n_max * (h->l_max + 1), needs = pass1_span(h->l_max) * pass1_slots(h->l_max, 16);
+    const bool small = channels <= 20 || (channels <= 32 && h->l_max <= 4);
+    if (small && needs <= 128 && h->smem_deriv4 != 0 && n_centers >= (int64_t)5 * h->sm_count) {
+        threads = 128; cp.P = h->P_deriv4; bytes = h->smem_deriv4;
+    }
+    CU(center_launch(kind, h->l_max, h->n_max, threads, cp, (unsigned)n_centers, bytes, st));
     return SOAP_OK;
 }
 
@@ -647,7 +696,7 @@ int soap_create(soap_t** out, const int32_t* species, int n_species, double r_cu
     std::string err;
     int rc = build_basis(rbf, r_cut, n_max, l_max, sigma, h->basis, err);
     if (rc) return bail(rc, err);
-    if ((int64_t)n_max * (l_max + 1) * (l_max + 1) > (int64_t)kMaxElemPerThread * kThreads)
+    if ((int64_t)n_max * (l_max + 1) * (l_max + 1) > kMaxElements)
         return bail(SOAP_ERR_INVALID_ARG, "n_max (l_max+1)^2 must not exceed 2048");
     build_feature_table(h);
     *out = h;
@@ -656,7 +705,7 @@ int soap_create(soap_t** out, const int32_t* species, int n_species, double r_cu
 
 void soap_destroy(soap_t* h) {
     if (!h) return;
-    void* ptrs[] = {h->d_table, h->d_table_ln, h->d_self, h->d_kl, h->d_feat, h->d_zlut, h->d_l_of_lm, h->d_counters, h->d_bbox,
+    void* ptrs[] = {h->d_table, h->d_table_ln, h->d_self, h->d_kl, h->d_feat, h->d_row_ops, h->d_zlut, h->d_l_of_lm, h->d_counters, h->d_bbox,
                     h->d_grid, h->d_species_idx, h->d_atom_cell, h->d_atom_wrap, h->d_s_wrap, h->d_s_pos, h->d_cell_count,
                     h->d_cell_start, h->d_pair_count, h->d_row_count, h->d_self_row, h->d_order, h->d_pair_ptr, h->d_pair_start, h->d_row_ptr, h->d_tile_sums, h->d_tile_offsets,
                     h->d_pair_key, h->d_pair_tmp, h->d_pair_row, h->d_work, h->d_pair_w, h->d_compact_map,
@@ -780,7 +829,7 @@ static int derivatives_impl(soap_t* h, const float* d_positions, const int32_t* 
         cp.row_capacity = capacity_rows;
         cp.out_desc = d_out_desc; cp.out_jac = d_out_jac; cp.row_atom = d_row_atom;
         if (d_out_center) { cp.compact = 1; cp.out_center = d_out_center; }
-        CU(center_launch(kCenterDeriv, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_deriv, st));
+        if ((rc = launch_deriv(h, kCenterDeriv, cp, n_centers, st))) return rc;
     }
     if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
     return SOAP_OK;
@@ -891,7 +940,7 @@ int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_
         cp.row_capacity = capacity_rows;
         cp.out_desc = d_out_desc; cp.out_jac = d_out_jac; cp.row_atom = d_row_atom;
         if (kind == SOAP_ROWS_COMPACT) { cp.compact = 1; cp.out_center = d_out_center; }
-        CU(center_launch(kind == SOAP_ROWS_COEFFICIENTS ? kCenterCoeff : kCenterDeriv, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_deriv, st));
+        if ((rc = launch_deriv(h, kind == SOAP_ROWS_COEFFICIENTS ? kCenterCoeff : kCenterDeriv, cp, n_centers, st))) return rc;
     }
     if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
     CU(cudaStreamSynchronize(st));
@@ -963,9 +1012,7 @@ int soap_set_crossover(soap_t* h, int crossover) {
     build_feature_table(h);
     if (h->tables_ready) {
         CU(cudaDeviceSynchronize());
-        cudaFree(h->d_feat);
-        h->d_feat = nullptr;
-        CU(upload(&h->d_feat, h->feat_pack));
+        if (int rc = upload_features(h)) return rc;
         if (h->d_compact_map) { cudaFree(h->d_compact_map); h->d_compact_map = nullptr; }
     }
     return SOAP_OK;
@@ -1036,7 +1083,7 @@ int soap_coefficient_derivatives(soap_t* h, const float* d_positions, const int3
         cp.row_ptr = (const long long*)d_row_ptr;
         cp.row_capacity = capacity_rows;
         cp.out_desc = d_out_coeff; cp.out_jac = d_out_jac; cp.row_atom = d_row_atom;
-        CU(center_launch(kCenterCoeff, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_deriv, st));
+        if ((rc = launch_deriv(h, kCenterCoeff, cp, n_centers, st))) return rc;
     }
     if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
     return SOAP_OK;
@@ -1111,7 +1158,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
         cp.out_jac = d_out_jac;
         cp.inner_rows = 1;
         cp.own_scale = (float)(1.0 / (double)n_centers);
-        CU(center_launch(kCenterInner, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_deriv, st));
+        CU(center_launch(kCenterInner, h->l_max, h->n_max, kThreads, cp, (unsigned)n_centers, h->smem_deriv, st));
         if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
         return SOAP_OK;
     }
@@ -1136,7 +1183,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
         cp.out_jac = d_out_jac;
         cp.own_scale = (float)(1.0 / (double)n_centers);
         cp.P = h->P_outer;
-        CU(center_launch(kCenterOuter, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_outer, st));
+        CU(center_launch(kCenterOuter, h->l_max, h->n_max, kThreads, cp, (unsigned)n_centers, h->smem_outer, st));
         if ((rc = column_mean(h, (const float*)(w + o_rows), n_centers, F, (double*)(w + o_partial), d_out_desc, st))) return rc;
         if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
         return SOAP_OK;
@@ -1178,7 +1225,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
     } else {
         cp.out_desc = (float*)(w + o_rows);
     }
-    CU(center_launch(kCenterDeriv, h->l_max, h->n_max, cp, (unsigned)n_centers, h->smem_deriv, st));
+    if ((rc = launch_deriv(h, kCenterDeriv, cp, n_centers, st))) return rc;
     if (!inner && (rc = column_mean(h, (const float*)(w + o_rows), n_centers, F, (double*)(w + o_partial), d_out_desc, st))) return rc;
     if (n_atoms > 0) {
         const int width3 = 3 * F;

@@ -7,9 +7,8 @@
 namespace soap {
 
 constexpr int kMaxSpecies = 8;
-constexpr int kThreads = 256;            // CTA size of the per-centre kernels
-constexpr int kWarps = kThreads / 32;
-constexpr int kMaxElemPerThread = 8;     // soap_create refuses n_max (l_max+1)^2 > 8 * kThreads (shared-memory budget of the tiles)
+constexpr int kThreads = 256;            // largest CTA of the per-centre derivative kernels
+constexpr int kMaxElements = 2048;       // soap_create refuses n_max (l_max+1)^2 above this (shared-memory budget of the tiles)
 
 // status bits (device, sticky until soap_status)
 constexpr int kStatusUnknownSpecies = 1;
@@ -65,16 +64,17 @@ struct CenterParams {
     long long pair_capacity, row_capacity;
     Counters* counters;
     // basis
-    const float* table;           // [nint][n_ch][6]
-    const float* table_ln;        // the same polynomials as [nint][l][n / 2][6][2], n padded to a multiple of 4 (descriptor-only kernel)
+    const float* table;           // [nint][l][n / 2][6][2], n padded to even: coefficients of two adjacent n interleaved (derivative kernels)
+    const float* table_ln;        // value polynomials on wider intervals as [nint][l][n / 2][6][2], n padded to a multiple of 4 (descriptor-only kernel)
     const float* self_term;       // [n_max]
     const int* l_of_lm;           // [lm] -> l
     const float* kl;
+    const unsigned* row_ops;      // [S][F] or null: operands of feature f in the row of a neighbour of species s: g | g' << 8 | u << 16 | u' << 24
     const int* feat_pack;         // [F] n | n'<<5 | mu<<10 | nu<<14 | l<<18
     double inv_h;                 // intervals per Angstrom of the radial table in use
     int n_intervals;
     int S, n_max, l_max, F;
-    int P;                        // pairs per staged chunk (<= 32)
+    int P;                        // pairs per staged chunk
     unsigned nch_magic;           // floor(2^32 / (n_max (l_max+1))) + 1: x / n_ch == umulhi(x, magic) for x < 65536
     // output mode
     int crossover;                // 0: only the species pairs mu == nu are features
@@ -136,10 +136,11 @@ __host__ __device__ inline void key_shift(unsigned long long k, int s[3]) {
 // single bank.
 constexpr int kGeoPairs = 128;           // pairs whose geometry is staged at once
 
-constexpr int kZeroWords = 1024;         // a block of zeros that bulk copies write into the structural-zero blocks of the rows
+constexpr int kMaxZeroWords = 1024;      // largest block of zeros that bulk copies write into the structural-zero blocks of the rows
 
 struct SmemLayout {
-    int c, geo, tri, xdec, zero, D, wUV, sSD, sG, total;
+    int c, geo, tri, xdec, zero, D, wUV, sSD, sG, slab, slab_words, total;
+    bool keep;                    // the slab is apart from the staging area: what pass 1 staged is still there in pass 2
 };
 // whether the cross-species blocks of the rows are written in table-driven sweeps (a decode table in shared
 // memory): several species, n_max from 9 to 12 and n_max (l_max+1) not a multiple of four (the other cases have
@@ -149,24 +150,47 @@ __host__ __device__ inline bool cross_table_wanted(int S, int n_max, int l_max) 
 }
 __host__ __device__ inline int align4(int x) { return (x + 3) & ~3; }
 constexpr int kGeoWords = kGeoPairs * 9 + 44;   // geometry (9 words per pair), species segments (9 + 32 words, padded)
-__host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, int P, bool deriv, bool weighted = false) {
-    const int L1 = l_max + 1, LMP = (L1 * L1) | 1, NCH = n_max * L1, CT = S * n_max * LMP;
+// words of zeros: the largest block (two species, all n, n', l), when there is more than one species
+__host__ __device__ inline int zero_words(int S, int n_max, int l_max) {
+    const int block = align4(n_max * n_max * (l_max + 1));
+    return S == 1 ? 0 : block < kMaxZeroWords ? block : kMaxZeroWords;
+}
+// Pass 1 of the per-centre kernel: threads that cover the lm index, and groups of them that split the n index.
+__host__ __device__ constexpr int pass1_span(int l_max) {
+    const int lm = (l_max + 1) * (l_max + 1);
+    return lm <= 8 ? 8 : lm <= 16 ? 16 : (lm + 31) / 32 * 32;
+}
+__host__ __device__ constexpr int pass1_slots(int l_max, int n_max) {
+    const int span = pass1_span(l_max), most = span <= 32 ? 64 / span : span <= 64 ? 2 : 256 / span;
+    const int want = l_max >= 8 && n_max < 4 ? 1 : l_max <= 3 ? n_max : (n_max + 1) / 2;
+    return want < most ? want : most;
+}
+// Bases whose Jacobian rows are written with the operands of every feature from a table (up to kKeepFeatures features).
+__host__ __device__ constexpr bool row_table_wanted(int n_max, int l_max) { return n_max <= 4 && n_max * (l_max + 1) <= 20; }
+// Features up to which the slab of the power spectrum has room of its own beside the staging area (16 bytes each).
+constexpr int kKeepFeatures = 512;
+__host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, int P, int warps, bool weighted) {
+    const int L1 = l_max + 1, LMP = (L1 * L1) | 1, NCH = n_max * L1, CT = S * n_max * LMP, F = S * n_max * (S * n_max + 1) / 2 * L1;
     SmemLayout o;
     int off = 0;
     o.c = off; off = align4(off + CT);
     o.geo = off; off = align4(off + kGeoWords + (weighted ? 2 * kGeoPairs : 0));   // + per-pair weights
-    o.tri = off; if (deriv) off = align4(off + ((n_max * (n_max + 1) / 2) * L1 + 1) / 2);   // 16-bit entries
-    o.xdec = off; if (deriv && cross_table_wanted(S, n_max, l_max)) off = align4(off + (n_max * NCH + 1) / 2);   // 16-bit entries
-    o.zero = off; if (deriv) off += kZeroWords;
+    o.tri = off; off = align4(off + ((n_max * (n_max + 1) / 2) * L1 + 1) / 2);   // 16-bit entries
+    o.xdec = off; if (cross_table_wanted(S, n_max, l_max)) off = align4(off + (n_max * NCH + 1) / 2);   // 16-bit entries
+    o.zero = off; off += zero_words(S, n_max, l_max);
     // the D tiles (pass 1, centre's row) and the per-warp U/V staging (pass 2) never live
     // at the same time and share space
     o.D = off; o.wUV = off;
-    if (deriv) {
-        const int a = 3 * CT, b = kWarps * S * NCH * 4;
+    {
+        const int a = 3 * CT, b = warps * S * NCH * 4;
         off = align4(off + (a > b ? a : b));
     }
-    o.sSD = off; off = align4(off + (deriv ? P * LMP * 4 : P * LMP));
-    o.sG = off; off = align4(off + (deriv ? P * NCH * 2 : P * NCH));
+    o.keep = F <= kKeepFeatures;
+    o.slab = off;
+    if (o.keep) { o.slab_words = 4 * F; off += 4 * F; }
+    o.sSD = off; off = align4(off + P * LMP * 4);
+    o.sG = off; off = align4(off + P * (NCH + (row_table_wanted(n_max, l_max) ? 1 : 0)) * 2);
+    if (!o.keep) o.slab_words = off - o.slab;
     o.total = off;
     return o;
 }
