@@ -113,23 +113,30 @@ int soap_neighbors(soap_t *h, const float *d_positions, const int32_t *d_numbers
                    const double *cell, const int32_t *d_centers, int64_t n_centers,
                    int64_t *n_pairs, int64_t *n_rows, void *stream);
 
-/* The two halves of a derivative call whose outputs the caller sizes exactly:
- * soap_search is soap_neighbors that also writes the row pointers of the
- * caller (d_row_ptr [n_centers+1]) and returns a device-side error at once
- * (and clears it); soap_derivatives_found then computes the derivatives of
- * what that search found, without searching again, and WAITS for the stream.
- * Both calls get the same structure (positions and centres unchanged, numbers
- * as well), and no other call on the handle comes between them.
+/* The parts of a derivative call whose outputs the caller sizes exactly.
+ * soap_search_start enqueues a neighbour search that also writes the caller's
+ * row pointers (d_row_ptr [n_centers+1]) and returns without waiting for it
+ * (the caller can allocate the outputs whose size it knows meanwhile);
+ * soap_search_finish, with the same arguments, WAITS, returns the totals like
+ * soap_neighbors (a search that met more pairs than the scratch holds is run
+ * again) and reports a device-side error at once (and clears it);
+ * soap_derivatives_found computes the derivatives of what that search found,
+ * without searching again, and WAITS for the stream.  All three get the same
+ * structure (positions and centres unchanged, numbers as well), and no other
+ * call on the handle comes between them.
  *   d_centers / d_sites   as in soap_derivatives / soap_derivatives_at (at most one of them)
  *   d_struct_ptr          as in soap_derivatives_batch, or NULL (one structure)
  *   kind                  what is written, as by soap_derivatives (SOAP_ROWS_FULL),
  *                         soap_derivatives_compact (d_out_center is used by this one only)
  *                         or soap_coefficient_derivatives */
 enum { SOAP_ROWS_FULL = 0, SOAP_ROWS_COMPACT = 1, SOAP_ROWS_COEFFICIENTS = 2 };
-int soap_search(soap_t *h, const float *d_positions, const int32_t *d_numbers, int64_t n_atoms,
-                const double *cell, const int32_t *d_centers, const float *d_sites, int64_t n_centers,
-                const int64_t *d_struct_ptr, int64_t n_structs,
-                int64_t *d_row_ptr, int64_t *n_pairs, int64_t *n_rows, void *stream);
+int soap_search_start(soap_t *h, const float *d_positions, const int32_t *d_numbers, int64_t n_atoms,
+                      const double *cell, const int32_t *d_centers, const float *d_sites, int64_t n_centers,
+                      const int64_t *d_struct_ptr, int64_t n_structs, int64_t *d_row_ptr, void *stream);
+int soap_search_finish(soap_t *h, const float *d_positions, const int32_t *d_numbers, int64_t n_atoms,
+                       const double *cell, const int32_t *d_centers, const float *d_sites, int64_t n_centers,
+                       const int64_t *d_struct_ptr, int64_t n_structs, int64_t *d_row_ptr,
+                       int64_t *n_pairs, int64_t *n_rows, void *stream);
 int soap_derivatives_found(soap_t *h, int kind, const float *d_positions, int64_t n_atoms, const double *cell,
                            const int32_t *d_centers, const float *d_sites, int64_t n_centers,
                            float *d_out_desc, float *d_out_center, float *d_out_jac, int64_t capacity_rows,

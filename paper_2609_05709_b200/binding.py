@@ -20,7 +20,7 @@ EXPORTED_SYMBOLS = [
     "soap_neighbors_at", "soap_descriptor_at", "soap_derivatives_at",
     "soap_rows_dense", "soap_neighbors_batch", "soap_descriptor_batch", "soap_derivatives_batch",
     "soap_num_compact_features", "soap_compact_feature_map", "soap_derivatives_compact", "soap_compact_expand",
-    "soap_measure_fp32_peak", "soap_search", "soap_derivatives_found",
+    "soap_measure_fp32_peak", "soap_search_start", "soap_search_finish", "soap_derivatives_found",
 ]
 
 ROWS_FULL, ROWS_COMPACT, ROWS_COEFFICIENTS = 0, 1, 2
@@ -80,7 +80,9 @@ def load_library() -> C.CDLL:
     lib.soap_neighbors_batch.argtypes = [vp, vp, vp, i64, vp, i64, C.POINTER(i64), C.POINTER(i64), vp]
     lib.soap_descriptor_batch.argtypes = [vp, vp, vp, i64, vp, i64, vp, vp]
     lib.soap_derivatives_batch.argtypes = [vp, vp, vp, i64, vp, i64, vp, vp, i64, vp, vp, vp]
-    lib.soap_search.argtypes = [vp, vp, vp, i64, C.POINTER(C.c_double), vp, vp, i64, vp, i64, vp, C.POINTER(i64), C.POINTER(i64), vp]
+    found = [vp, vp, vp, i64, C.POINTER(C.c_double), vp, vp, i64, vp, i64, vp]
+    lib.soap_search_start.argtypes = found + [vp]
+    lib.soap_search_finish.argtypes = found + [C.POINTER(i64), C.POINTER(i64), vp]
     lib.soap_derivatives_found.argtypes = [vp, i32, vp, i64, C.POINTER(C.c_double), vp, vp, i64, vp, vp, vp, i64, vp, vp, vp]
     lib.soap_set_crossover.argtypes = [vp, i32]
     lib.soap_set_weighting.argtypes = [vp, i32] + [C.c_double] * 5
@@ -198,8 +200,11 @@ class Soap:
 
     @staticmethod
     def _stream():
+        # the current stream of the current device, as a number: making a torch.cuda.Stream object for it costs as much as
+        # a launch
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
 
     @staticmethod
     def _cell(cell):
@@ -283,21 +288,25 @@ class Soap:
             c, sptr = sites.shape[0], sites.data_ptr()
         if struct_ptr is not None:
             bptr, n_structs = struct_ptr.data_ptr(), struct_ptr.shape[0] - 1
-        dev, stream, pos = positions.device, self._stream(), positions.data_ptr()
+        dev, stream, pos, lib = positions.device, self._stream(), positions.data_ptr(), self._lib
         row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
-        npairs, nrows = C.c_int64(), C.c_int64()
-        self._check(self._lib.soap_search(self._h, pos, numbers.data_ptr(), n, cellp, cptr, sptr, c, bptr, n_structs,
-                                          row_ptr.data_ptr(), C.byref(npairs), C.byref(nrows), stream))
-        rows = nrows.value
+        search = (self._h, pos, numbers.data_ptr(), n, cellp, cptr, sptr, c, bptr, n_structs, row_ptr.data_ptr())
+        self._check(lib.soap_search_start(*search, stream))
+        # the outputs whose size is known, while the search runs
         compact = kind == ROWS_COMPACT
         values = torch.empty((c, self.n_coefficients if kind == ROWS_COEFFICIENTS else self.n_features), dtype=torch.float32, device=dev)
         center_rows = torch.empty((c, 3, self.n_features), dtype=torch.float32, device=dev) if compact else None
+        npairs, nrows = C.c_int64(), C.c_int64()
+        self._check(lib.soap_search_finish(*search, C.byref(npairs), C.byref(nrows), stream))
+        rows = nrows.value
         jac = torch.empty((max(rows, 1), 3, width), dtype=torch.float32, device=dev)
         row_atom = torch.empty(max(rows, 1), dtype=torch.int32, device=dev)
-        self._check(self._lib.soap_derivatives_found(self._h, kind, pos, n, cellp, cptr, sptr, c, values.data_ptr(),
-                                                     center_rows.data_ptr() if compact else None, jac.data_ptr(), jac.shape[0],
-                                                     row_ptr.data_ptr(), row_atom.data_ptr(), stream))
-        return values, center_rows, jac[:rows], row_ptr, row_atom[:rows]
+        self._check(lib.soap_derivatives_found(self._h, kind, pos, n, cellp, cptr, sptr, c, values.data_ptr(),
+                                               center_rows.data_ptr() if compact else None, jac.data_ptr(), jac.shape[0],
+                                               row_ptr.data_ptr(), row_atom.data_ptr(), stream))
+        if rows == 0:
+            jac, row_atom = jac[:0], row_atom[:0]
+        return values, center_rows, jac, row_ptr, row_atom
 
     def derivatives(self, positions, numbers, cell=None, centers=None) -> Derivatives:
         """Sizes the Jacobian with one neighbour search, then computes it."""

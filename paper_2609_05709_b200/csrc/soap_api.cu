@@ -126,7 +126,8 @@ struct soap_handle {
     int64_t last_centers = 0;
     bool list_sorted = false;            // whether the pair list of the last search is sorted (descriptor-only calls skip that)
     bool ordered = false;                // whether the last search with rows left a launch order
-    int64_t found_atoms = -1, found_centers = -1;   // sizes of the search soap_search left for soap_derivatives_found; -1: none
+    int64_t started_atoms = -1, started_centers = -1;   // sizes of the search soap_search_start left for soap_search_finish; -1: none
+    int64_t found_atoms = -1, found_centers = -1;   // sizes of the search soap_search_finish left for soap_derivatives_found; -1: none
     int P_deriv4 = 16;                   // ... with CTAs of 128 threads
     size_t smem_deriv4 = 0;
     int P_deriv = 16, P_outer = 16;      // pairs per staged chunk: derivative kernels, kernel of the outer average
@@ -393,7 +394,7 @@ struct Batch {
 int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g,
                      const int32_t* centers, const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st,
                      const Batch& batch = Batch(), bool rows = true, bool publish = false) {
-    h->found_atoms = h->found_centers = -1;
+    h->found_atoms = h->found_centers = h->started_atoms = h->started_centers = -1;
     Counters* const host = publish ? h->h_counters : nullptr;
     // A small non-periodic structure with every atom a centre is searched by brute force, without a cell list.
     // (C == N: the brute-force kernel writes the per-centre arrays for every atom, and those are sized from C)
@@ -478,12 +479,17 @@ int check_inputs(soap_t* h, const float* pos, const int32_t* num, int64_t N, con
 // kernel of the search, so that the host waits for the stream and nothing else.  (A call that sizes its own outputs used
 // to search three times and wait five times; searching once took the 24-atom call from 129 to 65 us and the call on
 // 3000 atoms with 274 neighbours each from 1712 to 1374 us.)
+// A caller with something else to do meanwhile takes it in two steps: `start` enqueues the search, `finish` (the same
+// arguments) waits for it.
+enum class Search { whole, start, finish };
 int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g, const int32_t* centers,
-                    const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st, const Batch& batch = Batch()) {
+                    const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st, const Batch& batch = Batch(),
+                    Search step = Search::whole) {
     int rc = ensure_scratch(h, N, C, 0, st);
     if (rc) return rc;
     for (int attempt = 0; attempt < 2; ++attempt) {
-        if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
+        if ((step != Search::finish || attempt > 0) && (rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
+        if (step == Search::start) return SOAP_OK;
         CU(cudaStreamSynchronize(st));
         const int64_t pairs = h->h_counters->n_pairs;
         h->pairs_per_center_hint = C > 0 ? (pairs + C - 1) / C : 0;
@@ -743,7 +749,7 @@ int soap_radial_table(const soap_t* h, double d, double* G, double* Ghat) {
 
 static int neighbors_impl(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
                           const int32_t* d_centers, const float* d_sites, int64_t n_centers, int64_t* n_pairs, int64_t* n_rows,
-                          void* stream, const Batch& batch = Batch(), long long* row_ptr_out = nullptr) {
+                          void* stream, const Batch& batch = Batch(), long long* row_ptr_out = nullptr, Search step = Search::whole) {
     int rc = check_inputs(h, d_positions, d_numbers, n_atoms, d_centers, n_centers, d_sites);
     if (rc) return rc;
     if (batch.struct_ptr && (h->pbc[0] || h->pbc[1] || h->pbc[2]))
@@ -751,7 +757,7 @@ static int neighbors_impl(soap_t* h, const float* d_positions, const int32_t* d_
     if ((rc = ensure_device(h))) return rc;
     Geometry g;
     if ((rc = make_geometry(h, cell, g))) return rc;
-    if ((rc = search_and_size(h, d_positions, d_numbers, n_atoms, g, d_centers, d_sites, n_centers, row_ptr_out, (cudaStream_t)stream, batch))) return rc;
+    if ((rc = search_and_size(h, d_positions, d_numbers, n_atoms, g, d_centers, d_sites, n_centers, row_ptr_out, (cudaStream_t)stream, batch, step))) return rc;
     if (n_pairs) *n_pairs = h->h_counters->n_pairs;
     if (n_rows) *n_rows = h->h_counters->n_rows;
     return SOAP_OK;
@@ -895,9 +901,9 @@ int soap_derivatives_batch(soap_t* h, const float* d_positions, const int32_t* d
 }
 
 // ---- a search, then the derivatives of what it found ----
-int soap_search(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
-                const int32_t* d_centers, const float* d_sites, int64_t n_centers, const int64_t* d_struct_ptr, int64_t n_structs,
-                int64_t* d_row_ptr, int64_t* n_pairs, int64_t* n_rows, void* stream) {
+static int search_impl(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
+                       const int32_t* d_centers, const float* d_sites, int64_t n_centers, const int64_t* d_struct_ptr, int64_t n_structs,
+                       int64_t* d_row_ptr, int64_t* n_pairs, int64_t* n_rows, void* stream, Search step) {
     if (h && !d_row_ptr) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
     if (h && d_struct_ptr && (d_centers || d_sites || n_centers != n_atoms))
         return fail(h, SOAP_ERR_INVALID_ARG, "in a batch of structures every atom is a centre");
@@ -906,7 +912,28 @@ int soap_search(soap_t* h, const float* d_positions, const int32_t* d_numbers, i
     b.n_structs = n_structs;
     int rc = d_struct_ptr ? check_batch(h, d_struct_ptr, n_structs, n_atoms) : SOAP_OK;
     if (rc) return rc;
-    if ((rc = neighbors_impl(h, d_positions, d_numbers, n_atoms, cell, d_centers, d_sites, n_centers, n_pairs, n_rows, stream, b, (long long*)d_row_ptr))) return rc;
+    return neighbors_impl(h, d_positions, d_numbers, n_atoms, cell, d_centers, d_sites, n_centers, n_pairs, n_rows, stream, b, (long long*)d_row_ptr, step);
+}
+
+int soap_search_start(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
+                      const int32_t* d_centers, const float* d_sites, int64_t n_centers, const int64_t* d_struct_ptr, int64_t n_structs,
+                      int64_t* d_row_ptr, void* stream) {
+    const int rc = search_impl(h, d_positions, d_numbers, n_atoms, cell, d_centers, d_sites, n_centers, d_struct_ptr, n_structs, d_row_ptr,
+                               nullptr, nullptr, stream, Search::start);
+    if (!rc) { h->started_atoms = n_atoms; h->started_centers = n_centers; }
+    return rc;
+}
+
+int soap_search_finish(soap_t* h, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
+                       const int32_t* d_centers, const float* d_sites, int64_t n_centers, const int64_t* d_struct_ptr, int64_t n_structs,
+                       int64_t* d_row_ptr, int64_t* n_pairs, int64_t* n_rows, void* stream) {
+    if (!h) return SOAP_ERR_INVALID_ARG;
+    if (h->started_atoms != n_atoms || h->started_centers != n_centers)
+        return fail(h, SOAP_ERR_INVALID_ARG, "no search of this size is under way: call soap_search_start first");
+    int rc = search_impl(h, d_positions, d_numbers, n_atoms, cell, d_centers, d_sites, n_centers, d_struct_ptr, n_structs, d_row_ptr, n_pairs,
+                         n_rows, stream, Search::finish);
+    h->started_atoms = h->started_centers = -1;
+    if (rc) return rc;
     if (h->h_counters->status) {
         CU(cudaMemsetAsync(&h->d_counters->status, 0, sizeof(int), (cudaStream_t)stream));
         return status_error(h, h->h_counters->status);
@@ -921,7 +948,7 @@ int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_
     if (!h) return SOAP_ERR_INVALID_ARG;
     if (kind != SOAP_ROWS_FULL && kind != SOAP_ROWS_COMPACT && kind != SOAP_ROWS_COEFFICIENTS) return fail(h, SOAP_ERR_INVALID_ARG, "unknown kind of rows");
     if (h->found_atoms != n_atoms || h->found_centers != n_centers)
-        return fail(h, SOAP_ERR_INVALID_ARG, "no neighbour search of this size is at hand: call soap_search first");
+        return fail(h, SOAP_ERR_INVALID_ARG, "no neighbour search of this size is at hand: call soap_search_start and soap_search_finish first");
     if (!d_row_ptr || capacity_rows < 0) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
     if (n_centers > 0 && (!d_out_desc || !d_out_jac || !d_row_atom)) return fail(h, SOAP_ERR_INVALID_ARG, "output pointers must not be NULL");
     if (n_centers > 0 && kind == SOAP_ROWS_COMPACT && !d_out_center) return fail(h, SOAP_ERR_INVALID_ARG, "d_out_center must not be NULL");

@@ -1,5 +1,5 @@
-"""The search whose totals come back to the host, and the derivatives of what it found (soap_search,
-soap_derivatives_found), through the calls of the binding that size their own outputs."""
+"""The search whose totals come back to the host, and the derivatives of what it found (soap_search_start,
+soap_search_finish, soap_derivatives_found), through the calls of the binding that size their own outputs."""
 import numpy as np
 import pytest
 
@@ -78,16 +78,23 @@ def test_derivatives_of_a_search_need_that_search(pkg):
         soap._check(soap._lib.soap_derivatives_found(soap._h, 0, pos.data_ptr(), n, cellp, None, None, n, out.data_ptr(), None,
                                                      out.data_ptr(), 1, out.data_ptr(), out.data_ptr(), soap._stream()))
 
-    with pytest.raises(pkg.SoapError) as e:               # no search yet
-        found(60)
-    assert e.value.code == -1
+    def finish(n):
+        out64 = torch.empty(n + 1, dtype=torch.int64, device="cuda")
+        soap._check(soap._lib.soap_search_finish(soap._h, pos.data_ptr(), num.data_ptr(), n, cellp, None, None, n, None, 0,
+                                                 out64.data_ptr(), None, None, soap._stream()))
+
+    for call in (found, finish):
+        with pytest.raises(pkg.SoapError) as e:           # no search yet
+            call(60)
+        assert e.value.code == -1
     soap.derivatives(pos, num, s.cell)
     with pytest.raises(pkg.SoapError):                     # a search of another size
         found(59)
     soap.derivatives(pos, num, s.cell)
     soap.descriptor(pos, num, s.cell)                      # a call in between
-    with pytest.raises(pkg.SoapError):
-        found(60)
+    for call in (found, finish):
+        with pytest.raises(pkg.SoapError):
+            call(60)
 
 
 def all_pairs(pos, r_cut):
