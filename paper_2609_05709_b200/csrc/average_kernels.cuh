@@ -16,6 +16,7 @@ column_partial_kernel(const float* __restrict__ in, long long rows, int width, l
     if (col >= width) return;
     const long long r0 = (long long)blockIdx.y * chunk_rows, r1 = min(rows, r0 + chunk_rows);
     double s = 0.0;
+#pragma unroll 8
     for (long long r = r0; r < r1; ++r) s += (double)in[r * width + col];
     partial[(size_t)blockIdx.y * width + col] = s;
 }
@@ -26,6 +27,7 @@ column_finish_kernel(const double* __restrict__ partial, int chunks, int width, 
     const int col = blockIdx.x * kMeanThreads + threadIdx.x;
     if (col >= width) return;
     double s = 0.0;
+#pragma unroll 16
     for (int c = 0; c < chunks; ++c) s += partial[(size_t)c * width + col];
     out[col] = (float)(s * scale);
 }
