@@ -261,135 +261,19 @@ __global__ void bin_fill_kernel(const float* __restrict__ pos, long long N, cons
     }
 }
 
-// Small structures: species lookup, bounding box, grid choice, binning, bin scan and the sort of
-// the atoms by bin in ONE launch of a single CTA (five dependent launches otherwise; at a few
-// thousand atoms the launches, not the work, set the time).
-constexpr int kPrepThreads = 1024;
-constexpr long long kSmallPrepAtoms = 4096;
+// Species lookup, bounding box, grid choice, binning, bin scan and the sort of the atoms by bin in ONE launch (seven
+// dependent launches otherwise; up to some ten thousand atoms the launches, not the work, set the time): of a single CTA
+// up to kSmallPrepAtoms, bin counters on chip as long as they fit; of a thread-block cluster up to kPrepAtoms, whose CTAs
+// exchange the bounding box and the totals of the bin scan through each other's shared memory, bin counters in global
+// memory, zero before and after the call (the scan clears what it reads).  A thread keeps its atoms' positions, bins and
+// places in registers through the phases; without a free axis there is no bounding box to form (whole search of 431
+// atoms in a periodic box 22.2 -> 17.9 us with the pair kernel's loads ahead, 3000 atoms of water 25.5 -> 23.9 us).  At
+// 4096 atoms and below the cluster is no faster (1111 atoms 11.0 against 12.0 us, 3000 atoms 14.5 us both); at 30,000
+// atoms it takes 20 us, the seven launches 31 us and their gaps.
+constexpr int kPrepThreads = 1024, kPrepCtas = 8, kPrepPerThread = 8, kSmallPrepPerThread = 4;
+constexpr long long kPrepAtoms = (long long)kPrepThreads * kPrepCtas * kPrepPerThread, kSmallPrepAtoms = (long long)kPrepThreads * kSmallPrepPerThread;
 constexpr int kPrepSmemCells = 4096;
-__global__ void __launch_bounds__(kPrepThreads)
-small_prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long long N, Geometry geom,
-                  const int* __restrict__ z_lut, int* __restrict__ species_idx, int cell_cap, GridParams* grid_out,
-                  int* __restrict__ atom_cell, int* __restrict__ atom_wrap, int* cell_count, int* cell_start,
-                  float4* __restrict__ s_pos, int* __restrict__ s_wrap, Counters* counters) {
-    __shared__ double red[6][32];
-    __shared__ GridParams sg;
-    __shared__ long long warp_sums[32];
-    __shared__ long long carry_s;
-    __shared__ int s_cnt[kPrepSmemCells + 1], s_start[kPrepSmemCells + 1];   // bin counters on chip when they fit
-    grid_dependency_launch();                                                // the pair kernel may move in and wait
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    // ---- species and bounding box of the fractional coordinates ----
-    double hi[3] = {-1e300, -1e300, -1e300}, lo[3] = {-1e300, -1e300, -1e300};
-    bool bad = false;
-    for (long long i = tid; i < N; i += kPrepThreads) {
-        int z = numbers ? numbers[i] : 0;
-        int s = numbers ? ((z >= 0 && z < 128) ? z_lut[z] : -1) : 0;
-        if (s < 0) { bad = true; s = 0; }
-        if (species_idx) species_idx[i] = s;
-        double f[3];
-        frac_coords(geom, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], f);
-        for (int a = 0; a < 3; ++a) { hi[a] = fmax(hi[a], f[a]); lo[a] = fmax(lo[a], -f[a]); }
-    }
-    if (bad) atomicOr(&counters->status, kStatusUnknownSpecies);
-    for (int a = 0; a < 3; ++a) {
-        for (int o = 16; o > 0; o >>= 1) {
-            hi[a] = fmax(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-            lo[a] = fmax(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-        }
-        if (lane == 0) { red[a][wid] = hi[a]; red[3 + a][wid] = lo[a]; }
-    }
-    __syncthreads();
-    if (wid == 0) {
-        // the 32 warps' maxima, one per lane
-        for (int a = 0; a < 6; ++a) {
-            double v = red[a][lane];
-            for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (lane == 0) red[a][0] = v;
-        }
-    }
-    __syncthreads();
-    if (wid == 0) {
-        const int a = min(lane, 2);
-        choose_grid(red[a][0], -red[3 + a][0], geom, N, cell_cap, &sg);
-        if (lane == 0) {
-            *grid_out = sg;
-            carry_s = 0;
-            counters->n_pairs = 0;                                            // the pair cursor of this call
-            counters->n_rows = 0;
-        }
-    }
-    __syncthreads();
-    const GridParams g = sg;
-    const bool on_chip = g.n_cells <= kPrepSmemCells;
-    int* cnt = on_chip ? s_cnt : cell_count;
-    // ---- bin counts ----
-    for (int c = tid; c <= g.n_cells; c += kPrepThreads) cnt[c] = 0;
-    __syncthreads();
-    for (long long i = tid; i < N; i += kPrepThreads) {
-        int b[3], w[3];
-        bin_of(geom, g, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], b, w);
-        if (abs(w[0]) > 100 || abs(w[1]) > 100 || abs(w[2]) > 100) {
-            atomicOr(&counters->status, kStatusShiftRange);
-            w[0] = w[1] = w[2] = 0;
-        }
-        const int cell = (b[2] * g.nb[1] + b[1]) * g.nb[0] + b[0];
-        atom_cell[i] = cell;
-        atom_wrap[i] = pack3(w);
-        atomicAdd(&cnt[cell], 1);
-    }
-    __syncthreads();
-    // ---- exclusive scan of the bin counts ----
-    for (int base = 0; base < g.n_cells; base += kPrepThreads) {
-        const int i = base + tid;
-        const long long v = i < g.n_cells ? (long long)cnt[i] : 0;
-        long long x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) warp_sums[wid] = x;
-        __syncthreads();
-        if (wid == 0) {
-            long long sacc = warp_sums[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long y = __shfl_up_sync(0xffffffffu, sacc, o);
-                if (lane >= o) sacc += y;
-            }
-            warp_sums[lane] = sacc;
-        }
-        __syncthreads();
-        const long long carry = carry_s;
-        if (i < g.n_cells) {
-            const int st = (int)(carry + (wid > 0 ? warp_sums[wid - 1] : 0) + x - v);
-            cell_start[i] = st;
-            if (on_chip) s_start[i] = st;
-        }
-        __syncthreads();
-        if (tid == kPrepThreads - 1) carry_s = carry + warp_sums[31];
-        __syncthreads();
-    }
-    if (tid == 0) cell_start[g.n_cells] = (int)carry_s;
-    __syncthreads();
-    // ---- atoms sorted by bin ----
-    const int* starts = on_chip ? s_start : cell_start;
-    for (long long i = tid; i < N; i += kPrepThreads) {
-        const int cell = atom_cell[i];
-        const int slot = starts[cell] + atomicSub(&cnt[cell], 1) - 1;
-        s_pos[slot] = make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __int_as_float((int)i));
-        s_wrap[slot] = atom_wrap[i];
-    }
-}
-
-// Structures of kSmallPrepAtoms to kPrepAtoms atoms: the same steps, species lookup, bounding box, grid choice, binning, bin scan and the sort of
-// the atoms by bin, in ONE launch of a thread-block cluster (seven dependent launches otherwise; up to some ten thousand
-// atoms the launches, not the work, set the time).  The CTAs exchange the bounding box and the totals of the bin scan
-// through each other's shared memory; the bin counters are in global memory, zero before and after the call (the scan
-// clears what it reads).  Below kSmallPrepAtoms one CTA with its counters on chip is as fast or faster (1111 atoms 11.0
-// against 12.0 us, 3000 atoms 14.5 us both); at 30,000 atoms this takes 20 us, the seven launches 31 us and
-// their gaps.
-constexpr int kPrepCtas = 8, kPrepPerThread = 8;
-constexpr long long kPrepAtoms = (long long)kPrepThreads * kPrepCtas * kPrepPerThread;
+template <bool CLUSTER, int PER_THREAD>
 __global__ void __launch_bounds__(kPrepThreads)
 prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long long N, Geometry geom,
             const int* __restrict__ z_lut, int* __restrict__ species_idx, int cell_cap, GridParams* grid_out,
@@ -400,42 +284,68 @@ prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long
     __shared__ double red[6][32], box[6];
     __shared__ GridParams sg;
     __shared__ int warp_sums[32], cta_total;
+    __shared__ int s_count[CLUSTER ? 1 : kPrepSmemCells];
     grid_dependency_launch();                                                // the pair kernel may move in and wait
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
+    const int rank = CLUSTER ? (int)cluster.block_rank() : 0, ctas = CLUSTER ? (int)cluster.num_blocks() : 1;
     const int stride = ctas * kPrepThreads, first = rank * kPrepThreads + tid, n = (int)N;
+    if (!CLUSTER)
+        for (int c = tid; c < kPrepSmemCells; c += kPrepThreads) s_count[c] = 0;
     // ---- species and bounding box of the fractional coordinates ----
-    double m[6] = {-1e300, -1e300, -1e300, -1e300, -1e300, -1e300};           // max s, max -s
+    // (with more than four atoms per thread the positions do not fit the registers and are read again)
+    constexpr int KEPT = PER_THREAD <= 4 ? PER_THREAD : 1;
+    float x[KEPT], y[KEPT], z[KEPT];
+    auto position = [&](int k, int i, float& px, float& py, float& pz) {
+        if (PER_THREAD <= 4) { px = x[k % KEPT]; py = y[k % KEPT]; pz = z[k % KEPT]; }
+        else { px = pos[3 * i]; py = pos[3 * i + 1]; pz = pos[3 * i + 2]; }
+    };
     bool bad = false;
-    for (int i = first; i < n; i += stride) {
-        const int z = numbers[i];
-        int s = (z >= 0 && z < 128) ? z_lut[z] : -1;
-        if (s < 0) { bad = true; s = 0; }
-        species_idx[i] = s;
-        double f[3];
-        frac_coords(geom, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], f);
-        for (int a = 0; a < 3; ++a) { m[a] = fmax(m[a], f[a]); m[3 + a] = fmax(m[3 + a], -f[a]); }
+#pragma unroll
+    for (int k = 0; k < PER_THREAD; ++k) {
+        const int i = first + k * stride;
+        x[k % KEPT] = y[k % KEPT] = z[k % KEPT] = 0.f;
+        if (i < n) {
+            if (PER_THREAD <= 4) { x[k % KEPT] = pos[3 * i]; y[k % KEPT] = pos[3 * i + 1]; z[k % KEPT] = pos[3 * i + 2]; }
+            const int number = numbers[i];
+            int s = (number >= 0 && number < 128) ? z_lut[number] : -1;
+            if (s < 0) { bad = true; s = 0; }
+            species_idx[i] = s;
+        }
     }
     if (bad) atomicOr(&counters->status, kStatusUnknownSpecies);
-    for (int a = 0; a < 6; ++a) {
-        for (int o = 16; o > 0; o >>= 1) m[a] = fmax(m[a], __shfl_xor_sync(0xffffffffu, m[a], o));
-        if (lane == 0) red[a][wid] = m[a];
+    const bool free_axis = !(geom.pbc[0] && geom.pbc[1] && geom.pbc[2]);
+    if (free_axis) {
+        double m[6] = {-1e300, -1e300, -1e300, -1e300, -1e300, -1e300};       // max s, max -s
+#pragma unroll
+        for (int k = 0; k < PER_THREAD; ++k)
+            if (first + k * stride < n) {
+                float px, py, pz;
+                position(k, first + k * stride, px, py, pz);
+                double f[3];
+                frac_coords(geom, px, py, pz, f);
+                for (int a = 0; a < 3; ++a) { m[a] = fmax(m[a], f[a]); m[3 + a] = fmax(m[3 + a], -f[a]); }
+            }
+        for (int a = 0; a < 6; ++a) {
+            for (int o = 16; o > 0; o >>= 1) m[a] = fmax(m[a], __shfl_xor_sync(0xffffffffu, m[a], o));
+            if (lane == 0) red[a][wid] = m[a];
+        }
+        __syncthreads();
+        if (wid < 6) {
+            double v = red[wid][lane];
+            for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (lane == 0) box[wid] = v;
+        }
+        if (CLUSTER) cluster.sync(); else __syncthreads();
     }
-    __syncthreads();
-    if (wid < 6) {
-        double v = red[wid][lane];
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (lane == 0) box[wid] = v;
-    }
-    cluster.sync();
     if (wid == 0) {
         // every CTA makes the same choice from the boxes of all of them
         const int a = min(lane, 2);
         double hi = -1e300, lo = -1e300;
-        for (int r = 0; r < ctas; ++r) {
-            const double* other = cluster.map_shared_rank(box, r);
-            hi = fmax(hi, other[a]); lo = fmax(lo, other[3 + a]);
-        }
+        if (free_axis)
+            for (int r = 0; r < ctas; ++r) {
+                const double* other = CLUSTER ? cluster.map_shared_rank(box, r) : box;
+                hi = fmax(hi, other[a]); lo = fmax(lo, other[3 + a]);
+            }
         choose_grid(hi, -lo, geom, N, cell_cap, &sg);
         if (rank == 0 && lane == 0) {
             *grid_out = sg;
@@ -445,66 +355,74 @@ prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long
     }
     __syncthreads();
     const GridParams g = sg;
+    int* const count = !CLUSTER && g.n_cells <= kPrepSmemCells ? s_count : cell_count;
     // ---- bin counts; the count an atom finds is its place within the bin ----
-    int cell[kPrepPerThread], place[kPrepPerThread];
+    int cell[KEPT], place[PER_THREAD];
 #pragma unroll
-    for (int k = 0; k < kPrepPerThread; ++k) {
+    for (int k = 0; k < PER_THREAD; ++k) {
         const int i = first + k * stride;
-        cell[k] = place[k] = 0;
+        cell[k % KEPT] = place[k] = 0;
         if (i < n) {
+            float px, py, pz;
+            position(k, i, px, py, pz);
             int b[3], w[3];
-            bin_of(geom, g, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], b, w);
+            bin_of(geom, g, px, py, pz, b, w);
             if (abs(w[0]) > 100 || abs(w[1]) > 100 || abs(w[2]) > 100) {      // positions absurdly far outside the cell
                 atomicOr(&counters->status, kStatusShiftRange);
                 w[0] = w[1] = w[2] = 0;
             }
-            cell[k] = (b[2] * g.nb[1] + b[1]) * g.nb[0] + b[0];
-            atom_cell[i] = cell[k];
+            const int own = (b[2] * g.nb[1] + b[1]) * g.nb[0] + b[0];
+            if (PER_THREAD <= 4) cell[k % KEPT] = own;
+            atom_cell[i] = own;
             atom_wrap[i] = pack3(w);
-            place[k] = atomicAdd(&cell_count[cell[k]], 1);
+            place[k] = atomicAdd(&count[own], 1);
         }
     }
-    cluster.sync();
+    if (CLUSTER) cluster.sync(); else __syncthreads();
     // ---- exclusive scan of the bin counts: a contiguous range of bins per CTA and per thread ----
     const int per_cta = (g.n_cells + ctas - 1) / ctas, c_end = min(g.n_cells, (rank + 1) * per_cta);
     const int per_thread = (per_cta + kPrepThreads - 1) / kPrepThreads;
     const int c0 = min(c_end, rank * per_cta + tid * per_thread), c1 = min(c_end, c0 + per_thread);
     int mine = 0;
-    for (int c = c0; c < c1; ++c) mine += cell_count[c];
+    for (int c = c0; c < c1; ++c) mine += count[c];
     int incl = mine;
     for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
+        const int up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
     }
     if (lane == 31) warp_sums[wid] = incl;
     __syncthreads();
     if (wid == 0) {
         int w = warp_sums[lane];
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
+            const int up = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += up;
         }
         warp_sums[lane] = w;
         if (lane == 31) cta_total = w;
     }
-    cluster.sync();
+    if (CLUSTER) cluster.sync(); else __syncthreads();
     int at = (wid > 0 ? warp_sums[wid - 1] : 0) + incl - mine;
-    for (int r = 0; r < rank; ++r) at += *cluster.map_shared_rank(&cta_total, r);
+    if (CLUSTER)
+        for (int r = 0; r < rank; ++r) at += *cluster.map_shared_rank(&cta_total, r);
     for (int c = c0; c < c1; ++c) {
-        const int v = cell_count[c];
+        const int v = count[c];
         cell_start[c] = at;
-        cell_count[c] = 0;
+        count[c] = count == s_count ? at : 0;                                // (on chip: the bin's start, for the sort)
         at += v;
     }
     if (rank == 0 && tid == 0) cell_start[g.n_cells] = n;
-    cluster.sync();
+    if (CLUSTER) cluster.sync(); else __syncthreads();
     // ---- atoms sorted by bin ----
+    const int* const start = count == s_count ? s_count : cell_start;
 #pragma unroll
-    for (int k = 0; k < kPrepPerThread; ++k) {
+    for (int k = 0; k < PER_THREAD; ++k) {
         const int i = first + k * stride;
         if (i < n) {
-            const int slot = cell_start[cell[k]] + place[k];
-            s_pos[slot] = make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __int_as_float(i));
+            float px, py, pz;
+            position(k, i, px, py, pz);
+            const int slot = start[PER_THREAD <= 4 ? cell[k % KEPT] : atom_cell[i]] + place[k];
+            s_pos[slot] = make_float4(px, py, pz, __int_as_float(i));
             s_wrap[slot] = atom_wrap[i];
         }
     }
@@ -516,13 +434,44 @@ __device__ inline void wrap_bin(int b, int nb, int& cell, int& image) {
     cell = b - image * nb;
 }
 
+// Whether the atom pj (bin wrap `wrap`, in a bin at image `img`) is a neighbour of the centre, and its key.
+__device__ __forceinline__ bool look_at(const Geometry& geom, bool any_periodic, float4 pj, int wrap, int img, float xi, float yi, float zi,
+                                        const int wi[3], Counters* counters, unsigned long long& key) {
+    int wj[3], im[3];
+    unpack3(wrap, wj);
+    unpack3(img, im);
+    // translation on the raw (unwrapped) inputs
+    const int na = im[0] - wj[0] + wi[0], nb = im[1] - wj[1] + wi[1], nc = im[2] - wj[2] + wi[2];
+    double dx = __dsub_rn((double)pj.x, (double)xi);
+    double dy = __dsub_rn((double)pj.y, (double)yi);
+    double dz = __dsub_rn((double)pj.z, (double)zi);
+    if (any_periodic) {
+        // T = (n_a a + n_b b) + n_c c, each product and sum rounded on its own
+        const double fa = (double)na, fb = (double)nb, fc = (double)nc;
+        double tx = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[0]), __dmul_rn(fb, geom.cell[3])), __dmul_rn(fc, geom.cell[6]));
+        double ty = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[1]), __dmul_rn(fb, geom.cell[4])), __dmul_rn(fc, geom.cell[7]));
+        double tz = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[2]), __dmul_rn(fb, geom.cell[5])), __dmul_rn(fc, geom.cell[8]));
+        dx = __dadd_rn(dx, tx); dy = __dadd_rn(dy, ty); dz = __dadd_rn(dz, tz);
+    }
+    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    bool valid = (d2 < geom.rc2) && (d2 > 0.0);
+    if (valid && (abs(na) > 127 || abs(nb) > 127 || abs(nc) > 127)) {
+        atomicOr(&counters->status, kStatusShiftRange);
+        valid = false;
+    }
+    key = ((unsigned long long)(unsigned)__float_as_int(pj.w) << 24) |
+          ((unsigned long long)(na + 128) << 16) | ((unsigned long long)(nb + 128) << 8) |
+          (unsigned long long)(nc + 128);
+    return valid;
+}
+
 // Calls f(valid, key) for every lane in lock step, over all candidates of one centre.
 // key encodes (atom, lattice translation on the raw inputs); valid says whether this
 // lane holds a pair inside the cutoff.
 // The stencil is walked 32 bins at a time: each lane fetches the atom range of one bin (a single
 // memory round trip for all of them), a warp scan turns the counts into offsets, and the lanes
-// then run over the concatenated candidates, so they stay busy whatever the bin occupancy.
-template <class F>
+// then run over the concatenated candidates, so they stay busy whatever the bin occupancy, AHEAD of them per lane at once.
+template <int AHEAD = 1, class F>
 __device__ inline void for_each_candidate(const Geometry& geom, const GridParams& g, const int* __restrict__ cell_start,
                                           const float4* __restrict__ s_pos, const int* __restrict__ s_wrap,
                                           float xi, float yi, float zi, const int bi[3], const int wi[3],
@@ -556,49 +505,35 @@ __device__ inline void for_each_candidate(const Geometry& geom, const GridParams
             if (lane >= d) incl += y;
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        for (int t0 = 0; t0 < total; t0 += 32) {
-            const int t = t0 + lane;
-            // bin of candidate t: the first lane whose inclusive offset exceeds t (binary search by shuffles)
-            int lo = 0;
-            for (int step = 16; step > 0; step >>= 1) {
-                const int probe = __shfl_sync(0xffffffffu, incl, lo + step - 1);
-                if (probe <= t) lo += step;
-            }
-            lo = min(lo, 31);
-            const int b_incl = __shfl_sync(0xffffffffu, incl, lo), b_cnt = __shfl_sync(0xffffffffu, cnt, lo);
-            const int b_start = __shfl_sync(0xffffffffu, start, lo), b_img = __shfl_sync(0xffffffffu, img, lo);
-            bool valid = false;
-            unsigned long long key = 0;
-            if (t < total) {
-                const int at = b_start + (t - (b_incl - b_cnt));
-                const float4 pj = s_pos[at];
-                int wj[3], im[3];
-                unpack3(s_wrap[at], wj);
-                unpack3(b_img, im);
-                // translation on the raw (unwrapped) inputs
-                const int na = im[0] - wj[0] + wi[0], nb = im[1] - wj[1] + wi[1], nc = im[2] - wj[2] + wi[2];
-                double dx = __dsub_rn((double)pj.x, (double)xi);
-                double dy = __dsub_rn((double)pj.y, (double)yi);
-                double dz = __dsub_rn((double)pj.z, (double)zi);
-                if (any_periodic) {
-                    // T = (n_a a + n_b b) + n_c c, each product and sum rounded on its own
-                    const double fa = (double)na, fb = (double)nb, fc = (double)nc;
-                    double tx = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[0]), __dmul_rn(fb, geom.cell[3])), __dmul_rn(fc, geom.cell[6]));
-                    double ty = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[1]), __dmul_rn(fb, geom.cell[4])), __dmul_rn(fc, geom.cell[7]));
-                    double tz = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[2]), __dmul_rn(fb, geom.cell[5])), __dmul_rn(fc, geom.cell[8]));
-                    dx = __dadd_rn(dx, tx); dy = __dadd_rn(dy, ty); dz = __dadd_rn(dz, tz);
+        for (int t0 = 0; t0 < total; t0 += 32 * AHEAD) {
+            // where the lane's next AHEAD candidates are, and their loads, before any of them is looked at
+            float4 pj[AHEAD];
+            int wrap[AHEAD], b_img[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                const int t = t0 + 32 * u + lane;
+                // bin of candidate t: the first lane whose inclusive offset exceeds t (binary search by shuffles)
+                int lo = 0;
+                for (int step = 16; step > 0; step >>= 1) {
+                    const int probe = __shfl_sync(0xffffffffu, incl, lo + step - 1);
+                    if (probe <= t) lo += step;
                 }
-                const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-                valid = (d2 < geom.rc2) && (d2 > 0.0);
-                if (valid && (abs(na) > 127 || abs(nb) > 127 || abs(nc) > 127)) {
-                    atomicOr(&counters->status, kStatusShiftRange);
-                    valid = false;
+                lo = min(lo, 31);
+                const int b_incl = __shfl_sync(0xffffffffu, incl, lo), b_cnt = __shfl_sync(0xffffffffu, cnt, lo);
+                const int b_start = __shfl_sync(0xffffffffu, start, lo);
+                b_img[u] = __shfl_sync(0xffffffffu, img, lo);
+                if (AHEAD == 1 || t < total) {
+                    const int at = t < total ? b_start + (t - (b_incl - b_cnt)) : 0;
+                    pj[u] = s_pos[at];
+                    wrap[u] = s_wrap[at];
                 }
-                key = ((unsigned long long)(unsigned)__float_as_int(pj.w) << 24) |
-                      ((unsigned long long)(na + 128) << 16) | ((unsigned long long)(nb + 128) << 8) |
-                      (unsigned long long)(nc + 128);
             }
-            f(valid, key);
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                unsigned long long key = 0;
+                const bool valid = t0 + 32 * u + lane < total && look_at(geom, any_periodic, pj[u], wrap[u], b_img[u], xi, yi, zi, wi, counters, key);
+                f(valid, key);
+            }
         }
     }
 }
@@ -685,7 +620,11 @@ constexpr int kFillWarps = 4;
 // word says so; the caller plans again with the totals.
 // ROWS = false (descriptor-only calls, which sum over the pairs in any order and have no Jacobian rows): the keys
 // go out as they were found, unsorted, and the row bookkeeping is left out.
-template <int KEYS, bool ROWS>
+// AHEAD: candidates per lane whose loads are in flight at once where images have to be looked up: one on many centres (the
+// warps hide each other's loads, and more cost registers), four on few, where a call waits for the longest warp (search
+// of 60 atoms in a periodic box 31.6 -> 26.0 us, 431 atoms 21.1 -> 19.6 us, 2000 atoms 27.8 -> 26.0 us, 5000 atoms
+// 35.7 -> 37.7 us).
+template <int KEYS, bool ROWS, int AHEAD>
 __global__ void __launch_bounds__(kFillWarps * 32)
 pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, const float* __restrict__ sites, long long C, Geometry geom,
              const GridParams* __restrict__ gp, const int* __restrict__ atom_cell, const int* __restrict__ atom_wrap,
@@ -730,7 +669,7 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
     };
     const bool runs = !(g.periodic[0] | g.periodic[1] | g.periodic[2]) && g.R[0] <= 1 && g.R[1] <= 1 && g.R[2] <= 1;
     if (runs) for_each_candidate_runs(geom, g, cell_start, s_pos, xi, yi, zi, bi, lane, collect);
-    else for_each_candidate(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, collect);
+    else for_each_candidate<AHEAD>(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, collect);
     long long base = 0;
     if (lane == 0) base = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&counters->n_pairs), (unsigned long long)k);
     base = __shfl_sync(0xffffffffu, base, 0);

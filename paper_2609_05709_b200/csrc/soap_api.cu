@@ -413,12 +413,10 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
         if (N > 0) batch_pairs_kernel<<<(unsigned)((N + kFillWarps - 1) / kFillWarps), kFillWarps * 32, 0, st>>>(
             pos, num, h->d_zlut, h->d_species_idx, batch.struct_ptr, batch.n_structs, N, g.rc2, h->cap_pairs, h->d_pair_key,
             h->d_pair_row, h->d_pair_start, h->d_pair_count, h->d_row_count, h->d_self_row, h->d_counters);
-    } else if (N <= kSmallPrepAtoms) {
-        small_prep_kernel<<<1, kPrepThreads, 0, st>>>(pos, num, N, g, h->d_zlut, h->d_species_idx, (int)h->cap_cells, h->d_grid,
-                                                      h->d_atom_cell, h->d_atom_wrap, h->d_cell_count, h->d_cell_start,
-                                                      h->d_s_pos, h->d_s_wrap, h->d_counters);
     } else if (N <= kPrepAtoms) {
-        CU(launch_cluster(prep_kernel, kPrepCtas, kPrepThreads, st, false, pos, num, N, g, h->d_zlut, h->d_species_idx, (int)h->cap_cells,
+        const bool one = N <= kSmallPrepAtoms, kept = N <= kPrepCtas * kSmallPrepAtoms;
+        auto kernel = one ? prep_kernel<false, kSmallPrepPerThread> : kept ? prep_kernel<true, kSmallPrepPerThread> : prep_kernel<true, kPrepPerThread>;
+        CU(launch_cluster(kernel, one ? 1 : kPrepCtas, kPrepThreads, st, false, pos, num, N, g, h->d_zlut, h->d_species_idx, (int)h->cap_cells,
                           h->d_grid, h->d_atom_cell, h->d_atom_wrap, h->d_cell_count, h->d_cell_start, h->d_s_pos, h->d_s_wrap, h->d_counters));
     } else {
         CU(cudaMemsetAsync(h->d_bbox, 0, 64, st));
@@ -443,10 +441,12 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
 #define SOAP_PAIRS_ARGS pos, centers, sites, C, g, h->d_grid, h->d_atom_cell, h->d_atom_wrap, h->d_cell_start, h->d_s_pos, h->d_s_wrap, \
         h->cap_pairs, h->d_pair_tmp, h->d_pair_key, h->d_pair_row, h->d_pair_start, h->d_pair_count, h->d_row_count, h->d_self_row, h->d_counters
         // (these kernels wait for the kernel before them on the device: their launch overlaps its tail)
-        if (small_keys && rows) CU(launch_dependent(pairs_kernel<kFillSmemKeysSmall, true>, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
-        else if (small_keys) CU(launch_dependent(pairs_kernel<kFillSmemKeysSmall, false>, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
-        else if (rows) CU(launch_dependent(pairs_kernel<kFillSmemKeys, true>, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
-        else CU(launch_dependent(pairs_kernel<kFillSmemKeys, false>, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
+        const bool few = C <= (int64_t)16 * h->sm_count;
+#define SOAP_PAIRS(KEYS, ROWS) (few ? pairs_kernel<KEYS, ROWS, 4> : pairs_kernel<KEYS, ROWS, 1>)
+        auto kernel = small_keys ? (rows ? SOAP_PAIRS(kFillSmemKeysSmall, true) : SOAP_PAIRS(kFillSmemKeysSmall, false))
+                                 : (rows ? SOAP_PAIRS(kFillSmemKeys, true) : SOAP_PAIRS(kFillSmemKeys, false));
+        CU(launch_dependent(kernel, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
+#undef SOAP_PAIRS
 #undef SOAP_PAIRS_ARGS
     }
     if (!rows) {

@@ -123,7 +123,7 @@ def check_search(pkg, pos, r_cut):
 
 # one, two, four and eight CTAs of the brute-force search; one CTA, a cluster and many launches for the cell list;
 # one CTA and a cluster for the row pointers, and the tiled scan
-@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 65, 127, 129, 255, 257, 511, 512, 513, 4095, 4096, 4097, 8193, 65536, 65537])
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 65, 127, 129, 255, 257, 511, 512, 513, 2369, 4095, 4096, 4097, 8193, 32768, 32769, 65536, 65537])
 def test_sizes_at_which_the_search_changes(pkg, n):
     rng = np.random.default_rng(n)
     edge = (n / 0.6) ** (1 / 3)
@@ -141,3 +141,27 @@ def test_sort_of_a_centre_s_pairs(pkg, n_ball, spread):
         ids[-1] = n - 1
     pos[ids] = (rng.random((n_ball, 3)) * 1.0).astype(np.float32)
     check_search(pkg, pos, 2.5)
+
+
+@pytest.mark.parametrize("n", [7, 60, 431, 2368, 2369, 4097])
+@pytest.mark.parametrize("pbc", [(True, True, True), (True, False, True)])
+def test_periodic_search_of_few_and_many_atoms(pkg, n, pbc):
+    """With and without a free axis, one and several candidates per lane in flight, against a k-d tree over replicas."""
+    from scipy.spatial import cKDTree
+    rng = np.random.default_rng(n)
+    edge, r_cut = (n / 0.3) ** (1 / 3), 2.2
+    cell = np.eye(3) * edge
+    pos = (rng.random((n, 3)) * edge).astype(np.float32)
+    soap = pkg.Soap([1], r_cut, 1, 0, 0.5, pkg.GTO, pbc)
+    p, num = torch.from_numpy(pos).cuda(), torch.ones(n, dtype=torch.int32, device="cuda")
+    images = [(a, b, c) for a in (-1, 0, 1) for b in ((-1, 0, 1) if pbc[1] else (0,)) for c in (-1, 0, 1)]
+    x = pos.astype(np.float64)
+    tree = cKDTree(np.concatenate([x + np.array(t) @ cell for t in images]))
+    want = [sorted((j % n, *images[j // n]) for j in near if j != i + n * images.index((0, 0, 0)))
+            for i, near in enumerate(tree.query_ball_point(x, r_cut))]
+    for _ in range(2):
+        ptr, atom, shift = (t.cpu().numpy() for t in soap.neighbor_list(p, num, cell))
+        got = np.concatenate([atom[:, None], shift], axis=1)
+        assert ptr[-1] == sum(len(w) for w in want)
+        for i in range(n):
+            assert got[ptr[i]:ptr[i + 1]].tolist() == [list(w) for w in want[i]]
