@@ -146,7 +146,8 @@ __device__ __forceinline__ void harmonics_tiles(float x, float y, float z, float
 }
 
 // NP: n_max rounded up to a multiple of four.  PLAIN: the default configuration (atom centres, no weighting, every
-// species pair, power spectrum out).  TS: the radial table is in shared memory.
+// species pair, power spectrum out).  TS: the radial table is in shared memory (not with a weighting: a staged pair then
+// has no word for the weight).
 // TEAM: few centres, a CTA per centre: its warps take the chunks of pairs in turn, each into a tile of its own, and the
 // tiles are added up; the blocks of Eq. 4 are spread over all of them.
 template <int L, int NP, bool PLAIN, bool TS, bool TEAM>
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
                             v = __ffma2_rn(v, tt, make_float2(B.x, B.y));
                             v = __ffma2_rn(v, tt, make_float2(A.z, A.w));
                             v = __ffma2_rn(v, tt, make_float2(A.x, A.y));
-                            if (!PLAIN) { const float wgt = __int_as_float(gi.w); v.x *= wgt; v.y *= wgt; }
+                            if (!PLAIN && !TS) { const float wgt = __int_as_float(gi.w); v.x *= wgt; v.y *= wgt; }
                             *reinterpret_cast<float2*>(sG + pr * GROW + g_word(cp)) = v;
                             // 32 further down the list
                             pr += 32 / CPAIRS; cp += 32 % CPAIRS;

@@ -11,9 +11,8 @@ namespace soap {
 #define SOAP_CAT2(a, b) a##b
 #define SOAP_CAT(a, b) SOAP_CAT2(a, b)
 
-// the default configuration runs with the table in shared memory or in global memory, or with a team of warps per
-// centre; calls that use an option always read the table from global memory, a warp per centre
-#define SOAP_DESC_VARIANTS(X, NP) X(NP, true, true, false) X(NP, true, false, false) X(NP, false, false, false) X(NP, true, false, true) X(NP, false, false, true)
+// a warp per centre with the table in shared memory or in global memory, or a team of warps per centre
+#define SOAP_DESC_VARIANTS(X, NP) X(NP, true, true, false) X(NP, true, false, false) X(NP, false, true, false) X(NP, false, false, false) X(NP, true, false, true) X(NP, false, false, true)
 
 template <int NP>
 static cudaError_t set_np(int bytes) {
@@ -30,7 +29,8 @@ static cudaError_t launch_np(bool plain, bool ts, bool team, const CenterParams&
     // (the kernel waits on the device for the kernel before it: launch and table staging overlap that kernel's tail)
     if (team && plain) return launch_dependent(desc_kernel<SOAP_L, NP, true, false, true>, grid, block, smem, st, p);
     if (team) return launch_dependent(desc_kernel<SOAP_L, NP, false, false, true>, grid, block, smem, st, p);
-    if (plain && ts) return launch_dependent(desc_kernel<SOAP_L, NP, true, true, false>, grid, block, smem, st, p);
+    if (ts && !plain) return launch_dependent(desc_kernel<SOAP_L, NP, false, true, false>, grid, block, smem, st, p);
+    if (ts) return launch_dependent(desc_kernel<SOAP_L, NP, true, true, false>, grid, block, smem, st, p);
     if (plain) return launch_dependent(desc_kernel<SOAP_L, NP, true, false, false>, grid, block, smem, st, p);
     return launch_dependent(desc_kernel<SOAP_L, NP, false, false, false>, grid, block, smem, st, p);
 }

@@ -553,7 +553,7 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     const size_t fixed_ts = (size_t)with_table.warp0 * 4, warp_bytes_ts = (size_t)with_table.per_warp * 4;
     const int warps_ts = h->desc_table_bytes > 0 && fixed_ts + warp_bytes_ts <= (size_t)h->max_smem
                              ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed_ts) / warp_bytes_ts) : 0;
-    const bool ts = plain && warps_ts >= 6 && n_work >= (int64_t)4 * h->sm_count;
+    const bool ts = !cp.pair_w && warps_ts >= 6 && n_work >= (int64_t)4 * h->sm_count;
     int warps = ts ? warps_ts : warps_fit;
     warps = (int)std::max<int64_t>(1, std::min<int64_t>(warps, (n_work + h->sm_count - 1) / h->sm_count));
     const unsigned grid = (unsigned)std::min<int64_t>(h->sm_count, (n_work + warps - 1) / warps);

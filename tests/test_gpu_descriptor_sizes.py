@@ -75,3 +75,25 @@ def test_centres_with_no_one_few_and_very_many_neighbours(pkg):
         s.positions = np.concatenate([ball, [[50, 0, 0], [80, 0, 0], [81, 0, 0]]]).astype(np.float32)
         s.numbers = rng.choice([1, 8], size=n_ball + 3).astype(np.int32)
         check(pkg, s, ([1, 8], 4.0, 6, 5, 0.5, GTO), [0, n_ball - 1, n_ball, n_ball + 1, n_ball + 2])
+
+
+@pytest.mark.parametrize("n_centers", [600, 745])
+def test_options_on_many_centres(pkg, n_centers):
+    """The kernel that honours the options, with the table in shared memory (from 592 centres on, no weighting) and not."""
+    from oracle import modes
+    s = water_cluster(250, 4)
+    pos, num = torch.from_numpy(s.positions).cuda(), torch.from_numpy(s.numbers).cuda()
+    centers = np.random.default_rng(3).permutation(s.n_atoms)[:n_centers].tolist()
+    cen = torch.tensor(centers, dtype=torch.int32, device="cuda")
+    sample = [0, 11, n_centers - 1]
+    of = [centers[k] for k in sample]
+    args = ([1, 8], 4.5, 6, 5, 0.5, GTO)
+    soap, oracle = pkg.Soap(*args), SoapOracle(*args)
+    got = soap.coefficients(pos, num, None, cen)
+    ref = modes.coefficient_derivatives(oracle, s.positions, s.numbers, None, of).descriptor
+    assert col_err(got[sample].cpu().numpy(), ref) < DESC_TOL
+    weighting = {"function": "pow", "r0": 3.0, "c": 1.5, "d": 1.0, "m": 2.0, "w0": 0.7}
+    for kw in ({"crossover": False}, {"weighting": weighting}):
+        soap, oracle = pkg.Soap(*args, **kw), SoapOracle(*args, **kw)
+        got = soap.descriptor(pos, num, None, cen)
+        assert col_err(got[sample].cpu().numpy(), oracle.descriptor(s.positions, s.numbers, None, of)) < DESC_TOL
