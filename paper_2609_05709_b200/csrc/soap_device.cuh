@@ -167,8 +167,11 @@ __host__ __device__ constexpr int pass1_slots(int l_max, int n_max) {
 }
 // Bases whose Jacobian rows are written with the operands of every feature from a table (up to kKeepFeatures features).
 __host__ __device__ constexpr bool row_table_wanted(int n_max, int l_max) { return n_max <= 4 && n_max * (l_max + 1) <= 20; }
-// Features up to which the slab of the power spectrum has room of its own beside the staging area (16 bytes each).
-constexpr int kKeepFeatures = 512;
+// Features and l_max up to which the slab of the power spectrum has room of its own beside the staging area (16 bytes
+// each), so that a centre's pairs can stay staged for pass 2.  With 100 harmonics and more a chunk holds 8 to 16 pairs, no
+// centre's pairs fit, and the room halves the chunk (kernel, 3000 centres of 68 pairs, with and without the room: (3, 9)
+// 445 -> 425 us, (4, 12) 851 -> 820 us, (3, 9) crossover off 373 -> 340 us; at l_max 8 and below 0.89 to 1.1 by the pairs).
+constexpr int kKeepFeatures = 512, kKeepLmax = 8;
 __host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, int P, int warps, bool weighted) {
     const int L1 = l_max + 1, LMP = (L1 * L1) | 1, NCH = n_max * L1, CT = S * n_max * LMP, F = S * n_max * (S * n_max + 1) / 2 * L1;
     SmemLayout o;
@@ -185,7 +188,7 @@ __host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, i
         const int a = 3 * CT, b = warps * S * NCH * 4;
         off = align4(off + (a > b ? a : b));
     }
-    o.keep = F <= kKeepFeatures;
+    o.keep = F <= kKeepFeatures && l_max <= kKeepLmax;
     o.slab = off;
     if (o.keep) { o.slab_words = 4 * F; off += 4 * F; }
     o.sSD = off; off = align4(off + P * LMP * 4);

@@ -80,3 +80,10 @@ def test_neighbour_counts(pkg, n_ball, n_max, l_max):
     args = ([1, 8], 4.0, n_max, l_max, 0.5, GTO)
     check(pkg, s, args, list(range(n_ball)), [0, n_ball - 1])
     check(pkg, s, args, list(range(n_ball + 800)), [0, n_ball - 1, n_ball, n_ball + 799])
+
+
+@pytest.mark.parametrize("n_ball", [9, 32, 33, 34, 65])
+@pytest.mark.parametrize("n_max,l_max", [(2, 2), (4, 4), (2, 8), (3, 9), (4, 12)])
+def test_staging_limits(pkg, n_ball, n_max, l_max):
+    """Chunks of up to 32 and of more pairs; with and without a slab of its own (l_max 8 and 9)."""
+    test_neighbour_counts(pkg, n_ball, n_max, l_max)
