@@ -18,6 +18,7 @@
 #include "desc_kernel.cuh"
 #include "desc_launch.h"
 #include "neighbor_kernels.cuh"
+#include "smem_plan.h"
 #include "soap.h"
 #include "weight_kernel.cuh"
 
@@ -207,34 +208,12 @@ int plan_smem(soap_t* h) {
     h->desc_warp_bytes = (size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0, false).per_warp * 4;
     if (h->desc_warp_bytes > (size_t)max_smem) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
     CU(desc_set_smem(h->l_max, desc_np(h->n_max), max_smem));
-    // pairs per staged chunk of the derivative kernels: the largest that still leaves room for all the CTAs per SM that
-    // the registers allow (three of 256 threads), else two thirds of them, else whatever fits (`extra` bytes follow the
-    // usual layout); false if nothing fits.  Where the slab has room of its own a chunk may hold 96 pairs, so that most
-    // centres are staged once for both passes (3000 atoms of 68 neighbours at (4, 3): 218 -> 193 us).
-    // CTAs of 128 threads stop at 32 pairs where a pair takes 96 words and more: six larger chunks leave the L1 too little
-    // for the radial table (64 or more against 32 pairs: 36,000 centres of 18 pairs at (4, 3) 682 -> 658 us, 3000 of 68 at
-    // (4, 4) 241 -> 224 us, at (2, 8) 327 -> 313 us; (2, 2), 48 words a pair, goes the other way, 83 against 93 us).
-    auto plan_chunk = [&](int warps, size_t extra, int& P_out, size_t& bytes_out) -> bool {
-        const int ctas = 24 / warps;
-        auto bytes_of = [&](int P) { return (size_t)make_layout(h->S, h->n_max, h->l_max, P, warps, h->weight.fn != 0).total * 4 + extra; };
-        const bool keep = make_layout(h->S, h->n_max, h->l_max, 32, warps, false).keep;
-        const int L1 = h->l_max + 1, pair_words = 4 * ((L1 * L1) | 1) + 2 * h->n_max * L1;
-        const int most = warps == 4 && pair_words >= 96 ? 32 : 32 * warps;
-        int P = 4;
-        for (int pass = 0; pass < 3; ++pass) {
-            const size_t budget = pass == 2 ? (size_t)max_smem : (size_t)228 * 1024 / (pass == 0 ? ctas : (2 * ctas + 2) / 3) - 1024;
-            for (const int candidate : {96, 80, 64, 56, 48, 40, 32, 24, 16, 8, 4}) {
-                P = candidate;
-                if ((keep ? P <= most && (P != 24 || h->l_max < 8) : P <= 32 && P != 24) && bytes_of(P) <= budget) break;
-            }
-            if (P >= (pass == 2 ? 4 : 8) && bytes_of(P) <= budget) break;
-        }
-        P_out = P; bytes_out = bytes_of(P);
-        return bytes_out <= (size_t)max_smem;
+    auto plan = [&](int warps, size_t extra, int& P, size_t& bytes) {
+        return plan_chunk(h->S, h->n_max, h->l_max, h->weight.fn != 0, warps, extra, (size_t)max_smem, P, bytes);
     };
     // 256 threads, and the smaller CTAs that this basis may run with
-    if (!plan_chunk(8, 0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
-    if (!plan_chunk(4, 0, h->P_deriv4, h->smem_deriv4)) h->smem_deriv4 = 0;
+    if (!plan(8, 0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
+    if (!plan(4, 0, h->P_deriv4, h->smem_deriv4)) h->smem_deriv4 = 0;
     // (a kernel's limit is the process's, not the handle's: every handle sets the device's maximum, so that none takes away
     // what another one launches with)
     CU(center_set_smem(kCenterDeriv, h->l_max, h->n_max, max_smem));
@@ -243,7 +222,7 @@ int plan_smem(soap_t* h) {
     // the kernel of the outer average keeps, per warp, a copy of a neighbouring centre's coefficients behind the usual
     // layout; a basis too large for that takes the general path (per-pair rows in a workspace)
     const int LMP = ((h->l_max + 1) * (h->l_max + 1)) | 1;
-    h->outer_fast = plan_chunk(kThreads / 32, (size_t)(kThreads / 32) * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
+    h->outer_fast = plan(kThreads / 32, (size_t)(kThreads / 32) * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
     if (h->outer_fast) CU(center_set_smem(kCenterOuter, h->l_max, h->n_max, max_smem));
     return SOAP_OK;
 }

@@ -87,3 +87,26 @@ def test_neighbour_counts(pkg, n_ball, n_max, l_max):
 def test_staging_limits(pkg, n_ball, n_max, l_max):
     """Chunks of up to 32 and of more pairs; with and without a slab of its own (l_max 8 and 9)."""
     test_neighbour_counts(pkg, n_ball, n_max, l_max)
+
+
+@pytest.mark.parametrize("repeats", [1, 10])
+@pytest.mark.parametrize("kw", [{}, {"weighting": {"function": "poly", "r0": 4.0, "c": 1.0, "m": 2.0, "w0": 1.0}}], ids=["plain", "weighted"])
+@pytest.mark.parametrize("n_max,l_max", [(4, 0), (4, 1), (3, 0), (2, 2)])
+def test_absent_operands_are_zero(pkg, n_max, l_max, kw, repeats):
+    """Eight species without crossover: rows by the table of operands though the slab shares the staging area ((4, 0) is
+    where the two meet).  Only the block of the neighbour's species may differ from zero in its row."""
+    s = multispecies_box(80, 1)
+    species = [1, 6, 7, 8, 9, 14, 16, 17]
+    s.numbers = np.random.default_rng(1).choice(species, size=s.n_atoms).astype(np.int32)
+    args = (species, 4.0, n_max, l_max, 0.4, POLYNOMIAL, (True, True, True))
+    centers = list(range(80)) * repeats
+    check(pkg, s, args, centers, [0, 33, 79], crossover=False, **kw)
+    soap = pkg.Soap(*args, crossover=False, **kw)
+    out = soap.derivatives(torch.from_numpy(s.positions).cuda(), torch.from_numpy(s.numbers).cuda(), s.cell, torch.tensor(centers, dtype=torch.int32, device="cuda"))
+    width = soap.n_features // 8
+    atom = out.row_atom.cpu().numpy()
+    center = np.repeat(centers, np.diff(out.row_ptr.cpu().numpy()))
+    block = np.searchsorted(species, s.numbers[atom])
+    jac = out.jacobian.cpu().numpy().reshape(-1, 3, 8, width)
+    jac[np.arange(atom.size), :, block] = 0.0
+    assert not jac[atom != center].any()
