@@ -1006,7 +1006,7 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
                   long long* __restrict__ row_ptr, int* __restrict__ order, Counters* counters, Counters* host) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ int warp_sums[32], cta_sum;
+    __shared__ long long warp_sums[32], cta_sum;                             // (a Jacobian may have more than 2^31 rows)
     __shared__ int hist[kSizeBins], total[kSizeBins], first_slot[kSizeBins];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
@@ -1017,7 +1017,8 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
     const int c_hi = min(C, (rank + 1) * per_cta), i0 = rank * per_cta + tid * per_thread;
     grid_dependency_wait();                                                  // the counts of the pair kernel
     __syncthreads();
-    int v[kRowsPerThread], bin[kRowsPerThread], mine = 0;
+    int v[kRowsPerThread], bin[kRowsPerThread];
+    long long mine = 0;
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; ++k) {
         v[k] = bin[k] = 0;
@@ -1028,17 +1029,17 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
         }
         mine += v[k];
     }
-    int incl = mine;
+    long long incl = mine;
     for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        const long long y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
     if (lane == 31) warp_sums[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-        int w = warp_sums[lane];
+        long long w = warp_sums[lane];
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, w, o);
+            const long long y = __shfl_up_sync(0xffffffffu, w, o);
             if (lane >= o) w += y;
         }
         warp_sums[lane] = w;
@@ -1058,7 +1059,7 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
             total[tid] = all;
         }
         for (int r = 0; r < ctas; ++r) {
-            const int t = *cluster.map_shared_rank(&cta_sum, r);
+            const long long t = *cluster.map_shared_rank(&cta_sum, r);
             if (r < rank) base += t;
             rows += t;
         }
