@@ -121,9 +121,13 @@ int soap_neighbors(soap_t *h, const float *d_positions, const int32_t *d_numbers
  * soap_neighbors (a search that met more pairs than the scratch holds is run
  * again) and reports a device-side error at once (and clears it);
  * soap_derivatives_found computes the derivatives of what that search found,
- * without searching again, and WAITS for the stream.  All three get the same
- * structure (positions and centres unchanged, numbers as well), and no other
- * call on the handle comes between them.
+ * without searching again, and WAITS for the stream (once or several times,
+ * say for two kinds); with capacity_rows below the rows found it writes
+ * nothing and returns SOAP_ERR_CAPACITY, and soap_status has nothing more to
+ * report.  All three get the same structure (positions and centres unchanged,
+ * numbers as well), and no other call on the handle comes between them: one
+ * that searches or changes an option (soap_set_crossover, soap_set_weighting)
+ * takes the search away, and the next step returns SOAP_ERR_INVALID_ARG.
  *   d_centers / d_sites   as in soap_derivatives / soap_derivatives_at (at most one of them)
  *   d_struct_ptr          as in soap_derivatives_batch, or NULL (one structure)
  *   kind                  what is written, as by soap_derivatives (SOAP_ROWS_FULL),

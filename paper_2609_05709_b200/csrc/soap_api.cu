@@ -128,7 +128,7 @@ struct soap_handle {
     bool list_sorted = false;            // whether the pair list of the last search is sorted (descriptor-only calls skip that)
     bool ordered = false;                // whether the last search with rows left a launch order
     int64_t started_atoms = -1, started_centers = -1;   // sizes of the search soap_search_start left for soap_search_finish; -1: none
-    int64_t found_atoms = -1, found_centers = -1;   // sizes of the search soap_search_finish left for soap_derivatives_found; -1: none
+    int64_t found_atoms = -1, found_centers = -1, found_rows = 0;   // sizes of the search soap_search_finish left for soap_derivatives_found; -1: none
     int P_deriv4 = 16;                   // ... with CTAs of 128 threads
     size_t smem_deriv4 = 0;
     int P_deriv = 16, P_outer = 16;      // pairs per staged chunk: derivative kernels, kernel of the outer average
@@ -155,6 +155,9 @@ int cuda_fail(soap_t* h, cudaError_t e, const char* what) {
         cudaError_t e_ = (call);                                   \
         if (e_ != cudaSuccess) return cuda_fail(h, e_, #call);     \
     } while (0)
+
+// No search is under way or at hand any more for the calls that compute from one.
+void forget_search(soap_t* h) { h->found_atoms = h->found_centers = h->started_atoms = h->started_centers = -1; }
 
 template <typename T>
 cudaError_t upload(T** dst, const std::vector<T>& src) {
@@ -378,7 +381,7 @@ struct Batch {
 int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g,
                      const int32_t* centers, const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st,
                      const Batch& batch = Batch(), bool rows = true, bool publish = false) {
-    h->found_atoms = h->found_centers = h->started_atoms = h->started_centers = -1;
+    forget_search(h);
     Counters* const host = publish ? h->h_counters : nullptr;
     // A small non-periodic structure with every atom a centre is searched by brute force, without a cell list.
     // (C == N: the brute-force kernel writes the per-centre arrays for every atom, and those are sized from C)
@@ -922,7 +925,7 @@ int soap_search_finish(soap_t* h, const float* d_positions, const int32_t* d_num
         CU(cudaMemsetAsync(&h->d_counters->status, 0, sizeof(int), (cudaStream_t)stream));
         return status_error(h, h->h_counters->status);
     }
-    h->found_atoms = n_atoms; h->found_centers = n_centers;
+    h->found_atoms = n_atoms; h->found_centers = n_centers; h->found_rows = h->h_counters->n_rows;
     return SOAP_OK;
 }
 
@@ -936,6 +939,7 @@ int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_
     if (!d_row_ptr || capacity_rows < 0) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
     if (n_centers > 0 && (!d_out_desc || !d_out_jac || !d_row_atom)) return fail(h, SOAP_ERR_INVALID_ARG, "output pointers must not be NULL");
     if (n_centers > 0 && kind == SOAP_ROWS_COMPACT && !d_out_center) return fail(h, SOAP_ERR_INVALID_ARG, "d_out_center must not be NULL");
+    if (capacity_rows < h->found_rows) return fail(h, SOAP_ERR_CAPACITY, "more Jacobian rows than capacity_rows");
     int rc = ensure_device(h);
     if (rc) return rc;
     Geometry g;
@@ -1020,6 +1024,7 @@ int soap_set_crossover(soap_t* h, int crossover) {
     crossover = crossover ? 1 : 0;
     if (crossover == h->crossover) return SOAP_OK;
     h->crossover = crossover;
+    forget_search(h);                    // (whoever has one under way sized its outputs for other features)
     build_feature_table(h);
     if (h->tables_ready) {
         CU(cudaDeviceSynchronize());
@@ -1039,6 +1044,7 @@ int soap_set_weighting(soap_t* h, int function, double r0, double c, double d, d
         if (function == SOAP_WEIGHT_EXP && !(d >= 0)) return fail(h, SOAP_ERR_INVALID_ARG, "exp weighting needs d >= 0");
     }
     const bool was = h->weight.fn != 0, now = function != SOAP_WEIGHT_NONE;
+    forget_search(h);
     h->weight = WeightParams{function, now ? r0 : 1.0, now ? c : 1.0, d, m};
     h->w0 = now ? w0 : 1.0;
     if (was != now) {
