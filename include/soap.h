@@ -396,9 +396,12 @@ int soap_neighbor_counts_static(const float *d_positions, int64_t n_atoms, doubl
                                 int32_t *d_counts, void *stream, char *message, int64_t message_len);
 
 /* Per-segment timing, the counterpart of the paper's companion profiler
- * (end of its architecture section).  With profiling enabled,
- * soap_descriptor and soap_derivatives record CUDA events on the caller's
- * stream around (a) the neighbour search and (b) the fused per-centre kernel.
+ * (end of its architecture section).  With profiling enabled, the calls
+ * that compute a descriptor, coefficients or derivatives record CUDA events on
+ * the caller's stream around (a) the neighbour search and the weights of its
+ * pairs and (b) the per-centre kernels.  A call in steps (soap_search_start to
+ * soap_derivatives_found) is one call: the host's work between its steps
+ * counts in neither.
  * soap_profile_read waits for the last call's events and returns both
  * durations in milliseconds.  Off by default: the kernels of a call are
  * launched so that each may start while the one before it finishes (they wait

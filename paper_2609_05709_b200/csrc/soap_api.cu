@@ -136,7 +136,9 @@ struct soap_handle {
     bool outer_fast = false;             // whether the kernel of the outer average fits the shared memory
     // optional per-segment timing (events on the caller's stream)
     bool profiling = false;
-    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // search begins, ends (per-centre kernel begins), kernel ends;
+                                         // of a call in steps: the weights begin, they end (per-centre kernel begins)
+    bool in_steps = false;               // whether the last call profiled searched in a step of its own
 };
 
 namespace {
@@ -475,7 +477,12 @@ int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, 
     int rc = ensure_scratch(h, N, C, 0, st);
     if (rc) return rc;
     for (int attempt = 0; attempt < 2; ++attempt) {
-        if ((step != Search::finish || attempt > 0) && (rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
+        if (step != Search::finish || attempt > 0) {
+            const bool timed = h->profiling && step != Search::whole;        // (a search inside a call: `prepare` times it)
+            if (timed) CU(cudaEventRecord(h->ev[0], st));
+            if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
+            if (timed) CU(cudaEventRecord(h->ev[1], st));
+        }
         if (step == Search::start) return SOAP_OK;
         CU(cudaStreamSynchronize(st));
         const int64_t pairs = h->h_counters->n_pairs;
@@ -617,7 +624,7 @@ int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const do
         return fail(h, SOAP_ERR_INVALID_ARG, "batches of structures are for non-periodic structures");
     if ((rc = ensure_device(h))) return rc;
     if ((rc = make_geometry(h, cell, g))) return rc;
-    if (h->profiling) CU(cudaEventRecord(h->ev[0], st));
+    if (h->profiling) { CU(cudaEventRecord(h->ev[0], st)); h->in_steps = false; }
     // search with the totals read back (grows the scratch: allocates and waits) when this structure is larger
     // than anything planned so far; smaller ones run in the scratch that is there, and if one of them turns out
     // to have more pairs than that holds the status word says so
@@ -945,9 +952,9 @@ int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_
     Geometry g;
     if ((rc = make_geometry(h, cell, g))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    if (h->profiling) CU(cudaEventRecord(h->ev[0], st));
+    if (h->profiling) { CU(cudaEventRecord(h->ev[3], st)); h->in_steps = true; }
     if ((rc = launch_weights(h, d_positions, d_centers, d_sites, n_centers, g, st))) return rc;
-    if (h->profiling) CU(cudaEventRecord(h->ev[1], st));
+    if (h->profiling) CU(cudaEventRecord(h->ev[4], st));
     if (n_centers > 0) {
         CenterParams cp;
         fill_center_params(h, cp, d_positions, d_centers, n_centers, g, true, d_sites);
@@ -1387,9 +1394,11 @@ int soap_profile(soap_t* h, int enable) {
 int soap_profile_read(soap_t* h, float* ms_neighbors, float* ms_center) {
     if (!h || !h->ev[2]) return SOAP_ERR_INVALID_ARG;
     CU(cudaEventSynchronize(h->ev[2]));
-    float a = 0.f, b = 0.f;
+    float a = 0.f, b = 0.f, weights = 0.f;
     CU(cudaEventElapsedTime(&a, h->ev[0], h->ev[1]));
-    CU(cudaEventElapsedTime(&b, h->ev[1], h->ev[2]));
+    if (h->in_steps) CU(cudaEventElapsedTime(&weights, h->ev[3], h->ev[4]));
+    CU(cudaEventElapsedTime(&b, h->ev[h->in_steps ? 4 : 1], h->ev[2]));
+    if (h->weight.fn) a += weights;      // (without a weighting nothing lies between the two events)
     if (ms_neighbors) *ms_neighbors = a;
     if (ms_center) *ms_center = b;
     return SOAP_OK;
