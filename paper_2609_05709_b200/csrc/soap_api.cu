@@ -18,6 +18,7 @@
 #include "desc_kernel.cuh"
 #include "desc_launch.h"
 #include "neighbor_kernels.cuh"
+#include "scratch.h"
 #include "smem_plan.h"
 #include "soap.h"
 #include "weight_kernel.cuh"
@@ -161,17 +162,18 @@ int cuda_fail(soap_t* h, cudaError_t e, const char* what) {
 // No search is under way or at hand any more for the calls that compute from one.
 void forget_search(soap_t* h) { h->found_atoms = h->found_centers = h->started_atoms = h->started_centers = -1; }
 
-template <typename T>
-cudaError_t upload(T** dst, const std::vector<T>& src) {
-    cudaError_t e = cudaMalloc((void**)dst, std::max<size_t>(src.size(), 1) * sizeof(T));
-    if (e != cudaSuccess) return e;
-    return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
+// cudaMalloc whose failure leaves a null pointer and no error behind for a later launch to report.
+cudaError_t allocate(void** ptr, size_t bytes) {
+    const cudaError_t e = cudaMalloc(ptr, std::max<size_t>(bytes, 1));
+    if (e != cudaSuccess) { *ptr = nullptr; cudaGetLastError(); }
+    return e;
 }
 
 template <typename T>
-cudaError_t regrow(T** ptr, size_t count) {
-    if (*ptr) { cudaFree(*ptr); *ptr = nullptr; }
-    return cudaMalloc((void**)ptr, std::max<size_t>(count, 1) * sizeof(T));
+cudaError_t upload(T** dst, const std::vector<T>& src) {
+    cudaError_t e = allocate((void**)dst, src.size() * sizeof(T));
+    if (e != cudaSuccess) return e;
+    return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
 
 bool invert3(const double m[9], double inv[9], double& det) {
@@ -259,7 +261,7 @@ int ensure_device(soap_t* h) {
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaGetDevice (is a CUDA device present? this library has no CPU path)");
     if (h->tables_ready) {
         if (dev != h->device) return fail(h, SOAP_ERR_INVALID_ARG, "handle was first used on another device");
-        return SOAP_OK;
+        return h->d_feat ? SOAP_OK : upload_features(h);        // (missing after a change of features that found no memory)
     }
     h->device = dev;
     {
@@ -315,42 +317,36 @@ int ensure_device(soap_t* h) {
 }
 
 int ensure_scratch(soap_t* h, int64_t N, int64_t C, int64_t pairs, cudaStream_t st) {
+    // A group that cannot grow is gone (its old buffers are given back first): nothing is planned any more, so that the next
+    // call allocates again, whatever its size, or fails here as well.
+    auto grow = [&](int64_t& capacity, int64_t want, std::initializer_list<ScratchBuffer> buffers) -> int {
+        cudaError_t e = cudaSuccess;
+        if (regrow_group(capacity, want, buffers, [&](void** ptr, size_t bytes) { return (e = allocate(ptr, bytes)) == cudaSuccess; },
+                         [](void* ptr) { cudaFree(ptr); })) return SOAP_OK;
+        h->planned_atoms = h->planned_centers = -1;
+        forget_search(h);
+        return cuda_fail(h, e, "cudaMalloc of the neighbour search's scratch");
+    };
+    auto of = [](auto** ptr, int64_t count) { return ScratchBuffer{(void**)ptr, (size_t)count * sizeof(**ptr)}; };
     if (N > h->cap_atoms || h->cap_atoms == 0) {
-        int64_t cap = N + N / 8 + 256;
-        CU(regrow(&h->d_species_idx, cap));
-        CU(regrow(&h->d_atom_cell, cap));
-        CU(regrow(&h->d_atom_wrap, cap));
-        CU(regrow(&h->d_s_wrap, cap));
-        CU(regrow(&h->d_s_pos, cap));
-        int64_t cells = std::min<int64_t>(std::max<int64_t>(2 * cap, 4096), (int64_t)1 << 26);
-        CU(regrow(&h->d_cell_count, cells + 1));
-        CU(regrow(&h->d_cell_start, cells + 1));
-        CU(regrow(&h->d_cell_tile_sums, cells / kScanTile + 2));
-        CU(regrow(&h->d_cell_tile_offsets, cells / kScanTile + 3));
-        CU(cudaMemsetAsync(h->d_cell_count, 0, (cells + 1) * sizeof(int), st));      // zero between calls
+        const int64_t cap = N + N / 8 + 256, cells = std::min<int64_t>(std::max<int64_t>(2 * cap, 4096), (int64_t)1 << 26);
+        if (int rc = grow(h->cap_atoms, cap, {of(&h->d_species_idx, cap), of(&h->d_atom_cell, cap), of(&h->d_atom_wrap, cap), of(&h->d_s_wrap, cap),
+                                              of(&h->d_s_pos, cap), of(&h->d_cell_count, cells + 1), of(&h->d_cell_start, cells + 1),
+                                              of(&h->d_cell_tile_sums, cells / kScanTile + 2), of(&h->d_cell_tile_offsets, cells / kScanTile + 3)})) return rc;
         h->cap_cells = cells;
-        h->cap_atoms = cap;
+        CU(cudaMemsetAsync(h->d_cell_count, 0, (cells + 1) * sizeof(int), st));      // zero between calls
     }
     if (C > h->cap_centers || h->cap_centers == 0) {
-        int64_t cap = C + C / 8 + 256;
-        CU(regrow(&h->d_pair_count, cap));
-        CU(regrow(&h->d_row_count, cap));
-        CU(regrow(&h->d_self_row, cap));
-        CU(regrow(&h->d_order, cap));
-        CU(regrow(&h->d_pair_ptr, cap + 1));
-        CU(regrow(&h->d_pair_start, cap));
-        CU(regrow(&h->d_row_ptr, cap + 1));
-        CU(regrow(&h->d_tile_sums, cap / kScanTile + 2));
-        CU(regrow(&h->d_tile_offsets, cap / kScanTile + 3));
-        h->cap_centers = cap;
+        const int64_t cap = C + C / 8 + 256;
+        if (int rc = grow(h->cap_centers, cap, {of(&h->d_pair_count, cap), of(&h->d_row_count, cap), of(&h->d_self_row, cap), of(&h->d_order, cap),
+                                                of(&h->d_pair_ptr, cap + 1), of(&h->d_pair_start, cap), of(&h->d_row_ptr, cap + 1),
+                                                of(&h->d_tile_sums, cap / kScanTile + 2), of(&h->d_tile_offsets, cap / kScanTile + 3)})) return rc;
     }
     if (pairs > h->cap_pairs || h->cap_pairs == 0) {
-        int64_t cap = pairs + pairs / 4 + 1024;
-        CU(regrow(&h->d_pair_key, cap));
-        CU(regrow(&h->d_pair_tmp, cap));
-        CU(regrow(&h->d_pair_row, cap));
-        if (h->weight.fn) CU(regrow(&h->d_pair_w, cap));
-        h->cap_pairs = cap;
+        const int64_t cap = pairs + pairs / 4 + 1024;
+        const int rc = h->weight.fn ? grow(h->cap_pairs, cap, {of(&h->d_pair_key, cap), of(&h->d_pair_tmp, cap), of(&h->d_pair_row, cap), of(&h->d_pair_w, cap)})
+                                    : grow(h->cap_pairs, cap, {of(&h->d_pair_key, cap), of(&h->d_pair_tmp, cap), of(&h->d_pair_row, cap)});
+        if (rc) return rc;
     }
     return SOAP_OK;
 }
@@ -1035,8 +1031,8 @@ int soap_set_crossover(soap_t* h, int crossover) {
     build_feature_table(h);
     if (h->tables_ready) {
         CU(cudaDeviceSynchronize());
-        if (int rc = upload_features(h)) return rc;
         if (h->d_compact_map) { cudaFree(h->d_compact_map); h->d_compact_map = nullptr; }
+        if (int rc = upload_features(h)) return rc;
     }
     return SOAP_OK;
 }
@@ -1060,7 +1056,12 @@ int soap_set_weighting(soap_t* h, int function, double r0, double c, double d, d
         if (h->tables_ready) {
             CU(cudaDeviceSynchronize());
             if (h->d_pair_w) { cudaFree(h->d_pair_w); h->d_pair_w = nullptr; }
-            if (now) CU(regrow(&h->d_pair_w, (size_t)std::max<int64_t>(h->cap_pairs, 1)));
+            if (now && h->cap_pairs > 0) {
+                const int64_t cap = h->cap_pairs;
+                h->cap_pairs = 0;        // (if the weights do not fit, the next search replaces the pair scratch as a whole)
+                CU(allocate((void**)&h->d_pair_w, (size_t)cap * sizeof(float2)));
+                h->cap_pairs = cap;
+            }
             if (int rc = plan_smem(h)) return rc;
         }
     }
