@@ -162,7 +162,10 @@ int soap_neighbor_list(soap_t *h, int64_t *d_pair_ptr, int32_t *d_pair_atom, int
  * work.  If such a call meets more pairs than the planned scratch holds (a
  * denser structure), soap_status reports SOAP_ERR_CAPACITY and the outputs
  * of that call are invalid: call soap_neighbors for that structure, then
- * repeat. */
+ * repeat.  The sums over a centre's pairs run in the order in which the search
+ * finds them, which is not fixed where atoms share a bin of the cell list: the
+ * last bits can differ from call to call (derivatives and averages repeat bit
+ * for bit). */
 int soap_descriptor(soap_t *h, const float *d_positions, const int32_t *d_numbers, int64_t n_atoms,
                     const double *cell, const int32_t *d_centers, int64_t n_centers,
                     float *d_out, void *stream);

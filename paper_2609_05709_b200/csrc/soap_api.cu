@@ -126,7 +126,7 @@ struct soap_handle {
     int64_t planned_atoms = -1, planned_centers = -1;
     int64_t pairs_per_center_hint = 0;   // average at the last plan (chooses the pair kernel variant)
     int64_t last_centers = 0;
-    bool list_sorted = false;            // whether the pair list of the last search is sorted (descriptor-only calls skip that)
+    bool list_sorted = false;            // whether the pair list of the last search is one to export (those of descriptor-only calls are not)
     bool ordered = false;                // whether the last search with rows left a launch order
     int64_t started_atoms = -1, started_centers = -1;   // sizes of the search soap_search_start left for soap_search_finish; -1: none
     int64_t found_atoms = -1, found_centers = -1, found_rows = 0;   // sizes of the search soap_search_finish left for soap_derivatives_found; -1: none
@@ -376,9 +376,12 @@ struct Batch {
     const long long* struct_ptr = nullptr;
     int64_t n_structs = 0;
 };
+// What a search leaves: the pairs of a centre in the order they were found in (which differs from run to run where atoms
+// share a bin); sorted; or sorted with row pointers and a launch order for the Jacobian's rows.
+enum class List { found, sorted, rows };
 int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N, const Geometry& g,
                      const int32_t* centers, const float* sites, int64_t C, long long* row_ptr_out, cudaStream_t st,
-                     const Batch& batch = Batch(), bool rows = true, bool publish = false) {
+                     const Batch& batch = Batch(), List list = List::rows, bool publish = false) {
     forget_search(h);
     Counters* const host = publish ? h->h_counters : nullptr;
     // A small non-periodic structure with every atom a centre is searched by brute force, without a cell list.
@@ -420,7 +423,7 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
     }
     if (C > 0 && !batch.struct_ptr) {
         // few pairs per centre at the last plan: the variant with the small on-chip key buffers (more warps resident);
-        // descriptor-only calls take the variants without sorting and row bookkeeping
+        // calls that need no order take the variants without sorting and row bookkeeping
         const bool small_keys = h->pairs_per_center_hint > 0 && h->pairs_per_center_hint <= kFillSmemKeysSmall * 3 / 4;
         const unsigned grid = (unsigned)((C + kFillWarps - 1) / kFillWarps);
 #define SOAP_PAIRS_ARGS pos, centers, sites, C, g, h->d_grid, h->d_atom_cell, h->d_atom_wrap, h->d_cell_start, h->d_s_pos, h->d_s_wrap, \
@@ -428,13 +431,14 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
         // (these kernels wait for the kernel before them on the device: their launch overlaps its tail)
         const bool few = C <= (int64_t)16 * h->sm_count;
 #define SOAP_PAIRS(KEYS, ROWS) (few ? pairs_kernel<KEYS, ROWS, 4> : pairs_kernel<KEYS, ROWS, 1>)
-        auto kernel = small_keys ? (rows ? SOAP_PAIRS(kFillSmemKeysSmall, true) : SOAP_PAIRS(kFillSmemKeysSmall, false))
-                                 : (rows ? SOAP_PAIRS(kFillSmemKeys, true) : SOAP_PAIRS(kFillSmemKeys, false));
+        const bool sorted = list != List::found;
+        auto kernel = small_keys ? (sorted ? SOAP_PAIRS(kFillSmemKeysSmall, true) : SOAP_PAIRS(kFillSmemKeysSmall, false))
+                                 : (sorted ? SOAP_PAIRS(kFillSmemKeys, true) : SOAP_PAIRS(kFillSmemKeys, false));
         CU(launch_dependent(kernel, grid, kFillWarps * 32, 0, st, SOAP_PAIRS_ARGS));
 #undef SOAP_PAIRS
 #undef SOAP_PAIRS_ARGS
     }
-    if (!rows) {
+    if (list != List::rows) {
         // no Jacobian rows wanted: no row pointers, no launch order
         CU(cudaGetLastError());
         return SOAP_OK;
@@ -476,7 +480,7 @@ int search_and_size(soap_t* h, const float* pos, const int32_t* num, int64_t N, 
         if (step != Search::finish || attempt > 0) {
             const bool timed = h->profiling && step != Search::whole;        // (a search inside a call: `prepare` times it)
             if (timed) CU(cudaEventRecord(h->ev[0], st));
-            if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, true, true))) return rc;
+            if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, List::rows, true))) return rc;
             if (timed) CU(cudaEventRecord(h->ev[1], st));
         }
         if (step == Search::start) return SOAP_OK;
@@ -613,7 +617,7 @@ int launch_weights(soap_t* h, const float* pos, const int32_t* centers, const fl
 // changed, the neighbour search.
 int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const double* cell, const int32_t* centers,
             int64_t C, long long* row_ptr_out, Geometry& g, cudaStream_t st, const float* sites = nullptr,
-            const Batch& batch = Batch(), bool rows = true) {
+            const Batch& batch = Batch(), List list = List::rows) {
     int rc = check_inputs(h, pos, num, N, centers, C, sites);
     if (rc) return rc;
     if (batch.struct_ptr && (h->pbc[0] || h->pbc[1] || h->pbc[2]))
@@ -626,10 +630,11 @@ int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const do
     // to have more pairs than that holds the status word says so
     const bool planned = h->planned_atoms >= 0 && N <= h->planned_atoms && C <= h->planned_centers;
     if (!planned && (rc = search_and_size(h, pos, num, N, g, centers, sites, C, row_ptr_out, st, batch))) return rc;
-    if (planned || !rows) {
-        // (a call without rows always takes the unsorted list, so that its sums run in the same order every time)
-        if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, rows))) return rc;
-        h->list_sorted = rows;
+    if (planned || list == List::found) {
+        // (a first call of its size has the sorted list already, and takes the pairs as found all the same: its result then
+        // differs from that of the calls after it no more than theirs do from one another)
+        if ((rc = launch_neighbors(h, pos, num, N, g, centers, sites, C, row_ptr_out ? row_ptr_out : h->d_row_ptr, st, batch, list))) return rc;
+        h->list_sorted = list == List::rows;
         h->last_centers = C;
     }
     if ((rc = launch_weights(h, pos, centers, sites, C, g, st))) return rc;
@@ -785,7 +790,7 @@ static int descriptor_impl(soap_t* h, const float* d_positions, const int32_t* d
     if (h && n_centers > 0 && !d_out) return fail(h, SOAP_ERR_INVALID_ARG, "d_out must not be NULL");
     Geometry g;
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, d_sites, batch, false);
+    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, d_sites, batch, List::found);
     if (rc) return rc;
     if (n_centers > 0) {
         CenterParams cp;
@@ -1079,7 +1084,7 @@ int soap_coefficients(soap_t* h, const float* d_positions, const int32_t* d_numb
     if (h && n_centers > 0 && !d_out) return fail(h, SOAP_ERR_INVALID_ARG, "d_out must not be NULL");
     Geometry g;
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, nullptr, Batch(), false);
+    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, nullptr, Batch(), List::found);
     if (rc) return rc;
     if (n_centers > 0) {
         CenterParams cp;
@@ -1122,7 +1127,7 @@ int soap_descriptor_average(soap_t* h, int mode, const float* d_positions, const
     if (!d_out) return fail(h, SOAP_ERR_INVALID_ARG, "d_out must not be NULL");
     Geometry g;
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, nullptr, Batch(), false);
+    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, nullptr, Batch(), List::sorted);      // (sorted: the average repeats bit for bit)
     if (rc) return rc;
     const int F = (int)h->F, W = h->S * h->n_max * (h->l_max + 1) * (h->l_max + 1);
     const bool inner = mode == SOAP_AVERAGE_INNER;

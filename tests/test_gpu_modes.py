@@ -419,3 +419,16 @@ def test_batch_of_structures(pkg, rbf):
     per = pkg.Soap([1, 8], 4.5, 2, 2, 0.5, GTO, (True, False, False))
     with pytest.raises(pkg.SoapError, match="non-periodic"):
         per.derivatives_batch(pos, num, ptr)
+
+
+@pytest.mark.parametrize("mode", ["inner", "outer"])
+@pytest.mark.parametrize("n_atoms,edge,kw", [(3000, 14.0, {}), (9000, 20.0, {}), (3000, 14.0, {"crossover": False})])
+def test_averages_repeat_bit_for_bit_where_bins_are_full(pkg, mode, n_atoms, edge, kw):
+    """Beyond the brute-force search the atoms of a bin are in no fixed order; the averages must not show it."""
+    rng = np.random.default_rng(n_atoms)
+    pos = torch.from_numpy((rng.random((n_atoms, 3)) * edge).astype(np.float32)).cuda()
+    num = torch.from_numpy(rng.choice([1, 8], size=n_atoms).astype(np.int32)).cuda()
+    soap = pkg.Soap([1, 8], 4.0, 4, 3, 0.5, **kw)
+    first = soap.descriptor_average(mode, pos, num)
+    for _ in range(20):
+        assert torch.equal(soap.descriptor_average(mode, pos, num), first)
