@@ -135,10 +135,10 @@ center_kernel(const CenterParams p) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int S = p.S, NMAX = NMAX_T ? NMAX_T : p.n_max, NCH = NMAX * L1, NE = NMAX * LM;
     const int CT = S * NMAX * LMP, P = p.P, F = p.F;
-    const SmemLayout lay = make_layout(S, NMAX, L, P, warps, o_pw != nullptr);
     constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
     // words pairs (G, Ghat) per staged pair: the channels, and with a row table a zero behind them
     constexpr bool kRowTable = KIND == 1 && NMAX_T != 0 && row_table_wanted(NMAX_T, L);
+    const SmemLayout lay = make_layout(S, NMAX, L, P, warps, o_pw != nullptr, kRowTable && p.row_ops != nullptr);
     const int GP = NCH + (row_table_wanted(NMAX, L) ? 1 : 0);
     const int CP = NMAX_T ? CP_T : (NMAX + 1) / 2 * L1;                     // channel pairs: (l, two adjacent n)
     float* c_t = smem + lay.c;                                             // [S][NMAX][LMP]
@@ -159,6 +159,10 @@ center_kernel(const CenterParams p) {
     const int zero_w = zero_words(S, NMAX, L);
     for (int e = tid; e < zero_w; e += threads) smem[lay.zero + e] = 0.f;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // the zero behind the channels of every staged pair, for the operands that a feature does not have in rows by table (the
+    // slab of the power spectrum ends before it, make_layout)
+    if (kRowTable)
+        for (int e = tid; e < P; e += threads) sG2[e * GP + NCH] = make_float2(0.f, 0.f);
 
     // same-species blocks: feature index -> (n1 L1 + l) | (n2 L1 + l) << 8, rows n1 of (NMAX - n1) L1 entries
     unsigned short* tri_dec = reinterpret_cast<unsigned short*>(smem + lay.tri);
@@ -778,12 +782,6 @@ center_kernel(const CenterParams p) {
             const int row = e / LM, lm = e - row * LM;
             c_t[row * LMP + lm] *= __ldg(p.kl + __ldg(p.l_of_lm + lm));
         }
-    // The zero behind the channels of every staged pair, for the operands that a feature does not have.  Written here, not
-    // with the set-up: without room of its own the slab of the power spectrum runs through the staging area (the first
-    // barrier of pass 2 orders it).
-    const bool by_table = kRowTable && p.row_ops != nullptr && !o_compact;
-    if (by_table)
-        for (int e = tid; e < P; e += threads) sG2[e * GP + NCH] = make_float2(0.f, 0.f);
 
     // =========================== pass 2: the Jacobian rows ===========================
     const int NI = S * NCH, SN = S * NMAX;
@@ -1038,6 +1036,8 @@ center_kernel(const CenterParams p) {
             else { o0[f] = vx; o1[f] = vy; o2[f] = vz; }
         }
     };
+
+    const bool by_table = kRowTable && p.row_ops != nullptr && !o_compact;
 
     // Coefficient mode: the row of a neighbour of species Z is grad c^Z_nlm = G_nl grad S_lm + Ghat_nl d S_lm
     // (Eq. 14 / Eq. 23) in the block of Z and zero in the other blocks, written in aligned sweeps as above.

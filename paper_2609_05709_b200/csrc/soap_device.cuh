@@ -172,7 +172,10 @@ __host__ __device__ constexpr bool row_table_wanted(int n_max, int l_max) { retu
 // centre's pairs fit, and the room halves the chunk (kernel, 3000 centres of 68 pairs, with and without the room: (3, 9)
 // 445 -> 425 us, (4, 12) 851 -> 820 us, (3, 9) crossover off 373 -> 340 us; at l_max 8 and below 0.89 to 1.1 by the pairs).
 constexpr int kKeepFeatures = 512, kKeepLmax = 8;
-__host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, int P, int warps, bool weighted) {
+// by_table: the handle has a table of the rows' operands, whose zero behind the channels of every staged pair outlives the
+// power spectrum: the slab must not reach it.  (Writing that zero behind the power spectrum would do as well, but costs the
+// kernel 14 of 660 us on 36,000 centres of 18 pairs at (4, 3), where the slab has room of its own anyway.)
+__host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, int P, int warps, bool weighted, bool by_table = false) {
     const int L1 = l_max + 1, LMP = (L1 * L1) | 1, NCH = n_max * L1, CT = S * n_max * LMP, F = S * n_max * (S * n_max + 1) / 2 * L1;
     SmemLayout o;
     int off = 0;
@@ -193,7 +196,7 @@ __host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, i
     if (o.keep) { o.slab_words = 4 * F; off += 4 * F; }
     o.sSD = off; off = align4(off + P * LMP * 4);
     o.sG = off; off = align4(off + P * (NCH + (row_table_wanted(n_max, l_max) ? 1 : 0)) * 2);
-    if (!o.keep) o.slab_words = off - o.slab;
+    if (!o.keep) o.slab_words = (by_table ? o.sG : off) - o.slab;
     o.total = off;
     return o;
 }

@@ -38,6 +38,9 @@ int main() {
                         // decode tables, zeros, D), and apart from what stays staged where pass 2 relies on that
                         ok = ok && o.slab % 4 == 0 && o.slab >= o.D + 3 * CT && o.slab >= o.wUV + uv && o.slab + o.slab_words <= o.total;
                         if (o.keep) ok = ok && o.slab + o.slab_words <= o.sSD;
+                        // rows by the table of operands: the zero behind a pair's channels, in sG, is never written again
+                        const SmemLayout t = make_layout(S, n, l, P, warps, weighted, true);
+                        ok = ok && t.slab_words > 0 && t.slab + t.slab_words <= t.sG && t.slab == o.slab && t.sG == o.sG && t.total == o.total;
                         if (!ok) printf("species %d n_max %d l_max %d weighted %d warps %d\n", S, n, l, weighted, warps);
                     }
             }
