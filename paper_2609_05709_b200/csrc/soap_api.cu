@@ -547,7 +547,12 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     const size_t fixed_ts = (size_t)with_table.warp0 * 4, warp_bytes_ts = (size_t)with_table.per_warp * 4;
     const int warps_ts = h->desc_table_bytes > 0 && fixed_ts + warp_bytes_ts <= (size_t)h->max_smem
                              ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed_ts) / warp_bytes_ts) : 0;
-    const bool ts = !cp.pair_w && warps_ts >= 6 && n_work >= (int64_t)4 * h->sm_count;
+    // The table pays from four centres per SM on, except where the warps it costs make a second round of centres that keeps
+    // less than a quarter of them busy (coefficients, table against none: 1500 atoms at (8, 8) 46.1 against 39.6 us, 1000
+    // atoms of three species at (6, 9) 48.2 against 36.8 us; with a fuller second round 48.1 against 48.5 us and less).
+    const int64_t sms = h->sm_count;
+    const bool straggling = n_work <= warps_fit * sms && n_work > warps_ts * sms && 4 * n_work <= 5 * warps_ts * sms;
+    const bool ts = !cp.pair_w && warps_ts >= 6 && n_work >= 4 * sms && !straggling;
     int warps = ts ? warps_ts : warps_fit;
     warps = (int)std::max<int64_t>(1, std::min<int64_t>(warps, (n_work + h->sm_count - 1) / h->sm_count));
     const unsigned grid = (unsigned)std::min<int64_t>(h->sm_count, (n_work + warps - 1) / warps);

@@ -97,3 +97,23 @@ def test_options_on_many_centres(pkg, n_centers):
         soap, oracle = pkg.Soap(*args, **kw), SoapOracle(*args, **kw)
         got = soap.descriptor(pos, num, None, cen)
         assert col_err(got[sample].cpu().numpy(), oracle.descriptor(s.positions, s.numbers, None, of)) < DESC_TOL
+
+
+# sixteen warps without the radial table in shared memory, ten or thirteen with it: which of the two runs depends on the
+# warps that a second round of centres would keep busy
+@pytest.mark.parametrize("crossover", [True, False])
+@pytest.mark.parametrize("n_centers", [1480, 1481, 1850, 1851, 2368, 2369])
+@pytest.mark.parametrize("n_max,l_max,sigma", [(8, 8, 0.4), (4, 9, 0.5)])
+def test_rounds_of_centres(pkg, n_max, l_max, sigma, n_centers, crossover):
+    s = water_cluster(100, 1)
+    args = ([1, 8], 4.8, n_max, l_max, sigma, GTO)
+    soap, oracle = pkg.Soap(*args, crossover=crossover), SoapOracle(*args, crossover=crossover)
+    pos, num = torch.from_numpy(s.positions).cuda(), torch.from_numpy(s.numbers).cuda()
+    centers = np.random.default_rng(n_centers).integers(0, s.n_atoms, n_centers)
+    got = soap.descriptor(pos, num, None, torch.from_numpy(centers.astype(np.int32)).cuda())
+    few = soap.descriptor(pos, num)
+    scale = few.abs().max(dim=0).values.clamp_min(1e-3 * float(few.abs().max()))
+    assert float(((got - few[torch.from_numpy(centers).cuda()]).abs() / scale).max()) < DESC_TOL
+    sample = [0, 1479, n_centers - 1]
+    ref = oracle.descriptor(s.positions, s.numbers, None, centers[sample].tolist())
+    assert col_err(got[sample].cpu().numpy(), ref) < DESC_TOL
