@@ -52,11 +52,11 @@ __host__ __device__ constexpr int desc_s_row(int l_max) { return 4 * (desc_tiles
 __host__ __device__ constexpr int desc_g_l(int np) { return np == 16 ? 20 : np; }
 __host__ __device__ constexpr int desc_g_swap(int np, int l) { return np == 8 ? (l >> 2) & 1 : 0; }
 
-// The centre's coefficient tile c[lm][species, n]: S NP / 4 16-byte chunks per row, and one more chunk of room after every
-// four rows: the lanes of a warp, which own rows four apart, then do not all hit one group of banks when they store
-// their sums.
-__host__ __device__ constexpr int desc_c_at(int row, int row_chunks) { return row * row_chunks + (row >> 2); }
-__host__ __device__ constexpr int desc_c_words(int S, int np, int lm) { return 4 * (desc_c_at(lm - 1, S * np / 4) + S * np / 4); }
+// The centre's coefficient tile c[lm][species, n]: S NP / 4 16-byte chunks per row, and with `pad` one more chunk of room
+// after every four rows: the lanes of a warp, which own rows four apart, then do not all hit one group of banks when they
+// store their sums.  (launch_desc leaves the room out where it would cost a round of centres.)
+__host__ __device__ constexpr int desc_c_at(int row, int row_chunks, bool pad) { return row * row_chunks + (pad ? row >> 2 : 0); }
+__host__ __device__ constexpr int desc_c_words(int S, int np, int lm, bool pad) { return 4 * (desc_c_at(lm - 1, S * np / 4, pad) + S * np / 4); }
 
 // Pairs staged at once by a warp: 32 where a staged pair is small, so that every lane has a pair's harmonics to form
 // (80 words: sixteen warps still fit beside the table for two species), else 16; a team deals its chunks out to its warps
@@ -85,14 +85,14 @@ struct DescBlock {
 struct DescLayout {
     int table, blocks, warp0, per_warp, c, sS, sG, ring, slab_words, total;
 };
-__host__ __device__ inline DescLayout make_desc_layout(int S, int np, int l_max, int warps, int table_words, bool team) {
+__host__ __device__ inline DescLayout make_desc_layout(int S, int np, int l_max, int warps, int table_words, bool team, bool pad) {
     const int L1 = l_max + 1, LM = L1 * L1, n_blocks = desc_blocks(S, np, true), kDescChunk = desc_chunk(l_max, np, team);
     DescLayout o;
     o.table = 0;
     o.blocks = (table_words + 3) & ~3;
     o.warp0 = o.blocks + (n_blocks <= kDescTableBlocks ? n_blocks * (int)(sizeof(DescBlock) / 4) : 0);
     int off = 0;
-    o.c = off; off += desc_c_words(S, np, LM);
+    o.c = off; off += desc_c_words(S, np, LM, pad);
     o.sS = off; off += kDescChunk * desc_s_row(l_max);
     o.sG = off; off += kDescChunk * L1 * desc_g_l(np);
     o.ring = off; off += kDescChunk * (table_words ? 5 : 8);
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     const float2* const o_pw = PLAIN ? nullptr : p.pair_w;
     const float o_w0 = PLAIN ? 1.f : p.w0;
     const int S = p.S, NMAX = p.n_max, F = p.F;
-    const DescLayout lay = make_desc_layout(S, NP, L, warps, TS ? p.n_intervals * NCHP * 6 : 0, TEAM);
+    const DescLayout lay = make_desc_layout(S, NP, L, warps, TS ? p.n_intervals * NCHP * 6 : 0, TEAM, p.tile_pad);
 
     if (TS) {
         const float4* src = reinterpret_cast<const float4*>(p.table_ln);
@@ -226,7 +226,8 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     float* const wbase = smem + lay.warp0 + wid * lay.per_warp;
     float* const c_t = wbase + lay.c;                                               // [LM] rows of RC chunks, skewed
     const int RC = S * NP / 4;
-    auto c_chunk = [&](int r, int k) { return desc_c_at(r, RC) + k; };              // 16-byte chunk k of row r
+    const bool pad = p.tile_pad;
+    auto c_chunk = [&](int r, int k) { return desc_c_at(r, RC, pad) + k; };              // 16-byte chunk k of row r
     auto c_word = [&](int r, int col) { return 4 * c_chunk(r, col >> 2) + (col & 3); };
     float4* const sS4 = reinterpret_cast<float4*>(wbase + lay.sS);                  // [chunk][SROW / 4] tiles of four m
     float* const sG = wbase + lay.sG;                                               // [chunk][L1][GL]
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
         const float xi = hd.xi, yi = hd.yi, zi = hd.zi;
         const int zi_species = hd.zsp, k_pairs = hd.k_pairs;
 
-        for (int e = lane; e < desc_c_at(LM - 1, RC) + RC; e += 32) reinterpret_cast<float4*>(c_t)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e = lane; e < desc_c_at(LM - 1, RC, pad) + RC; e += 32) reinterpret_cast<float4*>(c_t)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
 
         for (int g0 = 0; g0 < k_pairs; g0 += kDescGroup) {
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
         if (TEAM) {
             // the tiles of the team add up in the first warp's, in a fixed order
             __syncthreads();
-            for (int e = threadIdx.x; e < desc_c_at(LM - 1, RC) + RC; e += blockDim.x) {
+            for (int e = threadIdx.x; e < desc_c_at(LM - 1, RC, pad) + RC; e += blockDim.x) {
                 float4 v = sum4[e];
                 for (int w = 1; w < warps; ++w) {
                     const float4 o = sum4[e + w * (lay.per_warp / 4)];
@@ -572,7 +573,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
                 int r = l >= 0 ? l * l : 0;
                 const float4 *pa = sum4 + blk.ta, *pb = sum4 + blk.tb;
                 for (int m = 0; m < steps; ++m, ++r) {
-                    const int at = desc_c_at(r, RC);
+                    const int at = desc_c_at(r, RC, pad);
                     const float4 A = pa[at], B = pb[at];
                     const float2 a01 = make_float2(A.x, A.y), a23 = make_float2(A.z, A.w);
                     const float2 b[2] = {make_float2(B.x, B.y), make_float2(B.z, B.w)}, bs[2] = {make_float2(B.y, B.x), make_float2(B.w, B.z)};

@@ -117,3 +117,19 @@ def test_rounds_of_centres(pkg, n_max, l_max, sigma, n_centers, crossover):
     sample = [0, 1479, n_centers - 1]
     ref = oracle.descriptor(s.positions, s.numbers, None, centers[sample].tolist())
     assert col_err(got[sample].cpu().numpy(), ref) < DESC_TOL
+
+
+# (14, 8) and (6, 4) with six species: the padding of a centre's tile costs a warp, and is there only where that makes no
+# further round of centres
+@pytest.mark.parametrize("n_species,n_max,l_max", [(2, 14, 8), (6, 6, 4)])
+@pytest.mark.parametrize("n_centers", [1036, 1037, 1184, 1776, 1924, 3000])
+def test_padded_and_plain_tiles(pkg, n_species, n_max, l_max, n_centers):
+    s = multispecies_box(90, 2)
+    species = [1, 6, 7, 8, 9, 14][:n_species]
+    s.numbers = np.random.default_rng(2).choice(species, size=s.n_atoms).astype(np.int32)
+    args = (species, 4.0, n_max, l_max, 0.5, GTO, (True, True, True))
+    centers = np.random.default_rng(n_centers).integers(0, s.n_atoms, n_centers).tolist()
+    got = check(pkg, s, args, [0, n_centers // 2, n_centers - 1], centers)
+    few = check(pkg, s, args, [0, 50, 89])
+    scale = few.abs().max(dim=0).values.clamp_min(1e-3 * float(few.abs().max()))
+    assert float(((got - few[centers]).abs() / scale).max()) < DESC_TOL
