@@ -14,8 +14,8 @@ LIB = os.path.join(HERE, "libsoap_b200.so")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC", "-Xptxas", "-v", "-Xfatbin=-compress-all"]
 # compiled in parallel, the longest first (compile time grows with l_max): the per-centre kernels are compiled
-# once per l_max from one source each (-DSOAP_L=<l_max>)
-PER_L_SOURCES = ["center_kernels", "desc_kernels"]
+# once per l_max and family from one source each (-DSOAP_L=<l_max> -DSOAP_FAMILY=<0 ...>)
+PER_L_SOURCES = {"center_kernels": 4, "desc_kernels": 2}
 PLAIN_UNITS = ["soap_api", "peak_kernel"]
 
 
@@ -45,10 +45,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
              "-c", os.path.join(CSRC, "basis_host.cpp"), "-o", obj("basis_host")]]
     objects = []
     for l in range(12, -1, -1):
-        for src in PER_L_SOURCES:
-            name = f"{src}_l{l}"
-            objects.append(name)
-            cmds.append([nvcc, *NVCC_FLAGS, f"-DSOAP_L={l}", "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src + ".cu"), "-o", obj(name)])
+        for src, families in PER_L_SOURCES.items():
+            for family in range(families):
+                name = f"{src}_l{l}_f{family}"
+                objects.append(name)
+                cmds.append([nvcc, *NVCC_FLAGS, f"-DSOAP_L={l}", f"-DSOAP_FAMILY={family}", "-I", INCLUDE, "-I", CSRC,
+                             "-c", os.path.join(CSRC, src + ".cu"), "-o", obj(name)])
     for unit in PLAIN_UNITS:
         objects.append(unit)
         cmds.append([nvcc, *NVCC_FLAGS, "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, unit + ".cu"), "-o", obj(unit)])

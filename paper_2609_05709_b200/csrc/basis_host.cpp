@@ -311,19 +311,6 @@ int build_basis(int rbf, double r_cut, int n_max, int l_max, double sigma,
     out.self_term.resize(n_max);
     for (int n = 0; n < n_max; ++n)
         out.self_term[n] = (float)(vals[(size_t)nint * kTableCoef * n_ch + n * L1] / sqrtq(4 * M_PIq));
-    // harmonic normalisation sqrt((2l+1)/4pi (l-m)!/(l+m)!), times sqrt2 for m > 0
-    out.anorm.resize(L1 * (L1 + 1) / 2);
-    for (int l = 0; l < L1; ++l)
-        for (int m = 0; m <= l; ++m) {
-            quad ratio = 1;
-            for (int j = l - m + 1; j <= l + m; ++j) ratio /= j;
-            quad a = sqrtq((2 * l + 1) / (4 * M_PIq) * ratio);
-            if (m > 0) a *= sqrtq(2.0Q);
-            out.anorm[l * (l + 1) / 2 + m] = (float)a;
-        }
-    out.dfact.resize(L1);
-    quad df = 1;
-    for (int m = 0; m < L1; ++m) { if (m > 0) df *= (2 * m - 1); out.dfact[m] = (float)df; }
     out.kl.resize(L1);
     for (int l = 0; l < L1; ++l) out.kl[l] = (float)(M_PIq * sqrtq(8.0Q / (2 * l + 1)));   // prefactor of Eq. 4
     return 0;

@@ -24,8 +24,6 @@ struct HostBasis {
     double inv_h_values = 0;
     std::vector<float> table_values;
     std::vector<float> self_term;                  // on-site c_n00, [n_max]
-    std::vector<float> anorm;                      // harmonic normalisation, [(l,m), m<=l], sqrt2 folded in for m>0
-    std::vector<float> dfact;                      // (2m-1)!!, [l_max+1]
     std::vector<float> kl;                         // pi sqrt(8/(2l+1)), [l_max+1]
 };
 

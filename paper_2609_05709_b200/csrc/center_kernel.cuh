@@ -25,6 +25,7 @@
 #pragma once
 #include <type_traits>
 
+#include "harmonic_tables.h"
 #include "soap_device.cuh"
 
 constexpr int kTriUnroll = 2;          // sweeps of a same-species block in flight per warp
@@ -34,10 +35,23 @@ namespace soap {
 
 // Universal small tables for the harmonic recursion (l_max <= 12), read with
 // warp-uniform indices, hence constant memory.  Each translation unit that
-// includes this file gets its own copy, filled in at load time.
-__device__ __constant__ float2 kc_norm[91] = {0};    // [(l,m)] a_lm = sqrt((2l+1)/4pi (l-m)!/(l+m)!) (sqrt2 for m > 0), (l+m) a_lm
-__device__ __constant__ float4 kc_step[91] = {0};    // [(l,m)] coefficients that advance columns m and m+1 from l to l+1
-__device__ __constant__ float kc_dfact[16] = {0};    // [m] (2m-1)!!
+// includes this file gets its own copy.
+struct HarmonicConstants {
+    float2 norm[kHarmonicTerms];         // [(l,m)] a_lm, (l+m) a_lm
+    float4 step[kHarmonicTerms];         // [(l,m)]
+    float dfact[16];                     // [m]
+};
+constexpr HarmonicConstants harmonic_constants() {
+    constexpr HarmonicTables t = harmonic_tables();
+    HarmonicConstants c{};
+    for (int i = 0; i < kHarmonicTerms; ++i) {
+        c.norm[i].x = t.norm[i]; c.norm[i].y = t.norm_lm[i];
+        c.step[i].x = t.step[i][0]; c.step[i].y = t.step[i][1]; c.step[i].z = t.step[i][2]; c.step[i].w = t.step[i][3];
+    }
+    for (int m = 0; m < 16; ++m) c.dfact[m] = t.dfact[m];
+    return c;
+}
+__device__ __constant__ HarmonicConstants kc = harmonic_constants();
 
 // Degree-5 table lookup of two adjacent n of one l, whose coefficients lie interleaved: values and derivatives with
 // respect to the interval coordinate t, by packed multiply-adds.
@@ -67,12 +81,12 @@ __device__ __forceinline__ void harmonics_column(int L, int m, float x, float y,
         sm = x * sm + y * cm;
         cm = cn;
     }
-    float a1 = kc_dfact[m], a0 = 0.f;                           // Q_l^m, Q_{l-1}^m
+    float a1 = kc.dfact[m], a0 = 0.f;                           // Q_l^m, Q_{l-1}^m
     float b1 = 0.f, b0 = 0.f;                                   // Q_l^{m+1}, Q_{l-1}^{m+1}
     const float fm = (float)m;
     int t = m * (m + 1) / 2 + m;                                // index of (l, m), l = m
     for (int l = m; l <= L; ++l) {
-        const float2 nr = kc_norm[t];
+        const float2 nr = kc.norm[t];
         const float aq = nr.x * a1;
         const int lm0 = l * l + l;
         const float qz = nr.y * a0;                             // a (l+m) Q_{l-1}^m  (a0 = 0 when l = m)
@@ -82,10 +96,10 @@ __device__ __forceinline__ void harmonics_column(int L, int m, float x, float y,
         out4[lm0 + m] = make_float4(aq * cm, mq * cp - xq * cm, -mq * sp - yq * cm, qz * cm);
         if (m) out4[lm0 - m] = make_float4(aq * sm, mq * sp - xq * sm, mq * cp - yq * sm, qz * sm);
         // advance both columns to l + 1
-        const float4 st = kc_step[t];
+        const float4 st = kc.step[t];
         const float an = st.x * z * a1 - st.y * r2 * a0;
         a0 = a1; a1 = an;
-        const float bn = (l == m) ? kc_dfact[m + 1] : st.z * z * b1 - st.w * r2 * b0;
+        const float bn = (l == m) ? kc.dfact[m + 1] : st.z * z * b1 - st.w * r2 * b0;
         b0 = b1; b1 = bn;
         t += l + 1;
     }

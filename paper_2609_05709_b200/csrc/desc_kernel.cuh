@@ -22,6 +22,7 @@
 // At (8, 6) on 30,000 atoms the kernel takes 246 us; the shared-memory pipe is 77 % busy, the issue slots 57 %.
 // Nothing but the pair list is read from HBM and nothing but the descriptor row is written.
 #pragma once
+#include "harmonic_tables.h"
 #include "soap_device.cuh"
 
 namespace soap {
@@ -30,8 +31,15 @@ constexpr int kDescGroup = 64;                    // pairs whose geometry a warp
 constexpr int kDescMaxWarps = 16;                 // warps per CTA (one CTA per SM)
 constexpr int kDescTeamWarps = 4;                 // most warps of a CTA that works on one centre
 
-// harmonic normalisation up to l = 12, filled by desc_constants(): a_lm (sqrt2 folded in for m > 0), index l(l+1)/2 + m
-__device__ __constant__ float kd_norm[91] = {0};
+// harmonic normalisation up to l = 12: a_lm (sqrt2 folded in for m > 0), index l(l+1)/2 + m
+struct HarmonicNorm { float a[kHarmonicTerms]; };
+constexpr HarmonicNorm harmonic_norm() {
+    constexpr HarmonicTables t = harmonic_tables();
+    HarmonicNorm n{};
+    for (int i = 0; i < kHarmonicTerms; ++i) n.a[i] = t.norm[i];
+    return n;
+}
+__device__ __constant__ HarmonicNorm kd_norm = harmonic_norm();
 
 // tiles of four consecutive m of one l: tile index of the first tile of row l, and their number up to l_max
 __host__ __device__ constexpr int desc_tile_base(int l) {
@@ -135,7 +143,7 @@ __device__ __forceinline__ void harmonics_tiles(float x, float y, float z, float
             else q = (zl * q1[m] - (float)(l - 1 + m) * r2 * q2[m]) * (1.f / (float)(l - m));
             q2[m] = q1[m];
             q1[m] = q;
-            const float aq = kd_norm[l * (l + 1) / 2 + m] * q;
+            const float aq = kd_norm.a[l * (l + 1) / 2 + m] * q;
             row[l + m] = aq * cm[m];
             if (m) row[l - m] = aq * sm[m];
         }

@@ -3,18 +3,16 @@
 #include "soap_device.cuh"
 
 namespace soap {
-// harmonic normalisation up to l = 12: anorm[91] (index l(l+1)/2 + m)
-cudaError_t desc_constants(int l_max, const float* anorm91);
-cudaError_t desc_set_smem(int l_max, int np, int bytes);
-// plain: every option at its default (see desc_kernel); table_in_smem: the radial table is staged per CTA
-cudaError_t desc_launch(int l_max, int np, bool plain, bool table_in_smem, bool team, const CenterParams& p, unsigned grid,
-                        unsigned block, size_t smem, cudaStream_t st);
+using DescKernel = void (*)(CenterParams);
+// plain: every option at its default (see desc_kernel); table_in_smem: the radial table is staged per CTA; team: a CTA per
+// centre.  Null where there is none.  (It waits on the device for the kernel before it: launch it with launch_dependent,
+// launch and table staging overlap that kernel's tail.)
+DescKernel desc_kernel_of(int l_max, int np, bool plain, bool table_in_smem, bool team);
 
-#define SOAP_DECLARE_L(LV)                                                                                              \
-    cudaError_t desc_constants_l##LV(const float* anorm91);                                                             \
-    cudaError_t desc_set_smem_l##LV(int np, int bytes);                                                                 \
-    cudaError_t desc_launch_l##LV(int np, bool plain, bool table_in_smem, bool team, const CenterParams& p, unsigned grid,         \
-                                  unsigned block, size_t smem, cudaStream_t st);
+// compiled, and loaded, apart for the two values of `plain`
+#define SOAP_DECLARE_L(LV)                                                           \
+    DescKernel desc_kernel_l##LV##_f0(int np, bool table_in_smem, bool team);         \
+    DescKernel desc_kernel_l##LV##_f1(int np, bool table_in_smem, bool team);
 SOAP_DECLARE_L(0) SOAP_DECLARE_L(1) SOAP_DECLARE_L(2) SOAP_DECLARE_L(3) SOAP_DECLARE_L(4) SOAP_DECLARE_L(5) SOAP_DECLARE_L(6)
 SOAP_DECLARE_L(7) SOAP_DECLARE_L(8) SOAP_DECLARE_L(9) SOAP_DECLARE_L(10) SOAP_DECLARE_L(11) SOAP_DECLARE_L(12)
 #undef SOAP_DECLARE_L

@@ -26,54 +26,24 @@
 using namespace soap;
 
 namespace soap {
-cudaError_t center_constants(int l_max, const float* anorm91, const float* dfact16) {
-    switch (l_max) {
-#define X(LV) case LV: return center_constants_l##LV(anorm91, dfact16);
+CenterKernel center_kernel_of(int kind, bool plain, int l_max, int n_max) {
+    const int family = kind == kCenterDeriv ? (plain ? kFamilyPlain : kFamilyOptions) : kind == kCenterCoeff ? kFamilyCoeff : kFamilyAverage;
+    switch (4 * l_max + family) {
+#define X(LV)                                                                                                                     \
+    case 4 * LV: return center_kernel_l##LV##_f0(kind, n_max);     case 4 * LV + 1: return center_kernel_l##LV##_f1(kind, n_max); \
+    case 4 * LV + 2: return center_kernel_l##LV##_f2(kind, n_max); case 4 * LV + 3: return center_kernel_l##LV##_f3(kind, n_max);
         X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
 #undef X
     }
-    return cudaErrorInvalidValue;
+    return nullptr;
 }
-cudaError_t center_set_smem(int kind, int l_max, int n_max, int bytes) {
+DescKernel desc_kernel_of(int l_max, int np, bool plain, bool table_in_smem, bool team) {
     switch (l_max) {
-#define X(LV) case LV: return center_set_smem_l##LV(kind, n_max, bytes);
+#define X(LV) case LV: return plain ? desc_kernel_l##LV##_f0(np, table_in_smem, team) : desc_kernel_l##LV##_f1(np, table_in_smem, team);
         X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
 #undef X
     }
-    return cudaErrorInvalidValue;
-}
-cudaError_t center_launch(int kind, int l_max, int n_max, int threads, const CenterParams& p, unsigned grid, size_t smem, cudaStream_t st) {
-    switch (l_max) {
-#define X(LV) case LV: return center_launch_l##LV(kind, n_max, center_params_plain(p), threads, p, grid, smem, st);
-        X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
-#undef X
-    }
-    return cudaErrorInvalidValue;
-}
-cudaError_t desc_constants(int l_max, const float* anorm91) {
-    switch (l_max) {
-#define X(LV) case LV: return desc_constants_l##LV(anorm91);
-        X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
-#undef X
-    }
-    return cudaErrorInvalidValue;
-}
-cudaError_t desc_set_smem(int l_max, int np, int bytes) {
-    switch (l_max) {
-#define X(LV) case LV: return desc_set_smem_l##LV(np, bytes);
-        X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
-#undef X
-    }
-    return cudaErrorInvalidValue;
-}
-cudaError_t desc_launch(int l_max, int np, bool plain, bool table_in_smem, bool team, const CenterParams& p, unsigned grid, unsigned block,
-                        size_t smem, cudaStream_t st) {
-    switch (l_max) {
-#define X(LV) case LV: return desc_launch_l##LV(np, plain, table_in_smem, team, p, grid, block, smem, st);
-        X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
-#undef X
-    }
-    return cudaErrorInvalidValue;
+    return nullptr;
 }
 }  // namespace soap
 
@@ -93,6 +63,7 @@ struct soap_handle {
     int64_t Fc = 0, Fc_pitch = 0;
     int* d_compact_map = nullptr;
     std::string error;
+    std::vector<const void*> launchable;   // per-centre kernels that may take all the shared memory of the device
     // device state (created on first use)
     int device = -1;
     bool tables_ready = false;
@@ -214,23 +185,16 @@ int plan_smem(soap_t* h) {
     h->max_smem = max_smem;
     h->desc_warp_bytes = (size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0, false, false).per_warp * 4;
     if (h->desc_warp_bytes > (size_t)max_smem) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
-    CU(desc_set_smem(h->l_max, desc_np(h->n_max), max_smem));
     auto plan = [&](int warps, size_t extra, int& P, size_t& bytes) {
         return plan_chunk(h->S, h->n_max, h->l_max, h->weight.fn != 0, warps, extra, (size_t)max_smem, P, bytes);
     };
     // 256 threads, and the smaller CTAs that this basis may run with
     if (!plan(8, 0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
     if (!plan(4, 0, h->P_deriv4, h->smem_deriv4)) h->smem_deriv4 = 0;
-    // (a kernel's limit is the process's, not the handle's: every handle sets the device's maximum, so that none takes away
-    // what another one launches with)
-    CU(center_set_smem(kCenterDeriv, h->l_max, h->n_max, max_smem));
-    CU(center_set_smem(kCenterCoeff, h->l_max, h->n_max, max_smem));
-    CU(center_set_smem(kCenterInner, h->l_max, h->n_max, max_smem));
     // the kernel of the outer average keeps, per warp, a copy of a neighbouring centre's coefficients behind the usual
     // layout; a basis too large for that takes the general path (per-pair rows in a workspace)
     const int LMP = ((h->l_max + 1) * (h->l_max + 1)) | 1;
     h->outer_fast = plan(kThreads / 32, (size_t)(kThreads / 32) * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
-    if (h->outer_fast) CU(center_set_smem(kCenterOuter, h->l_max, h->n_max, max_smem));
     return SOAP_OK;
 }
 
@@ -304,14 +268,6 @@ int ensure_device(soap_t* h) {
     CU(cudaMalloc((void**)&h->d_grid, sizeof(GridParams)));
     CU(cudaMallocHost((void**)&h->h_counters, sizeof(Counters)));
     if (int rc = plan_smem(h)) return rc;
-    {
-        // universal harmonic tables up to l = 12 (the handle's own tables stop at its l_max)
-        std::vector<float> anorm(91, 0.f), dfact(16, 0.f);
-        for (size_t i = 0; i < h->basis.anorm.size(); ++i) anorm[i] = h->basis.anorm[i];
-        for (size_t i = 0; i < h->basis.dfact.size(); ++i) dfact[i] = h->basis.dfact[i];
-        CU(center_constants(h->l_max, anorm.data(), dfact.data()));
-        CU(desc_constants(h->l_max, anorm.data()));
-    }
     h->tables_ready = true;
     return SOAP_OK;
 }
@@ -520,6 +476,23 @@ void fill_center_params(soap_t* h, CenterParams& cp, const float* pos, const int
     cp.out_desc = nullptr; cp.out_jac = nullptr; cp.row_atom = nullptr;
 }
 
+// Launch of a per-centre kernel.  Its limit of dynamic shared memory is set with the handle's first launch of it, not with the
+// handle: that loads the kernel, and a handle launches one or two of the many of its basis (first call of a process at
+// (8, 6), best of four: derivatives of 24 atoms 36.9 -> 16.6 ms, descriptor of 3000 37.5 -> 13.3 ms).  The limit is the
+// process's, not the handle's: every handle sets the device's maximum, so that none takes away what another one launches with.
+int launch_per_center(soap_t* h, void (*kernel)(CenterParams), const CenterParams& cp, unsigned grid, unsigned threads, size_t smem, cudaStream_t st) {
+    const void* const key = (const void*)kernel;
+    if (std::find(h->launchable.begin(), h->launchable.end(), key) == h->launchable.end()) {
+        CU(cudaFuncSetAttribute(key, cudaFuncAttributeMaxDynamicSharedMemorySize, h->max_smem));
+        h->launchable.push_back(key);
+    }
+    CU(launch_dependent(kernel, grid, threads, smem, st, cp));
+    return SOAP_OK;
+}
+int launch_center(soap_t* h, int kind, const CenterParams& cp, int64_t n_centers, int threads, size_t smem, cudaStream_t st) {
+    return launch_per_center(h, center_kernel_of(kind, center_params_plain(cp), h->l_max, h->n_max), cp, (unsigned)n_centers, (unsigned)threads, smem, st);
+}
+
 // Launch of the descriptor-only kernel: persistent CTAs (one per SM) whose warps take the centres in turn.
 // The radial table goes to shared memory when it leaves room for at least six warps and there is enough
 // work to pay for staging it; small jobs use fewer warps per CTA so that they spread over the SMs, the smallest
@@ -538,8 +511,7 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
         const int64_t per_sm = std::min<int64_t>(team_warps == 2 ? 5 : 16 / kDescTeamWarps, (int64_t)(228 * 1024 / (bytes + 1024)));
         if (n_work > per_sm * h->sm_count || bytes > (size_t)h->max_smem) continue;
         cp.tile_pad = 1;
-        CU(desc_launch(h->l_max, h->desc_np, plain, false, true, cp, (unsigned)n_work, (unsigned)team_warps * 32, bytes, st));
-        return SOAP_OK;
+        return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true), cp, (unsigned)n_work, (unsigned)team_warps * 32, bytes, st);
     }
     // Warps that fit, beside the radial table or without it (with it a warp's region is a little smaller: its staged pairs are
     // five words, not eight), with and without the padded tile.
@@ -565,8 +537,7 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(fit(ts, cp.tile_pad), (n_work + sms - 1) / sms));
     const unsigned grid = (unsigned)std::min<int64_t>(sms, (n_work + warps - 1) / warps);
     const size_t smem = (size_t)layout(warps, ts, cp.tile_pad).total * 4;
-    CU(desc_launch(h->l_max, h->desc_np, plain, ts, false, cp, grid, (unsigned)warps * 32, smem, st));
-    return SOAP_OK;
+    return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, ts, false), cp, grid, (unsigned)warps * 32, smem, st);
 }
 
 // What the bits of the status word mean to a caller.
@@ -591,8 +562,7 @@ int launch_deriv(soap_t* h, int kind, CenterParams& cp, int64_t n_centers, cudaS
     if (small && needs <= 128 && h->smem_deriv4 != 0 && n_centers >= (int64_t)5 * h->sm_count) {
         threads = 128; cp.P = h->P_deriv4; bytes = h->smem_deriv4;
     }
-    CU(center_launch(kind, h->l_max, h->n_max, threads, cp, (unsigned)n_centers, bytes, st));
-    return SOAP_OK;
+    return launch_center(h, kind, cp, n_centers, threads, bytes, st);
 }
 
 // Feature table: species pairs mu <= nu (only mu == nu without crossover), radial pair (n' >= n on
@@ -1201,7 +1171,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
         cp.out_jac = d_out_jac;
         cp.inner_rows = 1;
         cp.own_scale = (float)(1.0 / (double)n_centers);
-        CU(center_launch(kCenterInner, h->l_max, h->n_max, kThreads, cp, (unsigned)n_centers, h->smem_deriv, st));
+        if ((rc = launch_center(h, kCenterInner, cp, n_centers, kThreads, h->smem_deriv, st))) return rc;
         if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
         return SOAP_OK;
     }
@@ -1226,7 +1196,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
         cp.out_jac = d_out_jac;
         cp.own_scale = (float)(1.0 / (double)n_centers);
         cp.P = h->P_outer;
-        CU(center_launch(kCenterOuter, h->l_max, h->n_max, kThreads, cp, (unsigned)n_centers, h->smem_outer, st));
+        if ((rc = launch_center(h, kCenterOuter, cp, n_centers, kThreads, h->smem_outer, st))) return rc;
         if ((rc = column_mean(h, (const float*)(w + o_rows), n_centers, F, (double*)(w + o_partial), d_out_desc, st))) return rc;
         if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
         return SOAP_OK;
