@@ -152,7 +152,7 @@ center_kernel(const CenterParams p) {
     constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
     // words pairs (G, Ghat) per staged pair: the channels, and with a row table a zero behind them
     constexpr bool kRowTable = KIND == 1 && NMAX_T != 0 && row_table_wanted(NMAX_T, L);
-    const SmemLayout lay = make_layout(S, NMAX, L, P, warps, o_pw != nullptr, kRowTable && p.row_ops != nullptr);
+    const SmemLayout lay = make_layout(S, NMAX, L, P, warps, o_pw != nullptr, kRowTable && !PLAIN && p.row_ops != nullptr);
     const int GP = NCH + (row_table_wanted(NMAX, L) ? 1 : 0);
     const int CP = NMAX_T ? CP_T : (NMAX + 1) / 2 * L1;                     // channel pairs: (l, two adjacent n)
     float* c_t = smem + lay.c;                                             // [S][NMAX][LMP]
@@ -174,7 +174,7 @@ center_kernel(const CenterParams p) {
     for (int e = tid; e < zero_w; e += threads) smem[lay.zero + e] = 0.f;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // the zero behind the channels of every staged pair, for the operands that a feature does not have in rows by table (the
-    // slab of the power spectrum ends before it, make_layout)
+    // slab of the power spectrum ends before it; with every species pair a feature it does so by itself, make_layout)
     if (kRowTable)
         for (int e = tid; e < P; e += threads) sG2[e * GP + NCH] = make_float2(0.f, 0.f);
 

@@ -174,8 +174,10 @@ __host__ __device__ constexpr bool row_table_wanted(int n_max, int l_max) { retu
 // 445 -> 425 us, (4, 12) 851 -> 820 us, (3, 9) crossover off 373 -> 340 us; at l_max 8 and below 0.89 to 1.1 by the pairs).
 constexpr int kKeepFeatures = 512, kKeepLmax = 8;
 // by_table: the handle has a table of the rows' operands, whose zero behind the channels of every staged pair outlives the
-// power spectrum: the slab must not reach it.  (Writing that zero behind the power spectrum would do as well, but costs the
-// kernel 14 of 660 us on 36,000 centres of 18 pairs at (4, 3), where the slab has room of its own anyway.)
+// power spectrum: the slab must not reach it.  With crossover that holds anyway (the table stops at kKeepFeatures features,
+// and what has no room of its own up to there has l_max above kKeepLmax and few features), so the plain kernels do not ask.
+// (Writing that zero behind the power spectrum would do as well, but costs the kernel 14 of 660 us on 36,000 centres of 18
+// pairs at (4, 3), where the slab has room of its own; asking there costs 4 us.)
 __host__ __device__ inline SmemLayout make_layout(int S, int n_max, int l_max, int P, int warps, bool weighted, bool by_table = false) {
     const int L1 = l_max + 1, LMP = (L1 * L1) | 1, NCH = n_max * L1, CT = S * n_max * LMP, F = S * n_max * (S * n_max + 1) / 2 * L1;
     SmemLayout o;

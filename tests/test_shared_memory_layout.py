@@ -39,6 +39,9 @@ int main() {
                         ok = ok && o.slab % 4 == 0 && o.slab >= o.D + 3 * CT && o.slab >= o.wUV + uv && o.slab + o.slab_words <= o.total;
                         if (o.keep) ok = ok && o.slab + o.slab_words <= o.sSD;
                         // rows by the table of operands: the zero behind a pair's channels, in sG, is never written again
+                        // (with crossover off: `t`; with crossover the layout does not ask, and the features must fit before it)
+                        const int F = S * n * (S * n + 1) / 2 * L1;
+                        if (row_table_wanted(n, l) && F <= kKeepFeatures) ok = ok && o.slab + (4 * F < o.slab_words ? 4 * F : o.slab_words) <= o.sG;
                         const SmemLayout t = make_layout(S, n, l, P, warps, weighted, true);
                         ok = ok && t.slab_words > 0 && t.slab + t.slab_words <= t.sG && t.slab == o.slab && t.sG == o.sG && t.total == o.total;
                         if (!ok) printf("species %d n_max %d l_max %d weighted %d warps %d\n", S, n, l, weighted, warps);
