@@ -1001,12 +1001,14 @@ brute_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, con
 // above that eight (36,000 centres: 46 us with one, 13 us with eight).
 constexpr int kSizeBins = 256, kSizeBinShift = 2;
 constexpr int kRowsCtas = 8, kRowsPerThread = 8, kRowsPerCta = 4096;
+// Sum: what holds the rows of a CTA's centres (launch_neighbors: 64 bits where centres times atoms say that 32 do not do).
+template <typename Sum>
 __global__ void __launch_bounds__(1024)
 rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pair_count, int C,
                   long long* __restrict__ row_ptr, int* __restrict__ order, Counters* counters, Counters* host) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ long long warp_sums[32], cta_sum;                             // (a Jacobian may have more than 2^31 rows)
+    __shared__ Sum warp_sums[32], cta_sum;
     __shared__ int hist[kSizeBins], total[kSizeBins], first_slot[kSizeBins];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
@@ -1018,7 +1020,7 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
     grid_dependency_wait();                                                  // the counts of the pair kernel
     __syncthreads();
     int v[kRowsPerThread], bin[kRowsPerThread];
-    long long mine = 0;
+    Sum mine = 0;
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; ++k) {
         v[k] = bin[k] = 0;
@@ -1029,17 +1031,17 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
         }
         mine += v[k];
     }
-    long long incl = mine;
+    Sum incl = mine;
     for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        const Sum y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
     if (lane == 31) warp_sums[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-        long long w = warp_sums[lane];
+        Sum w = warp_sums[lane];
         for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, w, o);
+            const Sum y = __shfl_up_sync(0xffffffffu, w, o);
             if (lane >= o) w += y;
         }
         warp_sums[lane] = w;
@@ -1059,7 +1061,7 @@ rows_order_kernel(const int* __restrict__ row_count, const int* __restrict__ pai
             total[tid] = all;
         }
         for (int r = 0; r < ctas; ++r) {
-            const long long t = *cluster.map_shared_rank(&cta_sum, r);
+            const Sum t = *cluster.map_shared_rank(&cta_sum, r);
             if (r < rank) base += t;
             rows += t;
         }

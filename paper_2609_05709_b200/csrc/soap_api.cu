@@ -401,8 +401,11 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
     }
     h->ordered = C <= kOrderMaxCenters;
     if (h->ordered) {
-        CU(launch_cluster(rows_order_kernel, C <= kRowsPerCta ? 1 : kRowsCtas, 1024, st, true, h->d_row_count, h->d_pair_count, (int)C, row_ptr_out, h->d_order,
-                          h->d_counters, host));
+        // A centre has a row per atom at most.  (Sums in 64 bits take 1.5 us longer on 3000 centres, 3 us on 36,000.)
+        const int ctas = C <= kRowsPerCta ? 1 : kRowsCtas;
+        const bool wide = (C + ctas - 1) / ctas * N > INT32_MAX;
+        CU(launch_cluster(wide ? rows_order_kernel<long long> : rows_order_kernel<int>, ctas, 1024, st, true, h->d_row_count, h->d_pair_count, (int)C,
+                          row_ptr_out, h->d_order, h->d_counters, host));
     } else {
         scan_counts(h, h->d_row_count, row_ptr_out, C, &h->d_counters->n_rows, st, h->d_counters, host);
     }
