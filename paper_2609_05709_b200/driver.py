@@ -114,12 +114,15 @@ def cuda_backend(rank: int, config: dict):
             host[k].copy_(v)
         return host
 
-    # warm-up: one tiny call so that module loading and first-launch costs are paid before the start signal
+    # warm-up: one tiny call of each kind that tasks make, so that module loading and first-launch costs are paid before the
+    # start signal (a descriptor job's kernels are not among those that the derivative call loads)
     sp = [int(z) for z in config["species"]]
     wpos = torch.tensor([[0.0, 0.0, 0.0], [0.9, 0.1, 0.0], [40.0, 0.0, 0.0]], dtype=torch.float32, device="cuda")
     wnum = torch.tensor([sp[0], sp[-1], sp[0]], dtype=torch.int32, device="cuda")
     periodic = any(config.get("pbc", (False, False, False)))
-    soap.derivatives(wpos, wnum, np.eye(3) * 100.0 if periodic else None)
+    wcell = np.eye(3) * 100.0 if periodic else None
+    soap.derivatives(wpos, wnum, wcell)
+    soap.descriptor(wpos, wnum, wcell)
     torch.cuda.synchronize()
     return run
 
