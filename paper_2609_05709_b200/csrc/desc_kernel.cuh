@@ -19,7 +19,7 @@
 //   * Eq. 4 is the Gram matrix of that tile per l: lanes take 4 x 4 blocks of (species, n) pairs,
 //     two 16-byte loads per 16 multiply-adds, and the feature row is put together in shared memory
 //     and handed to the copy engine.
-// At (8, 6) on 30,000 atoms the kernel takes 246 us; the shared-memory pipe is 77 % busy, the issue slots 57 %.
+// At (8, 6) on 30,000 atoms the kernel takes 229 us; the L1 data pipe is 76 % busy, the issue slots 58 %.
 // Nothing but the pair list is read from HBM and nothing but the descriptor row is written.
 #pragma once
 #include "harmonic_tables.h"
@@ -62,7 +62,12 @@ __host__ __device__ constexpr int desc_g_swap(int np, int l) { return np == 8 ? 
 
 // The centre's coefficient tile c[lm][species, n]: S NP / 4 16-byte chunks per row, and with `pad` one more chunk of room
 // after every four rows: the lanes of a warp, which own rows four apart, then do not all hit one group of banks when they
-// store their sums.  (launch_desc leaves the room out where it would cost a round of centres.)
+// store their sums.  Not in the plain kernel at l_max 8 with n_max 13 to 16, where two species keep eight warps without the
+// room and seven with it (9000 atoms at (14, 8) 430 -> 389 us, 30,000 at (16, 8) 1659 -> 1565 us; one, three, four and five
+// species, whose warps stay, 0 to 1.4 % faster).  Coefficients, read from the tile row by row, need it (899 centres 46
+// against 52 us).  As an option of the launch, wherever the room costs a warp, it took registers from the largest bases ((7,
+// 10) on 28,821 atoms 903 -> 988 us).
+__host__ __device__ constexpr bool desc_tile_pad(int np, int l_max, bool plain) { return !(plain && np == 16 && l_max == 8); }
 __host__ __device__ constexpr int desc_c_at(int row, int row_chunks, bool pad) { return row * row_chunks + (pad ? row >> 2 : 0); }
 __host__ __device__ constexpr int desc_c_words(int S, int np, int lm, bool pad) { return 4 * (desc_c_at(lm - 1, S * np / 4, pad) + S * np / 4); }
 
@@ -87,20 +92,20 @@ struct DescBlock {
 
 // Shared memory in 4-byte words: [table (optional)] [block table (few blocks)] then one region per warp:
 //   c [LM] rows | S staging [chunk][s_row] | G staging [chunk][L1 g_l] | pair staging [chunk][8 or 5]
-// The feature row is assembled on top of the staging area when it fits there.  With the table in shared memory (the
-// plain build on many centres) a staged pair is five words (dx, dy, dz, t; interval | species << 16) instead of
-// eight (dx, dy, dz, r; interval, t, species, weight): at the benchmark's basis that is what lets a 16th warp fit.
+// The feature row is assembled on top of the staging area when it fits there.  With the table in shared memory (many
+// centres, no radial weighting) a staged pair is five words (dx, dy, dz, t; interval | species << 16) instead of eight (dx,
+// dy, dz, r; interval, t, species, weight), for the room of it.
 struct DescLayout {
     int table, blocks, warp0, per_warp, c, sS, sG, ring, slab_words, total;
 };
-__host__ __device__ inline DescLayout make_desc_layout(int S, int np, int l_max, int warps, int table_words, bool team, bool pad) {
+__host__ __device__ inline DescLayout make_desc_layout(int S, int np, int l_max, int warps, int table_words, bool team, bool plain) {
     const int L1 = l_max + 1, LM = L1 * L1, n_blocks = desc_blocks(S, np, true), kDescChunk = desc_chunk(l_max, np, team);
     DescLayout o;
     o.table = 0;
     o.blocks = (table_words + 3) & ~3;
     o.warp0 = o.blocks + (n_blocks <= kDescTableBlocks ? n_blocks * (int)(sizeof(DescBlock) / 4) : 0);
     int off = 0;
-    o.c = off; off += desc_c_words(S, np, LM, pad);
+    o.c = off; off += desc_c_words(S, np, LM, desc_tile_pad(np, l_max, plain));
     o.sS = off; off += kDescChunk * desc_s_row(l_max);
     o.sG = off; off += kDescChunk * L1 * desc_g_l(np);
     o.ring = off; off += kDescChunk * (table_words ? 5 : 8);
@@ -178,7 +183,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     const float2* const o_pw = PLAIN ? nullptr : p.pair_w;
     const float o_w0 = PLAIN ? 1.f : p.w0;
     const int S = p.S, NMAX = p.n_max, F = p.F;
-    const DescLayout lay = make_desc_layout(S, NP, L, warps, TS ? p.n_intervals * NCHP * 6 : 0, TEAM, p.tile_pad);
+    const DescLayout lay = make_desc_layout(S, NP, L, warps, TS ? p.n_intervals * NCHP * 6 : 0, TEAM, PLAIN);
 
     if (TS) {
         const float4* src = reinterpret_cast<const float4*>(p.table_ln);
@@ -234,7 +239,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     float* const wbase = smem + lay.warp0 + wid * lay.per_warp;
     float* const c_t = wbase + lay.c;                                               // [LM] rows of RC chunks, skewed
     const int RC = S * NP / 4;
-    const bool pad = p.tile_pad;
+    constexpr bool pad = desc_tile_pad(NP, L, PLAIN);
     auto c_chunk = [&](int r, int k) { return desc_c_at(r, RC, pad) + k; };              // 16-byte chunk k of row r
     auto c_word = [&](int r, int col) { return 4 * c_chunk(r, col >> 2) + (col & 3); };
     float4* const sS4 = reinterpret_cast<float4*>(wbase + lay.sS);                  // [chunk][SROW / 4] tiles of four m

@@ -71,11 +71,11 @@ struct soap_handle {
     float* d_table_ln = nullptr;         // the radial table re-laid for the descriptor-only kernel
     int sm_count = 0, max_smem = 0;
     int desc_np = 0;                     // n_max rounded up to a multiple of four
-    size_t desc_table_bytes = 0, desc_warp_bytes = 0;
+    size_t desc_table_bytes = 0;
     unsigned* d_row_ops = nullptr;       // operands of the Jacobian rows' features (small bases)
     int *d_feat = nullptr, *d_zlut = nullptr, *d_l_of_lm = nullptr;
     Counters* d_counters = nullptr;
-    unsigned long long* d_bbox = nullptr;   // 6 words of bounding box (structures above 16384 atoms)
+    unsigned long long* d_bbox = nullptr;   // 6 words of bounding box (structures above kPrepAtoms atoms)
     int* d_order = nullptr;
     GridParams* d_grid = nullptr;
     Counters* h_counters = nullptr;      // pinned
@@ -183,8 +183,7 @@ int plan_smem(soap_t* h) {
     int max_smem = 0;
     CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     h->max_smem = max_smem;
-    h->desc_warp_bytes = (size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0, false, false).per_warp * 4;
-    if (h->desc_warp_bytes > (size_t)max_smem) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
+    if ((size_t)make_desc_layout(h->S, desc_np(h->n_max), h->l_max, 1, 0, false, false).total * 4 > (size_t)max_smem) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
     auto plan = [&](int warps, size_t extra, int& P, size_t& bytes) {
         return plan_chunk(h->S, h->n_max, h->l_max, h->weight.fn != 0, warps, extra, (size_t)max_smem, P, bytes);
     };
@@ -510,36 +509,27 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     // of the sizes).  Whole calls, (n_max, l_max) = (8, 6): 120 atoms 27 -> 17 us, 431 atoms of four species 66 -> 38 us,
     // 600 atoms 31.2 -> 29.2 us; (12, 8), 600 atoms 60 -> 43 us.
     for (const int team_warps : {kDescTeamWarps, 2}) {
-        const size_t bytes = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, team_warps, 0, true, true).total * 4;
+        const size_t bytes = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, team_warps, 0, true, plain).total * 4;
         const int64_t per_sm = std::min<int64_t>(team_warps == 2 ? 5 : 16 / kDescTeamWarps, (int64_t)(228 * 1024 / (bytes + 1024)));
         if (n_work > per_sm * h->sm_count || bytes > (size_t)h->max_smem) continue;
-        cp.tile_pad = 1;
         return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true), cp, (unsigned)n_work, (unsigned)team_warps * 32, bytes, st);
     }
-    // Warps that fit, beside the radial table or without it (with it a warp's region is a little smaller: its staged pairs are
-    // five words, not eight), with and without the padded tile.
-    const int words = (int)(h->desc_table_bytes / 4);
-    auto layout = [&](int warps, bool table, bool pad) { return make_desc_layout(h->S, h->desc_np, h->l_max, warps, table ? words : 0, false, pad); };
-    auto fit = [&](bool table, bool pad) {
-        const DescLayout o = layout(1, table, pad);
-        const size_t fixed = (size_t)o.warp0 * 4;
-        return fixed < (size_t)h->max_smem ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed) / ((size_t)o.per_warp * 4)) : 0;
-    };
-    const int warps_fit = fit(false, false), warps_ts = words > 0 ? fit(true, false) : 0;
+    const DescLayout alone = make_desc_layout(h->S, h->desc_np, h->l_max, 1, 0, false, plain);
+    const int warps_fit = (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - (size_t)alone.warp0 * 4) / ((size_t)alone.per_warp * 4));
+    // (with the table in shared memory a warp's region is a little smaller: its staged pairs are five words, not eight)
+    const DescLayout with_table = make_desc_layout(h->S, h->desc_np, h->l_max, 1, (int)(h->desc_table_bytes / 4), false, plain);
+    const size_t fixed_ts = (size_t)with_table.warp0 * 4, warp_bytes_ts = (size_t)with_table.per_warp * 4;
+    const int warps_ts = h->desc_table_bytes > 0 && fixed_ts + warp_bytes_ts <= (size_t)h->max_smem
+                             ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed_ts) / warp_bytes_ts) : 0;
     // The table pays from four centres per SM on, except where the warps it costs make a second round of centres that keeps
     // less than a quarter of them busy (coefficients, table against none: 1500 atoms at (8, 8) 46.1 against 39.6 us, 1000
     // atoms of three species at (6, 9) 48.2 against 36.8 us; with a fuller second round 48.1 against 48.5 us and less).
     const int64_t sms = h->sm_count;
     const bool straggling = n_work <= warps_fit * sms && n_work > warps_ts * sms && 4 * n_work <= 5 * warps_ts * sms;
     const bool ts = !cp.pair_w && warps_ts >= 6 && n_work >= 4 * sms && !straggling;
-    // The tile keeps its padding unless that costs a warp and so a round of centres ((14, 8), two species, seven warps against
-    // eight: 9000 atoms 424 against 388 us, 30,000 atoms 1308 against 1209 us; 4000 atoms, four rounds either way, 201
-    // against 202 us; six species at (6, 4), 4000 atoms, three rounds either way, 116 against 120 us).
-    auto rounds = [&](int warps) { return warps > 0 ? (n_work + sms * warps - 1) / (sms * warps) : INT64_MAX; };
-    cp.tile_pad = rounds(fit(ts, true)) <= rounds(fit(ts, false));
-    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(fit(ts, cp.tile_pad), (n_work + sms - 1) / sms));
+    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(ts ? warps_ts : warps_fit, (n_work + sms - 1) / sms));
     const unsigned grid = (unsigned)std::min<int64_t>(sms, (n_work + warps - 1) / warps);
-    const size_t smem = (size_t)layout(warps, ts, cp.tile_pad).total * 4;
+    const size_t smem = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, warps, ts ? (int)(h->desc_table_bytes / 4) : 0, false, plain).total * 4;
     return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, ts, false), cp, grid, (unsigned)warps * 32, smem, st);
 }
 

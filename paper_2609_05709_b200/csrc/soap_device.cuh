@@ -29,7 +29,7 @@ struct Geometry {                 // host-known, passed by value
     int pbc[3];
 };
 
-struct GridParams {               // device-resident, written by grid_setup_kernel
+struct GridParams {               // device-resident, written by prep_kernel (above kPrepAtoms atoms by grid_setup_kernel)
     int nb[3];                    // bins per axis
     int R[3];                     // stencil half-width in bins
     int periodic[3];
@@ -76,7 +76,6 @@ struct CenterParams {
     int S, n_max, l_max, F;
     int P;                        // pairs per staged chunk
     unsigned nch_magic;           // floor(2^32 / (n_max (l_max+1))) + 1: x / n_ch == umulhi(x, magic) for x < 65536
-    int tile_pad;                 // descriptor-only kernel: room after every four rows of the centre's tile (desc_c_at)
     // output mode
     int crossover;                // 0: only the species pairs mu == nu are features
     int emit_coeff;               // descriptor build: write the coefficients c^mu_nlm instead of the power spectrum

@@ -119,10 +119,9 @@ def test_rounds_of_centres(pkg, n_max, l_max, sigma, n_centers, crossover):
     assert col_err(got[sample].cpu().numpy(), ref) < DESC_TOL
 
 
-# (14, 8) and (6, 4) with six species: the padding of a centre's tile costs a warp, and is there only where that makes no
-# further round of centres
-@pytest.mark.parametrize("n_species,n_max,l_max", [(2, 14, 8), (6, 6, 4)])
-@pytest.mark.parametrize("n_centers", [1036, 1037, 1184, 1776, 1924, 3000])
+# a centre's tile without its padding, at l_max 8 with n_max 13 to 16, and beside it
+@pytest.mark.parametrize("n_species,n_max,l_max", [(1, 13, 8), (2, 14, 8), (6, 16, 8), (2, 12, 8), (2, 14, 7)])
+@pytest.mark.parametrize("n_centers", [90, 1036, 1037, 3000])
 def test_padded_and_plain_tiles(pkg, n_species, n_max, l_max, n_centers):
     s = multispecies_box(90, 2)
     species = [1, 6, 7, 8, 9, 14][:n_species]
