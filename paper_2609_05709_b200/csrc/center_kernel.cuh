@@ -150,9 +150,15 @@ center_kernel(const CenterParams p) {
     const int S = p.S, NMAX = NMAX_T ? NMAX_T : p.n_max, NCH = NMAX * L1, NE = NMAX * LM;
     const int CT = S * NMAX * LMP, P = p.P, F = p.F;
     constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
-    // words pairs (G, Ghat) per staged pair: the channels, and with a row table a zero behind them
     constexpr bool kRowTable = KIND == 1 && NMAX_T != 0 && row_table_wanted(NMAX_T, L);
-    const SmemLayout lay = make_layout(S, NMAX, L, P, warps, o_pw != nullptr, kRowTable && !PLAIN && p.row_ops != nullptr);
+    // The layout as the host put it together, and everything that depends on the centre's number alone on its way at once: with
+    // the tables that rows by table do without left out, 36,000 centres of 18 pairs 733 -> 711 us, compact rows of 1111 atoms at (6, 6)
+    // 325 -> 316, 3000 at (8, 6) 591 -> 583.  From n_max 9 on, where the rows are long and the registers few, the start of a
+    // centre weighs less than what it holds: (12, 10) 922 -> 927 to 946 us, (12, 6) 661 -> 664.
+    constexpr bool kEarly = NMAX_T <= 8;
+    const SmemLayout made = kEarly ? SmemLayout{} : make_layout(S, NMAX, L, P, warps, o_pw != nullptr, kRowTable && !PLAIN && p.row_ops != nullptr);
+    const SmemLayout& lay = kEarly ? p.lay : made;
+    // words pairs (G, Ghat) per staged pair: the channels, and with a row table a zero behind them
     const int GP = NCH + (row_table_wanted(NMAX, L) ? 1 : 0);
     const int CP = NMAX_T ? CP_T : (NMAX + 1) / 2 * L1;                     // channel pairs: (l, two adjacent n)
     float* c_t = smem + lay.c;                                             // [S][NMAX][LMP]
@@ -171,8 +177,11 @@ center_kernel(const CenterParams p) {
     // zeros for the bulk copies of pass 2 (made visible to the copy engine; the barriers of pass 1 order them)
     const float* zero_buf = smem + lay.zero;
     const int zero_w = zero_words(S, NMAX, L);
-    for (int e = tid; e < zero_w; e += threads) smem[lay.zero + e] = 0.f;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    const bool by_table = kRowTable && p.row_ops != nullptr && !o_compact;       // (rows by table use neither these nor tri_dec)
+    if (!by_table) {
+        for (int e = tid; e < zero_w; e += threads) smem[lay.zero + e] = 0.f;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
     // the zero behind the channels of every staged pair, for the operands that a feature does not have in rows by table (the
     // slab of the power spectrum ends before it; with every species pair a feature it does so by itself, make_layout)
     if (kRowTable)
@@ -180,7 +189,7 @@ center_kernel(const CenterParams p) {
 
     // same-species blocks: feature index -> (n1 L1 + l) | (n2 L1 + l) << 8, rows n1 of (NMAX - n1) L1 entries
     unsigned short* tri_dec = reinterpret_cast<unsigned short*>(smem + lay.tri);
-    if (!CC)
+    if (!CC && !by_table)
         for (int e = tid; e < (NMAX * (NMAX + 1) / 2) * L1; e += threads) {
             int n1 = 0, r = e;
             while (r >= (NMAX - n1) * L1) { r -= (NMAX - n1) * L1; ++n1; }
@@ -202,17 +211,24 @@ center_kernel(const CenterParams p) {
     grid_dependency_wait();
     const long long c_idx = p.order ? p.order[blockIdx.x] : blockIdx.x;
     // a failed neighbour build or an undersized output: write nothing
-    if (p.counters->n_pairs > p.pair_capacity) return;
-    if (p.row_ptr[p.n_centers] > p.row_capacity) {
+    const long long pairs_found = p.counters->n_pairs;
+    if (!kEarly && pairs_found > p.pair_capacity) return;
+    const long long rows_found = p.row_ptr[p.n_centers];
+    auto too_many_rows = [&]() {
+        if (rows_found <= p.row_capacity) return false;
         if (c_idx == 0 && tid == 0) atomicOr(&p.counters->status, kStatusRowCapacity);
-        return;
-    }
+        return true;
+    };
+    if (!kEarly && too_many_rows()) return;
+    long long row_base = kEarly ? p.row_ptr[c_idx] : 0;
+    int own_row = kEarly ? p.self_row[c_idx] : 0;
     const int ci = o_sites ? -1 : (p.centers ? p.centers[c_idx] : (int)c_idx);
     const float* pc = o_sites ? o_sites + 3 * c_idx : p.pos + 3 * (long long)ci;
     const float xi = pc[0], yi = pc[1], zi = pc[2];
     const int zi_species = o_sites ? 0 : p.species_idx[ci];
     const long long pair_base = p.pair_start[c_idx];
     const int k_pairs = p.pair_count[c_idx];
+    if (kEarly && (pairs_found > p.pair_capacity || too_many_rows())) return;
     const bool periodic = p.geom.pbc[0] | p.geom.pbc[1] | p.geom.pbc[2];
     // the pairs are taken in batches of geometry of equal size (a multiple of eight, at most kGeoPairs): 274 pairs are
     // 96 + 96 + 82, not 128 + 128 + 18
@@ -445,17 +461,17 @@ center_kernel(const CenterParams p) {
     // centre's row is minus the sum over its neighbours: -K_l sum_m (D^mu c^nu + c^mu D^nu).  Results
     // pass through the slab, so that global memory is written in
     // feature order, whole sectors at a time.
-    const long long row_base = p.row_ptr[c_idx];
+    if (!kEarly) { row_base = p.row_ptr[c_idx]; own_row = p.self_row[c_idx]; }
     const bool has_own = !o_sites;                   // a centre that is no atom has no row of its own
     if (CC) {
         // the centre's own row: minus the sum over the atoms that move relative to it
         if (has_own) {
-            float* own = p.out_jac + (size_t)(row_base + p.self_row[c_idx]) * 3 * W;
+            float* own = p.out_jac + (size_t)(row_base + own_row) * 3 * W;
             for (int e = tid; e < 3 * W; e += threads) {
                 const int k = e / W, r = e - k * W, row = r / LM;
                 own[e] = -D_t[k * CT + row * LMP + (r - row * LM)];
             }
-            if (tid == 0) p.row_atom[row_base + p.self_row[c_idx]] = ci;
+            if (tid == 0) p.row_atom[row_base + own_row] = ci;
         }
     } else {
         // with given mean coefficients every centre would write the same descriptor: the first one does
@@ -466,9 +482,9 @@ center_kernel(const CenterParams p) {
         float* own = !has_own ? nullptr
                      : o_atom_rows ? p.out_jac + (size_t)ci * 3 * F            // row of atom a in the (atoms, 3, F) result
                      : o_compact ? p.out_center + (size_t)c_idx * 3 * F
-                                 : p.out_jac + (size_t)(row_base + p.self_row[c_idx]) * 3 * F;
+                                 : p.out_jac + (size_t)(row_base + own_row) * 3 * F;
         if (has_own && o_compact) {
-            float* slot = p.out_jac + (size_t)(row_base + p.self_row[c_idx]) * 3 * RW;
+            float* slot = p.out_jac + (size_t)(row_base + own_row) * 3 * RW;
             for (int e = tid; e < 3 * RW; e += threads) slot[e] = 0.f;
         }
         float* slab = smem + lay.slab;
@@ -519,7 +535,7 @@ center_kernel(const CenterParams p) {
                 __syncthreads();
             }
         }
-        if (has_own && !o_atom_rows && tid == 0) p.row_atom[row_base + p.self_row[c_idx]] = ci;
+        if (has_own && !o_atom_rows && tid == 0) p.row_atom[row_base + own_row] = ci;
     }
     if (o_inner) return;             // the averaged row of this atom is complete: no per-pair rows
     __syncthreads();
@@ -1050,8 +1066,6 @@ center_kernel(const CenterParams p) {
             else { o0[f] = vx; o1[f] = vy; o2[f] = vz; }
         }
     };
-
-    const bool by_table = kRowTable && p.row_ops != nullptr && !o_compact;
 
     // Coefficient mode: the row of a neighbour of species Z is grad c^Z_nlm = G_nl grad S_lm + Ghat_nl d S_lm
     // (Eq. 14 / Eq. 23) in the block of Z and zero in the other blocks, written in aligned sweeps as above.

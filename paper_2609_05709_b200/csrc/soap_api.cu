@@ -101,10 +101,8 @@ struct soap_handle {
     bool ordered = false;                // whether the last search with rows left a launch order
     int64_t started_atoms = -1, started_centers = -1;   // sizes of the search soap_search_start left for soap_search_finish; -1: none
     int64_t found_atoms = -1, found_centers = -1, found_rows = 0;   // sizes of the search soap_search_finish left for soap_derivatives_found; -1: none
-    int P_deriv4 = 16;                   // ... with CTAs of 128 threads
-    size_t smem_deriv4 = 0;
+    int P_deriv4 = 0;                    // ... with CTAs of 128 threads (0: they do not fit)
     int P_deriv = 16, P_outer = 16;      // pairs per staged chunk: derivative kernels, kernel of the outer average
-    size_t smem_deriv = 0, smem_outer = 0;
     bool outer_fast = false;             // whether the kernel of the outer average fits the shared memory
     // optional per-segment timing (events on the caller's stream)
     bool profiling = false;
@@ -177,6 +175,9 @@ int make_geometry(soap_t* h, const double* cell, Geometry& g) {
     return SOAP_OK;
 }
 
+// Bytes of the copies of neighbouring centres' coefficients that the kernel of the outer average keeps, one per warp.
+size_t outer_extra(const soap_t* h) { return (size_t)(kThreads / 32) * h->S * h->n_max * (((h->l_max + 1) * (h->l_max + 1)) | 1) * 4; }
+
 // Shared-memory plan of the per-centre kernels (depends on the basis and on whether pairs carry weights).
 int plan_smem(soap_t* h) {
     // shared-memory plan of the per-centre kernels
@@ -188,12 +189,12 @@ int plan_smem(soap_t* h) {
         return plan_chunk(h->S, h->n_max, h->l_max, h->weight.fn != 0, warps, extra, (size_t)max_smem, P, bytes);
     };
     // 256 threads, and the smaller CTAs that this basis may run with
-    if (!plan(8, 0, h->P_deriv, h->smem_deriv)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
-    if (!plan(4, 0, h->P_deriv4, h->smem_deriv4)) h->smem_deriv4 = 0;
+    size_t bytes = 0;
+    if (!plan(8, 0, h->P_deriv, bytes)) return fail(h, SOAP_ERR_INVALID_ARG, "this basis does not fit the shared memory of the device");
+    if (!plan(4, 0, h->P_deriv4, bytes)) h->P_deriv4 = 0;
     // the kernel of the outer average keeps, per warp, a copy of a neighbouring centre's coefficients behind the usual
     // layout; a basis too large for that takes the general path (per-pair rows in a workspace)
-    const int LMP = ((h->l_max + 1) * (h->l_max + 1)) | 1;
-    h->outer_fast = plan(kThreads / 32, (size_t)(kThreads / 32) * h->S * h->n_max * LMP * 4, h->P_outer, h->smem_outer);
+    h->outer_fast = plan(kThreads / 32, outer_extra(h), h->P_outer, bytes);
     return SOAP_OK;
 }
 
@@ -491,8 +492,12 @@ int launch_per_center(soap_t* h, void (*kernel)(CenterParams), const CenterParam
     CU(launch_dependent(kernel, grid, threads, smem, st, cp));
     return SOAP_OK;
 }
-int launch_center(soap_t* h, int kind, const CenterParams& cp, int64_t n_centers, int threads, size_t smem, cudaStream_t st) {
-    return launch_per_center(h, center_kernel_of(kind, center_params_plain(cp), h->l_max, h->n_max), cp, (unsigned)n_centers, (unsigned)threads, smem, st);
+// Launch of a derivative kernel with the shared memory of the layout it is given; `extra` bytes follow that.
+int launch_center(soap_t* h, int kind, CenterParams& cp, int64_t n_centers, int threads, size_t extra, cudaStream_t st) {
+    const bool plain = center_params_plain(cp);
+    cp.lay = make_layout(h->S, h->n_max, h->l_max, cp.P, threads / 32, cp.pair_w != nullptr, cp.row_ops && !plain);
+    return launch_per_center(h, center_kernel_of(kind, plain, h->l_max, h->n_max), cp, (unsigned)n_centers, (unsigned)threads,
+                             (size_t)cp.lay.total * 4 + extra, st);
 }
 
 // Launch of the descriptor-only kernel: persistent CTAs (one per SM) whose warps take the centres in turn.
@@ -549,13 +554,12 @@ int status_error(soap_t* h, int s) {
 // does where pass 1 keeps 128 threads busy and the rows are long (4 species at (4, 7) 250 against 262 us).
 int launch_deriv(soap_t* h, int kind, CenterParams& cp, int64_t n_centers, cudaStream_t st) {
     int threads = kThreads;
-    size_t bytes = h->smem_deriv;
     const int channels = h->n_max * (h->l_max + 1), needs = pass1_span(h->l_max) * pass1_slots(h->l_max, 16);
     const bool small = channels <= 20 || (channels <= 32 && h->l_max <= 4);
-    if (small && needs <= 128 && h->smem_deriv4 != 0 && n_centers >= (int64_t)5 * h->sm_count) {
-        threads = 128; cp.P = h->P_deriv4; bytes = h->smem_deriv4;
+    if (small && needs <= 128 && h->P_deriv4 != 0 && n_centers >= (int64_t)5 * h->sm_count) {
+        threads = 128; cp.P = h->P_deriv4;
     }
-    return launch_center(h, kind, cp, n_centers, threads, bytes, st);
+    return launch_center(h, kind, cp, n_centers, threads, 0, st);
 }
 
 // Feature table: species pairs mu <= nu (only mu == nu without crossover), radial pair (n' >= n on
@@ -1164,7 +1168,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
         cp.out_jac = d_out_jac;
         cp.inner_rows = 1;
         cp.own_scale = (float)(1.0 / (double)n_centers);
-        if ((rc = launch_center(h, kCenterInner, cp, n_centers, kThreads, h->smem_deriv, st))) return rc;
+        if ((rc = launch_center(h, kCenterInner, cp, n_centers, kThreads, 0, st))) return rc;
         if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
         return SOAP_OK;
     }
@@ -1189,7 +1193,7 @@ int soap_derivatives_average(soap_t* h, int mode, const float* d_positions, cons
         cp.out_jac = d_out_jac;
         cp.own_scale = (float)(1.0 / (double)n_centers);
         cp.P = h->P_outer;
-        if ((rc = launch_center(h, kCenterOuter, cp, n_centers, kThreads, h->smem_outer, st))) return rc;
+        if ((rc = launch_center(h, kCenterOuter, cp, n_centers, kThreads, outer_extra(h), st))) return rc;
         if ((rc = column_mean(h, (const float*)(w + o_rows), n_centers, F, (double*)(w + o_partial), d_out_desc, st))) return rc;
         if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
         return SOAP_OK;

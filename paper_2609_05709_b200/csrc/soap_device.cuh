@@ -45,6 +45,12 @@ struct Counters {                 // device-resident
     long long n_rows;
 };
 
+// Shared memory of a per-centre derivative kernel (make_layout), offsets in 4-byte words.
+struct SmemLayout {
+    int c, geo, tri, xdec, zero, D, wUV, sSD, sG, slab, slab_words, total;
+    bool keep;                    // the slab is apart from the staging area: what pass 1 staged is still there in pass 2
+};
+
 struct CenterParams {
     // structure
     const float* pos;             // [N,3]
@@ -75,6 +81,7 @@ struct CenterParams {
     int n_intervals;
     int S, n_max, l_max, F;
     int P;                        // pairs per staged chunk
+    SmemLayout lay;               // shared memory of the derivative kernels, for this P
     unsigned nch_magic;           // floor(2^32 / (n_max (l_max+1))) + 1: x / n_ch == umulhi(x, magic) for x < 65536
     // output mode
     int crossover;                // 0: only the species pairs mu == nu are features
@@ -138,10 +145,6 @@ constexpr int kGeoPairs = 128;           // pairs whose geometry is staged at on
 
 constexpr int kMaxZeroWords = 1024;      // largest block of zeros that bulk copies write into the structural-zero blocks of the rows
 
-struct SmemLayout {
-    int c, geo, tri, xdec, zero, D, wUV, sSD, sG, slab, slab_words, total;
-    bool keep;                    // the slab is apart from the staging area: what pass 1 staged is still there in pass 2
-};
 // whether the cross-species blocks of the rows are written in table-driven sweeps (a decode table in shared
 // memory): several species, n_max from 9 to 12 and n_max (l_max+1) not a multiple of four (the other cases have
 // faster paths with an operand in registers)
