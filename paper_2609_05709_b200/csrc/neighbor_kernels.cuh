@@ -76,21 +76,37 @@ __global__ void species_bbox_kernel(const float* __restrict__ pos, const int* __
     if (bad) atomicOr(&counters->status, kStatusUnknownSpecies);
 }
 
+constexpr int kThinBins = 4;
+constexpr long long kThinAtoms = 65536;
+constexpr double kThinAround = 512.0;
 // Choose the bin grid; called by a whole warp, one lane per axis, the result in `g` (shared or global memory).  Bin
 // width (measured perpendicular to the cell faces) is at least r_cut (1 + 1e-6) wherever more than one bin fits, so a
-// stencil of +-1 bin covers the sphere; short periodic axes get one bin and a wider stencil of images.
-__device__ inline void choose_grid(double hi, double lo, const Geometry& geom, long long N, int cell_cap, GridParams* g) {
+// stencil of +-1 bin covers the sphere; short periodic axes get one bin and a wider stencil of images.  Without a periodic
+// axis, the axes at right angles, bins are a quarter as wide along axis 0 (stencil of +-4), where a row of bins is one run
+// of the sorted atoms that can be cut to the width of the sphere there: 14.5 r_cut^3 of candidates for a sphere of 4.2
+// instead of 27.  (Bins of r_cut / 2 along the other axes as well: 9.2, but 25 rows to look up instead of nine.)  That
+// pays above kThinAtoms atoms, where the bins are counted and scanned by kernels of their own, and with many atoms around a
+// centre; else the longer scan costs more than the candidates: descriptors of 1,000,002 atoms 8914 -> 8799 us, 3000 atoms of 274
+// neighbours 1177 -> 1166, but 24,000 atoms of 37 neighbours 2 us longer (of 120 to 170), 30,000 of 46 about even.
+// may_thin: the caller walks by such runs.
+__device__ inline void choose_grid(double hi, double lo, const Geometry& geom, long long N, int cell_cap, bool may_thin, GridParams* g) {
     const int a = threadIdx.x & 31;                       // lanes 3 .. 31 repeat axis 2
     const int ax = min(a, 2);
     const double rc = geom.r_cut * (1.0 + 1e-6);
     const bool periodic = geom.pbc[ax] != 0;
     if (N <= 0) { hi = 0.0; lo = 0.0; }
     const double span = hi - lo;
+    const double* const c = geom.cell;
+    const bool square = c[1] == 0.0 && c[2] == 0.0 && c[3] == 0.0 && c[5] == 0.0 && c[6] == 0.0 && c[7] == 0.0;
     double want = periodic ? floor(geom.height[ax] / rc) : floor(span * geom.height[ax] / rc);
     if (!(want >= 1.0)) want = 1.0;
+    auto of = [&](int axis) { return __shfl_sync(0xffffffffu, want, axis); };
+    const double around = 27.0 * (double)N / (of(0) * of(1) * of(2));          // atoms in a stencil of bins as wide as the cutoff
+    const bool thin = may_thin && square && !(geom.pbc[0] | geom.pbc[1] | geom.pbc[2]) && (N > kThinAtoms || around >= kThinAround);
+    const int split = thin && ax == 0 ? kThinBins : 1;
+    if (split > 1) want = fmax(1.0, floor(span * geom.height[ax] * split / rc));
     if (want > 1024.0) want = 1024.0;
     // respect the scratch capacity: shrink the grid uniformly
-    auto of = [&](int axis) { return __shfl_sync(0xffffffffu, want, axis); };
     for (int it = 0; it < 64; ++it) {
         const double w0 = of(0), w1 = of(1), w2 = of(2);
         if (!(w0 * w1 * w2 > (double)cell_cap)) break;
@@ -103,9 +119,9 @@ __device__ inline void choose_grid(double hi, double lo, const Geometry& geom, l
         g->periodic[a] = periodic;
         g->smin[a] = periodic ? 0.0 : lo;
         g->sscale[a] = periodic ? (double)nb : (span > 0 ? nb / span : 0.0);
-        g->R[a] = periodic ? (int)ceil(rc / (geom.height[a] / nb)) : (nb > 1 ? 1 : 0);
+        g->R[a] = periodic ? (int)ceil(rc / (geom.height[a] / nb)) : min(nb - 1, split);
     }
-    if (a == 0) g->n_cells = n0 * n1 * n2;
+    if (a == 0) { g->n_cells = n0 * n1 * n2; g->thin = thin; }
     __syncwarp();
 }
 
@@ -113,7 +129,7 @@ __global__ void __launch_bounds__(32) grid_setup_kernel(const unsigned long long
                                   Counters* counters) {
     if (counters && threadIdx.x == 0) { counters->n_pairs = 0; counters->n_rows = 0; }      // the pair cursor of this call
     const int a = min((int)threadIdx.x, 2);
-    choose_grid(dec_double(bbox[a]), -dec_double(bbox[3 + a]), geom, N, cell_cap, out);
+    choose_grid(dec_double(bbox[a]), -dec_double(bbox[3 + a]), geom, N, cell_cap, counters != nullptr, out);
 }
 
 __device__ inline void bin_of(const Geometry& geom, const GridParams& g, float x, float y, float z, int b[3], int w[3]) {
@@ -346,7 +362,7 @@ prep_kernel(const float* __restrict__ pos, const int* __restrict__ numbers, long
                 const double* other = CLUSTER ? cluster.map_shared_rank(box, r) : box;
                 hi = fmax(hi, other[a]); lo = fmax(lo, other[3 + a]);
             }
-        choose_grid(hi, -lo, geom, N, cell_cap, &sg);
+        choose_grid(hi, -lo, geom, N, cell_cap, true, &sg);
         if (rank == 0 && lane == 0) {
             *grid_out = sg;
             counters->n_pairs = 0;                                            // the pair cursor of this call
@@ -538,9 +554,10 @@ __device__ inline void for_each_candidate(const Geometry& geom, const GridParams
     }
 }
 
-// The same walk for the common case (no periodic axis, stencil of +-1 bin): the three bins of a stencil row along
-// x are neighbours in the sorted atom array, so the 27 bins are 9 contiguous runs.  Every lane keeps the nine run
-// boundaries in registers, and a candidate finds its run with compares instead of shuffles.
+// The same walk for the common case (no periodic axis, stencil of +-1 bin across the rows): the bins of a stencil row along
+// x are neighbours in the sorted atom array, so the stencil is 9 contiguous runs, each cut to the bins that the sphere
+// reaches in its row (GridParams::thin).  Every lane keeps the nine run boundaries in registers, and a candidate finds its
+// run with compares instead of shuffles.
 template <class F>
 __device__ inline void for_each_candidate_runs(const Geometry& geom, const GridParams& g, const int* __restrict__ cell_start,
                                                const float4* __restrict__ s_pos, float xi, float yi, float zi,
@@ -551,10 +568,30 @@ __device__ inline void for_each_candidate_runs(const Geometry& geom, const GridP
         const int cy = bi[1] + lane % 3 - g.R[1], cz = bi[2] + lane / 3 - g.R[2];
         const bool inside = cy >= 0 && cy < g.nb[1] && cz >= 0 && cz < g.nb[2] && (lane % 3 <= 2 * g.R[1]) && (lane / 3 <= 2 * g.R[2]);
         if (inside) {
-            const int x0 = max(bi[0] - g.R[0], 0), x1 = min(bi[0] + g.R[0], g.nb[0] - 1);
-            const int row = (cz * g.nb[1] + cy) * g.nb[0];
-            start = cell_start[row + x0];
-            cnt = cell_start[row + x1 + 1] - start;
+            int x0 = max(bi[0] - g.R[0], 0), x1 = min(bi[0] + g.R[0], g.nb[0] - 1);
+            if (g.thin) {
+                // how far the sphere reaches along x at the nearest point of this row of bins, a little rounded up (an
+                // atom's bin and its edges carry rounding errors of the coordinates' last places)
+                const double rc = geom.r_cut * (1.0 + 1e-6);
+                double s[3], rest = rc * rc;
+                frac_coords(geom, xi, yi, zi, s);
+                const int row[3] = {0, cy, cz};
+#pragma unroll
+                for (int a = 1; a < 3; ++a) {
+                    const double t = (s[a] - g.smin[a]) * g.sscale[a] - row[a];            // the bin is 0 .. 1
+                    const double away = fmax(fmax(-t, t - 1.0) - 1e-6, 0.0);
+                    if (away > 0.0) { const double d = away / g.sscale[a] * geom.height[a]; rest -= d * d; }
+                }
+                const double reach = rest > 0.0 ? sqrt(rest) / geom.height[0] : 0.0, at = s[0] - g.smin[0];
+                x0 = max(x0, (int)floor((at - reach) * g.sscale[0] - 1e-6));
+                x1 = min(x1, (int)floor((at + reach) * g.sscale[0] + 1e-6));
+                if (rest <= 0.0) x1 = x0 - 1;
+            }
+            if (x0 <= x1) {
+                const int first = (cz * g.nb[1] + cy) * g.nb[0];
+                start = cell_start[first + x0];
+                cnt = cell_start[first + x1 + 1] - start;
+            }
         }
     }
     int r_start[9], r_end[9], total = 0;                 // run r covers candidates r_end[r] - count .. r_end[r] - 1
@@ -624,8 +661,9 @@ constexpr int kFillWarps = 4;
 // warps hide each other's loads, and more cost registers), four on few, where a call waits for the longest warp (search
 // of 60 atoms in a periodic box 31.6 -> 26.0 us, 431 atoms 21.1 -> 19.6 us, 2000 atoms 27.8 -> 26.0 us, 5000 atoms
 // 35.7 -> 37.7 us).
+// Nine CTAs per SM where loads are not fetched ahead and the key buffers allow it: 56 registers, eight fewer than the compiler takes.
 template <int KEYS, bool ROWS, int AHEAD>
-__global__ void __launch_bounds__(kFillWarps * 32)
+__global__ void __launch_bounds__(kFillWarps * 32, AHEAD == 1 && (KEYS <= 128 || !ROWS) ? 9 : 6)
 pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, const float* __restrict__ sites, long long C, Geometry geom,
              const GridParams* __restrict__ gp, const int* __restrict__ atom_cell, const int* __restrict__ atom_wrap,
              const int* __restrict__ cell_start, const float4* __restrict__ s_pos, const int* __restrict__ s_wrap,
@@ -667,7 +705,7 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
         if (valid && at < KEYS) s_raw[wid][at] = key;
         k += __popc(m);
     };
-    const bool runs = !(g.periodic[0] | g.periodic[1] | g.periodic[2]) && g.R[0] <= 1 && g.R[1] <= 1 && g.R[2] <= 1;
+    const bool runs = !(g.periodic[0] | g.periodic[1] | g.periodic[2]) && g.R[0] <= kThinBins && g.R[1] <= 1 && g.R[2] <= 1;
     if (runs) for_each_candidate_runs(geom, g, cell_start, s_pos, xi, yi, zi, bi, lane, collect);
     else for_each_candidate<AHEAD>(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, collect);
     long long base = 0;
@@ -687,13 +725,14 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
     if (!in_smem) {
         // rare: more pairs than the on-chip buffer holds; walk again, now with a place to put them
         int at0 = 0;
-        for_each_candidate(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters,
-                           [&](bool valid, unsigned long long key) {
-                               const unsigned m = __ballot_sync(0xffffffffu, valid);
-                               const int at = at0 + __popc(m & ((1u << lane) - 1));
-                               if (valid && at < k) pair_tmp[base + at] = key;
-                               at0 += __popc(m);
-                           });
+        auto store = [&](bool valid, unsigned long long key) {
+            const unsigned m = __ballot_sync(0xffffffffu, valid);
+            const int at = at0 + __popc(m & ((1u << lane) - 1));
+            if (valid && at < k) pair_tmp[base + at] = key;
+            at0 += __popc(m);
+        };
+        if (runs) for_each_candidate_runs(geom, g, cell_start, s_pos, xi, yi, zi, bi, lane, store);
+        else for_each_candidate(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, store);
     }
     __syncwarp();
     if (!ROWS) {

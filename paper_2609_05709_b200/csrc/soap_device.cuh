@@ -36,6 +36,7 @@ struct GridParams {               // device-resident, written by prep_kernel (ab
     double smin[3];               // bin = (s - smin) * sscale
     double sscale[3];
     int n_cells;
+    int thin;                     // no periodic axis, axes at right angles: bins a quarter as wide along axis 0 (for_each_candidate_runs)
 };
 
 struct Counters {                 // device-resident
