@@ -23,6 +23,7 @@
 // Nothing but the pair list is read from HBM and nothing but the descriptor row is written.
 #pragma once
 #include "harmonic_tables.h"
+#include "pair_test.cuh"
 #include "soap_device.cuh"
 
 namespace soap {
@@ -30,6 +31,10 @@ namespace soap {
 constexpr int kDescGroup = 64;                    // pairs whose geometry a warp holds in registers (two per lane)
 constexpr int kDescMaxWarps = 16;                 // warps per CTA (one CTA per SM)
 constexpr int kDescTeamWarps = 4;                 // most warps of a CTA that works on one centre
+constexpr int kDescSearchAtoms = 1024;            // most atoms that a team searches for its centre's neighbours
+// atoms of a warp's share of such a search, and the bytes behind the layout: a slot per atom, and what each warp found
+__host__ __device__ inline int desc_search_share(long long n_atoms, int warps) { return (int)((n_atoms + 32 * warps - 1) / (32 * warps)) * 32; }
+__host__ __device__ inline size_t desc_search_bytes(long long n_atoms, int warps) { return n_atoms > 0 ? (size_t)desc_search_share(n_atoms, warps) * warps * 8 + kDescTeamWarps * 4 : 0; }
 
 // harmonic normalisation up to l = 12: a_lm (sqrt2 folded in for m > 0), index l(l+1)/2 + m
 struct HarmonicNorm { float a[kHarmonicTerms]; };
@@ -233,8 +238,9 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     }
     // the tables are this handle's own; everything below reads what the kernels before this one wrote
     grid_dependency_wait();
+    const bool searches = TEAM && p.numbers != nullptr;
     // a failed neighbour build: write nothing
-    if (p.counters->n_pairs > p.pair_capacity) return;
+    if (!searches && p.counters->n_pairs > p.pair_capacity) return;
 
     float* const wbase = smem + lay.warp0 + wid * lay.per_warp;
     float* const c_t = wbase + lay.c;                                               // [LM] rows of RC chunks, skewed
@@ -272,7 +278,70 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     constexpr int PPL = kDescGroup / 32;                                 // pairs per lane and group
     struct Head { float xi, yi, zi; int zsp; long long pair_base; int k_pairs; };
     struct Raw { unsigned long long key[PPL]; float wgt[PPL]; int spj[PPL]; float px[PPL], py[PPL], pz[PPL]; };
+    // A team may look for its centre's neighbours itself, among all atoms of a small structure whose periodic axes are at least two
+    // cutoffs high: an atom then has one image inside at most, the one nearest in each fractional coordinate.  The test is the
+    // pair kernel's.  A warp takes a contiguous share of the atoms and leaves its finds in its own slots, in order.
+    unsigned long long* const list = reinterpret_cast<unsigned long long*>(smem + lay.total);
+    const int share = searches ? desc_search_share(p.n_atoms, warps) : 0;
+    int* const s_found = reinterpret_cast<int*>(list + share * warps);
+    auto species_of = [&](int number) { return number >= 0 && number < 128 ? __ldg(p.z_lut + number) : -1; };
+    auto search = [&](int i) {
+        Head h;
+        h.xi = p.pos[3 * i]; h.yi = p.pos[3 * i + 1]; h.zi = p.pos[3 * i + 2];
+        h.zsp = species_of(p.numbers[i]);
+        h.pair_base = 0;
+        double fi[3] = {0.0, 0.0, 0.0};
+        int status = 0, k = 0;
+        if (h.zsp < 0) { status |= kStatusUnknownSpecies; h.zsp = 0; }
+        if (periodic) {
+            frac_coords(p.geom, h.xi, h.yi, h.zi, fi);
+            for (int a = 0; a < 3; ++a)
+                if (p.geom.pbc[a] && fabs(floor(fi[a])) > 100.0) status |= kStatusShiftRange;    // absurdly far outside the cell
+        }
+#pragma unroll 2
+        for (int t = 0; t < share; t += 32) {
+            const int j = wid * share + t + lane;
+            bool valid = false;
+            unsigned long long key = 0;
+            if (j < p.n_atoms) {
+                const float4 pj = make_float4(p.pos[3 * j], p.pos[3 * j + 1], p.pos[3 * j + 2], __int_as_float(j));
+                const int zj = p.numbers[j];
+                int n[3] = {0, 0, 0};
+                if (periodic) {
+                    double fj[3];
+                    frac_coords(p.geom, pj.x, pj.y, pj.z, fj);
+                    for (int a = 0; a < 3; ++a)
+                        if (p.geom.pbc[a]) n[a] = -(int)rint(fj[a] - fi[a]);
+                }
+                bool out_of_range;
+                valid = inside_cutoff(p.geom, periodic, pj, n, h.xi, h.yi, h.zi, key, out_of_range);
+                if (out_of_range) { status |= kStatusShiftRange; valid = false; }
+                if (valid) {
+                    const int sj = species_of(zj);                            // (its own team reports an unknown one)
+                    key |= (unsigned long long)max(sj, 0) << 56;
+                }
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, valid);
+            if (valid) list[wid * share + k + __popc(m & ((1u << lane) - 1))] = key;
+            k += __popc(m);
+        }
+        status = (int)__reduce_or_sync(0xffffffffu, (unsigned)status);
+        if (lane == 0) {
+            s_found[wid] = k;
+            if (status) atomicOr(&p.counters->status, status);
+        }
+        __syncthreads();
+        h.k_pairs = 0;
+        for (int w = 0; w < warps; ++w) h.k_pairs += s_found[w];
+        return h;
+    };
+    auto found_key = [&](int e) {
+        int w = 0;
+        while (w + 1 < warps && e >= s_found[w]) e -= s_found[w++];
+        return list[w * share + e];
+    };
     auto load_head = [&](long long c_idx) {
+        if (searches) return search((int)c_idx);
         Head h;
         const int ci = o_sites ? -1 : (p.centers ? p.centers[c_idx] : (int)c_idx);
         const float* pc = o_sites ? o_sites + 3 * c_idx : p.pos + 3 * (long long)ci;
@@ -286,7 +355,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
 #pragma unroll
         for (int b = 0; b < PPL; ++b) {
             const int e = g0 + 32 * b + lane;
-            r.key[b] = e < h.k_pairs ? p.pair_key[h.pair_base + e] : 0ull;
+            r.key[b] = e < h.k_pairs ? (searches ? found_key(e) : p.pair_key[h.pair_base + e]) : 0ull;
             r.wgt[b] = (o_pw && e < h.k_pairs) ? o_pw[h.pair_base + e].x : 1.f;
         }
     };
@@ -297,7 +366,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
             r.spj[b] = -1; r.px[b] = r.py[b] = r.pz[b] = 0.f;
             if (e < h.k_pairs) {
                 const int j = key_atom(r.key[b]);
-                r.spj[b] = S == 1 ? 0 : p.species_idx[j];
+                r.spj[b] = S == 1 ? 0 : searches ? (int)(r.key[b] >> 56) : p.species_idx[j];
                 r.px[b] = p.pos[3 * (long long)j]; r.py[b] = p.pos[3 * (long long)j + 1]; r.pz[b] = p.pos[3 * (long long)j + 2];
             }
         }
@@ -633,6 +702,21 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
         }
     }
     if (!TEAM && lane == 0) wait_row();                                      // the slab must outlive the copies that read it
+    if (searches && threadIdx.x == 0) {
+        // the last team leaves the totals of the call
+        int k = 0;
+        for (int w = 0; w < warps; ++w) k += s_found[w];
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.counters->found), (unsigned long long)k);
+        __threadfence();
+        if (atomicAdd(&p.counters->finished, 1) == (int)gridDim.x - 1) {
+            __threadfence();
+            const long long total = (long long)atomicExch(reinterpret_cast<unsigned long long*>(&p.counters->found), 0ull);
+            p.counters->finished = 0;
+            p.counters->n_pairs = total;
+            p.counters->n_rows = 0;
+            if (total > p.pair_capacity) atomicOr(&p.counters->status, kStatusPairCapacity);
+        }
+    }
 }
 
 }  // namespace soap

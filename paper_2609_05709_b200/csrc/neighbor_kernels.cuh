@@ -11,6 +11,7 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include "pair_test.cuh"
 #include "soap_device.cuh"
 
 namespace soap {
@@ -40,11 +41,6 @@ __device__ inline unsigned long long enc_double(double x) {
 __device__ inline double dec_double(unsigned long long e) {
     unsigned long long b = (e >> 63) ? (e & 0x7fffffffffffffffull) : ~e;
     return __longlong_as_double((long long)b);
-}
-
-__device__ inline void frac_coords(const Geometry& g, float x, float y, float z, double s[3]) {
-    for (int a = 0; a < 3; ++a)
-        s[a] = (double)x * g.inv[0 + a] + (double)y * g.inv[3 + a] + (double)z * g.inv[6 + a];
 }
 
 // species index per atom, and the bounding box of the fractional coordinates
@@ -457,27 +453,10 @@ __device__ __forceinline__ bool look_at(const Geometry& geom, bool any_periodic,
     unpack3(wrap, wj);
     unpack3(img, im);
     // translation on the raw (unwrapped) inputs
-    const int na = im[0] - wj[0] + wi[0], nb = im[1] - wj[1] + wi[1], nc = im[2] - wj[2] + wi[2];
-    double dx = __dsub_rn((double)pj.x, (double)xi);
-    double dy = __dsub_rn((double)pj.y, (double)yi);
-    double dz = __dsub_rn((double)pj.z, (double)zi);
-    if (any_periodic) {
-        // T = (n_a a + n_b b) + n_c c, each product and sum rounded on its own
-        const double fa = (double)na, fb = (double)nb, fc = (double)nc;
-        double tx = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[0]), __dmul_rn(fb, geom.cell[3])), __dmul_rn(fc, geom.cell[6]));
-        double ty = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[1]), __dmul_rn(fb, geom.cell[4])), __dmul_rn(fc, geom.cell[7]));
-        double tz = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[2]), __dmul_rn(fb, geom.cell[5])), __dmul_rn(fc, geom.cell[8]));
-        dx = __dadd_rn(dx, tx); dy = __dadd_rn(dy, ty); dz = __dadd_rn(dz, tz);
-    }
-    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    bool valid = (d2 < geom.rc2) && (d2 > 0.0);
-    if (valid && (abs(na) > 127 || abs(nb) > 127 || abs(nc) > 127)) {
-        atomicOr(&counters->status, kStatusShiftRange);
-        valid = false;
-    }
-    key = ((unsigned long long)(unsigned)__float_as_int(pj.w) << 24) |
-          ((unsigned long long)(na + 128) << 16) | ((unsigned long long)(nb + 128) << 8) |
-          (unsigned long long)(nc + 128);
+    const int n[3] = {im[0] - wj[0] + wi[0], im[1] - wj[1] + wi[1], im[2] - wj[2] + wi[2]};
+    bool out_of_range;
+    const bool valid = inside_cutoff(geom, any_periodic, pj, n, xi, yi, zi, key, out_of_range);
+    if (out_of_range) { atomicOr(&counters->status, kStatusShiftRange); return false; }
     return valid;
 }
 

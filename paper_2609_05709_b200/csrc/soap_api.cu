@@ -475,6 +475,7 @@ void fill_center_params(soap_t* h, CenterParams& cp, const float* pos, const int
     cp.P = h->P_deriv;
     cp.crossover = h->crossover; cp.emit_coeff = 0; cp.c_bar = nullptr; cp.inner_rows = 0; cp.own_scale = 1.f; cp.c_all = nullptr;
     cp.pair_w = h->weight.fn ? h->d_pair_w : nullptr; cp.w0 = (float)h->w0;
+    cp.numbers = nullptr; cp.z_lut = h->d_zlut; cp.n_atoms = 0;
     cp.compact = 0; cp.Fc = (int)h->Fc_pitch; cp.out_center = nullptr;
     cp.out_desc = nullptr; cp.out_jac = nullptr; cp.row_atom = nullptr;
 }
@@ -500,6 +501,23 @@ int launch_center(soap_t* h, int kind, CenterParams& cp, int64_t n_centers, int 
                              (size_t)cp.lay.total * 4 + extra, st);
 }
 
+// Few centres: a team of warps per centre, four if the CTAs then run side by side in one wave (four of them fit an
+// SM's registers), else two (eight; up to five centres per SM: beyond that a warp per centre is the faster one on half
+// of the sizes).  Whole calls, (n_max, l_max) = (8, 6): 120 atoms 27 -> 17 us, 431 atoms of four species 66 -> 38 us,
+// 600 atoms 31.2 -> 29.2 us; (12, 8), 600 atoms 60 -> 43 us.
+// search_atoms: the team looks for its neighbours among that many atoms (0: it reads them).  Returns its warps, 0: no team.
+size_t desc_team_bytes(const soap_t* h, bool plain, int team_warps, int64_t search_atoms) {
+    return (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, team_warps, 0, true, plain).total * 4 + desc_search_bytes(search_atoms, team_warps);
+}
+int desc_team(const soap_t* h, bool plain, int64_t n_work, int64_t search_atoms) {
+    for (const int team_warps : {kDescTeamWarps, 2}) {
+        const size_t bytes = desc_team_bytes(h, plain, team_warps, search_atoms);
+        const int64_t per_sm = std::min<int64_t>(team_warps == 2 ? 5 : 16 / kDescTeamWarps, (int64_t)(228 * 1024 / (bytes + 1024)));
+        if (n_work <= per_sm * h->sm_count && bytes <= (size_t)h->max_smem) return team_warps;
+    }
+    return 0;
+}
+
 // Launch of the descriptor-only kernel: persistent CTAs (one per SM) whose warps take the centres in turn.
 // The radial table goes to shared memory when it leaves room for at least six warps and there is enough
 // work to pay for staging it; small jobs use fewer warps per CTA so that they spread over the SMs, the smallest
@@ -509,16 +527,10 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     cp.table_ln = h->d_table_ln;
     cp.inv_h = h->basis.inv_h_values; cp.n_intervals = h->basis.n_intervals_values;      // the value table has intervals of its own
     const bool plain = center_params_plain(cp);
-    // Few centres: a team of warps per centre, four if the CTAs then run side by side in one wave (four of them fit an
-    // SM's registers), else two (eight; up to five centres per SM: beyond that a warp per centre is the faster one on half
-    // of the sizes).  Whole calls, (n_max, l_max) = (8, 6): 120 atoms 27 -> 17 us, 431 atoms of four species 66 -> 38 us,
-    // 600 atoms 31.2 -> 29.2 us; (12, 8), 600 atoms 60 -> 43 us.
-    for (const int team_warps : {kDescTeamWarps, 2}) {
-        const size_t bytes = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, team_warps, 0, true, plain).total * 4;
-        const int64_t per_sm = std::min<int64_t>(team_warps == 2 ? 5 : 16 / kDescTeamWarps, (int64_t)(228 * 1024 / (bytes + 1024)));
-        if (n_work > per_sm * h->sm_count || bytes > (size_t)h->max_smem) continue;
-        return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true), cp, (unsigned)n_work, (unsigned)team_warps * 32, bytes, st);
-    }
+    const int64_t search_atoms = cp.numbers ? cp.n_atoms : 0;
+    if (const int team = desc_team(h, plain, n_work, search_atoms))
+        return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true), cp, (unsigned)n_work, (unsigned)team * 32,
+                                 desc_team_bytes(h, plain, team, search_atoms), st);
     const DescLayout alone = make_desc_layout(h->S, h->desc_np, h->l_max, 1, 0, false, plain);
     const int warps_fit = (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - (size_t)alone.warp0 * 4) / ((size_t)alone.per_warp * 4));
     // (with the table in shared memory a warp's region is a little smaller: its staged pairs are five words, not eight)
@@ -597,7 +609,7 @@ int launch_weights(soap_t* h, const float* pos, const int32_t* centers, const fl
 // changed, the neighbour search.
 int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const double* cell, const int32_t* centers,
             int64_t C, long long* row_ptr_out, Geometry& g, cudaStream_t st, const float* sites = nullptr,
-            const Batch& batch = Batch(), List list = List::rows) {
+            const Batch& batch = Batch(), List list = List::rows, bool* searches_itself = nullptr) {
     int rc = check_inputs(h, pos, num, N, centers, C, sites);
     if (rc) return rc;
     if (batch.struct_ptr && (h->pbc[0] || h->pbc[1] || h->pbc[2]))
@@ -610,6 +622,20 @@ int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const do
     // to have more pairs than that holds the status word says so
     const bool planned = h->planned_atoms >= 0 && N <= h->planned_atoms && C <= h->planned_centers;
     if (!planned && (rc = search_and_size(h, pos, num, N, g, centers, sites, C, row_ptr_out, st, batch))) return rc;
+    // Descriptors of a small structure with every atom a centre: the kernel that computes them searches as well, where a team of
+    // warps has a centre each and no periodic axis is shorter than two cutoffs
+    if (searches_itself) {
+        bool can = !centers && !sites && !batch.struct_ptr && C > 0 && C <= kDescSearchAtoms && !h->weight.fn && desc_team(h, h->crossover, C, N) != 0;
+        for (int a = 0; a < 3; ++a) can = can && (!g.pbc[a] || g.height[a] >= 2.0 * g.r_cut * (1.0 + 1e-6));
+        *searches_itself = can;
+        if (can) {
+            forget_search(h);
+            h->list_sorted = false;
+            h->last_centers = 0;
+            if (h->profiling) CU(cudaEventRecord(h->ev[1], st));
+            return SOAP_OK;
+        }
+    }
     if (planned || list == List::found) {
         // (a first call of its size has the sorted list already, and takes the pairs as found all the same: its result then
         // differs from that of the calls after it no more than theirs do from one another)
@@ -770,11 +796,13 @@ static int descriptor_impl(soap_t* h, const float* d_positions, const int32_t* d
     if (h && n_centers > 0 && !d_out) return fail(h, SOAP_ERR_INVALID_ARG, "d_out must not be NULL");
     Geometry g;
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, d_sites, batch, List::found);
+    bool searches = false;
+    int rc = prepare(h, d_positions, d_numbers, n_atoms, cell, d_centers, n_centers, nullptr, g, st, d_sites, batch, List::found, &searches);
     if (rc) return rc;
     if (n_centers > 0) {
         CenterParams cp;
         fill_center_params(h, cp, d_positions, d_centers, n_centers, g, false, d_sites);
+        if (searches) { cp.numbers = d_numbers; cp.n_atoms = (int)n_atoms; }
         cp.out_desc = d_out;
         if ((rc = launch_desc(h, cp, n_centers, st))) return rc;
     }

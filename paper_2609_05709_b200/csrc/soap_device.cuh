@@ -41,9 +41,10 @@ struct GridParams {               // device-resident, written by prep_kernel (ab
 
 struct Counters {                 // device-resident
     int status;
-    int pad;
+    int finished;                 // CTAs of a descriptor kernel that searches for itself that are done ...
     long long n_pairs;
     long long n_rows;
+    long long found;              // ... and the pairs they found (both zero between calls)
 };
 
 // Shared memory of a per-centre derivative kernel (make_layout), offsets in 4-byte words.
@@ -59,6 +60,9 @@ struct CenterParams {
     const float* sites;           // [C,3] or null: centres at these points instead of at atoms (no on-site term, no own row)
     const int* order;             // [C] CTA -> centre slot (largest first) or null
     const int* species_idx;       // [N]
+    const int* numbers;           // [N] or null: the descriptor kernel looks for its centres' neighbours among all atoms itself ...
+    const int* z_lut;             // ... with the species of every atomic number below 128
+    int n_atoms;
     long long n_centers;
     Geometry geom;
     // neighbour data
