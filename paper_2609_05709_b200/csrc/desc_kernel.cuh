@@ -3,14 +3,14 @@
 //
 // This build is bound by FP32 issue slots and by shared-memory bandwidth, not by HBM, so the layout is
 // chosen for few instructions and few shared-memory wavefronts per pair:
-//   * the radial table (value polynomials, re-laid as [interval][l][n / 2][6][2]) sits in shared memory
-//     once per CTA when it fits; a lane evaluates two adjacent n at once from three conflict-free 16-byte
-//     loads and five packed multiply-adds (fma.rn.f32x2: one issue slot for two multiply-adds);
+//   * the radial table (value polynomials) sits in shared memory once per CTA when it fits; a lane evaluates four adjacent n
+//     at once from six 16-byte loads and ten packed multiply-adds (fma.rn.f32x2: one issue slot for two multiply-adds), or two
+//     from half as many, whichever fills more lanes (desc_quads);
 //   * the pairs of a centre (up to 64 at a time) have their geometry formed in registers, are ranked by species with
 //     ballots, and staged 16 or 32 at a time in species order: solid harmonics with a lane per pair from the fully
-//     unrolled Q_l^m recursion, radial factors with the lanes side by side on the list of all (pair, two channels) of
-//     the chunk (a round per pair left half of the lanes idle at l_max 3: 324,000 atoms at (4, 3) 2.03 -> 1.47 ms,
-//     215,000 at (6, 4) 2.90 -> 2.33 ms, with the chunks of 32);
+//     unrolled Q_l^m recursion, radial factors with the lanes side by side on the chunk's pairs and channels (a round per
+//     pair left half of the lanes idle at l_max 3: 324,000 atoms at (4, 3) 2.03 -> 1.47 ms, 215,000 at (6, 4) 2.90 -> 2.33 ms,
+//     with the chunks of 32);
 //   * accumulation c[l,m][n] += S_lm G_nl is register-tiled: a lane owns four consecutive m of one l
 //     times all n (an outer product of 4 x n_max per pair from one 16-byte load of S and n_max/4 of
 //     G); with at most 16 such tiles the two half-warps work on two pairs at once.  Sums stay in
@@ -75,6 +75,19 @@ __host__ __device__ constexpr int desc_g_swap(int np, int l) { return np == 8 ? 
 __host__ __device__ constexpr bool desc_tile_pad(int np, int l_max, bool plain) { return !(plain && np == 16 && l_max == 8); }
 __host__ __device__ constexpr int desc_c_at(int row, int row_chunks, bool pad) { return row * row_chunks + (pad ? row >> 2 : 0); }
 __host__ __device__ constexpr int desc_c_words(int S, int np, int lm, bool pad) { return 4 * (desc_c_at(lm - 1, S * np / 4, pad) + S * np / 4); }
+
+// How the radial factors of a staged pair are taken from the table.  As quads: four adjacent n of one l per lane, the table as
+// [interval][6][l][n], so that lanes side by side read side by side: 24 instructions for four values instead of 40 and no
+// conflicts while eight lanes stay within one pair.  They do where 7 or 8 of every 8 lanes have a quad (`desc_quad_span`:
+// a lane then keeps its quad), and conflicts weigh little with more than 16 quads; else two adjacent n per lane, the table as
+// [interval][l][n / 2][6][2], which fills more lanes.  24,000 atoms of water, whole calls, pairs against quads: (8, 6) 202 ->
+// 193 us, (8, 3) 148 -> 144, (14, 6) 714 -> 661, (2, 7) 175 -> 170, (10, 8) 623 -> 608; the other way, left as pairs,
+// (8, 4) 164 -> 172, (2, 4) 131 -> 138, (10, 2) 169 -> 179, (8, 5) and (10, 3) equal or slower.
+__host__ __device__ constexpr int desc_quad_span(int np, int l_max) {
+    const int quads = (l_max + 1) * np / 4, span = (quads + 7) / 8 * 8;
+    return span <= 32 && 32 % span == 0 && 8 * quads >= 7 * span ? span : 0;
+}
+__host__ __device__ constexpr bool desc_quads(int np, int l_max) { return desc_quad_span(np, l_max) > 0 || (l_max + 1) * np / 4 > 16; }
 
 // Pairs staged at once by a warp: 32 where a staged pair is small, so that every lane has a pair's harmonics to form
 // (80 words: sixteen warps still fit beside the table for two species), else 16; a team deals its chunks out to its warps
@@ -178,7 +191,8 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     constexpr int TPL = (T + LANES_T - 1) / LANES_T;                     // tiles per lane (1, or 2 from l_max = 10 on)
     constexpr int NB = (TPL * NP * 4 <= 64) ? NP : 64 / (4 * TPL);      // n handled per pass (at most 64 accumulators)
     constexpr int NPASS = (NP + NB - 1) / NB;
-    constexpr int CPAIRS = NCHP / 2;                                     // channel pairs: two adjacent n of one l
+    constexpr bool QUADS = desc_quads(NP, L);
+    constexpr int UNIT = QUADS ? 4 : 2, UNITS = NCHP / UNIT;             // units of the radial factors: adjacent n of one l
     constexpr int kDescChunk = desc_chunk(L, NP, TEAM);
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
@@ -266,10 +280,10 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
         while (t >= (2 * l + 4) / 4) { t -= (2 * l + 4) / 4; ++l; }
         t_l[tp] = l; t_lm0[tp] = l * l + 4 * t; t_kv[tp] = min(4, 2 * l + 1 - 4 * t);
     }
-    // where the radial factors of the channel pair cp = l NP/2 + n/2 go in a pair's staging row: words l GL + n, l GL + n + 1
-    auto g_word = [](int cp) {
-        const int l = cp / (NP / 2);
-        return (2 * cp + l * (GL - NP)) ^ (4 * desc_g_swap(NP, l));
+    // where the radial factors of unit u go in a pair's staging row, in words
+    auto g_word = [](int u) {
+        const int l = u / (NP / UNIT);
+        return (UNIT * u + l * (GL - NP)) ^ (4 * desc_g_swap(NP, l));
     };
     const bool periodic = p.geom.pbc[0] | p.geom.pbc[1] | p.geom.pbc[2];
     const long long n_work = o_cbar ? 1 : p.n_centers;
@@ -525,29 +539,55 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
                         const float4 d = ring_d[lane];
                         harmonics_tiles<L>(d.x, d.y, d.z, TS ? fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)) : d.w * d.w, sS4 + lane * (SROW / 4));
                     }
-                    // radial factors: the lanes walk down the (pair, channel pair) list side by side, a warp's width at a time
-                    {
-                        int pr = lane / CPAIRS, cp = lane - pr * CPAIRS;
-#pragma unroll 4
-                        for (int e = lane; e < n_stage * CPAIRS; e += 32) {
-                            int4 gi;
-                            if (TS) { gi = make_int4(ring_q[pr] & 0xffff, __float_as_int(ring_d[pr].w), 0, 0); }
-                            else gi = ring_i[pr];
-                            const float t = __int_as_float(gi.y);
-                            const float2 tt = make_float2(t, t);
-                            // coefficients of t^0 .. t^5 of two adjacent n, interleaved: (c0, c0', c1, c1'), (c2, c2', c3, c3'), (c4, c4', c5, c5')
-                            const float4* row = tab + (unsigned)(gi.x * CPAIRS + cp) * 3u;
+                    // radial factors of one unit of one pair
+                    auto radial = [&](int pr, int u) {
+                        int4 gi;
+                        if (TS) { gi = make_int4(ring_q[pr] & 0xffff, __float_as_int(ring_d[pr].w), 0, 0); }
+                        else gi = ring_i[pr];
+                        const float t = __int_as_float(gi.y), wgt = !PLAIN && !TS ? __int_as_float(gi.w) : 1.f;
+                        const float2 tt = make_float2(t, t);
+                        float* const to = sG + pr * GROW + g_word(u);
+                        if constexpr (QUADS) {
+                            const float4* row = tab + (unsigned)(gi.x * 6 * UNITS + u);   // the coefficients of t^0 .. t^5, UNITS apart
+                            float2 lo, hi;
+#pragma unroll
+                            for (int k = 5; k >= 0; --k) {
+                                const float4 c = TS ? row[k * UNITS] : __ldg(row + k * UNITS);
+                                const float2 c_lo = make_float2(c.x, c.y), c_hi = make_float2(c.z, c.w);
+                                lo = k == 5 ? c_lo : __ffma2_rn(lo, tt, c_lo);
+                                hi = k == 5 ? c_hi : __ffma2_rn(hi, tt, c_hi);
+                            }
+                            if (!PLAIN && !TS) { lo.x *= wgt; lo.y *= wgt; hi.x *= wgt; hi.y *= wgt; }
+                            *reinterpret_cast<float4*>(to) = make_float4(lo.x, lo.y, hi.x, hi.y);
+                        } else {
+                            // coefficients of t^0 .. t^5 of two adjacent n, interleaved: (c0, c0', c1, c1'), (c2, ..), (c4, ..)
+                            const float4* row = tab + (unsigned)(gi.x * UNITS + u) * 3u;
                             const float4 A = TS ? row[0] : __ldg(row), B = TS ? row[1] : __ldg(row + 1), C = TS ? row[2] : __ldg(row + 2);
                             float2 v = __ffma2_rn(make_float2(C.z, C.w), tt, make_float2(C.x, C.y));
                             v = __ffma2_rn(v, tt, make_float2(B.z, B.w));
                             v = __ffma2_rn(v, tt, make_float2(B.x, B.y));
                             v = __ffma2_rn(v, tt, make_float2(A.z, A.w));
                             v = __ffma2_rn(v, tt, make_float2(A.x, A.y));
-                            if (!PLAIN && !TS) { const float wgt = __int_as_float(gi.w); v.x *= wgt; v.y *= wgt; }
-                            *reinterpret_cast<float2*>(sG + pr * GROW + g_word(cp)) = v;
+                            if (!PLAIN && !TS) { v.x *= wgt; v.y *= wgt; }
+                            *reinterpret_cast<float2*>(to) = v;
+                        }
+                    };
+                    constexpr int SPAN = QUADS ? desc_quad_span(NP, L) : 0;
+                    if constexpr (SPAN > 0) {
+                        const int u = lane % SPAN;
+                        if (u < UNITS) {
+#pragma unroll 2
+                            for (int pr = lane / SPAN; pr < n_stage; pr += 32 / SPAN) radial(pr, u);
+                        }
+                    } else {
+                        // the lanes walk down the (pair, unit) list side by side, a warp's width at a time
+                        int pr = lane / UNITS, u = lane - pr * UNITS;
+#pragma unroll (QUADS ? 2 : 4)
+                        for (int e = lane; e < n_stage * UNITS; e += 32) {
+                            radial(pr, u);
                             // 32 further down the list
-                            pr += 32 / CPAIRS; cp += 32 % CPAIRS;
-                            if (cp >= CPAIRS) { cp -= CPAIRS; ++pr; }
+                            pr += 32 / UNITS; u += 32 % UNITS;
+                            if (u >= UNITS) { u -= UNITS; ++pr; }
                         }
                     }
                     __syncwarp();

@@ -229,23 +229,24 @@ int ensure_device(soap_t* h) {
     }
     h->device = dev;
     {
-        // [interval][l][n / 2][6][2]: the coefficients of two adjacent n interleaved (the kernels evaluate them with packed
-        // multiply-adds), n padded to a multiple of two for the derivative kernels and of four for the descriptor-only
-        // kernel; the padding channels are zero
-        const int L1 = h->l_max + 1, n_ch = h->n_max * L1;
-        auto interleaved = [&](const std::vector<float>& table, int intervals, int np) {
-            std::vector<float> out((size_t)intervals * L1 * np * kTableCoef, 0.f);
-            for (int q = 0; q < intervals; ++q)
-                for (int l = 0; l < L1; ++l)
-                    for (int n = 0; n < h->n_max; ++n)
-                        for (int k = 0; k < kTableCoef; ++k)
-                            out[((((size_t)q * L1 + l) * (np / 2) + n / 2) * kTableCoef + k) * 2 + (n & 1)] =
-                                table[((size_t)q * n_ch + n * L1 + l) * kTableCoef + k];
-            return out;
-        };
-        CU(upload(&h->d_table, interleaved(h->basis.table, h->basis.n_intervals, (h->n_max + 1) & ~1)));
+        // Derivative kernels: [interval][l][n / 2][6][2], the coefficients of two adjacent n interleaved (evaluated with packed
+        // multiply-adds), n padded to even.  Descriptor-only kernel: the same with n padded to a multiple of four, or by quads
+        // (desc_quads).  The padding channels are zero.
+        const int L1 = h->l_max + 1, n_ch = h->n_max * L1, even = (h->n_max + 1) & ~1;
         h->desc_np = desc_np(h->n_max);
-        const std::vector<float> values = interleaved(h->basis.table_values, h->basis.n_intervals_values, h->desc_np);
+        std::vector<float> both((size_t)h->basis.n_intervals * L1 * even * kTableCoef, 0.f), values((size_t)h->basis.n_intervals_values * L1 * h->desc_np * kTableCoef, 0.f);
+        for (int l = 0; l < L1; ++l)
+            for (int n = 0; n < h->n_max; ++n)
+                for (int k = 0; k < kTableCoef; ++k) {
+                    const size_t channel = n * L1 + l;
+                    for (size_t q = 0; q < (size_t)h->basis.n_intervals; ++q)
+                        both[(((q * L1 + l) * (even / 2) + n / 2) * kTableCoef + k) * 2 + (n & 1)] = h->basis.table[(q * n_ch + channel) * kTableCoef + k];
+                    for (size_t q = 0; q < (size_t)h->basis.n_intervals_values; ++q)
+                        values[desc_quads(h->desc_np, h->l_max) ? ((q * kTableCoef + k) * L1 + l) * h->desc_np + n
+                                                                : (((q * L1 + l) * (h->desc_np / 2) + n / 2) * kTableCoef + k) * 2 + (n & 1)] =
+                            h->basis.table_values[(q * n_ch + channel) * kTableCoef + k];
+                }
+        CU(upload(&h->d_table, both));
         CU(upload(&h->d_table_ln, values));
         h->desc_table_bytes = values.size() * sizeof(float);
     }

@@ -76,7 +76,7 @@ struct CenterParams {
     Counters* counters;
     // basis
     const float* table;           // [nint][l][n / 2][6][2], n padded to even: coefficients of two adjacent n interleaved (derivative kernels)
-    const float* table_ln;        // value polynomials on wider intervals as [nint][l][n / 2][6][2], n padded to a multiple of 4 (descriptor-only kernel)
+    const float* table_ln;        // value polynomials on wider intervals as [nint][l][n / 2][6][2] or [nint][6][l][n] (desc_quads), n padded to a multiple of 4 (descriptor-only kernel)
     const float* self_term;       // [n_max]
     const int* l_of_lm;           // [lm] -> l
     const float* kl;
