@@ -146,6 +146,16 @@ int soap_derivatives_found(soap_t *h, int kind, const float *d_positions, int64_
                            float *d_out_desc, float *d_out_center, float *d_out_jac, int64_t capacity_rows,
                            const int64_t *d_row_ptr, int32_t *d_row_atom, void *stream);
 
+/* The three in one call that waits once, for structures so small that the caller
+ * can do without the number of rows beforehand: capacity_rows must be at least
+ * n_centers * n_atoms, which no structure exceeds (else SOAP_ERR_CAPACITY).
+ * *n_rows is the number of rows written.  Device-side problems are returned, as
+ * by soap_search_finish. */
+int soap_derivatives_bounded(soap_t *h, int kind, const float *d_positions, const int32_t *d_numbers, int64_t n_atoms,
+                             const double *cell, const int32_t *d_centers, int64_t n_centers,
+                             float *d_out_desc, float *d_out_center, float *d_out_jac, int64_t capacity_rows,
+                             int64_t *d_row_ptr, int32_t *d_row_atom, int64_t *n_rows, void *stream);
+
 /* Exports the neighbour list of the last soap_neighbors / soap_descriptor /
  * soap_derivatives call: d_pair_ptr [n_centers+1]; for pair e of centre i
  * (d_pair_ptr[i] <= e < d_pair_ptr[i+1]) the neighbour atom d_pair_atom[e] and

@@ -20,10 +20,13 @@ EXPORTED_SYMBOLS = [
     "soap_neighbors_at", "soap_descriptor_at", "soap_derivatives_at",
     "soap_rows_dense", "soap_neighbors_batch", "soap_descriptor_batch", "soap_derivatives_batch",
     "soap_num_compact_features", "soap_compact_feature_map", "soap_derivatives_compact", "soap_compact_expand",
-    "soap_measure_fp32_peak", "soap_search_start", "soap_search_finish", "soap_derivatives_found",
+    "soap_measure_fp32_peak", "soap_search_start", "soap_search_finish", "soap_derivatives_found", "soap_derivatives_bounded",
 ]
 
 ROWS_FULL, ROWS_COMPACT, ROWS_COEFFICIENTS = 0, 1, 2
+# Jacobians with a row for every (centre, atom) up to this size are allocated so, without waiting for the number of rows first (the
+# result keeps that much memory; 24 atoms at (4, 3) take 1.0 MB of it)
+BOUNDED_BYTES = 2 << 20
 
 _ERRORS = {-1: "SOAP_ERR_INVALID_ARG", -2: "SOAP_ERR_UNKNOWN_SPECIES", -3: "SOAP_ERR_CAPACITY",
            -4: "SOAP_ERR_CUDA", -5: "SOAP_ERR_ALLOC"}
@@ -84,6 +87,7 @@ def load_library() -> C.CDLL:
     lib.soap_search_start.argtypes = found + [vp]
     lib.soap_search_finish.argtypes = found + [C.POINTER(i64), C.POINTER(i64), vp]
     lib.soap_derivatives_found.argtypes = [vp, i32, vp, i64, C.POINTER(C.c_double), vp, vp, i64, vp, vp, vp, i64, vp, vp, vp]
+    lib.soap_derivatives_bounded.argtypes = [vp, i32, vp, vp, i64, C.POINTER(C.c_double), vp, i64, vp, vp, vp, i64, vp, vp, C.POINTER(i64), vp]
     lib.soap_set_crossover.argtypes = [vp, i32]
     lib.soap_set_weighting.argtypes = [vp, i32] + [C.c_double] * 5
     lib.soap_num_coefficients.argtypes = [vp, C.POINTER(i64)]
@@ -290,6 +294,18 @@ class Soap:
             bptr, n_structs = struct_ptr.data_ptr(), struct_ptr.shape[0] - 1
         dev, stream, pos, lib = positions.device, self._stream(), positions.data_ptr(), self._lib
         row_ptr = torch.empty(c + 1, dtype=torch.int64, device=dev)
+        most = c * n
+        if sites is None and struct_ptr is None and 12 * most * width <= BOUNDED_BYTES:
+            # a row per centre and atom is little: one call, one wait, and the rows that it wrote
+            values = torch.empty((c, self.n_coefficients if kind == ROWS_COEFFICIENTS else self.n_features), dtype=torch.float32, device=dev)
+            center_rows = torch.empty((c, 3, self.n_features), dtype=torch.float32, device=dev) if kind == ROWS_COMPACT else None
+            jac = torch.empty((max(most, 1), 3, width), dtype=torch.float32, device=dev)
+            row_atom = torch.empty(max(most, 1), dtype=torch.int32, device=dev)
+            nrows = C.c_int64()
+            self._check(lib.soap_derivatives_bounded(self._h, kind, pos, numbers.data_ptr(), n, cellp, cptr, c, values.data_ptr(),
+                                                     None if center_rows is None else center_rows.data_ptr(), jac.data_ptr(), most,
+                                                     row_ptr.data_ptr(), row_atom.data_ptr(), C.byref(nrows), stream))
+            return values, center_rows, jac[:nrows.value], row_ptr, row_atom[:nrows.value]
         search = (self._h, pos, numbers.data_ptr(), n, cellp, cptr, sptr, c, bptr, n_structs, row_ptr.data_ptr())
         self._check(lib.soap_search_start(*search, stream))
         # the outputs whose size is known, while the search runs

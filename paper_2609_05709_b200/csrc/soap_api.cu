@@ -946,22 +946,13 @@ int soap_search_finish(soap_t* h, const float* d_positions, const int32_t* d_num
     return SOAP_OK;
 }
 
-int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_t n_atoms, const double* cell, const int32_t* d_centers,
-                           const float* d_sites, int64_t n_centers, float* d_out_desc, float* d_out_center, float* d_out_jac,
-                           int64_t capacity_rows, const int64_t* d_row_ptr, int32_t* d_row_atom, void* stream) {
-    if (!h) return SOAP_ERR_INVALID_ARG;
-    if (kind != SOAP_ROWS_FULL && kind != SOAP_ROWS_COMPACT && kind != SOAP_ROWS_COEFFICIENTS) return fail(h, SOAP_ERR_INVALID_ARG, "unknown kind of rows");
-    if (h->found_atoms != n_atoms || h->found_centers != n_centers)
-        return fail(h, SOAP_ERR_INVALID_ARG, "no neighbour search of this size is at hand: call soap_search_start and soap_search_finish first");
-    if (!d_row_ptr || capacity_rows < 0) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
-    if (n_centers > 0 && (!d_out_desc || !d_out_jac || !d_row_atom)) return fail(h, SOAP_ERR_INVALID_ARG, "output pointers must not be NULL");
-    if (n_centers > 0 && kind == SOAP_ROWS_COMPACT && !d_out_center) return fail(h, SOAP_ERR_INVALID_ARG, "d_out_center must not be NULL");
-    if (capacity_rows < h->found_rows) return fail(h, SOAP_ERR_CAPACITY, "more Jacobian rows than capacity_rows");
-    int rc = ensure_device(h);
-    if (rc) return rc;
+// The derivatives of the pairs that the last search leaves, behind it on the stream.
+static int enqueue_found(soap_t* h, int kind, const float* d_positions, const double* cell, const int32_t* d_centers, const float* d_sites,
+                         int64_t n_centers, float* d_out_desc, float* d_out_center, float* d_out_jac, int64_t capacity_rows,
+                         const int64_t* d_row_ptr, int32_t* d_row_atom, cudaStream_t st) {
     Geometry g;
-    if ((rc = make_geometry(h, cell, g))) return rc;
-    cudaStream_t st = (cudaStream_t)stream;
+    int rc = make_geometry(h, cell, g);
+    if (rc) return rc;
     if (h->profiling) { CU(cudaEventRecord(h->ev[3], st)); h->in_steps = true; }
     if ((rc = launch_weights(h, d_positions, d_centers, d_sites, n_centers, g, st))) return rc;
     if (h->profiling) CU(cudaEventRecord(h->ev[4], st));
@@ -975,7 +966,59 @@ int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_
         if ((rc = launch_deriv(h, kind == SOAP_ROWS_COEFFICIENTS ? kCenterCoeff : kCenterDeriv, cp, n_centers, st))) return rc;
     }
     if (h->profiling) CU(cudaEventRecord(h->ev[2], st));
-    CU(cudaStreamSynchronize(st));
+    return SOAP_OK;
+}
+
+int soap_derivatives_found(soap_t* h, int kind, const float* d_positions, int64_t n_atoms, const double* cell, const int32_t* d_centers,
+                           const float* d_sites, int64_t n_centers, float* d_out_desc, float* d_out_center, float* d_out_jac,
+                           int64_t capacity_rows, const int64_t* d_row_ptr, int32_t* d_row_atom, void* stream) {
+    if (!h) return SOAP_ERR_INVALID_ARG;
+    if (kind != SOAP_ROWS_FULL && kind != SOAP_ROWS_COMPACT && kind != SOAP_ROWS_COEFFICIENTS) return fail(h, SOAP_ERR_INVALID_ARG, "unknown kind of rows");
+    if (h->found_atoms != n_atoms || h->found_centers != n_centers)
+        return fail(h, SOAP_ERR_INVALID_ARG, "no neighbour search of this size is at hand: call soap_search_start and soap_search_finish first");
+    if (!d_row_ptr || capacity_rows < 0) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
+    if (n_centers > 0 && (!d_out_desc || !d_out_jac || !d_row_atom)) return fail(h, SOAP_ERR_INVALID_ARG, "output pointers must not be NULL");
+    if (n_centers > 0 && kind == SOAP_ROWS_COMPACT && !d_out_center) return fail(h, SOAP_ERR_INVALID_ARG, "d_out_center must not be NULL");
+    if (capacity_rows < h->found_rows) return fail(h, SOAP_ERR_CAPACITY, "more Jacobian rows than capacity_rows");
+    int rc = ensure_device(h);
+    if (rc) return rc;
+    if ((rc = enqueue_found(h, kind, d_positions, cell, d_centers, d_sites, n_centers, d_out_desc, d_out_center, d_out_jac, capacity_rows, d_row_ptr,
+                            d_row_atom, (cudaStream_t)stream))) return rc;
+    CU(cudaStreamSynchronize((cudaStream_t)stream));
+    return SOAP_OK;
+}
+
+int soap_derivatives_bounded(soap_t* h, int kind, const float* d_positions, const int32_t* d_numbers, int64_t n_atoms, const double* cell,
+                             const int32_t* d_centers, int64_t n_centers, float* d_out_desc, float* d_out_center, float* d_out_jac,
+                             int64_t capacity_rows, int64_t* d_row_ptr, int32_t* d_row_atom, int64_t* n_rows, void* stream) {
+    if (!h) return SOAP_ERR_INVALID_ARG;
+    if (kind != SOAP_ROWS_FULL && kind != SOAP_ROWS_COMPACT && kind != SOAP_ROWS_COEFFICIENTS) return fail(h, SOAP_ERR_INVALID_ARG, "unknown kind of rows");
+    if (!d_row_ptr || capacity_rows < 0) return fail(h, SOAP_ERR_INVALID_ARG, "d_row_ptr must not be NULL");
+    if (n_centers > 0 && (!d_out_desc || !d_out_jac || !d_row_atom)) return fail(h, SOAP_ERR_INVALID_ARG, "output pointers must not be NULL");
+    if (n_centers > 0 && kind == SOAP_ROWS_COMPACT && !d_out_center) return fail(h, SOAP_ERR_INVALID_ARG, "d_out_center must not be NULL");
+    int rc = check_inputs(h, d_positions, d_numbers, n_atoms, d_centers, n_centers);
+    if (rc) return rc;
+    if (n_atoms > 0 && n_centers > capacity_rows / n_atoms) return fail(h, SOAP_ERR_CAPACITY, "capacity_rows must hold a row per centre and atom");
+    auto search = [&](Search step) {
+        return neighbors_impl(h, d_positions, d_numbers, n_atoms, cell, d_centers, nullptr, n_centers, nullptr, n_rows, stream, Batch(),
+                              (long long*)d_row_ptr, step);
+    };
+    if ((rc = search(Search::start))) return rc;
+    auto compute = [&]() {
+        return enqueue_found(h, kind, d_positions, cell, d_centers, nullptr, n_centers, d_out_desc, d_out_center, d_out_jac, capacity_rows, d_row_ptr,
+                             d_row_atom, (cudaStream_t)stream);
+    };
+    // (with more pairs than the scratch holds the kernels behind the search write nothing, and run again after it was grown)
+    const int64_t held = h->cap_pairs;
+    if ((rc = compute()) || (rc = search(Search::finish))) return rc;
+    if (h->h_counters->status) {
+        CU(cudaMemsetAsync(&h->d_counters->status, 0, sizeof(int), (cudaStream_t)stream));
+        return status_error(h, h->h_counters->status);
+    }
+    if (h->h_counters->n_pairs > held) {
+        if ((rc = compute())) return rc;
+        CU(cudaStreamSynchronize((cudaStream_t)stream));
+    }
     return SOAP_OK;
 }
 
