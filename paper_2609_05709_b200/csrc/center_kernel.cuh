@@ -146,7 +146,7 @@ center_kernel(const CenterParams p) {
     constexpr int NPT = NPT_RAW < 8 ? NPT_RAW : 8;                // ... at most 8 at a time (register budget)
     extern __shared__ __align__(16) float smem[];
     const int threads = KIND <= 2 ? (int)blockDim.x : kThreads, warps = threads >> 5;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform in a warp, and the compiler sees it
     const int S = p.S, NMAX = NMAX_T ? NMAX_T : p.n_max, NCH = NMAX * L1, NE = NMAX * LM;
     const int CT = S * NMAX * LMP, P = p.P, F = p.F;
     constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
