@@ -74,7 +74,7 @@ __global__ void species_bbox_kernel(const float* __restrict__ pos, const int* __
 
 constexpr int kThinBins = 4;
 constexpr long long kThinAtoms = 65536;
-constexpr double kThinAround = 512.0;
+constexpr double kThinAround = 160.0;
 // Choose the bin grid; called by a whole warp, one lane per axis, the result in `g` (shared or global memory).  Bin
 // width (measured perpendicular to the cell faces) is at least r_cut (1 + 1e-6) wherever more than one bin fits, so a
 // stencil of +-1 bin covers the sphere; short periodic axes get one bin and a wider stencil of images.  Without a periodic
@@ -83,7 +83,7 @@ constexpr double kThinAround = 512.0;
 // instead of 27.  (Bins of r_cut / 2 along the other axes as well: 9.2, but 25 rows to look up instead of nine.)  That
 // pays above kThinAtoms atoms, where the bins are counted and scanned by kernels of their own, and with many atoms around a
 // centre; else the longer scan costs more than the candidates: descriptors of 1,000,002 atoms 8914 -> 8799 us, 3000 atoms of 274
-// neighbours 1177 -> 1166, but 24,000 atoms of 37 neighbours 2 us longer (of 120 to 170), 30,000 of 46 about even.
+// neighbours 1177 -> 1166, 30,000 of 46 neighbours (198 in a stencil) 280 -> 276, but 24,000 atoms of 37 (132) 1 to 2 us longer.
 // may_thin: the caller walks by such runs.
 __device__ inline void choose_grid(double hi, double lo, const Geometry& geom, long long N, int cell_cap, bool may_thin, GridParams* g) {
     const int a = threadIdx.x & 31;                       // lanes 3 .. 31 repeat axis 2
