@@ -327,12 +327,11 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
                     for (int a = 0; a < 3; ++a)
                         if (p.geom.pbc[a]) n[a] = -(int)rint(fj[a] - fi[a]);
                 }
-                bool out_of_range;
-                valid = inside_cutoff(p.geom, periodic, pj, n, h.xi, h.yi, h.zi, key, out_of_range);
-                if (out_of_range) { status |= kStatusShiftRange; valid = false; }
+                valid = inside_cutoff(p.geom, pair_distance2(p.geom, periodic, pj, n[0], n[1], n[2], h.xi, h.yi, h.zi));
+                if (valid && beyond_key(n[0], n[1], n[2])) { status |= kStatusShiftRange; valid = false; }
                 if (valid) {
                     const int sj = species_of(zj);                            // (its own team reports an unknown one)
-                    key |= (unsigned long long)max(sj, 0) << 56;
+                    key = pair_key_of(pj, n[0], n[1], n[2]) | (unsigned long long)max(sj, 0) << 56;
                 }
             }
             const unsigned m = __ballot_sync(0xffffffffu, valid);

@@ -453,10 +453,13 @@ __device__ __forceinline__ bool look_at(const Geometry& geom, bool any_periodic,
     unpack3(wrap, wj);
     unpack3(img, im);
     // translation on the raw (unwrapped) inputs
-    const int n[3] = {im[0] - wj[0] + wi[0], im[1] - wj[1] + wi[1], im[2] - wj[2] + wi[2]};
-    bool out_of_range;
-    const bool valid = inside_cutoff(geom, any_periodic, pj, n, xi, yi, zi, key, out_of_range);
-    if (out_of_range) { atomicOr(&counters->status, kStatusShiftRange); return false; }
+    const int na = im[0] - wj[0] + wi[0], nb = im[1] - wj[1] + wi[1], nc = im[2] - wj[2] + wi[2];
+    bool valid = inside_cutoff(geom, pair_distance2(geom, any_periodic, pj, na, nb, nc, xi, yi, zi));
+    if (valid && beyond_key(na, nb, nc)) {
+        atomicOr(&counters->status, kStatusShiftRange);
+        valid = false;
+    }
+    key = pair_key_of(pj, na, nb, nc);
     return valid;
 }
 
@@ -466,14 +469,15 @@ __device__ __forceinline__ bool look_at(const Geometry& geom, bool any_periodic,
 // The stencil is walked 32 bins at a time: each lane fetches the atom range of one bin (a single
 // memory round trip for all of them), a warp scan turns the counts into offsets, and the lanes
 // then run over the concatenated candidates, so they stay busy whatever the bin occupancy, AHEAD of them per lane at once.
-template <int AHEAD = 1, class F>
+// PERIODIC: an axis is periodic, as the caller knows; else that is looked up.
+template <int AHEAD = 1, bool PERIODIC = false, class F>
 __device__ inline void for_each_candidate(const Geometry& geom, const GridParams& g, const int* __restrict__ cell_start,
                                           const float4* __restrict__ s_pos, const int* __restrict__ s_wrap,
                                           float xi, float yi, float zi, const int bi[3], const int wi[3],
                                           int lane, Counters* counters, F f) {
     const int w0 = 2 * g.R[0] + 1, w1 = 2 * g.R[1] + 1, w2 = 2 * g.R[2] + 1;
     const int n_stencil = w0 * w1 * w2;
-    const bool any_periodic = g.periodic[0] | g.periodic[1] | g.periodic[2];
+    const bool any_periodic = PERIODIC || (g.periodic[0] | g.periodic[1] | g.periodic[2]);
     for (int q0 = 0; q0 < n_stencil; q0 += 32) {
         // ---- this lane's bin of the stencil ----
         const int q = q0 + lane;
@@ -640,9 +644,12 @@ constexpr int kFillWarps = 4;
 // warps hide each other's loads, and more cost registers), four on few, where a call waits for the longest warp (search
 // of 60 atoms in a periodic box 31.6 -> 26.0 us, 431 atoms 21.1 -> 19.6 us, 2000 atoms 27.8 -> 26.0 us, 5000 atoms
 // 35.7 -> 37.7 us).
-// Nine CTAs per SM where loads are not fetched ahead and the key buffers allow it: 56 registers, eight fewer than the compiler takes.
-template <int KEYS, bool ROWS, int AHEAD>
-__global__ void __launch_bounds__(kFillWarps * 32, AHEAD == 1 && (KEYS <= 128 || !ROWS) ? 9 : 6)
+// PERIODIC: an axis is periodic, and images have to be looked up; without one the centre walks runs of the sorted atoms.  A
+// kernel holds one of the two walks only: with both (and the runs a second time, in the rare second walk below) the compiler
+// spoilt the one that images take, at whatever bound on its registers (search and descriptors of a periodic box, r_cut 6, both
+// walks against one: 60 atoms 34.2 -> 31.0 us, 150 atoms 55.7 -> 49.0 us, 1200 atoms 41.1 -> 37.8 us).
+template <int KEYS, bool ROWS, bool PERIODIC, int AHEAD>
+__global__ void __launch_bounds__(kFillWarps * 32)
 pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, const float* __restrict__ sites, long long C, Geometry geom,
              const GridParams* __restrict__ gp, const int* __restrict__ atom_cell, const int* __restrict__ atom_wrap,
              const int* __restrict__ cell_start, const float4* __restrict__ s_pos, const int* __restrict__ s_wrap,
@@ -684,9 +691,10 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
         if (valid && at < KEYS) s_raw[wid][at] = key;
         k += __popc(m);
     };
-    const bool runs = !(g.periodic[0] | g.periodic[1] | g.periodic[2]) && g.R[0] <= kThinBins && g.R[1] <= 1 && g.R[2] <= 1;
-    if (runs) for_each_candidate_runs(geom, g, cell_start, s_pos, xi, yi, zi, bi, lane, collect);
-    else for_each_candidate<AHEAD>(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, collect);
+    // (that an axis is periodic is told where several candidates are in flight: 150 atoms 50.6 -> 49.1 us; with one it costs registers,
+    // 64 against 53, and 10,000 atoms 66.0 -> 68.0)
+    if constexpr (PERIODIC) for_each_candidate<AHEAD, (AHEAD > 1)>(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, collect);
+    else for_each_candidate_runs(geom, g, cell_start, s_pos, xi, yi, zi, bi, lane, collect);
     long long base = 0;
     if (lane == 0) base = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&counters->n_pairs), (unsigned long long)k);
     base = __shfl_sync(0xffffffffu, base, 0);
@@ -704,14 +712,13 @@ pairs_kernel(const float* __restrict__ pos, const int* __restrict__ centers, con
     if (!in_smem) {
         // rare: more pairs than the on-chip buffer holds; walk again, now with a place to put them
         int at0 = 0;
-        auto store = [&](bool valid, unsigned long long key) {
-            const unsigned m = __ballot_sync(0xffffffffu, valid);
-            const int at = at0 + __popc(m & ((1u << lane) - 1));
-            if (valid && at < k) pair_tmp[base + at] = key;
-            at0 += __popc(m);
-        };
-        if (runs) for_each_candidate_runs(geom, g, cell_start, s_pos, xi, yi, zi, bi, lane, store);
-        else for_each_candidate(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters, store);
+        for_each_candidate(geom, g, cell_start, s_pos, s_wrap, xi, yi, zi, bi, wi, lane, counters,
+                           [&](bool valid, unsigned long long key) {
+                               const unsigned m = __ballot_sync(0xffffffffu, valid);
+                               const int at = at0 + __popc(m & ((1u << lane) - 1));
+                               if (valid && at < k) pair_tmp[base + at] = key;
+                               at0 += __popc(m);
+                           });
     }
     __syncwarp();
     if (!ROWS) {

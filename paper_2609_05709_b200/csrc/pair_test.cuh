@@ -9,11 +9,9 @@ __device__ inline void frac_coords(const Geometry& g, float x, float y, float z,
         s[a] = (double)x * g.inv[0 + a] + (double)y * g.inv[3 + a] + (double)z * g.inv[6 + a];
 }
 
-// Whether the atom pj (its number in w), translated by n cells, lies inside the cutoff of the centre, and the pair's key.  Every
-// operation is rounded to fp64 on its own, on the raw fp32 inputs.  out_of_range: a neighbour too many cells away for the key.
-__device__ __forceinline__ bool inside_cutoff(const Geometry& geom, bool any_periodic, float4 pj, const int n[3], float xi, float yi, float zi,
-                                              unsigned long long& key, bool& out_of_range) {
-    const int na = n[0], nb = n[1], nc = n[2];
+// Squared distance of the atom pj, translated by (na, nb, nc) cells, from the centre.  Every operation is rounded to fp64 on its
+// own, on the raw fp32 inputs.
+__device__ __forceinline__ double pair_distance2(const Geometry& geom, bool any_periodic, float4 pj, int na, int nb, int nc, float xi, float yi, float zi) {
     double dx = __dsub_rn((double)pj.x, (double)xi);
     double dy = __dsub_rn((double)pj.y, (double)yi);
     double dz = __dsub_rn((double)pj.z, (double)zi);
@@ -25,13 +23,20 @@ __device__ __forceinline__ bool inside_cutoff(const Geometry& geom, bool any_per
         double tz = __dadd_rn(__dadd_rn(__dmul_rn(fa, geom.cell[2]), __dmul_rn(fb, geom.cell[5])), __dmul_rn(fc, geom.cell[8]));
         dx = __dadd_rn(dx, tx); dy = __dadd_rn(dy, ty); dz = __dadd_rn(dz, tz);
     }
-    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    const bool valid = (d2 < geom.rc2) && (d2 > 0.0);
-    out_of_range = valid && (abs(na) > 127 || abs(nb) > 127 || abs(nc) > 127);
-    key = ((unsigned long long)(unsigned)__float_as_int(pj.w) << 24) |
-          ((unsigned long long)(na + 128) << 16) | ((unsigned long long)(nb + 128) << 8) |
-          (unsigned long long)(nc + 128);
-    return valid;
+    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+
+// Inside the cutoff: 0 < d2 < r_cut^2 (an atom is no neighbour of itself, its images are).
+__device__ __forceinline__ bool inside_cutoff(const Geometry& geom, double d2) { return (d2 < geom.rc2) && (d2 > 0.0); }
+
+// Whether a neighbour is too many cells away for its key.
+__device__ __forceinline__ bool beyond_key(int na, int nb, int nc) { return abs(na) > 127 || abs(nb) > 127 || abs(nc) > 127; }
+
+// The pair's key: the atom's number (in pj.w) and its translation.
+__device__ __forceinline__ unsigned long long pair_key_of(float4 pj, int na, int nb, int nc) {
+    return ((unsigned long long)(unsigned)__float_as_int(pj.w) << 24) |
+           ((unsigned long long)(na + 128) << 16) | ((unsigned long long)(nb + 128) << 8) |
+           (unsigned long long)(nc + 128);
 }
 
 }  // namespace soap

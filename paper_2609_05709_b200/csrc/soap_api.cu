@@ -386,8 +386,8 @@ int launch_neighbors(soap_t* h, const float* pos, const int32_t* num, int64_t N,
 #define SOAP_PAIRS_ARGS pos, centers, sites, C, g, h->d_grid, h->d_atom_cell, h->d_atom_wrap, h->d_cell_start, h->d_s_pos, h->d_s_wrap, \
         h->cap_pairs, h->d_pair_tmp, h->d_pair_key, h->d_pair_row, h->d_pair_start, h->d_pair_count, h->d_row_count, h->d_self_row, h->d_counters
         // (these kernels wait for the kernel before them on the device: their launch overlaps its tail)
-        const bool few = C <= (int64_t)16 * h->sm_count;
-#define SOAP_PAIRS(KEYS, ROWS) (few ? pairs_kernel<KEYS, ROWS, 4> : pairs_kernel<KEYS, ROWS, 1>)
+        const bool periodic = g.pbc[0] | g.pbc[1] | g.pbc[2], few = C <= (int64_t)16 * h->sm_count;
+#define SOAP_PAIRS(KEYS, ROWS) (!periodic ? pairs_kernel<KEYS, ROWS, false, 1> : few ? pairs_kernel<KEYS, ROWS, true, 4> : pairs_kernel<KEYS, ROWS, true, 1>)
         const bool sorted = list != List::found;
         auto kernel = small_keys ? (sorted ? SOAP_PAIRS(kFillSmemKeysSmall, true) : SOAP_PAIRS(kFillSmemKeysSmall, false))
                                  : (sorted ? SOAP_PAIRS(kFillSmemKeys, true) : SOAP_PAIRS(kFillSmemKeys, false));
