@@ -181,7 +181,10 @@ __device__ __forceinline__ void harmonics_tiles(float x, float y, float z, float
 // has no word for the weight).
 // TEAM: few centres, a CTA per centre: its warps take the chunks of pairs in turn, each into a tile of its own, and the
 // tiles are added up; the blocks of Eq. 4 are spread over all of them.
-template <int L, int NP, bool PLAIN, bool TS, bool TEAM>
+// SEARCH: a team that looks for its centre's neighbours itself (CenterParams::numbers).  A kernel of its own: carried along by the
+// teams that read their pairs it cost those registers and start-up (coefficients of 570 atoms at (4, 4) 20.6 -> 22.6 us, 200
+// centres of 300 atoms 20.6 -> 21.6 us, 260 of 780 at (12, 2) 20.6 -> 22.7 us).
+template <int L, int NP, bool PLAIN, bool TS, bool TEAM, bool SEARCH>
 __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 32, TEAM ? 16 / kDescTeamWarps : 1) desc_kernel(const CenterParams p) {
     constexpr int L1 = L + 1, LM = L1 * L1;
     constexpr int NCHP = L1 * NP;                                        // channels (l, n), n padded
@@ -252,9 +255,8 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     }
     // the tables are this handle's own; everything below reads what the kernels before this one wrote
     grid_dependency_wait();
-    const bool searches = TEAM && p.numbers != nullptr;
     // a failed neighbour build: write nothing
-    if (!searches && p.counters->n_pairs > p.pair_capacity) return;
+    if (!SEARCH && p.counters->n_pairs > p.pair_capacity) return;
 
     float* const wbase = smem + lay.warp0 + wid * lay.per_warp;
     float* const c_t = wbase + lay.c;                                               // [LM] rows of RC chunks, skewed
@@ -292,11 +294,11 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
     constexpr int PPL = kDescGroup / 32;                                 // pairs per lane and group
     struct Head { float xi, yi, zi; int zsp; long long pair_base; int k_pairs; };
     struct Raw { unsigned long long key[PPL]; float wgt[PPL]; int spj[PPL]; float px[PPL], py[PPL], pz[PPL]; };
-    // A team may look for its centre's neighbours itself, among all atoms of a small structure whose periodic axes are at least two
+    // SEARCH: the team looks for its centre's neighbours itself, among all atoms of a small structure whose periodic axes are at least two
     // cutoffs high: an atom then has one image inside at most, the one nearest in each fractional coordinate.  The test is the
     // pair kernel's.  A warp takes a contiguous share of the atoms and leaves its finds in its own slots, in order.
     unsigned long long* const list = reinterpret_cast<unsigned long long*>(smem + lay.total);
-    const int share = searches ? desc_search_share(p.n_atoms, warps) : 0;
+    const int share = SEARCH ? desc_search_share(p.n_atoms, warps) : 0;
     int* const s_found = reinterpret_cast<int*>(list + share * warps);
     auto species_of = [&](int number) { return number >= 0 && number < 128 ? __ldg(p.z_lut + number) : -1; };
     auto search = [&](int i) {
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
         return list[w * share + e];
     };
     auto load_head = [&](long long c_idx) {
-        if (searches) return search((int)c_idx);
+        if constexpr (SEARCH) return search((int)c_idx);
         Head h;
         const int ci = o_sites ? -1 : (p.centers ? p.centers[c_idx] : (int)c_idx);
         const float* pc = o_sites ? o_sites + 3 * c_idx : p.pos + 3 * (long long)ci;
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
 #pragma unroll
         for (int b = 0; b < PPL; ++b) {
             const int e = g0 + 32 * b + lane;
-            r.key[b] = e < h.k_pairs ? (searches ? found_key(e) : p.pair_key[h.pair_base + e]) : 0ull;
+            r.key[b] = e < h.k_pairs ? (SEARCH ? found_key(e) : p.pair_key[h.pair_base + e]) : 0ull;
             r.wgt[b] = (o_pw && e < h.k_pairs) ? o_pw[h.pair_base + e].x : 1.f;
         }
     };
@@ -379,7 +381,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
             r.spj[b] = -1; r.px[b] = r.py[b] = r.pz[b] = 0.f;
             if (e < h.k_pairs) {
                 const int j = key_atom(r.key[b]);
-                r.spj[b] = S == 1 ? 0 : searches ? (int)(r.key[b] >> 56) : p.species_idx[j];
+                r.spj[b] = S == 1 ? 0 : SEARCH ? (int)(r.key[b] >> 56) : p.species_idx[j];
                 r.px[b] = p.pos[3 * (long long)j]; r.py[b] = p.pos[3 * (long long)j + 1]; r.pz[b] = p.pos[3 * (long long)j + 2];
             }
         }
@@ -741,7 +743,7 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
         }
     }
     if (!TEAM && lane == 0) wait_row();                                      // the slab must outlive the copies that read it
-    if (searches && threadIdx.x == 0) {
+    if (SEARCH && threadIdx.x == 0) {
         // the last team leaves the totals of the call
         int k = 0;
         for (int w = 0; w < warps; ++w) k += s_found[w];

@@ -11,21 +11,22 @@ namespace soap {
 #define SOAP_CAT2(a, b, c, d) a##b##c##d
 #define SOAP_CAT(a, b, c, d) SOAP_CAT2(a, b, c, d)
 
-// a warp per centre with the table in shared memory or in global memory, or a team of warps per centre
+// a warp per centre with the table in shared memory or in global memory, or a team of warps per centre, which may search itself
 template <int NP>
-static DescKernel of_np(bool ts, bool team) {
+static DescKernel of_np(bool ts, bool team, bool search) {
     constexpr bool PLAIN = SOAP_FAMILY == 0;
-    if (team) return desc_kernel<SOAP_L, NP, PLAIN, false, true>;
-    if (ts) return desc_kernel<SOAP_L, NP, PLAIN, true, false>;
-    return desc_kernel<SOAP_L, NP, PLAIN, false, false>;
+    if (search) return desc_kernel<SOAP_L, NP, PLAIN, false, true, true>;
+    if (team) return desc_kernel<SOAP_L, NP, PLAIN, false, true, false>;
+    if (ts) return desc_kernel<SOAP_L, NP, PLAIN, true, false, false>;
+    return desc_kernel<SOAP_L, NP, PLAIN, false, false, false>;
 }
 
-DescKernel SOAP_CAT(desc_kernel_l, SOAP_L, _f, SOAP_FAMILY)(int np, bool ts, bool team) {
+DescKernel SOAP_CAT(desc_kernel_l, SOAP_L, _f, SOAP_FAMILY)(int np, bool ts, bool team, bool search) {
     switch (np) {
-        case 4: return of_np<4>(ts, team);
-        case 8: return of_np<8>(ts, team);
-        case 12: return of_np<12>(ts, team);
-        case 16: return of_np<16>(ts, team);
+        case 4: return of_np<4>(ts, team, search);
+        case 8: return of_np<8>(ts, team, search);
+        case 12: return of_np<12>(ts, team, search);
+        case 16: return of_np<16>(ts, team, search);
     }
     return nullptr;
 }

@@ -37,9 +37,9 @@ CenterKernel center_kernel_of(int kind, bool plain, int l_max, int n_max) {
     }
     return nullptr;
 }
-DescKernel desc_kernel_of(int l_max, int np, bool plain, bool table_in_smem, bool team) {
+DescKernel desc_kernel_of(int l_max, int np, bool plain, bool table_in_smem, bool team, bool search) {
     switch (l_max) {
-#define X(LV) case LV: return plain ? desc_kernel_l##LV##_f0(np, table_in_smem, team) : desc_kernel_l##LV##_f1(np, table_in_smem, team);
+#define X(LV) case LV: return plain ? desc_kernel_l##LV##_f0(np, table_in_smem, team, search) : desc_kernel_l##LV##_f1(np, table_in_smem, team, search);
         X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
 #undef X
     }
@@ -530,7 +530,7 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     const bool plain = center_params_plain(cp);
     const int64_t search_atoms = cp.numbers ? cp.n_atoms : 0;
     if (const int team = desc_team(h, plain, n_work, search_atoms))
-        return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true), cp, (unsigned)n_work, (unsigned)team * 32,
+        return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true, cp.numbers != nullptr), cp, (unsigned)n_work, (unsigned)team * 32,
                                  desc_team_bytes(h, plain, team, search_atoms), st);
     const DescLayout alone = make_desc_layout(h->S, h->desc_np, h->l_max, 1, 0, false, plain);
     const int warps_fit = (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - (size_t)alone.warp0 * 4) / ((size_t)alone.per_warp * 4));
@@ -548,7 +548,7 @@ int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(ts ? warps_ts : warps_fit, (n_work + sms - 1) / sms));
     const unsigned grid = (unsigned)std::min<int64_t>(sms, (n_work + warps - 1) / warps);
     const size_t smem = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, warps, ts ? (int)(h->desc_table_bytes / 4) : 0, false, plain).total * 4;
-    return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, ts, false), cp, grid, (unsigned)warps * 32, smem, st);
+    return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, ts, false, false), cp, grid, (unsigned)warps * 32, smem, st);
 }
 
 // What the bits of the status word mean to a caller.
