@@ -82,7 +82,9 @@ __host__ __device__ constexpr int desc_c_words(int S, int np, int lm, bool pad) 
 // a lane then keeps its quad), and conflicts weigh little with more than 16 quads; else two adjacent n per lane, the table as
 // [interval][l][n / 2][6][2], which fills more lanes.  24,000 atoms of water, whole calls, pairs against quads: (8, 6) 202 ->
 // 193 us, (8, 3) 148 -> 144, (14, 6) 714 -> 661, (2, 7) 175 -> 170, (10, 8) 623 -> 608; the other way, left as pairs,
-// (8, 4) 164 -> 172, (2, 4) 131 -> 138, (10, 2) 169 -> 179, (8, 5) and (10, 3) equal or slower.
+// (8, 4) 164 -> 172, (2, 4) 131 -> 138, (10, 2) 169 -> 179, (8, 5) and (10, 3) equal or slower.  The bases that take quads do so
+// with the table in global memory too (weighted, 3000 atoms, (3, 6) 53.6 -> 51.5 us, (8, 6) 65.9 -> 61.7, (14, 6) 122 -> 118) and
+// in teams (300 atoms, (8, 6) 13.6 -> 12.4, (9, 4) 12.9 -> 12.1, (14, 6) 27.9 -> 27.3).
 __host__ __device__ constexpr int desc_quad_span(int np, int l_max) {
     const int quads = (l_max + 1) * np / 4, span = (quads + 7) / 8 * 8;
     return span <= 32 && 32 % span == 0 && 8 * quads >= 7 * span ? span : 0;
@@ -573,17 +575,19 @@ __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 3
                             *reinterpret_cast<float2*>(to) = v;
                         }
                     };
+                    // (a team's warp has few rounds, and two of them at once make it spill: coefficients of 60 atoms at (14, 3) 18.5 ->
+                    // 16.5 us, descriptors of 720 30.3 -> 27.8 us)
                     constexpr int SPAN = QUADS ? desc_quad_span(NP, L) : 0;
                     if constexpr (SPAN > 0) {
                         const int u = lane % SPAN;
                         if (u < UNITS) {
-#pragma unroll 2
+#pragma unroll (TEAM ? 1 : 2)
                             for (int pr = lane / SPAN; pr < n_stage; pr += 32 / SPAN) radial(pr, u);
                         }
                     } else {
                         // the lanes walk down the (pair, unit) list side by side, a warp's width at a time
                         int pr = lane / UNITS, u = lane - pr * UNITS;
-#pragma unroll (QUADS ? 2 : 4)
+#pragma unroll (!QUADS ? 4 : TEAM ? 1 : 2)
                         for (int e = lane; e < n_stage * UNITS; e += 32) {
                             radial(pr, u);
                             // 32 further down the list
