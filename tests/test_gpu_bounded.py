@@ -57,6 +57,21 @@ def test_periodic_with_centres(pkg, monkeypatch, weighted):
         assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("call", ["derivatives", "derivatives_compact", "coefficient_derivatives"])
+@pytest.mark.parametrize("n,centers,scale", [(24, 24, 1.0), (24, 24, 4.0), (120, 8, 1.0), (3000, 1, 1.0)])
+def test_results_do_not_keep_the_room(pkg, call, n, centers, scale):
+    """Whatever share of its room a call fills, its result holds at most twice the bytes of its rows."""
+    s = water_cluster((n + 2) // 3, 1)
+    pos, num = torch.from_numpy((scale * s.positions[:n]).astype(np.float32)).cuda(), torch.from_numpy(s.numbers[:n]).cuda()
+    soap = pkg.Soap([1, 8], 4.0, 2, 2, 0.5)
+    d = getattr(soap, call)(pos, num, None, torch.arange(centers, dtype=torch.int32, device="cuda"))
+    rows = int(d.row_ptr[-1])
+    assert d.jacobian.shape[0] == d.row_atom.shape[0] == rows > 0
+    again = getattr(soap, call)(pos, num, None, torch.arange(centers, dtype=torch.int32, device="cuda"))     # (the other way, after an empty room)
+    for x, y in ((d.jacobian, again.jacobian), (d.row_atom, again.row_atom)):
+        assert x.is_contiguous() and x.untyped_storage().nbytes() <= 2 * x.nbytes and torch.equal(x, y)
+
+
 def test_errors(pkg):
     s = water_cluster(4, 0)
     pos, num = torch.from_numpy(s.positions).cuda(), torch.from_numpy(s.numbers).cuda()
