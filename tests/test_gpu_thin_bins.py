@@ -25,8 +25,10 @@ def spread(kind, n, rng):
     if kind == "lattice":
         m = int(np.ceil(n ** (1 / 3)))
         return 0.75 * np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n]
+    if kind == "clumps":
+        return rng.random((n, 3)) * 18 + 1700.0 * (np.arange(n) % 2)[:, None]
     extent = {"cube": (18, 18, 18), "line x": (300, 1, 1), "line y": (1, 300, 1), "line z": (0, 0, 300), "plane": (40, 40, 0),
-              "point": (1.4, 1.4, 1.4), "far": (30, 9, 9)}[kind]
+              "point": (1.4, 1.4, 1.4), "far": (30, 9, 9), "sparse": (150, 150, 150), "long line": (1200, 1, 1)}[kind]
     return rng.random((n, 3)) * extent + (1.0e5 if kind == "far" else -7.0)
 
 
@@ -46,6 +48,13 @@ def test_pairs_are_exact(kind, n):
     ptr, atom, _ = soap.neighbor_list(at, torch.ones(n, dtype=torch.int32, device="cuda"), None, torch.from_numpy(centers).cuda())
     want_ptr, want = pairs_of(pos, pos[centers], 3.0)
     assert np.array_equal(ptr.cpu().numpy(), want_ptr) and np.array_equal(atom.cpu().numpy(), want)
+
+
+# where the grid is not the one that r_cut asks for: more bins than the scratch holds (158,012 for 70,000 atoms: 500,000 are wanted,
+# and 3e8), more than 1024 along an axis (1600), both
+@pytest.mark.parametrize("kind,n", [("sparse", 70000), ("long line", 5000), ("long line", 70000), ("clumps", 70000)])
+def test_pairs_are_exact_on_cut_grids(kind, n):
+    test_pairs_are_exact(kind, n)
 
 
 @pytest.mark.parametrize("cell", [np.diag([2.0, 0.5, 7.0]), np.array([[9.0, 1.0, 0.0], [0.0, 8.0, 2.0], [1.0, 0.0, 7.0]])], ids=["square", "skew"])
