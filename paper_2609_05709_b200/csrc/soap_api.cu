@@ -502,53 +502,19 @@ int launch_center(soap_t* h, int kind, CenterParams& cp, int64_t n_centers, int 
                              (size_t)cp.lay.total * 4 + extra, st);
 }
 
-// Few centres: a team of warps per centre, four if the CTAs then run side by side in one wave (four of them fit an
-// SM's registers), else two (eight; up to five centres per SM: beyond that a warp per centre is the faster one on half
-// of the sizes).  Whole calls, (n_max, l_max) = (8, 6): 120 atoms 27 -> 17 us, 431 atoms of four species 66 -> 38 us,
-// 600 atoms 31.2 -> 29.2 us; (12, 8), 600 atoms 60 -> 43 us.
-// search_atoms: the team looks for its neighbours among that many atoms (0: it reads them).  Returns its warps, 0: no team.
-size_t desc_team_bytes(const soap_t* h, bool plain, int team_warps, int64_t search_atoms) {
-    return (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, team_warps, 0, true, plain).total * 4 + desc_search_bytes(search_atoms, team_warps);
-}
-int desc_team(const soap_t* h, bool plain, int64_t n_work, int64_t search_atoms) {
-    for (const int team_warps : {kDescTeamWarps, 2}) {
-        const size_t bytes = desc_team_bytes(h, plain, team_warps, search_atoms);
-        const int64_t per_sm = std::min<int64_t>(team_warps == 2 ? 5 : 16 / kDescTeamWarps, (int64_t)(228 * 1024 / (bytes + 1024)));
-        if (n_work <= per_sm * h->sm_count && bytes <= (size_t)h->max_smem) return team_warps;
-    }
-    return 0;
+// How the descriptor-only kernel runs on n_work centres (search_atoms: of a structure of so many atoms, which it searches itself).
+DescPlan plan_desc(const soap_t* h, bool plain, bool weighted, int64_t n_work, int64_t search_atoms) {
+    return desc_plan(h->S, h->desc_np, h->l_max, plain, weighted, h->desc_table_bytes / 4, n_work, search_atoms, h->sm_count, (size_t)h->max_smem);
 }
 
-// Launch of the descriptor-only kernel: persistent CTAs (one per SM) whose warps take the centres in turn.
-// The radial table goes to shared memory when it leaves room for at least six warps and there is enough
-// work to pay for staging it; small jobs use fewer warps per CTA so that they spread over the SMs, the smallest
-// several warps per centre.
 int launch_desc(soap_t* h, CenterParams& cp, int64_t n_work, cudaStream_t st) {
     if (n_work <= 0) return SOAP_OK;
     cp.table_ln = h->d_table_ln;
     cp.inv_h = h->basis.inv_h_values; cp.n_intervals = h->basis.n_intervals_values;      // the value table has intervals of its own
-    const bool plain = center_params_plain(cp);
-    const int64_t search_atoms = cp.numbers ? cp.n_atoms : 0;
-    if (const int team = desc_team(h, plain, n_work, search_atoms))
-        return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, false, true, cp.numbers != nullptr), cp, (unsigned)n_work, (unsigned)team * 32,
-                                 desc_team_bytes(h, plain, team, search_atoms), st);
-    const DescLayout alone = make_desc_layout(h->S, h->desc_np, h->l_max, 1, 0, false, plain);
-    const int warps_fit = (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - (size_t)alone.warp0 * 4) / ((size_t)alone.per_warp * 4));
-    // (with the table in shared memory a warp's region is a little smaller: its staged pairs are five words, not eight)
-    const DescLayout with_table = make_desc_layout(h->S, h->desc_np, h->l_max, 1, (int)(h->desc_table_bytes / 4), false, plain);
-    const size_t fixed_ts = (size_t)with_table.warp0 * 4, warp_bytes_ts = (size_t)with_table.per_warp * 4;
-    const int warps_ts = h->desc_table_bytes > 0 && fixed_ts + warp_bytes_ts <= (size_t)h->max_smem
-                             ? (int)std::min<size_t>(kDescMaxWarps, ((size_t)h->max_smem - fixed_ts) / warp_bytes_ts) : 0;
-    // The table pays from four centres per SM on, except where the warps it costs make a second round of centres that keeps
-    // less than a quarter of them busy (coefficients, table against none: 1500 atoms at (8, 8) 46.1 against 39.6 us, 1000
-    // atoms of three species at (6, 9) 48.2 against 36.8 us; with a fuller second round 48.1 against 48.5 us and less).
-    const int64_t sms = h->sm_count;
-    const bool straggling = n_work <= warps_fit * sms && n_work > warps_ts * sms && 4 * n_work <= 5 * warps_ts * sms;
-    const bool ts = !cp.pair_w && warps_ts >= 6 && n_work >= 4 * sms && !straggling;
-    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(ts ? warps_ts : warps_fit, (n_work + sms - 1) / sms));
-    const unsigned grid = (unsigned)std::min<int64_t>(sms, (n_work + warps - 1) / warps);
-    const size_t smem = (size_t)make_desc_layout(h->S, h->desc_np, h->l_max, warps, ts ? (int)(h->desc_table_bytes / 4) : 0, false, plain).total * 4;
-    return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, ts, false, false), cp, grid, (unsigned)warps * 32, smem, st);
+    const bool plain = center_params_plain(cp), search = cp.numbers != nullptr;
+    const DescPlan plan = plan_desc(h, plain, cp.pair_w != nullptr, n_work, search ? cp.n_atoms : 0);
+    return launch_per_center(h, desc_kernel_of(h->l_max, h->desc_np, plain, plan.table, plan.team != 0, search), cp, plan.grid, (unsigned)plan.warps * 32,
+                             plan.bytes, st);
 }
 
 // What the bits of the status word mean to a caller.
@@ -626,7 +592,7 @@ int prepare(soap_t* h, const float* pos, const int32_t* num, int64_t N, const do
     // Descriptors of a small structure with every atom a centre: the kernel that computes them searches as well, where a team of
     // warps has a centre each and no periodic axis is shorter than two cutoffs
     if (searches_itself) {
-        bool can = !centers && !sites && !batch.struct_ptr && C > 0 && C <= kDescSearchAtoms && !h->weight.fn && desc_team(h, h->crossover, C, N) != 0;
+        bool can = !centers && !sites && !batch.struct_ptr && C > 0 && !h->weight.fn && plan_desc(h, h->crossover, false, C, N).team != 0;
         for (int a = 0; a < 3; ++a) can = can && (!g.pbc[a] || g.height[a] >= 2.0 * g.r_cut * (1.0 + 1e-6));
         *searches_itself = can;
         if (can) {
