@@ -115,6 +115,27 @@ __device__ __forceinline__ void bulk_store(float* dst, const float* src_shared, 
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
+// How a centre's CTA starts.  Early: with the layout as the host put it together, and everything that depends on the centre's
+// number alone on its way at once; with the tables that rows by table do without left out, 36,000 centres of 18 pairs 733 -> 711 us,
+// compact rows of 1111 atoms at (6, 6) 325 -> 316, 3000 at (8, 6) 591 -> 583.  It holds registers through pass 1, so where these
+// are short or the rows long the start weighs less than that.  Measured early against not, on 120 and 900 atoms:
+//   n_max from 9 on: (12, 10) 922 -> 927 to 946 us, (12, 6) 661 -> 664; coefficients 0.89 to 1.01 times as fast; up to n_max 8
+//   l_max from 11 on (the inner average from 9): 0.96 to 0.99;
+//   n_max at run time, which spills in any case: 0.93 to 1.0, but for rows at l_max 2 and 3 (1.03 to 1.17) and plain ones at 7 (1.2
+//   to 1.3 from n_max 13 on, 0.95 at n_max 1), and for the outer average up to l_max 7 (1.02 to 1.2).
+template <int KIND, int L, int NMAX_T, bool PLAIN>
+constexpr bool early_start() {
+    if (KIND == 2) return false;
+    if (NMAX_T != 0) return NMAX_T <= 8 && L <= (KIND == 3 ? 8 : 10);
+    return KIND == 4 ? L <= 7 : KIND == 1 && (L <= 3 || (PLAIN && L == 7));
+}
+// Whether the warp's number comes from lane 0, by which the compiler sees that it is uniform: addresses and branches that depend on
+// it alone leave the lanes' registers (36,000 centres of 18 pairs 709 -> 698 us, outer average of 3000 atoms 580 -> 574).  Not in
+// two corners where it lost: the outer average with n_max at run time from l_max 8 on (0.93 to 0.98 at 9 and 10), and rows from
+// l_max 11 on up to n_max 8 (0.92 to 1.0 at (2, 12)).
+template <int KIND, int L, int NMAX_T>
+constexpr bool uniform_warp() { return NMAX_T == 0 ? !(KIND == 4 && L >= 8) : !(KIND == 1 && L >= 11 && NMAX_T <= 8); }
+
 // KIND: 1 descriptor and Jacobian, 2 coefficients c^mu_nlm and their Jacobian, 3 Jacobian of the inner average
 // (every atom a centre; given mean coefficients; one row per atom, no per-pair rows), 4 Jacobian of the outer average
 // (every atom a centre; given the coefficients of all centres; one row per atom, no per-pair rows).
@@ -146,16 +167,12 @@ center_kernel(const CenterParams p) {
     constexpr int NPT = NPT_RAW < 8 ? NPT_RAW : 8;                // ... at most 8 at a time (register budget)
     extern __shared__ __align__(16) float smem[];
     const int threads = KIND <= 2 ? (int)blockDim.x : kThreads, warps = threads >> 5;
-    const int tid = threadIdx.x, lane = tid & 31, wid = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform in a warp, and the compiler sees it
+    const int tid = threadIdx.x, lane = tid & 31, wid = uniform_warp<KIND, L, NMAX_T>() ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5;
     const int S = p.S, NMAX = NMAX_T ? NMAX_T : p.n_max, NCH = NMAX * L1, NE = NMAX * LM;
     const int CT = S * NMAX * LMP, P = p.P, F = p.F;
     constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
     constexpr bool kRowTable = KIND == 1 && NMAX_T != 0 && row_table_wanted(NMAX_T, L);
-    // The layout as the host put it together, and everything that depends on the centre's number alone on its way at once: with
-    // the tables that rows by table do without left out, 36,000 centres of 18 pairs 733 -> 711 us, compact rows of 1111 atoms at (6, 6)
-    // 325 -> 316, 3000 at (8, 6) 591 -> 583.  From n_max 9 on, where the rows are long and the registers few, the start of a
-    // centre weighs less than what it holds: (12, 10) 922 -> 927 to 946 us, (12, 6) 661 -> 664.
-    constexpr bool kEarly = NMAX_T <= 8;
+    constexpr bool kEarly = early_start<KIND, L, NMAX_T, PLAIN>();
     const SmemLayout made = kEarly ? SmemLayout{} : make_layout(S, NMAX, L, P, warps, o_pw != nullptr, kRowTable && !PLAIN && p.row_ops != nullptr);
     const SmemLayout& lay = kEarly ? p.lay : made;
     // words pairs (G, Ghat) per staged pair: the channels, and with a row table a zero behind them
