@@ -156,8 +156,8 @@ int soap_derivatives_bounded(soap_t *h, int kind, const float *d_positions, cons
                              float *d_out_desc, float *d_out_center, float *d_out_jac, int64_t capacity_rows,
                              int64_t *d_row_ptr, int32_t *d_row_atom, int64_t *n_rows, void *stream);
 
-/* Exports the neighbour list of the last soap_neighbors / soap_descriptor /
- * soap_derivatives call: d_pair_ptr [n_centers+1]; for pair e of centre i
+/* Exports the neighbour list of the last soap_neighbors / soap_derivatives call
+ * (a descriptor call leaves none to export: SOAP_ERR_INVALID_ARG): d_pair_ptr [n_centers+1]; for pair e of centre i
  * (d_pair_ptr[i] <= e < d_pair_ptr[i+1]) the neighbour atom d_pair_atom[e] and
  * its lattice translation d_pair_shift[3e..3e+2] (multiples of a, b, c; may be
  * NULL).  Pairs of a centre are sorted by (atom, shift).  capacity_pairs is
@@ -172,10 +172,11 @@ int soap_neighbor_list(soap_t *h, int64_t *d_pair_ptr, int32_t *d_pair_atom, int
  * work.  If such a call meets more pairs than the planned scratch holds (a
  * denser structure), soap_status reports SOAP_ERR_CAPACITY and the outputs
  * of that call are invalid: call soap_neighbors for that structure, then
- * repeat.  The sums over a centre's pairs run in the order in which the search
- * finds them, which is not fixed where atoms share a bin of the cell list: the
- * last bits can differ from call to call (derivatives and averages repeat bit
- * for bit). */
+ * repeat (small structures, which the descriptor kernel searches itself, keep
+ * to that rule as well).  The sums over a centre's pairs run in the order in
+ * which the search finds them, which is not fixed where atoms share a bin of
+ * the cell list: the last bits can differ from call to call (derivatives and
+ * averages repeat bit for bit, and so do descriptors of small structures). */
 int soap_descriptor(soap_t *h, const float *d_positions, const int32_t *d_numbers, int64_t n_atoms,
                     const double *cell, const int32_t *d_centers, int64_t n_centers,
                     float *d_out, void *stream);
@@ -416,7 +417,8 @@ int soap_neighbor_counts_static(const float *d_positions, int64_t n_atoms, doubl
  * soap_derivatives_found) is one call: the host's work between its steps
  * counts in neither.
  * soap_profile_read waits for the last call's events and returns both
- * durations in milliseconds.  Off by default: the kernels of a call are
+ * durations in milliseconds (where the descriptor kernel searches itself, the
+ * search counts in (b)).  Off by default: the kernels of a call are
  * launched so that each may start while the one before it finishes (they wait
  * for it on the device), and an event recorded between two launches keeps the
  * second from starting early - a profiled call is a few microseconds slower,

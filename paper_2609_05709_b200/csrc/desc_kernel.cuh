@@ -19,7 +19,7 @@
 //   * Eq. 4 is the Gram matrix of that tile per l: lanes take 4 x 4 blocks of (species, n) pairs,
 //     two 16-byte loads per 16 multiply-adds, and the feature row is put together in shared memory
 //     and handed to the copy engine.
-// At (8, 6) on 30,000 atoms the kernel takes 229 us; the L1 data pipe is 76 % busy, the issue slots 58 %.
+// At (8, 6) on 30,000 atoms the kernel takes 212 us; the L1 data pipe is 82 % busy, the issue slots 50 %.
 // Nothing but the pair list is read from HBM and nothing but the descriptor row is written.
 #pragma once
 #include "desc_layout.h"
@@ -88,7 +88,7 @@ __device__ __forceinline__ void harmonics_tiles(float x, float y, float z, float
 // tiles are added up; the blocks of Eq. 4 are spread over all of them.
 // SEARCH: a team that looks for its centre's neighbours itself (CenterParams::numbers).  A kernel of its own: carried along by the
 // teams that read their pairs it cost those registers and start-up (coefficients of 570 atoms at (4, 4) 20.6 -> 22.6 us, 200
-// centres of 300 atoms 20.6 -> 21.6 us, 260 of 780 at (12, 2) 20.6 -> 22.7 us).
+// centres of 570 atoms 20.6 -> 22.6).
 template <int L, int NP, bool PLAIN, bool TS, bool TEAM, bool SEARCH>
 __global__ void __launch_bounds__(TEAM ? kDescTeamWarps * 32 : kDescMaxWarps * 32, TEAM ? 16 / kDescTeamWarps : 1) desc_kernel(const CenterParams p) {
     constexpr int L1 = L + 1, LM = L1 * L1;
