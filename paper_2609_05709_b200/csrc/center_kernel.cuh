@@ -131,10 +131,14 @@ constexpr bool early_start() {
 }
 // Whether the warp's number comes from lane 0, by which the compiler sees that it is uniform: addresses and branches that depend on
 // it alone leave the lanes' registers (36,000 centres of 18 pairs 709 -> 698 us, outer average of 3000 atoms 580 -> 574).  Not in
-// two corners where it lost: the outer average with n_max at run time from l_max 8 on (0.93 to 0.98 at 9 and 10), and rows from
-// l_max 11 on up to n_max 8 (0.92 to 1.0 at (2, 12)).
-template <int KIND, int L, int NMAX_T>
-constexpr bool uniform_warp() { return NMAX_T == 0 ? !(KIND == 4 && L >= 8) : !(KIND == 1 && L >= 11 && NMAX_T <= 8); }
+// three corners where it lost: the outer average with n_max at run time from l_max 8 on (0.93 to 0.98 at 9 and 10), rows from
+// l_max 11 on up to n_max 8 (0.92 to 1.0 at (2, 12)), and rows with options at l_max 8 from n_max 7 on (compact rows of 600 atoms
+// of four species, (7, 8) 371 -> 360 us without, (8, 8) 379 -> 372; smaller n_max equal or slower without).
+template <int KIND, int L, int NMAX_T, bool PLAIN>
+constexpr bool uniform_warp() {
+    if (NMAX_T == 0) return !(KIND == 4 && L >= 8);
+    return !(KIND == 1 && (NMAX_T <= 8 ? L >= 11 || (!PLAIN && L == 8 && NMAX_T >= 7) : false));
+}
 
 // KIND: 1 descriptor and Jacobian, 2 coefficients c^mu_nlm and their Jacobian, 3 Jacobian of the inner average
 // (every atom a centre; given mean coefficients; one row per atom, no per-pair rows), 4 Jacobian of the outer average
@@ -167,7 +171,7 @@ center_kernel(const CenterParams p) {
     constexpr int NPT = NPT_RAW < 8 ? NPT_RAW : 8;                // ... at most 8 at a time (register budget)
     extern __shared__ __align__(16) float smem[];
     const int threads = KIND <= 2 ? (int)blockDim.x : kThreads, warps = threads >> 5;
-    const int tid = threadIdx.x, lane = tid & 31, wid = uniform_warp<KIND, L, NMAX_T>() ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = uniform_warp<KIND, L, NMAX_T, PLAIN>() ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5;
     const int S = p.S, NMAX = NMAX_T ? NMAX_T : p.n_max, NCH = NMAX * L1, NE = NMAX * LM;
     const int CT = S * NMAX * LMP, P = p.P, F = p.F;
     constexpr int CP_T = (NMAX_T + 1) / 2 * L1;
